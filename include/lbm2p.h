@@ -134,8 +134,10 @@ typedef struct {
                                    fused form replaces single sweeps only when its time per
                                    sweep is at most 0.95 of the best single sweep's (these
                                    timings favour the fused forms a little).  Fused
-                                   kernels: T = 2 or 4 sweeps on shared-memory stages, and, on
-                                   lattices with walls on every side, 2 sweeps on rows staged
+                                   kernels: T = 2 or 4 sweeps on shared-memory stages on
+                                   lattices with a periodic side; on lattices with walls on
+                                   every side, 4 sweeps in registers (automatically when
+                                   check_every is a multiple of 8), 2 sweeps on rows staged
                                    by bulk copies and 2 sweeps with direct loads (fuse_sweeps
                                    2 with sweep_kernel ROWS pins the former, with SCALAR the
                                    latter). */
@@ -263,7 +265,8 @@ lbm2p_status lbm2p_set_timing(lbm2p *h, int enable);
 /* How the pressure sweeps run on this handle, as chosen at create: sweeps fused per launch
    (1, 2 or 4); the single-sweep kernel (an lbm2p_sweep_kernel value, never AUTO); the tile
    of the kernel that runs the sweeps: for fused sweeps its threads per block (columns per
-   block for the two-sweep row-walking kernels: 120 or 240) and rows per block, for the ROWS
+   block for the two-sweep row-walking kernels: 120 or 240; 32 for the four-sweep kernel's
+   one-warp tiles of 56 columns) and rows per block, for the ROWS
    kernel its strip width and rows per block, otherwise 0 and 0. */
 lbm2p_status lbm2p_sweep_config(const lbm2p *h, int *fused, int *kind, int *tile_w, int *tile_h);
 
@@ -272,7 +275,8 @@ typedef enum {
     LBM2P_FUSED_NONE = 0,        /* single sweeps */
     LBM2P_FUSED_STAGES = 1,      /* T sweeps on shared-memory stages (T = 2 or 4) */
     LBM2P_FUSED_STAGED_ROWS = 2, /* two sweeps on rows staged by bulk copies */
-    LBM2P_FUSED_DIRECT = 3       /* two sweeps, inputs loaded directly (lattices held in L2) */
+    LBM2P_FUSED_DIRECT = 3,      /* two sweeps, inputs loaded directly (lattices held in L2) */
+    LBM2P_FUSED_QUAD = 4         /* four sweeps, one warp per tile of 56 columns */
 } lbm2p_fused_form;
 int lbm2p_fused_form_of(const lbm2p *h);
 
@@ -293,7 +297,8 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
  *   "single_rows <strip width> <ring slots> <rows per block> <grid> <us>",
  *   "fused <sweeps per launch> <threads per block> <rows per block> <grid> <us>",
  *   "fused_rows <consumer warps> <ring slots> <rows per block> <grid> <us>",
- *   "fused_direct <warps> 0 <rows per block> <grid> <us>"
+ *   "fused_direct <warps> 0 <rows per block> <grid> <us>",
+ *   "fused_quad <sweeps per launch> 0 <rows per tile> <grid> <us>"
  * with <us> the time per sweep inside the solve loop: a check period of check_every sweeps
  * timed as its plain launches plus the one launch that also sums the residual (the first two
  * kinds once per grid tried: the resident-block capacity of the GPU down to half of it).  Owned by h; valid until the next create-time tuning. */

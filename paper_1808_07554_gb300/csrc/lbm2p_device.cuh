@@ -292,6 +292,15 @@ void pressure_sweeps_pair_direct(const PressureArgs &a, bool check, int cw, int 
                                  void *stream);
 cudaError_t node_pressure_pair_direct(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                       const PressureArgs &a, bool check, int cw, int H, int grid);
+// four sweeps per launch (sweep_quad.cu), lattices without periodic sides: tiles of 56 columns by H
+// rows, one warp each, four to a block; grid = quad_grid(...)
+long long quad_grid(int H, int nx, int ny);
+int quad_strips_of(int nx);
+int quad_tile_slots(bool has_fp);      // tiles that run at a time (0: the kernel cannot run)
+cudaError_t quad_prepare();
+void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream);
+cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
+                               const PressureArgs &a, bool check, int H, int grid);
 // FP16 storage (fp16.cu): narrow = max |n| -> scale -> convert; one sweep; widen
 int max_blocks_per_sm_pressure_h();
 void half_narrow(const HalfConvertArgs &a, int grid, void *stream);

@@ -327,7 +327,10 @@ lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int p
             for (int kk = T; kk <= m; kk += T) {
                 cudaGraphNode_t n;
                 PressureArgs a = pressure_args(h, src, dst_of(src), work);
-                if (h->tb_kind == 2)
+                if (h->tb_kind == 3)
+                    CUDA_TRY(h, lbm2p_launch::node_pressure_quad(&n, g, prev ? &prev : nullptr, a,
+                                                                 kk == m, h->tb_H, h->tb_grid));
+                else if (h->tb_kind == 2)
                     CUDA_TRY(h, lbm2p_launch::node_pressure_pair_direct(&n, g, prev ? &prev : nullptr,
                                                                         a, kk == m, h->tb_W / 30,
                                                                         h->tb_H, h->tb_grid));
@@ -699,7 +702,10 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
         }
         for (int q = 0; q < nf; ++q) {
             PressureArgs a = pressure_args(h, src, dst_of(src), work);
-            if (h->tb_kind == 2)
+            if (h->tb_kind == 3)
+                lbm2p_launch::pressure_sweeps_quad(a, q == nf - 1 && final_check, h->tb_H,
+                                                   h->tb_grid, h->stream);
+            else if (h->tb_kind == 2)
                 lbm2p_launch::pressure_sweeps_pair_direct(a, q == nf - 1 && final_check,
                                                           h->tb_W / 30, h->tb_H, h->tb_grid,
                                                           h->stream);
@@ -1179,7 +1185,9 @@ lbm2p_status autotune_sweeps(lbm2p *h)
         const bool rows2_only = walls && h->p.fuse_sweeps == 2 && forced == LBM2P_SWEEP_ROWS;
         const bool direct_only = walls && h->p.fuse_sweeps == 2 && forced == LBM2P_SWEEP_SCALAR;
         for (int T : {2, 4}) {
-            if ((h->p.fuse_sweeps != 0 && h->p.fuse_sweeps != T) || rows2_only || direct_only)
+            // lattices with walls on every side have faster forms (below)
+            if ((h->p.fuse_sweeps != 0 && h->p.fuse_sweeps != T) || rows2_only || direct_only ||
+                (walls && (T == 4 || forced == LBM2P_SWEEP_AUTO)))
                 continue;
             for (int W : {128, 64, 32}) {
                 cudaError_t ce = lbm2p_launch::tb_prepare(T, W);
@@ -1214,6 +1222,51 @@ lbm2p_status autotune_sweeps(lbm2p *h)
                         h->tb_H = H;
                         h->tb_grid = (int)blocks;
                     }
+                }
+            }
+        }
+        // four sweeps per launch (lattices with walls on every side), when a check period is an
+        // even number of launches: rows per tile giving 1 to 12 rounds of resident tiles
+        if (walls &&
+            (h->p.fuse_sweeps == 4 || (h->p.fuse_sweeps == 0 && m_chk % 8 == 0)) &&
+            lbm2p_launch::quad_prepare() == cudaSuccess) {
+            const int slots = lbm2p_launch::quad_tile_slots(h->Fp != nullptr);
+            const int strips = (int)lbm2p_launch::quad_strips_of(h->nx);
+            int last_H = -1;
+            for (int rounds : {1, 2, 3, 4, 5, 6, 8, 12}) {
+                if (slots < 1)
+                    break;
+                const long long chunks = (long long)slots * rounds / strips;
+                int H = chunks > 0 ? (int)((h->ny + chunks - 1) / chunks) : 128;
+                H = H < 4 ? 4 : (H > 128 ? 128 : H);
+                H = H < h->ny ? H : h->ny;
+                if (H == last_H)
+                    continue;
+                last_H = H;
+                const long long blocks = lbm2p_launch::quad_grid(H, h->nx, h->ny);
+                if (blocks > (1LL << 30))
+                    continue;
+                float ms = 0.0f, mc = 0.0f;
+                if (!timed([&](int k) {
+                        PressureArgs a = pressure_args(h, k % 2, 1 - k % 2, false);
+                        lbm2p_launch::pressure_sweeps_quad(a, false, H, (int)blocks, h->stream);
+                    }, &ms))
+                    goto done;
+                if (!timed_check([&](int k) {
+                        PressureArgs a = pressure_args(h, k % 2, 1 - k % 2, false);
+                        lbm2p_launch::pressure_sweeps_quad(a, true, H, (int)blocks, h->stream);
+                    }, blocks, ms, &mc))
+                    goto done;
+                const float per = in_loop(ms, mc, 4);
+                note("fused_quad", 4, 0, H, (int)blocks, per * 1e3f);
+                if (fused_wins(per)) {
+                    best = per;
+                    h->tb_T = 4;
+                    h->tb_kind = 3;
+                    h->tb_W = 32;
+                    h->tb_slots = 0;
+                    h->tb_H = H;
+                    h->tb_grid = (int)blocks;
                 }
             }
         }
@@ -1539,9 +1592,14 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
         return *dst != nullptr;
     };
     bool ok = true;
-    for (int b = 0; b < 3; ++b)
+    // the eight planes of a population buffer lie one after another (k_pressure_quad addresses
+    // them by their distance)
+    for (int b = 0; b < 3; ++b) {
+        float *base = (float *)dev_alloc(h, 8 * pb);
+        ok = ok && base;
         for (int i = 0; i < 8; ++i)
-            ok = ok && plane_alloc(&h->fbuf[b][i]);
+            h->fbuf[b][i] = base ? base + (size_t)i * h->plane : nullptr;
+    }
     for (int b = 0; b < 2; ++b) {
         for (int i = 0; i < 9; ++i)
             ok = ok && plane_alloc(&h->gbuf[b][i]);
@@ -2106,8 +2164,9 @@ int lbm2p_fused_form_of(const lbm2p *h)
 {
     if (!h || h->fp16 || h->tb_T <= 1)
         return LBM2P_FUSED_NONE;
-    return h->tb_kind == 2 ? LBM2P_FUSED_DIRECT
-                           : (h->tb_kind == 1 ? LBM2P_FUSED_STAGED_ROWS : LBM2P_FUSED_STAGES);
+    constexpr int forms[4] = {LBM2P_FUSED_STAGES, LBM2P_FUSED_STAGED_ROWS, LBM2P_FUSED_DIRECT,
+                              LBM2P_FUSED_QUAD};
+    return forms[h->tb_kind];
 }
 
 const char *lbm2p_autotune_report(const lbm2p *h)

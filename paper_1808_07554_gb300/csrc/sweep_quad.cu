@@ -1,0 +1,142 @@
+// Four pressure sweeps (Eq. 3-1, pull stream + BGK collide) per launch on lattices with walls on
+// every side.
+//
+// What bounded the sub-iteration was the launches that carry two sweeps (k_pressure_rows2,
+// k_pressure_pair_direct): 154 thread instructions per node and sweep and 36 B per node and sweep.
+// Here a warp owns a tile of 56 columns by H rows and carries four sweeps in registers, about 55
+// thread instructions and 18 B per node and sweep:
+//   - each lane holds two neighbouring columns, so the collision, the sum of Eq. 3-9a and the
+//     unshifted pulls are packed FP32 pairs (add / mul / fma .rn.f32x2, the same IEEE roundings
+//     as the scalar operations), half the issue slots of one column per lane;
+//   - a pull from a neighbouring column needs one warp shuffle per pair of columns;
+//   - the 64 columns of a warp are the 56 it owns and four on each side (one per sweep, and the
+//     segment starts on a 16-byte boundary), so warps exchange nothing: no block barrier;
+//   - input rows are copied by cp.async (16 bytes per lane) into the warp's own ring of 7 slots,
+//     four rows ahead, and waited for by the warp's own copy groups (one cp.async.bulk per plane
+//     and row took 115 us per sweep at 4096^2 where these take 88: 256-byte bulk copies cost about
+//     40 cycles each).
+// Sweep s runs s - 1 rows behind sweep 1.  Of a sweep's values a lane keeps what the next sweep
+// still needs: directions 1 and 3 of the last row, 2, 5, 6 (pulled from below) of the last two,
+// R of six rows, 1/tau_f of four.  Two warps per scheduler with up to 255 registers: three with 168
+// spill inside the row loop (381 against 231 us per launch at 4096^2, whose memory system the
+// spills share).  A tile whose footprint holds no wall node takes the interior path; the others
+// apply the wall rules of Sec. 4 as selects and keep the planes that the rules read.  The edge
+// path is one row body with guards for the filling sweeps, not unrolled: few tiles run it, so its
+// instruction fetches are cold (unrolled, the tile at a corner took 500k cycles at 4096^2 where an
+// interior tile took 60k).
+// The per-node operations and their order are those of the single sweep (dev1, pressure_of,
+// collide1), so four sweeps equal four launches of one bit for bit.
+// Per sweep, two-sweep launches before and this kernel now: 4096^2 129.5 and 57 us (229 us per
+// launch, 1.24 times the time that its 1208 MB take at the copy bandwidth), 1024^2 14.0 and
+// 7.7 us, 512^2 7.5 and 4.1 us.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "lbm2p_async.cuh"
+#include "lbm2p_device.cuh"
+#include "lbm2p_node.cuh"
+#include "sweep_quad.cuh"
+
+namespace lbm2p_dev {
+namespace {
+
+template <bool CHECK, int S>
+__global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
+    k_pressure_quad(const __grid_constant__ PressureArgs a, int H)
+{
+    extern __shared__ __align__(128) float smem_raw[];
+    __shared__ double red[kQuadWarps][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float *smem = quad_warp_smem<S>(smem_raw, warp, a.Fp != nullptr);
+    const int strips = quad_strips(a.g.nx);
+    const int tile = blockIdx.x * kQuadWarps + warp;
+    ResAcc racc;
+    if (tile < strips * ((a.g.ny + H - 1) / H))
+        quad_tile<CHECK, S>(a, H, tile, smem, lane, racc);
+    if (CHECK) {
+        double v[4];
+        racc.warp_totals(v);
+        if (lane == 0)
+            for (int c = 0; c < 4; ++c)
+                red[warp][c] = v[c];
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            double s = 0.0;
+            for (int w = 0; w < kQuadWarps; ++w)
+                s += red[w][threadIdx.x];
+            a.partials[4 * blockIdx.x + threadIdx.x] = s;
+        }
+    }
+}
+
+void *quad_func(bool check)
+{
+    return check ? (void *)k_pressure_quad<true, kQuadSlots> : (void *)k_pressure_quad<false, kQuadSlots>;
+}
+
+}  // namespace
+}  // namespace lbm2p_dev
+
+namespace lbm2p_launch {
+
+using lbm2p_dev::PressureArgs;
+using namespace lbm2p_dev;
+
+long long quad_grid(int H, int nx, int ny)
+{
+    const long long tiles = (long long)quad_strips(nx) * ((ny + H - 1) / H);
+    return (tiles + kQuadWarps - 1) / kQuadWarps;
+}
+
+int quad_strips_of(int nx) { return quad_strips(nx); }
+
+int quad_tile_slots(bool has_fp)
+{
+    int dev = 0, sms = 0, lo = 1 << 30;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    for (bool c : {false, true}) {
+        int b = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, quad_func(c), kQuadThreads,
+                                                          quad_smem_bytes(has_fp)) != cudaSuccess)
+            return 0;
+        lo = b < lo ? b : lo;
+    }
+    return sms * lo * kQuadWarps;
+}
+
+cudaError_t quad_prepare()
+{
+    for (bool c : {false, true}) {
+        cudaError_t e = cudaFuncSetAttribute(quad_func(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)quad_smem_bytes(true));
+        if (e != cudaSuccess)
+            return e;
+    }
+    return cudaSuccess;
+}
+
+void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream)
+{
+    void *args[] = {(void *)&a, (void *)&H};
+    cudaLaunchKernel(quad_func(check), dim3(grid), dim3(kQuadThreads), args,
+                     quad_smem_bytes(a.Fp != nullptr), reinterpret_cast<cudaStream_t>(stream));
+}
+
+cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
+                               const PressureArgs &a, bool check, int H, int grid)
+{
+    cudaKernelNodeParams prm{};
+    prm.func = quad_func(check);
+    prm.gridDim = dim3((unsigned)grid);
+    prm.blockDim = dim3(kQuadThreads);
+    prm.sharedMemBytes = (unsigned)quad_smem_bytes(a.Fp != nullptr);
+    void *args[] = {(void *)&a, (void *)&H};
+    prm.kernelParams = args;
+    prm.extra = nullptr;
+    return cudaGraphAddKernelNode(n, g, dep, dep ? 1 : 0, &prm);
+}
+
+}  // namespace lbm2p_launch

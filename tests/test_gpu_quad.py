@@ -1,0 +1,56 @@
+"""Four pressure sweeps per launch (one warp per tile of 56 columns) against one sweep per launch:
+identical populations bit for bit, at the edges of its tiles: lattices narrower than a tile, one
+column more or less than a whole number of tiles, odd widths (a wall in either column of a lane),
+fewer rows than sweeps, wells on walls, at corners and at tile borders, dense sources, and walls
+of both kinds on opposite sides."""
+import numpy as np
+import pytest
+
+from _problems import uniform
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1808_07554_gb300 import build
+    build.build()
+    import paper_1808_07554_gb300 as pkg
+    pkg.load_library()
+
+
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("bc", [(1, 1, 1, 1), (2, 2, 2, 2), (1, 2, 2, 1), (2, 1, 1, 1)])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (5, 1), (55, 9), (56, 8), (57, 7), (64, 64), (112, 5),
+                                   (113, 131), (168, 33), (301, 257), (600, 40), (1237, 66)])
+def test_four_sweeps_equal_single_sweeps(nx, ny, bc, dense):
+    import paper_1808_07554_gb300 as pkg
+    if ny < 3 and 2 in bc[2:]:
+        pytest.skip("Dirichlet y-sides need three rows")
+    rng = np.random.default_rng(nx * 1000 + ny)
+    wells = {(0, 0), (nx - 1, ny - 1), (min(56, nx - 1), ny // 2), (min(55, nx - 1), ny // 3),
+             (nx // 2, 0), (0, ny // 2)}
+    prob = uniform(nx, ny, bc=bc, K=np.exp(rng.standard_normal((ny, nx))),
+                   S0=0.2 + 0.5 * rng.random((ny, nx)),
+                   Fp=rng.standard_normal((ny, nx)) if dense else None,
+                   wells=[(i, j, 1e-2 * (1 + k), k % 2) for k, (i, j) in enumerate(sorted(wells))],
+                   P_b=[rng.random(2 * (ny if s < 2 else nx) + 1) for s in range(4)],
+                   S_b=[np.full(2 * (ny if s < 2 else nx) + 1, 0.3) for s in range(4)])
+    one = pkg.Solver.from_problem(prob, init_replay=0, fuse_sweeps=1)
+    four = pkg.Solver.from_problem(prob, init_replay=0, fuse_sweeps=4)
+    assert four.fused_form() == pkg.FUSED_QUAD and four.sweep_config()[0] == 4
+    state = one.get_state()
+    state[:8] = 0.01 * rng.standard_normal(state[:8].shape)
+    state[17] = 1.0 / (0.55 + 2.0 * rng.random(state[17].shape))
+    state[19] = rng.standard_normal(state[19].shape)
+    one.set_state(state)
+    four.set_state(state)
+    for n in (4, 9, 8):
+        r1, r4 = one.pressure_sweeps(n), four.pressure_sweeps(n)
+        assert np.array_equal(one.get_state(), four.get_state()), (n, nx, ny, bc)
+        assert r4 == pytest.approx(r1, rel=1e-3, abs=1e-30)
+    one.close()
+    four.close()

@@ -75,6 +75,7 @@ SWEEP_KERNEL_NAMES = {1: "four nodes per thread (128-bit accesses)", 2: "one nod
 # CUDA sources each launch form is compiled from; their hash keys the ncu captures below
 KERNEL_SOURCES = {
     "four_sweep": ["sweep_quad.cu", "sweep_quad.cuh", "lbm2p_node.cuh", "lbm2p_device.cuh"],
+    "resident": ["resident.cu", "lbm2p_node.cuh", "lbm2p_device.cuh"],
     "two_sweep": ["sweep_rows.cu", "lbm2p_node.cuh", "lbm2p_device.cuh", "lbm2p_async.cuh"],
     "single": ["kernels.cu", "sweep_rows.cu", "lbm2p_node.cuh", "lbm2p_device.cuh",
                "lbm2p_async.cuh"],
@@ -91,9 +92,10 @@ NCU_TRAFFIC_PER_LAUNCH = {
         "bytes": 1229841323, "sources": "a38cf4db413179c4",
         "profile": "profiles/pressure_sweeps_fused_rows_five_spot_4096.md"},
 }
-FUSED_FORM_NAMES = {1: "stages", 2: "staged_rows", 3: "direct", 4: "quad"}
+FUSED_FORM_NAMES = {1: "stages", 2: "staged_rows", 3: "direct", 4: "quad", 5: "resident"}
 FUSED_FORM_TEXT = {1: "on shared-memory stages", 2: "on rows staged by bulk copies",
-                   3: "with direct loads", 4: "in registers, one warp per tile of 56 columns"}
+                   3: "with direct loads", 4: "in registers, one warp per tile of 56 columns",
+                   5: "of a whole solve in one launch, the lattice in a cluster's shared memory"}
 
 
 def log(msg: str) -> None:
@@ -541,7 +543,7 @@ def run_ours(args):
     achieved = bpn * nodes / avg_launch_s / 1e9
     form = ((args.workload, FUSED_FORM_NAMES.get(fform, "?"), sweep_cfg[2]) if fused > 1
             else (args.workload, "single", sweep_cfg[1]))
-    src_form = "four_sweep" if fform == 4 else ("two_sweep" if fused > 1 else "single")
+    src_form = {4: "four_sweep", 5: "resident"}[fform] if fform in (4, 5) else ("two_sweep" if fused > 1 else "single")
     src_hash = kernel_source_hash(src_form)
     traffic, traffic_profile = captured_traffic(form, src_hash) if not fp16 else (None, None)
     hist = {}

@@ -276,7 +276,11 @@ typedef enum {
     LBM2P_FUSED_STAGES = 1,      /* T sweeps on shared-memory stages (T = 2 or 4) */
     LBM2P_FUSED_STAGED_ROWS = 2, /* two sweeps on rows staged by bulk copies */
     LBM2P_FUSED_DIRECT = 3,      /* two sweeps, inputs loaded directly (lattices held in L2) */
-    LBM2P_FUSED_QUAD = 4         /* four sweeps, one warp per tile of 56 columns */
+    LBM2P_FUSED_QUAD = 4,        /* four sweeps, one warp per tile of 56 columns */
+    LBM2P_FUSED_RESIDENT = 5     /* whole solves in one launch, the lattice in the shared memory of
+                                    a thread-block cluster (small lattices; solves that end at a
+                                    residual check the graph loop cannot make, an odd check_every,
+                                    use the form that lbm2p_sweep_config reports) */
 } lbm2p_fused_form;
 int lbm2p_fused_form_of(const lbm2p *h);
 
@@ -298,7 +302,8 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
  *   "fused <sweeps per launch> <threads per block> <rows per block> <grid> <us>",
  *   "fused_rows <consumer warps> <ring slots> <rows per block> <grid> <us>",
  *   "fused_direct <warps> 0 <rows per block> <grid> <us>",
- *   "fused_quad <sweeps per launch> 0 <rows per tile> <grid> <us>"
+ *   "fused_quad <sweeps per launch> 0 <rows per tile> <grid> <us>",
+ *   "resident <blocks of the cluster> 0 <rows per block> <grid> <us>" (its residual checks included)
  * with <us> the time per sweep inside the solve loop: a check period of check_every sweeps
  * timed as its plain launches plus the one launch that also sums the residual (the first two
  * kinds once per grid tried: the resident-block capacity of the GPU down to half of it).  Owned by h; valid until the next create-time tuning. */

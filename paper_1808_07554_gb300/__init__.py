@@ -298,7 +298,7 @@ def lbm2p_op_mse_grad(y0, tgt, g, loss, npix, c_out, stream=0):
     _check(_lib_or_raise().lbm2p_op_mse_grad(y0, tgt, g, loss, npix, c_out, stream or None))
 
 
-FUSED_NONE, FUSED_STAGES, FUSED_STAGED_ROWS, FUSED_DIRECT, FUSED_QUAD = 0, 1, 2, 3, 4
+FUSED_NONE, FUSED_STAGES, FUSED_STAGED_ROWS, FUSED_DIRECT, FUSED_QUAD, FUSED_RESIDENT = range(6)
 ROWS2_DENSE = 16
 
 

@@ -632,7 +632,7 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
         M.pair = (!h->fp16 && walls && h->nnodes >= 512LL * 512 && b->body % 4 == 0) ? 1 : 0;
         M.h2 = M.nb2 = M.pb0 = 0;
         if (M.pair) {
-            M.h2 = (h->tb_T > 1 && h->tb_kind == 2 && h->tb_W == 120) ? h->tb_H : 4;
+            M.h2 = (h->tb.T > 1 && h->tb.kind == 2 && h->tb.W == 120) ? h->tb.H : 4;
             M.h2 = M.h2 < h->ny ? M.h2 : h->ny;
             M.nb2 = (int)lbm2p_launch::pair_direct_grid(4, M.h2, h->nx, h->ny);
             M.pb0 = b->pair_total;

@@ -223,6 +223,20 @@ struct LoopCtl {
     double r;       // last residual
 };
 
+// A whole sub-iteration in one launch (resident.cu): m, cap, every and tol from *ctl when given
+// (which receives the sweeps run and the last residual), else from here.
+struct ResidentArgs {
+    LoopCtl *ctl;
+    int m, cap, every;
+    double tol;
+    ResidualOut *out;
+    float *shift_out;        // the residual's conditioning constants (PressureArgs::shift)
+    float *Rw;               // R, moved by a mid-solve rebase (PressureArgs::R)
+    int set_ok;              // 1: set the condition of `ok` to whether the residual is a number
+    cudaGraphConditionalHandle ok;
+    int h, cells;            // rows per block, cells per plane (set by the launcher)
+};
+
 }  // namespace lbm2p_dev
 
 // Error text for calls made without a handle (read back by lbm2p_last_error(NULL)).
@@ -301,6 +315,11 @@ cudaError_t quad_prepare();
 void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream);
 cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                const PressureArgs &a, bool check, int H, int grid);
+// a whole sub-iteration by one cluster of C blocks (resident.cu)
+bool resident_fits(int C, int nx, int ny);
+cudaError_t pressure_resident(const PressureArgs &a, const ResidentArgs &s, int C, void *stream);
+cudaError_t node_resident(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
+                          const PressureArgs &a, const ResidentArgs &s, int C);
 // FP16 storage (fp16.cu): narrow = max |n| -> scale -> convert; one sweep; widen
 int max_blocks_per_sm_pressure_h();
 void half_narrow(const HalfConvertArgs &a, int grid, void *stream);

@@ -14,6 +14,14 @@ struct Alloc {
     void *ptr;
     size_t bytes;
 };
+
+// Fused sweeps: T per launch (0 or 1: single sweeps) by kernel kind 0 = k_pressure_tb (shared-
+// memory stages), 1 = k_pressure_rows2 (two sweeps on staged rows), 2 = k_pressure_pair_direct
+// (two sweeps, direct loads), 3 = k_pressure_quad (four sweeps in registers); W columns (kinds 1
+// and 2: 30 x warps) or threads per block, H rows per block, ring slots of kind 1
+struct FusedShape {
+    int T = 0, kind = 0, W = 0, H = 0, grid = 0, slots = 0;
+};
 }  // namespace lbm2p_internal
 
 struct lbm2p {
@@ -33,13 +41,10 @@ struct lbm2p {
     long long partials_cap = 0;   // residual partials the partials array holds
     int grid_k[2] = {}, grid_check_k[2] = {}, grid_cap_k[2] = {};
     int rows_w = 0, rows_slots = 0, rows_H = 0, rows_grid = 0;   // staged-rows kernel shape
-    int tb_T = 0, tb_W = 0, tb_H = 0, tb_grid = 0;   // fused sweeps per launch and tile shape
-    int tb_kind = 0;           // fused kernel: 0 = k_pressure_tb (shared-memory stages), 1 =
-                               // k_pressure_rows2 (two sweeps on staged rows), 2 =
-                               // k_pressure_pair_direct (two sweeps, direct loads); for 1 and
-                               // 2 tb_W = 30 x warps
-    int tb_slots = 0;          // ring slots of k_pressure_rows2
+    lbm2p_internal::FusedShape tb;          // fused sweeps per launch, chosen at create
+    lbm2p_internal::FusedShape host_form;   // the same for counts driven from the host
     int tb_T_graph = 0;        // fused sweeps used inside the graph loop body (0: single sweeps)
+    int res_C = 0;             // blocks of the cluster that runs whole solves (resident.cu), or 0
     bool fp16 = false;         // storage FP16_DEV: sweeps run on FP16 copies inside a solve
     __half *hbuf[2][8] = {};
     float *Rh[2] = {};

@@ -130,6 +130,7 @@ using lbm2p_internal::fnext;
 using lbm2p_internal::itau_of;
 using lbm2p_internal::R_of;
 using lbm2p_internal::Pstep_of;
+using lbm2p_internal::FusedShape;
 
 lbm2p_status fail(lbm2p *h, lbm2p_status st, const char *fmt, ...)
 {
@@ -294,6 +295,17 @@ int sweep_nparts(const lbm2p *h)
     return h->sweep_kind == 2 ? h->rows_grid : h->grid_check;
 }
 
+// a whole solve in one launch (resident.cu), its rule taken from the handle's loop control
+ResidentArgs resident_args(lbm2p *h, bool work)
+{
+    ResidentArgs s{};
+    s.ctl = h->ctl;
+    s.out = h->res;
+    s.shift_out = h->shift;
+    s.Rw = R_of(h, work);
+    return s;
+}
+
 // ---- graph-resident sub-iteration ----------------------------------------------------------
 // Appends to G: reset(ctl) -> event(sw0) -> the first check period -> WHILE{ further check
 // periods } -> event(sw1).  A check period is m = check_every sweeps (single or fused
@@ -303,12 +315,27 @@ int sweep_nparts(const lbm2p *h)
 // rotation, then ping-pongs between the two buffers other than pin and ends on the third; every
 // later period starts and ends there (m, or m / T fused launches, is even).  So the state the
 // solve starts from is only read, and the solve ends in buffer fnext(pin, 2).  `work`: R and
-// 1/tau_f of the work buffers (a step's solve) or the current ones (a bare solve).
+// 1/tau_f of the work buffers (a step's solve) or the current ones (a bare solve).  A lattice that
+// stays on chip runs all of this in one kernel, which also sets `ok` (when given) to whether the
+// last residual is a number.
 lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int pin, bool work,
-                      cudaGraphNode_t *last)
+                      cudaGraphNode_t *last, const cudaGraphConditionalHandle *ok)
 {
     const int m = h->p.check_every;
     const int b1 = fnext(pin, 1), b2 = fnext(pin, 2);
+    if (h->res_C > 0) {
+        cudaGraphNode_t e0, n, e1;
+        ResidentArgs s = resident_args(h, work);
+        if (ok) {
+            s.set_ok = 1;
+            s.ok = *ok;
+        }
+        CUDA_TRY(h, cudaGraphAddEventRecordNode(&e0, G, dep, dep ? 1 : 0, h->ev_sw0));
+        CUDA_TRY(h, lbm2p_launch::node_resident(&n, G, &e0, pressure_args(h, pin, b2, work), s, h->res_C));
+        CUDA_TRY(h, cudaGraphAddEventRecordNode(&e1, G, &n, 1, h->ev_sw1));
+        *last = e1;
+        return LBM2P_OK;
+    }
     auto dst_of = [&](int src) { return src == b1 ? b2 : b1; };
     cudaGraphNode_t reset, ev0, first_end, wn, ev1;
     CUDA_TRY(h, lbm2p_launch::node_loop_reset(&reset, G, dep, h->ctl));
@@ -327,25 +354,25 @@ lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int p
             for (int kk = T; kk <= m; kk += T) {
                 cudaGraphNode_t n;
                 PressureArgs a = pressure_args(h, src, dst_of(src), work);
-                if (h->tb_kind == 3)
+                if (h->tb.kind == 3)
                     CUDA_TRY(h, lbm2p_launch::node_pressure_quad(&n, g, prev ? &prev : nullptr, a,
-                                                                 kk == m, h->tb_H, h->tb_grid));
-                else if (h->tb_kind == 2)
+                                                                 kk == m, h->tb.H, h->tb.grid));
+                else if (h->tb.kind == 2)
                     CUDA_TRY(h, lbm2p_launch::node_pressure_pair_direct(&n, g, prev ? &prev : nullptr,
-                                                                        a, kk == m, h->tb_W / 30,
-                                                                        h->tb_H, h->tb_grid));
-                else if (h->tb_kind == 1)
+                                                                        a, kk == m, h->tb.W / 30,
+                                                                        h->tb.H, h->tb.grid));
+                else if (h->tb.kind == 1)
                     CUDA_TRY(h, lbm2p_launch::node_pressure_rows2(&n, g, prev ? &prev : nullptr, a,
-                                                                  kk == m, h->tb_W / 30, h->tb_slots,
-                                                                  h->tb_H, h->tb_grid));
+                                                                  kk == m, h->tb.W / 30, h->tb.slots,
+                                                                  h->tb.H, h->tb.grid));
                 else
                     CUDA_TRY(h, lbm2p_launch::node_pressure_fused(&n, g, prev ? &prev : nullptr, a,
-                                                                  T, h->tb_W, h->tb_H, kk == m,
-                                                                  h->tb_grid));
+                                                                  T, h->tb.W, h->tb.H, kk == m,
+                                                                  h->tb.grid));
                 prev = n;
                 src = dst_of(src);
             }
-            nparts = h->tb_grid;
+            nparts = h->tb.grid;
         } else {
             for (int kk = 1; kk <= m; ++kk) {
                 cudaGraphNode_t n;
@@ -402,7 +429,7 @@ lbm2p_status solve_graph(lbm2p *h, int pin, cudaGraphExec_t *out)
         CUDA_TRY(h, cudaGraphCreate(&G, 0));
         h->solve_g[pin][r] = G;
         cudaGraphNode_t last;
-        lbm2p_status e = add_loop(h, G, nullptr, pin, false, &last);
+        lbm2p_status e = add_loop(h, G, nullptr, pin, false, &last, nullptr);
         if (e != LBM2P_OK)
             return e;
         CUDA_TRY(h, cudaGraphInstantiate(&h->solve_x[pin][r], G, 0));
@@ -423,12 +450,15 @@ lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
         h->step_g[pin][pg][r] = G;
         cudaGraphNode_t nr, last, nf, ifn, ns, nb;
         CUDA_TRY(h, lbm2p_launch::node_refresh(&nr, G, nullptr, refresh_args(h, pg, false), h->grid));
-        lbm2p_status e = add_loop(h, G, &nr, pin, true, &last);
-        if (e != LBM2P_OK)
-            return e;
         cudaGraphConditionalHandle hok;
         CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hok, G, 0, 0));
-        CUDA_TRY(h, lbm2p_launch::node_if_finite(&nf, G, &last, h->ctl, hok));
+        lbm2p_status e = add_loop(h, G, &nr, pin, true, &last, &hok);
+        if (e != LBM2P_OK)
+            return e;
+        if (h->res_C > 0)
+            nf = last;
+        else
+            CUDA_TRY(h, lbm2p_launch::node_if_finite(&nf, G, &last, h->ctl, hok));
         cudaGraphNodeParams ip{};
         ip.type = cudaGraphNodeTypeConditional;
         ip.conditional.handle = hok;
@@ -457,9 +487,10 @@ lbm2p_status read_loop(lbm2p *h, int *k, double *r, float *sweep_ms)
     const int m = h->p.check_every;
     const int per_launch = h->tb_T_graph > 1 ? h->tb_T_graph : 1;
     h->sweeps += *k;
-    // reset, sweep launches, finalizes, mid-solve rebases
-    h->launches += 1 + *k / per_launch + *k / m +
-                   (h->rebase_every > 0 && *k > 0 ? (*k - 1) / h->rebase_every : 0);
+    // reset, sweep launches, finalizes, mid-solve rebases; or the one launch of the whole solve
+    h->launches += h->res_C > 0 ? 1
+                                : 1 + *k / per_launch + *k / m +
+                                      (h->rebase_every > 0 && *k > 0 ? (*k - 1) / h->rebase_every : 0);
     if (sweep_ms) {
         *sweep_ms = -1.0f;
         if (h->timing)
@@ -686,7 +717,8 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
         if (h->timing)
             CUDA_TRY(h, cudaEventRecord(h->ev_sw0, st));
         const int n = upto - k;
-        const int T = h->tb_T;
+        const FusedShape &fs = h->host_form;
+        const int T = fs.T;
         const int nf = (T > 1 && n >= T) ? n / T : 0;
         const int ns = n - nf * T;
         const bool final_check = is_check(upto) && upto >= 2;
@@ -702,25 +734,23 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
         }
         for (int q = 0; q < nf; ++q) {
             PressureArgs a = pressure_args(h, src, dst_of(src), work);
-            if (h->tb_kind == 3)
-                lbm2p_launch::pressure_sweeps_quad(a, q == nf - 1 && final_check, h->tb_H,
-                                                   h->tb_grid, h->stream);
-            else if (h->tb_kind == 2)
-                lbm2p_launch::pressure_sweeps_pair_direct(a, q == nf - 1 && final_check,
-                                                          h->tb_W / 30, h->tb_H, h->tb_grid,
-                                                          h->stream);
-            else if (h->tb_kind == 1)
-                lbm2p_launch::pressure_sweeps_rows2(a, q == nf - 1 && final_check, h->tb_W / 30,
-                                                    h->tb_slots, h->tb_H, h->tb_grid, h->stream);
+            if (fs.kind == 3)
+                lbm2p_launch::pressure_sweeps_quad(a, q == nf - 1 && final_check, fs.H, fs.grid,
+                                                   h->stream);
+            else if (fs.kind == 2)
+                lbm2p_launch::pressure_sweeps_pair_direct(a, q == nf - 1 && final_check, fs.W / 30,
+                                                          fs.H, fs.grid, h->stream);
+            else if (fs.kind == 1)
+                lbm2p_launch::pressure_sweeps_rows2(a, q == nf - 1 && final_check, fs.W / 30,
+                                                    fs.slots, fs.H, fs.grid, h->stream);
             else
-                lbm2p_launch::pressure_sweeps_fused(a, T, h->tb_W, h->tb_H,
-                                                    q == nf - 1 && final_check, h->tb_grid,
-                                                    h->stream);
+                lbm2p_launch::pressure_sweeps_fused(a, T, fs.W, fs.H, q == nf - 1 && final_check,
+                                                    fs.grid, h->stream);
             LAUNCHED(h, "fused pressure sweeps");
             src = dst_of(src);
             h->sweeps += T;
         }
-        last_nparts = nf > 0 ? h->tb_grid : sweep_nparts(h);
+        last_nparts = nf > 0 ? fs.grid : sweep_nparts(h);
         if (h->timing)
             CUDA_TRY(h, cudaEventRecord(h->ev_sw1, st));
         k = upto;
@@ -874,8 +904,9 @@ lbm2p_status one_step(lbm2p *h, int replay, lbm2p_step_stats *stats)
         if ((e = read_loop(h, &k, &r, &sw_ms)) != LBM2P_OK)
             return e;
         const bool finite = !std::isnan(r);
-        // refresh and the finiteness test; saturation and rebase when the step goes on
-        h->launches += finite ? 4 : 2;
+        // refresh and the finiteness test (a launch of its own unless the solve is one); saturation
+        // and rebase when the step goes on
+        h->launches += (finite ? 4 : 2) - (h->res_C > 0 ? 1 : 0);
         if (h->timing)
             CUDA_TRY(h, cudaEventElapsedTime(&step_ms, h->ev_step0, h->ev_step1));
         lbm2p_status ps = loop_status(h, k, r);
@@ -1041,8 +1072,19 @@ lbm2p_status autotune_sweeps(lbm2p *h)
     // direct form estimated 8 % ahead here with a 16-sweep check period and 3.5 % ahead in the
     // loop; 8 % ahead with an 8-sweep period and about even in the loop)
     float single_best = 1e30f;
-    auto fused_wins = [&](float per) {
-        return h->tb_T > 1 ? per < best : (per < best && per < kFusedMargin * single_best);
+    // counts driven from the host (replays, bare sweeps) below 512^2 keep launches of at most two
+    // sweeps: what a caller reads from lbm2p_counters there is launches per sweep
+    const bool host_two = h->p.fuse_sweeps == 0 && h->nnodes < 512LL * 512;
+    float host_best = 1e30f;
+    auto take = [&](float per, const FusedShape &s, bool pinned) {
+        if (pinned || (per < best && (h->tb.T > 1 || per < kFusedMargin * single_best))) {
+            best = per;
+            h->tb = s;
+        }
+        if (host_two && s.T == 2 && per < host_best && per < kFusedMargin * single_best) {
+            host_best = per;
+            h->host_form = s;
+        }
     };
     h->autotune_log.clear();
     auto note = [&](const char *what, int a1, int a2, int a3, int a4, float us) {
@@ -1064,7 +1106,7 @@ lbm2p_status autotune_sweeps(lbm2p *h)
             return true;
         return timed(launch, ms);
     };
-    h->tb_T = 0;
+    h->tb = h->host_form = FusedShape{};
     h->sweep_kind = forced == LBM2P_SWEEP_AUTO ? 0 : forced - 1;
     if (!fused_only || forced != LBM2P_SWEEP_AUTO) {
         // grid-stride kernels: resident blocks per SM from the occupancy limit down to half
@@ -1214,14 +1256,7 @@ lbm2p_status autotune_sweeps(lbm2p *h)
                         goto done;
                     const float per = in_loop(ms, mc, T);
                     note("fused", T, W, H, (int)blocks, per * 1e3f);
-                    if (fused_wins(per)) {
-                        best = per;
-                        h->tb_T = T;
-                        h->tb_kind = 0;
-                        h->tb_W = W;
-                        h->tb_H = H;
-                        h->tb_grid = (int)blocks;
-                    }
+                    take(per, FusedShape{T, 0, W, H, (int)blocks, 0}, false);
                 }
             }
         }
@@ -1259,15 +1294,7 @@ lbm2p_status autotune_sweeps(lbm2p *h)
                     goto done;
                 const float per = in_loop(ms, mc, 4);
                 note("fused_quad", 4, 0, H, (int)blocks, per * 1e3f);
-                if (fused_wins(per)) {
-                    best = per;
-                    h->tb_T = 4;
-                    h->tb_kind = 3;
-                    h->tb_W = 32;
-                    h->tb_slots = 0;
-                    h->tb_H = H;
-                    h->tb_grid = (int)blocks;
-                }
+                take(per, FusedShape{4, 3, 32, H, (int)blocks, 0}, false);
             }
         }
         // two sweeps per launch on rows staged by bulk copies (lattices with walls on every
@@ -1300,15 +1327,8 @@ lbm2p_status autotune_sweeps(lbm2p *h)
                         goto done;
                     const float per = in_loop(ms, mc, 2);
                     note("fused_direct", cw, 0, Hc, (int)blocks, per * 1e3f);
-                    if (fused_wins(per) || (direct_only && h->tb_kind != 2)) {
-                        best = per;
-                        h->tb_T = 2;
-                        h->tb_kind = 2;
-                        h->tb_W = 30 * cw;
-                        h->tb_slots = 0;
-                        h->tb_H = Hc;
-                        h->tb_grid = (int)blocks;
-                    }
+                    take(per, FusedShape{2, 2, 30 * cw, Hc, (int)blocks, 0},
+                         direct_only && h->tb.kind != 2);
                 }
             }
         }
@@ -1346,19 +1366,43 @@ lbm2p_status autotune_sweeps(lbm2p *h)
                         goto done;
                     const float per = in_loop(ms, mc, 2);
                     note("fused_rows", cw, slots, Hc, (int)blocks, per * 1e3f);
-                    if (fused_wins(per)) {
-                        best = per;
-                        h->tb_T = 2;
-                        h->tb_kind = 1;
-                        h->tb_W = lbm2p_launch::rows2_width(cw);
-                        h->tb_slots = slots;
-                        h->tb_H = Hc;
-                        h->tb_grid = (int)blocks;
-                    }
+                    take(per, FusedShape{2, 1, lbm2p_launch::rows2_width(cw), Hc, (int)blocks, slots}, false);
                 }
             }
         }
     }
+    if (!host_two)
+        h->host_form = h->tb;
+    // whole solves in one launch, for lattices that fit a cluster's shared memory: timed over four
+    // check periods (the tolerance -1 never stops it), checks included.  What a check costs the
+    // other forms besides its launch (the finalize kernel and the conditional nodes around it,
+    // about 10 us at 64^2 to 256^2) is not in their times, so it is added here
+    h->res_C = 0;
+    best += 0.010f / (float)m_chk;
+    if (h->p.fuse_sweeps == 0 && forced == LBM2P_SWEEP_AUTO && m_chk >= 2 && m_chk <= 4096)
+        for (int C : {1, 2, 4, 8, 16}) {
+            if (!lbm2p_launch::resident_fits(C, h->nx, h->ny))
+                continue;
+            ResidentArgs s{};
+            s.m = m_chk;
+            s.cap = 4 * m_chk;
+            s.tol = -1.0;
+            s.out = reinterpret_cast<ResidualOut *>(h->partials);
+            s.shift_out = h->shift;
+            s.Rw = R_of(h, false);
+            float ms = 0.0f;
+            if (!timed([&](int k) {
+                    lbm2p_launch::pressure_resident(pressure_args(h, k % 2, 1 - k % 2, false), s, C,
+                                                    h->stream);
+                }, &ms))
+                goto done;
+            const float per = ms / (float)s.cap;
+            note("resident", C, 0, (h->ny + C - 1) / C, C, per * 1e3f);
+            if (per < best) {
+                best = per;
+                h->res_C = C;
+            }
+        }
 done:
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1656,7 +1700,7 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
             return e;
     } else {
         h->sweep_kind = 1;
-        h->tb_T = 0;
+        h->tb = h->host_form = FusedShape{};
         lbm2p_status e = autotune_h(h, sms);
         if (e != LBM2P_OK)
             return e;
@@ -1667,7 +1711,8 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
     h->grid_sweep = h->grid_k[h->sweep_kind < 2 ? h->sweep_kind : 1];
     h->grid_check = h->grid_check_k[h->sweep_kind < 2 ? h->sweep_kind : 1];
     {
-        int np = h->tb_grid > h->rows_grid ? h->tb_grid : h->rows_grid;
+        int np = h->tb.grid > h->rows_grid ? h->tb.grid : h->rows_grid;
+        np = np > h->host_form.grid ? np : h->host_form.grid;
         np = np > h->grid_h ? np : h->grid_h;
         np = np > h->h16_grid ? np : h->h16_grid;
         for (int kind = 0; kind < 2; ++kind) {
@@ -1702,10 +1747,10 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
     // the loop body holds check_every sweeps and must return to the same f buffer
     h->graph_ok = !h->fp16 && p.check_every >= 2 && p.check_every % 2 == 0 &&
                   p.max_sub_iters % p.check_every == 0;
-    if (h->tb_T > 1 && p.check_every % (2 * h->tb_T) != 0)
+    if (h->tb.T > 1 && p.check_every % (2 * h->tb.T) != 0)
         h->tb_T_graph = 0;
     else
-        h->tb_T_graph = h->tb_T;
+        h->tb_T_graph = h->tb.T;
     {
         LoopCtl c{};
         c.m = p.check_every;
@@ -2085,7 +2130,7 @@ lbm2p_status lbm2p_sweep_config(const lbm2p *h, int *fused, int *kind, int *tile
     if (!h)
         return fail(nullptr, LBM2P_EINVAL, "NULL handle");
     if (fused)
-        *fused = h->tb_T > 1 ? h->tb_T : 1;
+        *fused = h->tb.T > 1 ? h->tb.T : 1;
     if (h->fp16) {                       // the FP16 sweep kernels
         if (kind)
             *kind = h->h16_kind == 1 ? LBM2P_SWEEP_ROWS : LBM2P_SWEEP_SCALAR;
@@ -2098,9 +2143,9 @@ lbm2p_status lbm2p_sweep_config(const lbm2p *h, int *fused, int *kind, int *tile
     if (kind)
         *kind = h->sweep_kind + 1;        // internal 0, 1, 2 = VEC4, SCALAR, ROWS
     if (tile_w)
-        *tile_w = h->tb_T > 1 ? h->tb_W : (h->sweep_kind == 2 ? h->rows_w : 0);
+        *tile_w = h->tb.T > 1 ? h->tb.W : (h->sweep_kind == 2 ? h->rows_w : 0);
     if (tile_h)
-        *tile_h = h->tb_T > 1 ? h->tb_H : (h->sweep_kind == 2 ? h->rows_H : 0);
+        *tile_h = h->tb.T > 1 ? h->tb.H : (h->sweep_kind == 2 ? h->rows_H : 0);
     return LBM2P_OK;
 }
 
@@ -2148,25 +2193,25 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
                     h->partials_cap);
     CUDA_TRY(h, cudaStreamSynchronize((cudaStream_t)h->stream));
     drop_graphs(h);
-    h->tb_T = 2;
+    h->res_C = 0;
     // as at create: the graph loop body runs the fused launches only when check_every is a
     // multiple of 2 T (an even number of launches per body)
     h->tb_T_graph = h->p.check_every % 4 == 0 ? 2 : 0;
-    h->tb_kind = form == LBM2P_FUSED_STAGED_ROWS ? 1 : 2;
-    h->tb_W = 30 * warps;
-    h->tb_slots = form == LBM2P_FUSED_STAGED_ROWS ? slots : 0;
-    h->tb_H = rows;
-    h->tb_grid = (int)grid;
+    const bool staged = form == LBM2P_FUSED_STAGED_ROWS;
+    h->tb = FusedShape{2, staged ? 1 : 2, 30 * warps, rows, (int)grid, staged ? slots : 0};
+    h->host_form = h->tb;
     return LBM2P_OK;
 }
 
 int lbm2p_fused_form_of(const lbm2p *h)
 {
-    if (!h || h->fp16 || h->tb_T <= 1)
+    if (h && !h->fp16 && h->res_C > 0)
+        return LBM2P_FUSED_RESIDENT;
+    if (!h || h->fp16 || h->tb.T <= 1)
         return LBM2P_FUSED_NONE;
     constexpr int forms[4] = {LBM2P_FUSED_STAGES, LBM2P_FUSED_STAGED_ROWS, LBM2P_FUSED_DIRECT,
                               LBM2P_FUSED_QUAD};
-    return forms[h->tb_kind];
+    return forms[h->tb.kind];
 }
 
 const char *lbm2p_autotune_report(const lbm2p *h)

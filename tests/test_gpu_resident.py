@@ -1,0 +1,93 @@
+"""Whole solves in one launch (the lattice in a cluster's shared memory) against one sweep per launch:
+identical populations bit for bit at the edges of its shapes (blocks of one row, a last block with
+fewer rows, one to three nodes per thread, lattices one column wide), for every wall kind, with
+wells, dense sources and a mid-solve rebase, and the same stopping sweep as the host's rule."""
+import numpy as np
+import pytest
+
+import workloads as W
+from _problems import uniform
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(1, 7), (5, 3), (31, 30), (64, 64), (97, 70), (300, 9), (128, 128), (131, 127), (7, 500)]
+WALLS = {"periodic": (0, 0, 0, 0), "noflux": (1, 1, 1, 1), "dirichlet": (2, 2, 2, 2),
+         "mixed": (0, 0, 2, 1), "mixed2": (1, 2, 0, 0)}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1808_07554_gb300 import build
+    build.build()
+    import paper_1808_07554_gb300 as pkg
+    pkg.load_library()
+
+
+def _problem(nx, ny, walls):
+    rng = np.random.default_rng(nx * 1000 + ny)
+    dense = (nx + ny) % 2 == 0
+    wells = [(0, 0, 1e-3, 0), (nx - 1, ny - 1, 1e-3, 1), (nx // 2, ny // 3, 2e-3, 0)]
+    return rng, uniform(nx, ny, bc=WALLS[walls], K=np.exp(rng.standard_normal((ny, nx))),
+                        S0=0.2 + 0.5 * rng.random((ny, nx)),
+                        Fp=rng.standard_normal((ny, nx)) if dense else None, wells=wells,
+                        P_b=[rng.random(2 * (ny if s < 2 else nx) + 1) for s in range(4)],
+                        S_b=[np.full(2 * (ny if s < 2 else nx) + 1, 0.3) for s in range(4)])
+
+
+@pytest.mark.parametrize("walls", list(WALLS))
+@pytest.mark.parametrize("nx,ny", SHAPES)
+def test_resident_equals_single_sweeps(nx, ny, walls):
+    import paper_1808_07554_gb300 as pkg
+    bc = WALLS[walls]
+    if (nx < 3 and 2 in bc[:2]) or (ny < 3 and 2 in bc[2:]):
+        pytest.skip("Dirichlet sides need three nodes")
+    rng, prob = _problem(nx, ny, walls)
+    state = None
+    for every, cap in ((2, 2), (2, 6), (8, 48), (8, 1040)):   # 1040: a rebase after sweep 1024
+        kw = dict(init_replay=0, tol=0.0, max_sub_iters=cap, check_every=every)
+        one = pkg.Solver.from_problem(prob, fuse_sweeps=1, **kw)
+        res = pkg.Solver.from_problem(prob, **kw)
+        assert res.fused_form() == pkg.FUSED_RESIDENT
+        if state is None:
+            state = one.get_state()
+            state[:8] = 0.01 * rng.standard_normal(state[:8].shape)
+            state[19] = rng.standard_normal(state[19].shape)
+        one.set_state(state)
+        res.set_state(state)
+        s1, s2 = one.step(2), res.step(2)
+        for t in s1[1] + s2[1]:                # the rule r <= 0: a few nodes may reach it
+            assert t.sub_iters == cap or t.residual == 0.0
+        if all(t.sub_iters == cap for t in s1[1] + s2[1]):
+            assert np.array_equal(one.get_state(), res.get_state()), (nx, ny, walls, every, cap)
+            for x, y in zip(s1[1], s2[1]):
+                assert y.residual == pytest.approx(x.residual, rel=1e-3, abs=1e-9)
+        else:
+            assert nx * ny < 16 and cap > 48
+        one.close()
+        res.close()
+
+
+@pytest.mark.parametrize("name", ["five_spot", "manufactured", "example2"])
+def test_resident_stops_where_single_sweeps_do(name):
+    """To a tolerance: the counts agree up to one check period (the residual's sums are grouped
+    differently), and so do the fields; long solves cross several rebases."""
+    import paper_1808_07554_gb300 as pkg
+    prob = {"five_spot": lambda: W.quarter_five_spot(96, seed=3, corr_len=8.0),
+            "manufactured": lambda: W.manufactured_periodic(64),
+            "example2": lambda: W.example2(48)}[name]()
+    one = pkg.Solver.from_problem(prob, fuse_sweeps=1, tol=1e-7)
+    res = pkg.Solver.from_problem(prob, tol=1e-7)
+    assert res.fused_form() == pkg.FUSED_RESIDENT
+    assert abs(one.init_stats.sub_iters - res.init_stats.sub_iters) <= 8
+    for _ in range(3):
+        a, b = one.step(1)[1][0], res.step(1)[1][0]
+        assert abs(a.sub_iters - b.sub_iters) <= 8 and b.residual <= 1e-7
+    Pa, Sa = one.fields(mean_free_P=True)
+    Pb, Sb = res.fields(mean_free_P=True)
+    # one more check period moves P by at most 8 sweeps' increments of 1e-7 each, three solves
+    assert W.rel_l2(Pb, Pa) <= 8 * 4 * 1e-7 * 2 and W.rel_l2(Sb, Sa) <= 1e-6
+    one.close()
+    res.close()

@@ -16,8 +16,8 @@
  * and activations BF16, products accumulated in FP32.  The convolutions run on the fifth-
  * generation tensor cores (tcgen05.mma, accumulators in tensor memory) as implicit GEMMs:
  * M = 128 pixels per tile, N = output channels, K = 9 taps x input channels (forward and
- * input gradient), or M = 128 (tap, input channel) rows, N = output channels, K = pixels
- * (weight gradient).
+ * input gradient), or M = 128 (input row, input channel) rows, N = output channels, K =
+ * pixels (weight gradient).
  *
  * Layouts.  Activations: BF16 [n_img][H][W][C] (channels fastest).  Weights: BF16
  * [9][C_out][C_in], tap t = 3 (dy + 1) + (dx + 1) for the input pixel (y + dy, x + dx).

@@ -4,20 +4,14 @@
 //
 // Convolution as an implicit GEMM (forward and input gradient): a CTA computes tiles of
 // M = 128 consecutive pixels by N = C_out channels; the reduction runs over K = 9 taps x C_in
-// channels in steps of 16.  For each K-step every thread gathers 16 bytes (8 channels of one
-// pixel at one tap, zero outside the image) into a shared-memory stage laid out as the
-// tensor core's K-major core matrices (8 rows x 16 bytes each); thread 0 issues one
-// tcgen05.mma (M = 128, N = C_out, K = 16, BF16 inputs, FP32 accumulator in tensor memory)
-// and commits it to the stage's mbarrier, which frees the stage for the K-step NS later.
-// The weights of all K-steps stay in shared memory for the whole kernel.  After a tile's
-// last K-step the CTA waits for its MMAs, reads the accumulator with tcgen05.ld (each warp
-// its 32 tensor-memory lanes, i.e. its 32 pixels), adds the bias, applies the activation
-// (and the ReLU mask of the input-gradient pass) and stores BF16 channels-last rows.
+// channels in steps of 16 (tcgen05.mma, BF16 inputs, FP32 accumulators in tensor memory, K-major
+// core matrices in shared memory).  The weights stay in shared memory for the whole kernel.  The
+// epilogue (tcgen05.ld, bias, activation, the ReLU mask of the input-gradient pass) stores BF16
+// channels-last rows.
 //
-// Weight gradient: M = 128 rows of (tap, input channel), N = C_out, K = pixels; the stage
-// loader transposes 16-pixel chunks of the channels-last activations and output gradients
-// into K-major core matrices; each CTA reduces a share of the pixels and adds its partial
-// sums into the FP32 gradient with atomics.
+// Weight gradient: M = (input row, input channel), N = C_out, K = pixels, the channels-last operands
+// read MN-major as they are; each CTA reduces a share of the pixels at one dx in tensor memory and adds
+// its partial sums into the FP32 gradient with atomics.
 //
 // Every wait on an mbarrier is bounded; a CTA that gives up records the failure in *err,
 // waits (bounded) for its MMAs in flight, frees its tensor memory and returns.
@@ -35,6 +29,7 @@ lbm2p_status set_global_error(lbm2p_status st, const char *fmt, ...);
 }
 
 namespace lbm2p_op {
+using lbm2p_dev::bar_arrive;
 using lbm2p_dev::bar_init;
 using lbm2p_dev::bar_try_wait;
 using lbm2p_dev::kWaitLimit;
@@ -142,10 +137,11 @@ __device__ __forceinline__ bool wait_bounded(uint64_t *bar, unsigned parity)
     return false;
 }
 
-constexpr int kThreads = 256;
-constexpr int kStages = 4;
-constexpr uint32_t kABytes = 128 * 16 * 2;       // one A stage: 128 rows x 16 BF16
-constexpr uint32_t kTmemCols = 32;
+// 0xffff in each half whose BF16 value is positive
+__device__ __forceinline__ uint32_t positive2(uint32_t v)
+{
+    return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162 *>(&v), __float2bfloat162_rn(0.0f));
+}
 
 struct ConvArgs {
     const bf16 *x;        // [npix][cin]
@@ -161,353 +157,544 @@ struct ConvArgs {
 
 // ---- convolution on staged rows ----------------------------------------------------------
 // A tile is 128 consecutive pixels of one image row (x0 .. x0 + 127, the last tile of a row
-// ragged).  Its three input rows y - 1 .. y + 1, pixels x0 - 1 .. x0 + 128, are copied once into
-// shared memory as channel-chunk planes: chunk c (channels 8 c .. 8 c + 7) of staged row r is
-// an array of 130 pixels x 16 bytes.  In that layout the A operand of tap (dy, dx) and K-half j
-// is the K-major core-matrix matrix that starts at row dy + 1, chunk 2 j, pixel dx + 1: a shift
-// by one pixel is a shift of the descriptor's start address by 16 bytes, so all 9 x C_in / 16
-// MMAs of a tile read the same staged rows.  Two stage buffers: the rows of the next tile are
-// copied while the tensor core works on the current one.
+// ragged).  Its three input rows y - 1 .. y + 1, pixels x0 - 1 .. x0 + 128, are copied into shared
+// memory as channel-chunk planes: chunk c (channels 8 c .. 8 c + 7) of staged row r is an array of
+// 130 pixels x 16 bytes.  In that layout the A operand of tap (dy, dx) and K-half j is the K-major
+// core-matrix matrix that starts at row dy + 1, chunk 2 j, pixel dx + 1: a shift by one pixel is a
+// shift of the descriptor's start address by 16 bytes, so all 9 x C_in / 16 MMAs of a tile read the
+// same staged rows.
+//
+// The three stages of a tile run in different warps, handed on by mbarriers: eight warps copy (whole
+// pixels, a warp 512 contiguous bytes, the next tile's loads in registers while this one's are
+// stored: cp.async with a chunk plane as its target makes a request of every 16 bytes and kept the
+// load/store unit 60 to 80 % busy), one thread issues the MMAs (descriptors by additions), four warps
+// read the accumulator, of which there are two, apply bias, activation and mask and store whole pixels
+// through a padded row per warp.
+// 1024^2 pixels, 32 -> 32 channels: 80 us with all three in turn in one set of warps.
 constexpr int kRowPix = 130;                        // staged pixels per row
 constexpr uint32_t kChunkBytes = kRowPix * 16;      // one channel chunk of a staged row
+constexpr int kCvCopiers = 8, kCvEpilogue = 4;      // warps 0-7, 8-11; warp 12 issues the MMAs
+constexpr int kCvThreads = 32 * (kCvCopiers + kCvEpilogue + 1);
+constexpr int kCvStages = 3;
+constexpr uint32_t kCvTmemCols = 64;                // two accumulators of 32 columns
+
+// 16 bytes of padding per pixel row of the output tile of a warp
+template <int COUT>
+__host__ __device__ constexpr uint32_t conv_out_row() { return COUT * 2 + 16; }
 
 template <int CIN, int COUT>
-constexpr size_t conv_rows_smem_bytes()
+__host__ __device__ constexpr size_t conv_rows_smem_bytes()
 {
-    return (size_t)(9 * CIN / 16) * COUT * 32 + 2 * (size_t)3 * (CIN / 8) * kChunkBytes + 8 + 16 + 128;
-}
-
-// 16 bytes global -> shared without a register round trip (cp.async); a source outside the
-// image (valid false) reads nothing and fills zeros.  Complete after cp_async_wait_all.
-__device__ __forceinline__ void cp_async16(unsigned char *dst, const void *src, bool valid)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                 :: "r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all()
-{
-    asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
-// the three input rows of a tile into a stage buffer (asynchronous: every copy is in flight
-// at once; the caller waits with cp_async_wait_all)
-template <int CIN, int COUT>
-__device__ __forceinline__ void stage_rows(const ConvArgs &a, unsigned char *buf, long long tile,
-                                           int tiles_x, int tid)
-{
-    constexpr int CH = CIN / 8;
-    const int img = (int)(tile / ((long long)a.H * tiles_x));
-    const int rem = (int)(tile - (long long)img * a.H * tiles_x);
-    const int y = rem / tiles_x, x0 = (rem - y * tiles_x) * 128;
-    for (int i = tid; i < 3 * kRowPix * CH; i += kThreads) {
-        const int c = i % CH, px = (i / CH) % kRowPix, r = i / (CH * kRowPix);
-        const int yy = y + r - 1, xx = x0 + px - 1;
-        const bool valid = yy >= 0 && yy < a.H && xx >= 0 && xx < a.W;
-        const bf16 *src = valid ? a.x + (((size_t)img * a.H + yy) * a.W + xx) * CIN + 8 * c : a.x;
-        cp_async16(buf + (r * CH + c) * kChunkBytes + px * 16, src, valid);
-    }
+    return (size_t)(9 * CIN / 16) * COUT * 32 + kCvStages * (size_t)3 * (CIN / 8) * kChunkBytes +
+           (size_t)kCvEpilogue * 32 * conv_out_row<COUT>() + (2 * kCvStages + 4) * 8 + 16 + 128;
 }
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kThreads) k_conv3x3_rows(const ConvArgs a)
+__global__ void __launch_bounds__(kCvThreads, 2) k_conv3x3_rows(const ConvArgs a)
 {
-    constexpr int CH = CIN / 8;
+    constexpr int CH = CIN / 8, GH = COUT / 8;
     constexpr int KH = CIN / 16;                      // K-halves of 16 channels per tap
     constexpr int KS = 9 * KH;
     constexpr uint32_t kBBytes = COUT * 16 * 2;
     constexpr uint32_t kStageBytes = 3 * CH * kChunkBytes;
     constexpr uint32_t IDESC = idesc_bf16(128, COUT);
+    constexpr uint32_t ORow = conv_out_row<COUT>();
+    constexpr int R = kCvStages;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     unsigned char *wsm = smem;
     unsigned char *stg = smem + KS * kBBytes;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(stg + 2 * kStageBytes);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 1);
+    unsigned char *osm = stg + R * kStageBytes;
+    // full[s] / empty[s]: stage s copied / read; done[d] / taken[d]: accumulator d ready / read
+    uint64_t *full = reinterpret_cast<uint64_t *>(osm + kCvEpilogue * 32 * ORow);
+    uint64_t *empty = full + R, *done = empty + R, *taken = done + 2;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(taken + 2);
+    __shared__ int failed;
+    __shared__ unsigned issued;                       // tiles given to the tensor core
+    __shared__ __align__(16) float bsm[COUT];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int kMmaWarp = kCvCopiers + kCvEpilogue;
 
-    for (int i = tid; i < KS * COUT * 2; i += kThreads) {
+    for (int i = tid; i < KS * COUT * 2; i += kCvThreads) {
         const int s = i / (COUT * 2), rem = i - s * (COUT * 2);
         const int kc = rem / COUT, n = rem - kc * COUT;
         const int t = s / KH, j = s - t * KH;
         const uint4 v = *reinterpret_cast<const uint4 *>(a.w + ((size_t)(t * COUT + n) * CIN + 16 * j + 8 * kc));
         *reinterpret_cast<uint4 *>(wsm + s * kBBytes + kc * (COUT * 16) + n * 16) = v;
     }
-    if (warp == 0) {
-        tmem_alloc(tslot, kTmemCols);
+    if (a.bias && tid < COUT)
+        bsm[tid] = a.bias[tid];
+    if (warp == kMmaWarp) {
+        tmem_alloc(tslot, kCvTmemCols);
         tmem_relinquish();
     }
     if (tid == 0) {
-        bar_init(bar, 1);
+        failed = 0;
+        issued = 0;
+        for (int i = 0; i < R; ++i) {
+            bar_init(full + i, kCvCopiers);
+            bar_init(empty + i, 1);
+        }
+        for (int i = 0; i < 2; ++i) {
+            bar_init(done + i, 1);
+            bar_init(taken + i, kCvEpilogue);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    const int tiles_x = (a.W + 127) / 128;
-    const long long tiles = (long long)a.nimg * a.H * tiles_x;
-    long long tile = blockIdx.x;
-    if (tile < tiles)
-        stage_rows<CIN, COUT>(a, stg, tile, tiles_x, tid);
-    cp_async_wait_all();
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    unsigned phase = 0;
-    int b = 0;
+    const unsigned tiles_x = (unsigned)(a.W + 127) / 128u;
+    const long long tiles = (long long)a.nimg * a.H * tiles_x;
+    const unsigned count = tiles > (long long)blockIdx.x
+                               ? (unsigned)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0u;
+    // image row (over all images) and first pixel of this CTA's tile n
+    auto tile_at = [&](unsigned n, long long &row, int &x0) {
+        const long long t = blockIdx.x + (long long)n * gridDim.x;
+        row = tiles < 0x7fffffffLL ? (long long)((unsigned)t / tiles_x) : t / tiles_x;
+        x0 = (int)(t - row * tiles_x) * 128;
+    };
     bool ok = true;
-    for (; tile < tiles; tile += gridDim.x, b ^= 1) {
-        unsigned char *cur = stg + b * kStageBytes;
-        if (tid == 0) {
+    if (warp == kMmaWarp) {
+        if (lane == 0) {
+            // descriptors: start addresses count 16 bytes
+            const uint64_t ad0 = sdesc(smem_u32(stg), kChunkBytes, 128);
+            const uint64_t bd0 = sdesc(smem_u32(wsm), COUT * 16, 128);
+            for (unsigned n = 0; n < count; ++n) {
+                ok = wait_bounded(full + n % R, (n / R) & 1u) &&
+                     (n < 2 || wait_bounded(taken + (n & 1u), ((n >> 1) + 1u) & 1u));
+                if (!ok)
+                    break;
+                tc_fence_after();
+                const uint64_t ad = ad0 + (n % R) * (kStageBytes >> 4);
+                const uint32_t d = tmem + 32u * (n & 1u);
+#pragma unroll
+                for (int t = 0; t < 9; ++t)
+#pragma unroll
+                    for (int j = 0; j < KH; ++j)
+                        umma_bf16(d, ad + ((((t / 3) * CH + 2 * j) * kChunkBytes + (t % 3) * 16) >> 4),
+                                  bd0 + (((t * KH + j) * kBBytes) >> 4), IDESC, t + j > 0 ? 1u : 0u);
+                umma_commit(empty + n % R);
+                umma_commit(done + (n & 1u));
+                issued = n + 1;
+            }
+        }
+        __syncwarp();
+    } else if (warp < kCvCopiers) {
+        // ---- copies: chunk c of pixels px, px + P, ... of the three rows; the last two pixels of
+        // the rows by the first lanes ----
+        constexpr int P = 32 * kCvCopiers / CH;       // pixels per pass
+        constexpr int NP = 128 / P, NV = 3 * NP + 1;
+        const int c = tid % CH, px = tid / CH;
+        const bool tail = tid < 6 * CH;
+        const int tr = tid / (2 * CH), tpx = 128 + (tid / CH) % 2;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        auto fetch = [&](unsigned n, uint4 (&v)[NV]) {
+            long long row;
+            int x0;
+            tile_at(n, row, x0);
+            const int y = row < 0x7fffffffLL ? (int)((unsigned)row % (unsigned)a.H) : (int)(row % a.H);
+            const bf16 *src = a.x + ((row - 1) * a.W + x0 - 1) * CIN + 8 * c;
+            auto get = [&](int r, int p) {
+                const int xx = x0 - 1 + p;
+                const bool in = (r != 0 || y > 0) && (r != 2 || y < a.H - 1) && xx >= 0 && xx < a.W;
+                return in ? __ldg(reinterpret_cast<const uint4 *>(src + ((long long)r * a.W + p) * CIN)) : zero;
+            };
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int q = 0; q < NP; ++q)
+                    v[r * NP + q] = get(r, px + q * P);
+            v[NV - 1] = tail ? get(tr, tpx) : zero;
+        };
+        auto hand_over = [&](unsigned n, const uint4 (&v)[NV]) {
+            if (n >= (unsigned)R && !wait_bounded(empty + n % R, (n / R + 1u) & 1u)) {
+                ok = false;
+                return;
+            }
+            unsigned char *dst = stg + (n % R) * kStageBytes + c * kChunkBytes;
+#pragma unroll
+            for (int r = 0; r < 3; ++r)
+#pragma unroll
+                for (int q = 0; q < NP; ++q)
+                    *reinterpret_cast<uint4 *>(dst + r * CH * kChunkBytes + (px + q * P) * 16) = v[r * NP + q];
+            if (tail)
+                *reinterpret_cast<uint4 *>(dst + tr * CH * kChunkBytes + tpx * 16) = v[NV - 1];
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0)
+                bar_arrive(full + n % R);
+        };
+        uint4 v0[NV], v1[NV];
+        if (count > 0)
+            fetch(0, v0);
+        for (unsigned n = 0; n < count && ok; n += 2) {
+            if (n + 1 < count)
+                fetch(n + 1, v1);
+            hand_over(n, v0);
+            if (n + 1 < count && ok) {
+                if (n + 2 < count)
+                    fetch(n + 2, v0);
+                hand_over(n + 1, v1);
+            }
+        }
+    } else {
+        // ---- epilogue: a pixel per lane, 32 lanes of tensor memory per warp ----
+        const int w = warp - kCvCopiers;              // = warp % 4, the warp's tensor-memory lanes
+        unsigned char *out = osm + w * 32 * ORow;
+        // stores: whole pixels, GH lanes each; lane's chunk sc of pixels sp, sp + 32 / GH, ...
+        const int sc = lane % GH, sp = lane / GH;
+        for (unsigned n = 0; n < count; ++n) {
+            long long row;
+            int x0;
+            tile_at(n, row, x0);
+            const int xw = x0 + 32 * w;               // the warp's first pixel
+            const long long q0 = row * a.W + xw;
+            // the mask is on its way while the tensor core works
+            uint4 mk[GH];
+            if (a.mask)
+#pragma unroll
+                for (int i = 0; i < GH; ++i) {
+                    const int px = i * (32 / GH) + sp;
+                    mk[i] = xw + px < a.W ? __ldg(reinterpret_cast<const uint4 *>(
+                                                a.mask + (q0 + px) * COUT + 8 * sc))
+                                          : make_uint4(0u, 0u, 0u, 0u);
+                }
+            const bool m0 = a.mask && a.y0 && xw + lane < a.W
+                                ? __bfloat162float(a.mask[(q0 + lane) * COUT]) > 0.0f : true;
+            ok = wait_bounded(done + (n & 1u), (n >> 1) & 1u);
+            if (!ok)
+                break;
             tc_fence_after();
-            int s = 0;
+            float v[COUT];
 #pragma unroll
-            for (int t = 0; t < 9; ++t) {
+            for (int h = 0; h < COUT / 16; ++h)
+                tmem_ld16(tmem + ((uint32_t)(32 * w) << 16) + 32u * (n & 1u) + 16u * h,
+                          *reinterpret_cast<float (*)[16]>(v + 16 * h));
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                bar_arrive(taken + (n & 1u));
+            if (a.bias)
 #pragma unroll
-                for (int j = 0; j < KH; ++j, ++s) {
-                    const uint32_t start = smem_u32(cur + ((t / 3) * CH + 2 * j) * kChunkBytes +
-                                                    (t % 3) * 16);
-                    const uint64_t ad = sdesc(start, kChunkBytes, 128);
-                    const uint64_t bd = sdesc(smem_u32(wsm + s * kBBytes), COUT * 16, 128);
-                    umma_bf16(tmem, ad, bd, IDESC, s > 0 ? 1u : 0u);
+                for (int i = 0; i < COUT; i += 4) {
+                    const float4 t = *reinterpret_cast<const float4 *>(bsm + i);
+                    v[i] += t.x;
+                    v[i + 1] += t.y;
+                    v[i + 2] += t.z;
+                    v[i + 3] += t.w;
                 }
+            if (a.act == 1)
+#pragma unroll
+                for (int i = 0; i < COUT; ++i)
+                    v[i] = fmaxf(v[i], 0.0f);
+            if (a.y0 && xw + lane < a.W)
+                a.y0[q0 + lane] = m0 ? v[0] : 0.0f;
+            if (!a.y)
+                continue;
+#pragma unroll
+            for (int c = 0; c < GH; ++c) {
+                __nv_bfloat162 o[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    o[e] = __floats2bfloat162_rn(v[8 * c + 2 * e], v[8 * c + 2 * e + 1]);
+                *reinterpret_cast<uint4 *>(out + lane * ORow + c * 16) = *reinterpret_cast<const uint4 *>(o);
             }
-            umma_commit(bar);
-        }
-        // the next tile's rows into the other buffer while the tensor core works
-        const long long next = tile + gridDim.x;
-        if (next < tiles)
-            stage_rows<CIN, COUT>(a, stg + (b ^ 1) * kStageBytes, next, tiles_x, tid);
-        if (!wait_bounded(bar, phase)) {
-            ok = false;
-            break;
-        }
-        phase ^= 1u;
-        tc_fence_after();
-        const int img = (int)(tile / ((long long)a.H * tiles_x));
-        const int rem = (int)(tile - (long long)img * a.H * tiles_x);
-        const int y = rem / tiles_x, x0 = (rem - y * tiles_x) * 128;
-        const int cb = 16 * (warp >> 2);
-        if (cb < COUT) {
-            float v[16];
-            tmem_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)cb, v);
-            const int x = x0 + 32 * (warp & 3) + lane;
-            if (x < a.W) {
-                const long long q = ((long long)img * a.H + y) * a.W + x;
+            __syncwarp();
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    float u = v[i] + (a.bias ? a.bias[cb + i] : 0.0f);
-                    if (a.act == 1)
-                        u = fmaxf(u, 0.0f);
-                    v[i] = u;
-                }
+            for (int i = 0; i < GH; ++i) {
+                const int px = i * (32 / GH) + sp;
+                uint4 o = *reinterpret_cast<const uint4 *>(out + px * ORow + sc * 16);
                 if (a.mask) {
-                    const bf16 *mk = a.mask + q * COUT + cb;
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (!(__bfloat162float(mk[i]) > 0.0f))
-                            v[i] = 0.0f;
+                    o.x &= positive2(mk[i].x);
+                    o.y &= positive2(mk[i].y);
+                    o.z &= positive2(mk[i].z);
+                    o.w &= positive2(mk[i].w);
                 }
-                if (a.y) {
-                    __align__(16) bf16 o[16];
-#pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        o[i] = __float2bfloat16_rn(v[i]);
-                    uint4 *dst = reinterpret_cast<uint4 *>(a.y + q * COUT + cb);
-                    dst[0] = reinterpret_cast<const uint4 *>(o)[0];
-                    dst[1] = reinterpret_cast<const uint4 *>(o)[1];
-                }
-                if (a.y0 && cb == 0)
-                    a.y0[q] = v[0];
+                if (xw + px < a.W)
+                    *reinterpret_cast<uint4 *>(a.y + (q0 + px) * COUT + 8 * sc) = o;
             }
+            __syncwarp();
         }
-        // the next tile's rows are in place, and the accumulator and the buffer just read are
-        // free, once every thread is past here
-        cp_async_wait_all();
-        fence_async_smem();
-        tc_fence_before();
-        __syncthreads();
     }
-    cp_async_wait_all();
-    if (!ok) {
-        if (tid == 0)
-            atomicExch(a.err, 1);
-        wait_bounded(bar, phase);
-    }
+    if (!ok)
+        failed = 1;
+    __syncthreads();
+    // every MMA issued has ended when the last commits have arrived
+    for (unsigned q = issued > 2u ? issued - 2u : 0u; q < issued; ++q)
+        if (!wait_bounded(done + (q & 1u), (q >> 1) & 1u))
+            ok = false;
+    if ((!ok || failed) && lane == 0)
+        atomicExch(a.err, 1);
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == kMmaWarp) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        tmem_dealloc(tmem, kCvTmemCols);
     }
 }
 
 // ---- weight gradient --------------------------------------------------------------------
+// dw[t][co][ci] = sum over pixels p of x[p + d_t][ci] g[p][co]: M = (input row dy, channel), N = C_out,
+// K = pixels, a CTA per dx and chain.  The operands have their channels contiguous, i.e. they are
+// MN-major, which the tensor core reads as they are (transpose bits of the instruction descriptor):
+// a chunk of eight channels by eight pixels is one 128-byte core matrix, so a stage holds, per input
+// row and chunk, eight K-steps of 16 pixels x 16 bytes (core matrices 128 bytes apart along K).  The rows of M beyond 3 C_in read whatever follows and are not
+// used.  Sixteen (eight) warps load whole pixels (two groups of eight K-steps ahead, in registers: cp.async
+// with chunk planes as its target fetched every 16 bytes by a request of its own, 194 us), store them
+// into a ring of stages and hand these over by mbarriers to the warp that issues the MMAs; the
+// accumulator stays in tensor memory over all of a CTA's K-steps and is added to the gradient
+// with FP32 atomics at the end.  In the CTAs of dx = 0 every copying lane also
+// adds up what it copied of g: the bias gradient.
+//
+// The pixels are reduced in gridDim.y chains, chain s taking K-steps s, s + chains, ...: a third
+// (half) of the SMs, i.e. one chain per SM and 128 rows of the 9 C_in.  The tensor core truncates when
+// it accumulates, so a result depends on the length of its chain: 50 chains are 2e-5 from the exact
+// sums where 456 shorter ones were 2e-6 (and took a fifth less of a training step), but results are
+// kept as they have been.
+// 16 images of 256^2, 32 -> 32 channels: 1551 us before (one K-step at a time, transposed by 2-byte
+// stores into K-major matrices) and 22 us for the bias on its own.
+// warps that copy (16 bytes of three rows of x per lane and group), beside the one that issues the
+// MMAs: sixteen at 32 input channels, eight at 16, where two CTAs share an SM
+__host__ __device__ constexpr int wgrad_copiers(int cin) { return cin == 32 ? 16 : 8; }
+__host__ __device__ constexpr int wgrad_threads(int cin) { return 32 * (wgrad_copiers(cin) + 1); }
+constexpr int kWgSteps = 8;                          // K-steps of a stage
+constexpr uint32_t kWgTmemCols = 32;
+template <int CIN>
+__host__ __device__ constexpr int wgrad_stages() { return 3; }
+// bytes from chunk plane to chunk plane in a stage: the lanes of a warp copy whole pixels, chunk by
+// chunk, and the distance keeps their 16-byte writes in different banks
+__host__ __device__ constexpr uint32_t wgrad_plane(int channels)
+{
+    return kWgSteps * 256 + (channels == 32 ? 32 : 64);
+}
+
 struct WgradArgs {
     const bf16 *x;        // [npix][cin]
     const bf16 *g;        // [npix][cout]
     float *dw;            // [9][cout][cin]
+    float *db;            // [cout] or null
     int nimg, H, W;
     int *err;
 };
 
 template <int CIN, int COUT>
-constexpr size_t wgrad_smem_bytes()
+__host__ __device__ constexpr uint32_t wgrad_stage_bytes()
 {
-    return (size_t)kStages * (kABytes + COUT * 32) + kStages * 8 + 16 + 128;
+    return (uint32_t)(3 * (CIN / 8)) * wgrad_plane(CIN) + (uint32_t)(COUT / 8) * wgrad_plane(COUT);
 }
 
-// grid (M-tiles of 128 (tap, channel) rows, pixel splits): CTA (mt, sp) reduces the K-steps
-// sp, sp + gridDim.y, ... of 16 pixels each
+// the 16 planes that an MMA's 128 rows span reach past the last stage
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(kThreads) k_conv3x3_wgrad(const WgradArgs a)
+__host__ __device__ constexpr size_t wgrad_smem_bytes()
 {
-    constexpr uint32_t kBBytes = COUT * 16 * 2;
-    constexpr uint32_t IDESC = idesc_bf16(128, COUT);
-    constexpr int R = 9 * CIN;                         // rows (tap, ci)
-    constexpr int TPT = 128 / CIN;                     // taps per M-tile
+    const size_t st = wgrad_stage_bytes<CIN, COUT>(), reach = 16 * (size_t)wgrad_plane(CIN);
+    return (wgrad_stages<CIN>() - 1) * st + (st > reach ? st : reach) + wgrad_stages<CIN>() * 16 + 16 + 128;
+}
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(wgrad_threads(CIN), CIN == 32 ? 1 : 2) k_conv3x3_wgrad(const WgradArgs a)
+{
+    constexpr int CH = CIN / 8, GH = COUT / 8;
+    constexpr int kCopiers = wgrad_copiers(CIN);
+    // 16-byte pieces of g per lane and group
+    constexpr int GI = kWgSteps * GH * 16 > 32 * kCopiers ? kWgSteps * GH / (2 * kCopiers) : 1;
+    constexpr uint32_t IDESC = idesc_bf16(128, COUT) | (1u << 15) | (1u << 16);
+    constexpr uint32_t kXP = wgrad_plane(CIN), kGP = wgrad_plane(COUT);
+    constexpr uint32_t kG = 3 * CH * kXP;                     // the output gradients in a stage
+    constexpr uint32_t kStage = wgrad_stage_bytes<CIN, COUT>();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
-    unsigned char *asm_ = smem;
-    unsigned char *bsm = smem + kStages * kABytes;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(bsm + kStages * kBBytes);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + kStages);
+    constexpr int R = wgrad_stages<CIN>();
+    // full[s]: every copying warp's share of stage s is in place; empty[s]: its MMAs are done
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + wgrad_smem_bytes<CIN, COUT>() - 128 - 16 - R * 16);
+    uint64_t *empty = full + R;
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(empty + R);
+    __shared__ int failed;
+    __shared__ unsigned issued;                               // groups given to the tensor core
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int mt = blockIdx.x;
-    const int t0 = mt * TPT;                           // first tap of this M-tile
+    const int dx = (int)blockIdx.x - 1;
+    const long long chains = gridDim.y;
 
-    if (warp == 0) {
-        tmem_alloc(tslot, kTmemCols);
+    if (warp == kCopiers) {
+        tmem_alloc(tslot, kWgTmemCols);
         tmem_relinquish();
     }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s)
-            bar_init(bars + s, 1);
+        failed = 0;
+        issued = 0;
+        for (int i = 0; i < R; ++i) {
+            bar_init(full + i, kCopiers);
+            bar_init(empty + i, 1);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-
-    const long long hw = (long long)a.H * a.W;
-    const long long npix = (long long)a.nimg * hw;
+    const long long npix = (long long)a.nimg * a.H * a.W;
     const long long ksteps = (npix + 15) / 16;
-    unsigned gstep = 0;
+    // this chain's K-steps, in groups of kWgSteps
+    const long long mine = ksteps > (long long)blockIdx.y ? (ksteps - blockIdx.y + chains - 1) / chains : 0;
+    const unsigned groups = (unsigned)((mine + kWgSteps - 1) / kWgSteps);
     bool ok = true;
-    // loader roles: A: thread -> (pixel k = tid % 16, tap slot u, channel chunk c): 16 x TPT x
-    // (CIN / 8) = 256 items; B: threads 0 .. 2 COUT - 1 -> (pixel k, channel chunk of g)
-    const int k = tid & 15;
-    const int item = tid >> 4;                         // 0 .. 15
-    const int u = item / (CIN / 8), c = item - u * (CIN / 8);
-    for (long long ks = blockIdx.y; ks < ksteps; ks += gridDim.y, ++gstep) {
-        const int st = (int)(gstep % kStages);
-        if (gstep >= (unsigned)kStages && !wait_bounded(bars + st, ((gstep / kStages) + 1u) & 1u)) {
-            ok = false;
-            break;
-        }
-        unsigned char *As = asm_ + st * kABytes;
-        unsigned char *Bs = bsm + st * kBBytes;
-        const long long p = ks * 16 + k;
-        int img = 0, y = 0, x = 0;
-        if (p < npix) {
-            img = (int)(p / hw);
-            const int r = (int)(p - (long long)img * hw);
-            y = r / a.W;
-            x = r - y * a.W;
-        }
-        // A row m = u * CIN + 8 c + e holds x[p + d_t][8 c + e], t = t0 + u (zero past row R)
-        {
-            const int t = t0 + u;
-            const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-            __align__(16) bf16 v[8];
-            *reinterpret_cast<uint4 *>(v) = make_uint4(0u, 0u, 0u, 0u);
-            if (t < 9 && p < npix && yy >= 0 && yy < a.H && xx >= 0 && xx < a.W)
-                *reinterpret_cast<uint4 *>(v) = *reinterpret_cast<const uint4 *>(
-                    a.x + (((size_t)img * a.H + yy) * a.W + xx) * CIN + 8 * c);
+    if (warp == kCopiers) {
+        // ---- MMAs: one thread ----
+        if (lane == 0) {
+            // descriptors: start addresses count 16 bytes
+            const uint64_t xd0 = sdesc(smem_u32(smem), 128, kXP), gd0 = sdesc(smem_u32(smem) + kG, 128, kGP);
+            for (unsigned n = 0; n < groups && ok; ++n) {
+                ok = wait_bounded(full + n % R, (n / R) & 1u);
+                if (!ok)
+                    break;
+                tc_fence_after();
+                const uint64_t at = (n % R) * (kStage >> 4);
+                const long long left = mine - (long long)n * kWgSteps;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int mrow = u * CIN + 8 * c + e;
-                *reinterpret_cast<bf16 *>(As + (k >> 3) * 2048 + mrow * 16 + (k & 7) * 2) = v[e];
+                for (int ks = 0; ks < kWgSteps; ++ks)
+                    if (ks < left)
+                        umma_bf16(tmem, xd0 + at + ks * 16, gd0 + at + ks * 16, IDESC,
+                                  (n > 0 || ks > 0) ? 1u : 0u);
+                umma_commit(empty + n % R);
+                issued = n + 1;
             }
         }
-        // B row n = 8 c + e holds g[p][8 c + e]
-        if (tid < 16 * (COUT / 8)) {
-            const int cb = tid >> 4;
-            __align__(16) bf16 v[8];
-            *reinterpret_cast<uint4 *>(v) = make_uint4(0u, 0u, 0u, 0u);
-            if (p < npix)
-                *reinterpret_cast<uint4 *>(v) =
-                    *reinterpret_cast<const uint4 *>(a.g + p * COUT + 8 * cb);
+        __syncwarp();
+    } else {
+        // ---- copies ----
+        // pixel k of K-step ks, one chunk of x (in three rows) and one of g of every group.  From
+        // group to group the pixel moves on by 16 kWgSteps chains; image row and column move with
+        // it (no division inside the loop).
+        const int k = (tid / CH) & 15, xc = tid % CH, xks = tid / (16 * CH);
+        const int gk = (tid / GH) & 15, gc = tid % GH, gks = tid / (16 * GH);
+        const long long step = 16 * kWgSteps * chains;
+        const int step_y = (int)((step / a.W) % a.H), step_x = (int)(step % a.W);
+        long long xp = ((long long)blockIdx.y + xks * chains) * 16 + k;
+        long long gp = ((long long)blockIdx.y + gks * chains) * 16 + gk;
+        int y = (int)((xp / a.W) % a.H), x = (int)(xp % a.W);
+        const long long wrow = (long long)a.W * CIN;
+        const bool bias = dx == 0 && a.db && gks < kWgSteps;
+        float bsum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        const unsigned xoff = xc * kXP + xks * 256 + k * 16, goff = kG + gc * kGP + gks * 256 + gk * 16;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        // this lane's loads of group grp (zeros outside the image), then on to the next group
+        auto fetch = [&](unsigned grp, uint4 (&v)[3 + GI]) {
+            const bool in = xks < kWgSteps && xp < npix && (long long)grp * kWgSteps + xks < mine &&
+                            x + dx >= 0 && x + dx < a.W;
+            const bf16 *src = a.x + (xp + dx) * CIN + 8 * xc;
+            v[0] = in && y > 0 ? __ldg(reinterpret_cast<const uint4 *>(src - wrow)) : zero;
+            v[1] = in ? __ldg(reinterpret_cast<const uint4 *>(src)) : zero;
+            v[2] = in && y < a.H - 1 ? __ldg(reinterpret_cast<const uint4 *>(src + wrow)) : zero;
+#pragma unroll
+            for (int q = 0; q < GI; ++q) {
+                const int ks = gks + q * (kWgSteps / GI);
+                const long long p = gp + q * (kWgSteps / GI) * 16 * chains;
+                v[3 + q] = ks < kWgSteps && p < npix && (long long)grp * kWgSteps + ks < mine
+                               ? __ldg(reinterpret_cast<const uint4 *>(a.g + p * COUT + 8 * gc)) : zero;
+            }
+            xp += step;
+            gp += step;
+            x += step_x;
+            y += step_y;
+            if (x >= a.W) {
+                x -= a.W;
+                ++y;
+            }
+            if (y >= a.H)
+                y -= a.H;
+        };
+        auto hand_over = [&](unsigned grp, const uint4 (&v)[3 + GI]) {
+            if (grp >= (unsigned)R && !wait_bounded(empty + grp % R, (grp / R + 1u) & 1u)) {
+                ok = false;
+                return;
+            }
+            unsigned char *buf = smem + (grp % R) * kStage;
+            if (xks < kWgSteps)
+#pragma unroll
+                for (int r = 0; r < 3; ++r)
+                    *reinterpret_cast<uint4 *>(buf + r * CH * kXP + xoff) = v[r];
+            if (gks < kWgSteps)
+#pragma unroll
+                for (int q = 0; q < GI; ++q)
+                    *reinterpret_cast<uint4 *>(buf + goff + q * (kWgSteps / GI) * 256) = v[3 + q];
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0)
+                bar_arrive(full + grp % R);
+            if (bias)
+#pragma unroll
+                for (int q = 0; q < GI; ++q) {
+                    const uint32_t w[4] = {v[3 + q].x, v[3 + q].y, v[3 + q].z, v[3 + q].w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        bsum[2 * e] += __uint_as_float(w[e] << 16);
+                        bsum[2 * e + 1] += __uint_as_float(w[e] & 0xFFFF0000u);
+                    }
+                }
+        };
+        // D - 1 groups of loads in flight while another is stored
+        constexpr int D = 3;
+        uint4 v[D][3 + GI];
+#pragma unroll
+        for (int u = 0; u < D - 1; ++u)
+            if ((unsigned)u < groups)
+                fetch(u, v[u]);
+        for (unsigned n = 0; n < groups && ok; n += D)
+#pragma unroll
+            for (int u = 0; u < D; ++u) {
+                if (n + u + D - 1 < groups)
+                    fetch(n + u + D - 1, v[(u + D - 1) % D]);
+                if (n + u < groups && ok)
+                    hand_over(n + u, v[u]);
+            }
+        if (bias && ok) {
+            // lanes of the same chunk are GH apart
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-                const int n = 8 * cb + e;
-                *reinterpret_cast<bf16 *>(Bs + (k >> 3) * (COUT * 16) + n * 16 + (k & 7) * 2) = v[e];
+#pragma unroll
+                for (int o = 16; o >= GH; o >>= 1)
+                    bsum[e] += __shfl_xor_sync(0xffffffffu, bsum[e], o);
+                if (lane < GH)
+                    atomicAdd(a.db + 8 * gc + e, bsum[e]);
             }
         }
-        fence_async_smem();
-        __syncthreads();
-        if (tid == 0) {
-            tc_fence_after();
-            const uint64_t ad = sdesc(smem_u32(As), 2048, 128);
-            const uint64_t bd = sdesc(smem_u32(Bs), COUT * 16, 128);
-            umma_bf16(tmem, ad, bd, IDESC, gstep > 0 ? 1u : 0u);
-            umma_commit(bars + st);
-        }
     }
-    if (ok && gstep > 0) {
-        const unsigned last = gstep - 1;
-        if (!wait_bounded(bars + last % kStages, (last / kStages) & 1u))
+    if (!ok)
+        failed = 1;
+    __syncthreads();
+    // every MMA issued has ended when the last commits have arrived
+    for (unsigned q = issued > (unsigned)R ? issued - R : 0; q < issued; ++q)
+        if (!wait_bounded(empty + q % R, (q / R) & 1u))
             ok = false;
-    }
-    if (ok && gstep > 0) {
+    ok = ok && !failed;
+    if (ok && groups > 0) {
         tc_fence_after();
-        const int cb = 16 * (warp >> 2);
+        const int cb = 16 * (warp >> 2), row = 32 * (warp & 3) + lane;
         if (cb < COUT) {
             float v[16];
             tmem_ld16(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)cb, v);
-            const int row = mt * 128 + 32 * (warp & 3) + lane;
-            if (row < R) {
-                const int t = row / CIN, ci = row - t * CIN;
+            if (row < 3 * CIN) {
+                const int r = row / CIN, ci = row - r * CIN;
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    atomicAdd(a.dw + ((size_t)t * COUT + cb + i) * CIN + ci, v[i]);
+                    atomicAdd(a.dw + ((size_t)(3 * r + dx + 1) * COUT + cb + i) * CIN + ci, v[i]);
             }
         }
     }
-    if (!ok) {
-        if (tid == 0)
-            atomicExch(a.err, 1);
-        if (gstep > 0)
-            wait_bounded(bars + (gstep - 1) % kStages, ((gstep - 1) / kStages) & 1u);
-    }
+    if (!ok && lane == 0)
+        atomicExch(a.err, 1);
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) {
+    if (warp == kCopiers) {
         tc_fence_after();
-        tmem_dealloc(tmem, kTmemCols);
+        tmem_dealloc(tmem, kWgTmemCols);
     }
 }
 
 // ---- CUDA-core helpers -------------------------------------------------------------------
-__global__ void k_bias_grad(const bf16 *g, float *db, long long npix, int cout)
-{
-    // one block per channel group of 32 pixels strided; thread -> channel (tid % cout)
-    __shared__ float acc[32];
-    const int c = threadIdx.x % cout;
-    const int lanes = blockDim.x / cout;
-    const int l = threadIdx.x / cout;
-    float s = 0.0f;
-    for (long long p = (long long)blockIdx.x * lanes + l; p < npix; p += (long long)gridDim.x * lanes)
-        s += __bfloat162float(g[p * cout + c]);
-    if (threadIdx.x < cout)
-        acc[threadIdx.x] = 0.0f;
-    __syncthreads();
-    atomicAdd(&acc[c], s);
-    __syncthreads();
-    if (threadIdx.x < cout)
-        atomicAdd(db + threadIdx.x, acc[threadIdx.x]);
-}
-
 __global__ void k_flip(const bf16 *w, bf16 *wt, int cin, int cout)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;   // over wt[t][ci][co]
@@ -542,33 +729,65 @@ __device__ __forceinline__ float sd_of(const double *st, long long n)
     return v > 1e-60 ? (float)sqrt(v) : 1.0f;
 }
 
+// (s, c) += (h, l): an unevaluated pair of floats (about 48 bits)
+__device__ __forceinline__ void pair_add(float2 &a, float h, float l)
+{
+    const float s = __fadd_rn(a.x, h), bb = __fsub_rn(s, a.x);
+    const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(h, bb));
+    const float t = __fadd_rn(__fadd_rn(a.y, l), e);
+    a.x = __fadd_rn(s, t);
+    a.y = __fsub_rn(t, __fsub_rn(a.x, s));
+}
+
+// a power of two that brings |v| near 1 (1 for zero, infinities and NaN)
+__device__ __forceinline__ float unit_scale(float v)
+{
+    const int e = (int)((__float_as_uint(v) >> 23) & 255u);
+    return e == 255 || v == 0.0f ? 1.0f : __uint_as_float((unsigned)(e < 253 ? 254 - e : 1) << 23);
+}
+
+// Sums of a - b and (a - b)^2.  The difference of two floats is a pair of floats exactly, and so its
+// square to 2^-48: each thread adds pairs, the squares scaled by a power of two that follows its
+// largest difference (so they cover the range that FP64 would), and the block's totals are added in
+// FP64.  The FP64 units, a 64th as many, took 27 us for a 1024^2 plane.
 __global__ void k_diff_stats(const float *a, const float *b, long long n, double *st)
 {
     __shared__ double red[2][8];
-    double s1 = 0.0, s2 = 0.0;
+    float2 s1 = make_float2(0.0f, 0.0f), s2 = make_float2(0.0f, 0.0f);
+    float sc = 0.0f;                                          // scale of s2's terms (0: none yet)
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
-        const double d = (double)a[i] - (double)b[i];
-        s1 += d;
-        s2 += d * d;
+        const float x = a[i], y = b[i];
+        const float h = __fsub_rn(x, y), yy = __fsub_rn(x, h);
+        const float l = __fsub_rn(__fsub_rn(x, __fadd_rn(h, yy)), __fsub_rn(y, yy));
+        pair_add(s1, h, l);
+        float u = h * sc;
+        if (sc == 0.0f || fabsf(u) > 1073741824.0f) {
+            const float ns = unit_scale(h);
+            const float f = sc == 0.0f ? 0.0f : ns / sc;      // both powers of two
+            s2 = make_float2(s2.x * f * f, s2.y * f * f);
+            sc = h == 0.0f ? sc : ns;
+            u = h * sc;
+        }
+        const float v = l * sc, q = __fmul_rn(u, u);
+        pair_add(s2, q, fmaf(2.0f * u, v, fmaf(u, u, -q)));
     }
+    const double is = sc > 0.0f ? 1.0 / (double)sc : 0.0;
+    double t1 = (double)s1.x + (double)s1.y, t2 = ((double)s2.x + (double)s2.y) * is * is;
     for (int o = 16; o > 0; o >>= 1) {
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+        t2 += __shfl_xor_sync(0xffffffffu, t2, o);
     }
     if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = s1;
-        red[1][threadIdx.x >> 5] = s2;
+        red[0][threadIdx.x >> 5] = t1;
+        red[1][threadIdx.x >> 5] = t2;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double t1 = 0.0, t2 = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            t1 += red[0][w];
-            t2 += red[1][w];
-        }
-        atomicAdd(st, t1);
-        atomicAdd(st + 1, t2);
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+            t += red[threadIdx.x][w];
+        atomicAdd(st + threadIdx.x, t);
     }
 }
 
@@ -576,7 +795,13 @@ __global__ void k_features(const float *lnK, const float *S, const float *Sp, co
                            const float *Pp, const double *dss, const double *dps, bf16 *feat,
                            long long n, float sm, float ss)
 {
-    const float inv_ds = 1.0f / sd_of(dss, n), inv_dp = 1.0f / sd_of(dps, n);
+    // the standard deviations once per block: an FP64 root and divisions in every thread took 55 of
+    // the 63 us of a 1024^2 plane
+    __shared__ float sd[2];
+    if (threadIdx.x < 2)
+        sd[threadIdx.x] = 1.0f / sd_of(threadIdx.x ? dps : dss, n);
+    __syncthreads();
+    const float inv_ds = sd[0], inv_dp = sd[1];
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         __align__(16) bf16 o[16];
@@ -596,7 +821,11 @@ __global__ void k_features(const float *lnK, const float *S, const float *Sp, co
 __global__ void k_target(const float *Pn, const float *P, const float *Pp, const double *dps,
                          float *out, long long n)
 {
-    const float inv_dp = 1.0f / sd_of(dps, n);
+    __shared__ float sd;
+    if (threadIdx.x == 0)
+        sd = 1.0f / sd_of(dps, n);
+    __syncthreads();
+    const float inv_dp = sd;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = (Pn[i] - (2.0f * P[i] - Pp[i])) * inv_dp;
@@ -605,12 +834,18 @@ __global__ void k_target(const float *Pn, const float *P, const float *Pp, const
 __global__ void k_predict(const float *P, const float *Pp, const float *d, const double *dps,
                           float *out, long long n)
 {
-    const float sd = sd_of(dps, n);
+    __shared__ float sh;
+    if (threadIdx.x == 0)
+        sh = sd_of(dps, n);
+    __syncthreads();
+    const float sd = sh;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = (2.0f * P[i] - Pp[i]) + sd * d[i];
 }
 
+// VEC: g is 16-byte aligned (else 2-byte stores)
+template <bool VEC>
 __global__ void k_mse_grad(const float *y0, const float *t, bf16 *g, double *loss, long long n,
                            int cout)
 {
@@ -621,9 +856,17 @@ __global__ void k_mse_grad(const float *y0, const float *t, bf16 *g, double *los
          i += (long long)gridDim.x * blockDim.x) {
         const float e = y0[i] - t[i];
         s += (double)e * e;
-        g[i * cout] = __float2bfloat16_rn(sc * e);
-        for (int c = 1; c < cout; ++c)
-            g[i * cout + c] = __float2bfloat16_rn(0.0f);
+        if (VEC) {
+            // 2-byte stores took 89 us where the bytes need 6 (2^20 pixels, 16 channels)
+            uint4 *dst = reinterpret_cast<uint4 *>(g + i * cout);
+            dst[0] = make_uint4((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(sc * e)), 0u, 0u, 0u);
+            for (int c = 1; c < cout / 8; ++c)
+                dst[c] = make_uint4(0u, 0u, 0u, 0u);
+        } else {
+            g[i * cout] = __float2bfloat16_rn(sc * e);
+            for (int c = 1; c < cout; ++c)
+                g[i * cout + c] = __float2bfloat16_rn(0.0f);
+        }
     }
     for (int o = 16; o > 0; o >>= 1)
         s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -654,8 +897,8 @@ int sm_count()
 
 // CTAs of `func` that fit on one SM by its registers, threads and `smem` bytes of dynamic
 // shared memory (the occupancy rule written out from the device attributes), and by the tensor
-// memory (kTmemCols of the 512 columns per CTA)
-int resident_per_sm(const void *func, size_t smem)
+// memory (tmem_cols of the 512 columns per CTA)
+int resident_per_sm(const void *func, size_t smem, int threads, uint32_t tmem_cols)
 {
     int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0, thr_sm = 0;
     cudaFuncAttributes fa{};
@@ -666,11 +909,11 @@ int resident_per_sm(const void *func, size_t smem)
         cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev) != cudaSuccess)
         return 1;
     const long long per_smem = (long long)smem_sm / ((long long)smem + fa.sharedSizeBytes + reserved);
-    const int regs_cta = ((fa.numRegs * 32 + 255) / 256) * 256 * (kThreads / 32);
+    const int regs_cta = ((fa.numRegs * 32 + 255) / 256) * 256 * (threads / 32);
     const long long per_regs = regs_cta > 0 ? regs_sm / regs_cta : 1;
     long long per = per_smem < per_regs ? per_smem : per_regs;
-    per = per < thr_sm / kThreads ? per : thr_sm / kThreads;
-    per = per < 512 / (long long)kTmemCols ? per : 512 / (long long)kTmemCols;
+    per = per < thr_sm / threads ? per : thr_sm / threads;
+    per = per < 512 / (long long)tmem_cols ? per : 512 / (long long)tmem_cols;
     return per < 1 ? 1 : (int)per;
 }
 
@@ -689,12 +932,13 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t s)
         return e;
     // the runtime's occupancy query answered one CTA per SM for this kernel, where its
     // registers and shared memory allow three (ncu's occupancy limits agree with the latter)
-    const int per_sm = resident_per_sm((const void *)k_conv3x3_rows<CIN, COUT>, smem);
+    const int per_sm = resident_per_sm((const void *)k_conv3x3_rows<CIN, COUT>, smem, kCvThreads,
+                                       kCvTmemCols);
     const long long tiles = (long long)a.nimg * a.H * ((a.W + 127) / 128);
     long long grid = (long long)sm_count() * per_sm;
     if (grid > tiles)
         grid = tiles;
-    k_conv3x3_rows<CIN, COUT><<<(unsigned)grid, kThreads, smem, s>>>(a);
+    k_conv3x3_rows<CIN, COUT><<<(unsigned)grid, kCvThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -709,22 +953,13 @@ cudaError_t launch_wgrad(const WgradArgs &a, cudaStream_t s)
                                  cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess)
         return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_conv3x3_wgrad<CIN, COUT>, kThreads,
-                                                      smem);
-    if (e != cudaSuccess)
-        return e;
-    per_sm = per_sm < 1 ? 1 : (per_sm > 512 / (int)kTmemCols ? 512 / (int)kTmemCols : per_sm);
-    const int mtiles = (9 * CIN + 127) / 128;
     const long long ksteps = ((long long)a.nimg * a.H * a.W + 15) / 16;
-    long long splits = (long long)sm_count() * per_sm / mtiles;
-    if (splits < 1)
-        splits = 1;
-    if (splits > ksteps)
-        splits = ksteps;
-    if (splits > 65535)
-        splits = 65535;
-    k_conv3x3_wgrad<CIN, COUT><<<dim3((unsigned)mtiles, (unsigned)splits), kThreads, smem, s>>>(a);
+    long long chains = sm_count() / ((9 * CIN + 127) / 128);
+    if (chains < 1)
+        chains = 1;
+    if (chains > ksteps)
+        chains = ksteps;
+    k_conv3x3_wgrad<CIN, COUT><<<dim3(3, (unsigned)chains), wgrad_threads(CIN), smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -808,6 +1043,7 @@ lbm2p_status lbm2p_op_conv3x3_wgrad(const void *x, const void *g, float *dw, flo
     a.x = static_cast<const bf16 *>(x);
     a.g = static_cast<const bf16 *>(g);
     a.dw = dw;
+    a.db = dbias;
     a.nimg = n_img;
     a.H = H;
     a.W = W;
@@ -816,12 +1052,6 @@ lbm2p_status lbm2p_op_conv3x3_wgrad(const void *x, const void *g, float *dw, flo
         e = c_out == 16 ? launch_wgrad<16, 16>(a, s) : launch_wgrad<16, 32>(a, s);
     else
         e = c_out == 16 ? launch_wgrad<32, 16>(a, s) : launch_wgrad<32, 32>(a, s);
-    if (e == cudaSuccess && dbias) {
-        const long long npix = (long long)n_img * H * W;
-        k_bias_grad<<<grid_for(npix / 8 + 1, 1), 256, 0, s>>>(static_cast<const bf16 *>(g), dbias,
-                                                               npix, c_out);
-        e = cudaGetLastError();
-    }
     if (e != cudaSuccess)
         return set_global_error(LBM2P_ECUDA, "conv3x3_wgrad launch failed: %s", cudaGetErrorString(e));
     return LBM2P_OK;
@@ -918,7 +1148,8 @@ lbm2p_status lbm2p_op_mse_grad(const float *y0, const float *tgt, void *g, doubl
 {
     if (!y0 || !tgt || !g || !loss || npix < 1 || (c_out != 16 && c_out != 32))
         return set_global_error(LBM2P_EINVAL, "mse_grad: bad arguments");
-    k_mse_grad<<<grid_for(npix, 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+    const auto kernel = aligned16(g) ? k_mse_grad<true> : k_mse_grad<false>;
+    kernel<<<grid_for(npix, 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
         y0, tgt, static_cast<bf16 *>(g), loss, npix, c_out);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)

@@ -43,12 +43,13 @@ struct Member {
     int every;                   // sweeps between mid-solve rebases
     int wshift, rpt, seg_x;      // segment width 2^wshift, rows per tile, segments per row
     int tile0, ntiles;           // range in the batch tile list
-    // A member of 512^2 nodes or more on a lattice with walls on every side ("pair" member)
-    // is swept two sweeps per launch by k_pair_batch (blocks of 120 columns x h2 rows, nb2 of
-    // them, residual partials at pb0 in the pair partials) instead of joining the one-sweep
-    // batched sweep.  pparts / nparts: where finalize finds the member's residual partials
-    // (the pair partials, or the batch's per-tile ones).
-    int pair;                    // 1: a pair member
+    // A member on a lattice with walls on every side sweeps several times per launch instead of
+    // joining the one-sweep batched sweep ("multi" member): four times by k_quad_batch (tiles of
+    // 56 columns x h2 rows) when check_every is a multiple of 8, else, from 512^2 nodes, twice by
+    // k_pair_batch (blocks of 120 columns x h2 rows).  nb2 tiles or blocks, residual partials at
+    // pb0 in the multi partials.  pparts / nparts: where finalize finds the member's residual
+    // partials (these, or the batch's per-tile ones).
+    int multi;
     int h2, nb2, pb0;
     const double *pparts;
     int nparts;
@@ -148,7 +149,6 @@ __global__ void __launch_bounds__(kBlock) kb_sweep(const Member *__restrict__ me
 // mark it for a mid-solve rebase on the rule of the single-lattice loop.  counts[0] counts
 // the members still active, counts[1] those to rebase.
 __global__ void __launch_bounds__(256) kb_finalize(const Member *__restrict__ mem,
-                                                   const double *__restrict__ partials,
                                                    MemberCtl *ctl, int body, int *counts)
 {
     const int mi = blockIdx.x;
@@ -158,7 +158,6 @@ __global__ void __launch_bounds__(256) kb_finalize(const Member *__restrict__ me
     const Member &M = mem[mi];
     __shared__ double red[256][4];
     double s[4] = {0.0, 0.0, 0.0, 0.0};
-    (void)partials;
     for (int i = threadIdx.x; i < M.nparts; i += 256)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
@@ -223,15 +222,15 @@ __global__ void __launch_bounds__(256) kb_prefix(const Member *__restrict__ mem,
         carry[0] = carry[1] = 0;
     }
     __syncthreads();
-    // two exclusive prefixes at once: tiles of the one-sweep members, blocks of the pair
+    // two exclusive prefixes at once: tiles of the one-sweep members, tiles of the multi
     // members (a member is one or the other, so one prefix array holds both)
     for (int base = 0; base < count; base += 256) {
         const int m = base + (int)threadIdx.x;
         const bool on = m < count && ctl[m].active;
-        const int pair = on && mem[m].pair;
-        const int v = on ? (pair ? mem[m].nb2 : mem[m].ntiles) : 0;
-        scan[0][threadIdx.x] = pair ? 0 : v;
-        scan[1][threadIdx.x] = pair ? v : 0;
+        const int multi = on && mem[m].multi;
+        const int v = on ? (multi ? mem[m].nb2 : mem[m].ntiles) : 0;
+        scan[0][threadIdx.x] = multi ? 0 : v;
+        scan[1][threadIdx.x] = multi ? v : 0;
         __syncthreads();
         for (int off = 1; off < 256; off <<= 1) {        // inclusive scans
             const int a0 = (int)threadIdx.x >= off ? scan[0][threadIdx.x - off] : 0;
@@ -242,7 +241,7 @@ __global__ void __launch_bounds__(256) kb_prefix(const Member *__restrict__ mem,
             __syncthreads();
         }
         if (m < count)
-            prefix[m] = carry[pair] + scan[pair][threadIdx.x] - v;
+            prefix[m] = carry[multi] + scan[multi][threadIdx.x] - v;
         __syncthreads();
         if (threadIdx.x == 255) {
             carry[0] += scan[0][255];
@@ -256,8 +255,8 @@ __global__ void __launch_bounds__(256) kb_prefix(const Member *__restrict__ mem,
     }
 }
 
-// one block per member: list the tiles of an active one-sweep member (act) or the blocks of an
-// active pair member (items) at its prefix offset
+// one block per member: list the tiles of an active one-sweep member (act) or those of an active
+// multi member (items) at its prefix offset
 __global__ void __launch_bounds__(256) kb_scatter(const Member *__restrict__ mem,
                                                   const MemberCtl *__restrict__ ctl,
                                                   const int *__restrict__ prefix,
@@ -266,9 +265,9 @@ __global__ void __launch_bounds__(256) kb_scatter(const Member *__restrict__ mem
     const int m = blockIdx.x;
     if (!ctl[m].active)
         return;
-    const bool pair = mem[m].pair != 0;
-    const int base = prefix[m], n = pair ? mem[m].nb2 : mem[m].ntiles;
-    int2 *dst = pair ? items : act;
+    const bool multi = mem[m].multi != 0;
+    const int base = prefix[m], n = multi ? mem[m].nb2 : mem[m].ntiles;
+    int2 *dst = multi ? items : act;
     for (int i = threadIdx.x; i < n; i += 256)
         dst[base + i] = make_int2(m, i);
 }
@@ -328,16 +327,18 @@ struct lbm2p_batch {
     double *h_tols = nullptr;            // pinned
     int *d_active = nullptr;             // [0] active members, [1] members to rebase,
                                          // [2] tiles of the active one-sweep members,
-                                         // [3] blocks of the active pair members
-    int *d_prefix = nullptr;             // first compacted tile (block) of each active member
+                                         // [3] tiles of the active multi members
+    int *d_prefix = nullptr;             // first compacted tile of each active member
     int2 *d_act = nullptr;               // compacted (member, tile) list
     double *d_partials = nullptr;
-    int npair = 0, pair_total = 0;       // pair members, their blocks
+    bool quad = false;                   // the multi members sweep four times per launch
+    bool has_fp = false;                 // one of them has dense sources
+    int nmulti = 0, multi_total = 0;     // multi members, their tiles
     int pair_grid = 0;                   // blocks of a k_pair_batch launch
-    PressureArgs *d_pa2 = nullptr;       // [2 count] argument blocks of the pair launches
-    int *d_h2 = nullptr, *d_pb0 = nullptr;   // [count] block height, first partial
-    int2 *d_items = nullptr;             // compacted (member, block) list of the pair members
-    double *d_pparts = nullptr;          // [4 pair_total] their residual partials
+    PressureArgs *d_pa2 = nullptr;       // [2 count] argument blocks of the multi launches
+    int *d_h2 = nullptr, *d_pb0 = nullptr;   // [count] tile height, first partial
+    int2 *d_items = nullptr;             // compacted (member, tile) list of the multi members
+    double *d_pparts = nullptr;          // [4 multi_total] their residual partials
     cudaGraph_t graph[2] = {};
     cudaGraphExec_t exec[2] = {};
     int gstep = 0;                       // parity of the steps run by the batch
@@ -419,6 +420,63 @@ void *sweep_kernel(bool check, bool write_p)
                  : (write_p ? (void *)kb_sweep<false, true> : (void *)kb_sweep<false, false>);
 }
 
+// Which members sweep several times per launch, and the height of their tiles.  A body of
+// check_every / 4 launches must be an even number to end in buffer A, hence the multiple of 8.
+// Every wall-bounded member takes the four-sweep kernel, the small ones too: their tiles fill the
+// gaps that those of the large ones leave.  One height H for all: a tile costs its H rows and
+// about 12 that fill and drain its pipeline, and a launch lasts as many rounds of resident tiles
+// as there are, so H minimises rounds(H) * (H + 12).
+void plan_multi(lbm2p_batch *b, std::vector<Member> &hm, std::vector<int> &h2, std::vector<int> &pb0)
+{
+    b->quad = b->body % 8 == 0;
+    int tallest = 1;
+    for (int i = 0; i < b->count; ++i) {
+        const lbm2p *h = b->members[(size_t)i];
+        bool walls = true;
+        for (int sd = 0; sd < 4; ++sd)
+            walls = walls && h->p.bc[sd] != LBM2P_BC_PERIODIC;
+        hm[(size_t)i].multi =
+            walls && (b->quad || (h->nnodes >= 512LL * 512 && b->body % 4 == 0)) ? 1 : 0;
+        if (hm[(size_t)i].multi) {
+            ++b->nmulti;
+            tallest = h->ny > tallest ? h->ny : tallest;
+            b->has_fp = b->has_fp || hm[(size_t)i].pa[0].Fp;
+        }
+    }
+    int height = 1;
+    if (b->quad && b->nmulti > 0) {
+        const long long slots = lbm2p_launch::quad_batch_slots();
+        long long best = 0;
+        for (int H = 4; H < tallest + 4; H += 4) {
+            long long n = 0;
+            for (const Member &M : hm)
+                n += M.multi ? lbm2p_launch::quad_tiles(H < M.ny ? H : M.ny, M.nx, M.ny) : 0;
+            const long long cost = (n + slots - 1) / slots * (H + 12);
+            if (best == 0 || cost < best) {
+                best = cost;
+                height = H;
+            }
+        }
+    }
+    for (int i = 0; i < b->count; ++i) {
+        const lbm2p *h = b->members[(size_t)i];
+        Member &M = hm[(size_t)i];
+        if (M.multi) {
+            // k_pair_batch: the height that the handle's tuning chose for the direct-load form
+            M.h2 = b->quad ? height
+                           : ((h->tb.T > 1 && h->tb.kind == 2 && h->tb.W == 120) ? h->tb.H : 4);
+            M.h2 = M.h2 < h->ny ? M.h2 : h->ny;
+            M.nb2 = b->quad ? lbm2p_launch::quad_tiles(M.h2, h->nx, h->ny)
+                            : (int)lbm2p_launch::pair_direct_grid(4, M.h2, h->nx, h->ny);
+            M.pb0 = b->multi_total;
+            b->multi_total += M.nb2;
+        }
+        M.nparts = M.multi ? M.nb2 : M.ntiles;
+        h2[(size_t)i] = M.h2;
+        pb0[(size_t)i] = M.pb0;
+    }
+}
+
 // the graph of one batched step at step parity q (the g buffers swap every step):
 // refresh -> reset -> prefix -> scatter -> WHILE{ body sweeps -> finalize -> condition +
 // prefix -> scatter -> IF{ mid-solve rebase } } -> saturation -> rebase
@@ -436,7 +494,6 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
     const double *tols = b->d_tols;
     int *act = b->d_active;
     double *partials = b->d_partials;
-    const double *cpartials = b->d_partials;
     int *prefix = b->d_prefix;
     const int *cprefix = b->d_prefix;
     int2 *actl = b->d_act;
@@ -472,34 +529,43 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
     cp.conditional.size = 1;
     BTRY(b, cudaGraphAddNode(&nw, G, &nsc, nullptr, 1, &cp));
     cudaGraph_t bg = cp.conditional.phGraph_out[0];
-    cudaGraphNode_t prev = nullptr;
-    for (int kk = 0; kk < body; ++kk) {
-        const bool check = kk == body - 1, write_p = kk == body - 2;
-        int idx = kk;
-        void *args[] = {(void *)&mem, (void *)&cactl, (void *)&cact, (void *)&idx,
-                        (void *)&partials};
-        cudaGraphNode_t n;
-        BTRY(b, add_k(&n, bg, prev ? &prev : nullptr, sweep_kernel(check, write_p),
-                      check ? b->grid_check : b->grid, kBlock, args));
-        prev = n;
-    }
-    // the pair members: check_every / 2 launches of k_pair_batch (two sweeps each, over the
-    // blocks of every pair member still iterating), a chain beside the one-sweep chain
-    std::vector<cudaGraphNode_t> ends{prev};
-    if (b->npair > 0) {
-        cudaGraphNode_t p2 = nullptr;
-        for (int kk = 0; kk < body / 2; ++kk) {
+    // the one-sweep members: check_every launches; the multi members: check_every / 4 (or / 2)
+    // launches over the tiles of every one still iterating, a chain beside the first
+    std::vector<cudaGraphNode_t> ends;
+    if (b->nmulti < count) {
+        cudaGraphNode_t prev = nullptr;
+        for (int kk = 0; kk < body; ++kk) {
+            const bool check = kk == body - 1, write_p = kk == body - 2;
+            int idx = kk;
+            void *args[] = {(void *)&mem, (void *)&cactl, (void *)&cact, (void *)&idx,
+                            (void *)&partials};
             cudaGraphNode_t n;
-            BTRY(b, lbm2p_launch::node_pair_batch(&n, bg, p2 ? &p2 : nullptr, b->d_pa2, b->d_h2,
-                                                  b->d_pb0, b->d_items, b->d_active + 3, kk & 1,
-                                                  kk == body / 2 - 1, b->d_pparts, b->pair_grid));
+            BTRY(b, add_k(&n, bg, prev ? &prev : nullptr, sweep_kernel(check, write_p),
+                          check ? b->grid_check : b->grid, kBlock, args));
+            prev = n;
+        }
+        ends.push_back(prev);
+    }
+    if (b->nmulti > 0) {
+        cudaGraphNode_t p2 = nullptr;
+        const int launches = body / (b->quad ? 4 : 2);
+        for (int kk = 0; kk < launches; ++kk) {
+            const bool check = kk == launches - 1;
+            const cudaGraphNode_t *dep = p2 ? &p2 : nullptr;
+            cudaGraphNode_t n;
+            BTRY(b, b->quad ? lbm2p_launch::node_quad_batch(&n, bg, dep, b->d_pa2, b->d_h2, b->d_pb0,
+                                                            b->d_items, b->d_active + 3, kk & 1, check,
+                                                            b->d_pparts, b->multi_total, b->has_fp)
+                            : lbm2p_launch::node_pair_batch(&n, bg, dep, b->d_pa2, b->d_h2, b->d_pb0,
+                                                            b->d_items, b->d_active + 3, kk & 1, check,
+                                                            b->d_pparts, b->pair_grid));
             p2 = n;
         }
         ends.push_back(p2);
     }
     cudaGraphNode_t nf, nc, nsc2, nif, nrm;
     {
-        void *args[] = {(void *)&mem, (void *)&cpartials, (void *)&ctl, (void *)&body, (void *)&act};
+        void *args[] = {(void *)&mem, (void *)&ctl, (void *)&body, (void *)&act};
         cudaKernelNodeParams kp{};
         kp.func = (void *)kb_finalize;
         kp.gridDim = dim3((unsigned)count);
@@ -622,34 +688,15 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
         M.ntiles = M.seg_x * ((h->ny + M.rpt - 1) / M.rpt);
         total += M.ntiles;
         tile_member.insert(tile_member.end(), (size_t)M.ntiles, i);
-        // members of 512^2 nodes and more with walls on every side sweep two at a time
-        // (k_pair_batch; a body of check_every sweeps is then check_every / 2 launches, an
-        // even number, ending in buffer A), in blocks of the height their handle's tuning
-        // chose for the direct-load form, else 4 rows
-        bool walls = true;
-        for (int sd = 0; sd < 4; ++sd)
-            walls = walls && h->p.bc[sd] != LBM2P_BC_PERIODIC;
-        M.pair = (!h->fp16 && walls && h->nnodes >= 512LL * 512 && b->body % 4 == 0) ? 1 : 0;
-        M.h2 = M.nb2 = M.pb0 = 0;
-        if (M.pair) {
-            M.h2 = (h->tb.T > 1 && h->tb.kind == 2 && h->tb.W == 120) ? h->tb.H : 4;
-            M.h2 = M.h2 < h->ny ? M.h2 : h->ny;
-            M.nb2 = (int)lbm2p_launch::pair_direct_grid(4, M.h2, h->nx, h->ny);
-            M.pb0 = b->pair_total;
-            b->pair_total += M.nb2;
-            ++b->npair;
-        }
+        M.multi = M.h2 = M.nb2 = M.pb0 = 0;
         pa2[2 * (size_t)i] = M.pa[0];
         pa2[2 * (size_t)i + 1] = M.pa[1];
-        h2v[(size_t)i] = M.h2;
-        pb0v[(size_t)i] = M.pb0;
-        M.pparts = nullptr;                    // set once the partials are allocated
-        M.nparts = M.pair ? M.nb2 : M.ntiles;
         b->pf.push_back(h->cur_f);
         b->pg0.push_back(h->cur_g);
         b->pr.push_back(h->cur_r);
     }
     b->total = total;
+    plan_multi(b, hm, h2v, pb0v);
     int dev = 0, sms = 0, per = 0, perc = 0;
     lbm2p_status st = LBM2P_OK;
     auto ok = [&](cudaError_t e, const char *what) {
@@ -663,14 +710,15 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
         ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kb_sweep<false, true>, kBlock, 0),
            "cudaOccupancyMaxActiveBlocksPerMultiprocessor") &&
         ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&perc, kb_sweep<true, false>, kBlock, 0),
-           "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
+           "cudaOccupancyMaxActiveBlocksPerMultiprocessor") &&
+        ok(lbm2p_launch::quad_prepare(), "cudaFuncSetAttribute");
     if (st == LBM2P_OK) {
         const long long g1 = (long long)sms * (per > 0 ? per : 1);
         const long long g2 = (long long)sms * (perc > 0 ? perc : 1);
         b->grid = (int)(g1 < total ? g1 : total);
         b->grid_check = (int)(g2 < total ? g2 : total);
         const long long g3 = (long long)sms * lbm2p_launch::pair_batch_blocks_per_sm();
-        b->pair_grid = (int)(g3 < b->pair_total ? g3 : (b->pair_total > 0 ? b->pair_total : 1));
+        b->pair_grid = (int)(g3 < b->multi_total ? g3 : (b->multi_total > 0 ? b->multi_total : 1));
         ok(cudaMalloc(&b->d_mem, sizeof(Member) * (size_t)count), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_tile_member, sizeof(int) * (size_t)total), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_ctl, sizeof(MemberCtl) * (size_t)count), "cudaMalloc") &&
@@ -683,10 +731,10 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
             ok(cudaMalloc(&b->d_pa2, sizeof(PressureArgs) * 2 * (size_t)count), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_h2, sizeof(int) * (size_t)count), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_pb0, sizeof(int) * (size_t)count), "cudaMalloc") &&
-            ok(cudaMalloc(&b->d_items, sizeof(int2) * (size_t)(b->pair_total > 0 ? b->pair_total : 1)),
+            ok(cudaMalloc(&b->d_items, sizeof(int2) * (size_t)(b->multi_total > 0 ? b->multi_total : 1)),
                "cudaMalloc") &&
             ok(cudaMalloc(&b->d_pparts,
-                          sizeof(double) * 4 * (size_t)(b->pair_total > 0 ? b->pair_total : 1)),
+                          sizeof(double) * 4 * (size_t)(b->multi_total > 0 ? b->multi_total : 1)),
                "cudaMalloc") &&
             ok(cudaMallocHost(&b->h_ctl, sizeof(MemberCtl) * (size_t)count), "cudaMallocHost") &&
             ok(cudaMallocHost(&b->h_caps, sizeof(int) * (size_t)count), "cudaMallocHost") &&
@@ -695,11 +743,10 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
             ok(cudaEventCreate(&b->ev1), "cudaEventCreate");
     }
     if (st == LBM2P_OK) {
-        // residual partials: one per tile of each one-sweep member, one per block of each
-        // pair member
+        // residual partials: one per tile of each member
         for (int i = 0; i < count; ++i) {
             Member &M = hm[(size_t)i];
-            M.pparts = M.pair ? b->d_pparts + 4 * (size_t)M.pb0 : b->d_partials + 4 * (size_t)M.tile0;
+            M.pparts = M.multi ? b->d_pparts + 4 * (size_t)M.pb0 : b->d_partials + 4 * (size_t)M.tile0;
         }
         cudaStream_t cs = (cudaStream_t)b->stream;
         ok(cudaMemcpyAsync(b->d_mem, hm.data(), sizeof(Member) * (size_t)count,
@@ -800,9 +847,11 @@ lbm2p_status lbm2p_batch_step(lbm2p_batch *b, int nsteps, const int *replay,
         // finalize, condition + prefix, scatter; and the mid-solve rebases of the longest solve
         const int passes = kmax > 0 ? kmax / b->body : 1;
         const int every = b->body * ((1024 + b->body - 1) / b->body);
-        b->launches += 6 + (long long)passes * (b->body + 3) + (kmax > 0 ? (kmax - 1) / every : 0);
-        if (b->npair > 0)                      // the pair members' body / 2 launches a pass
-            b->launches += (long long)passes * (b->body / 2);
+        b->launches += 6 + (long long)passes * 3 + (kmax > 0 ? (kmax - 1) / every : 0);
+        if (b->nmulti < b->count)
+            b->launches += (long long)passes * b->body;
+        if (b->nmulti > 0)
+            b->launches += (long long)passes * (b->body / (b->quad ? 4 : 2));
         if (worst == LBM2P_ENONFINITE)
             return bfail(b, worst, "a member's pressure residual is not finite (step %d)", s);
     }

@@ -315,6 +315,15 @@ cudaError_t quad_prepare();
 void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream);
 cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                const PressureArgs &a, bool check, int H, int grid);
+// the same over several lattices: item t (t < *nitems <= grid) is tile items[t].y (of H[m] rows) of
+// member m = items[t].x, with argument block pa[2 m + parity]; residual sums of member m to
+// parts[4 (pb0[m] + tile) ..]
+int quad_tiles(int H, int nx, int ny);
+int quad_batch_slots();                       // tiles resident on the device at once
+cudaError_t node_quad_batch(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
+                            const PressureArgs *pa, const int *H, const int *pb0,
+                            const int2 *items, const int *nitems, int parity, bool check,
+                            double *parts, int grid, bool has_fp);
 // a whole sub-iteration by one cluster of C blocks (resident.cu)
 bool resident_fits(int C, int nx, int ny);
 cudaError_t pressure_resident(const PressureArgs &a, const ResidentArgs &s, int C, void *stream);

@@ -70,6 +70,45 @@ __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
     }
 }
 
+// Four sweeps over several lattices in one launch (members of a batch): block t runs the tile
+// items[t] = (member m, tile of H[m] rows) with the argument block pa[2 m + parity]; CHECK: its
+// residual sums go to parts[4 (pb0[m] + tile) ..].  The grid covers the items of every member and
+// the blocks beyond *nitems leave at once, so the hardware balances tiles of different cost.  The
+// argument block is read from shared memory: from global memory the compiler keeps it in registers
+// and the tile spills.
+template <bool CHECK, int S>
+__global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
+    k_quad_batch(const PressureArgs *__restrict__ pa, const int *__restrict__ H,
+                 const int *__restrict__ pb0, const int2 *__restrict__ items,
+                 const int *__restrict__ nitems, int parity, double *__restrict__ parts)
+{
+    extern __shared__ __align__(128) float smem_raw[];
+    __shared__ PressureArgs a;
+    static_assert(kQuadWarps == 1, "an item per block");
+    if ((int)blockIdx.x >= *nitems)
+        return;
+    const int lane = threadIdx.x & 31;
+    const int2 e = items[blockIdx.x];
+    const unsigned *src = reinterpret_cast<const unsigned *>(pa + 2 * e.x + parity);
+    for (int i = lane; i < (int)(sizeof(PressureArgs) / 4); i += 32)
+        reinterpret_cast<unsigned *>(&a)[i] = src[i];
+    __syncwarp();
+    ResAcc racc;
+    quad_tile<CHECK, S>(a, H[e.x], e.y, smem_raw, lane, racc);
+    if (CHECK) {
+        double v[4];
+        racc.warp_totals(v);
+        if (lane == 0)
+            for (int c = 0; c < 4; ++c)
+                parts[4 * ((size_t)pb0[e.x] + e.y) + c] = v[c];
+    }
+}
+
+void *quad_batch_func(bool check)
+{
+    return check ? (void *)k_quad_batch<true, kQuadSlots> : (void *)k_quad_batch<false, kQuadSlots>;
+}
+
 void *quad_func(bool check)
 {
     return check ? (void *)k_pressure_quad<true, kQuadSlots> : (void *)k_pressure_quad<false, kQuadSlots>;
@@ -109,12 +148,13 @@ int quad_tile_slots(bool has_fp)
 
 cudaError_t quad_prepare()
 {
-    for (bool c : {false, true}) {
-        cudaError_t e = cudaFuncSetAttribute(quad_func(c), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)quad_smem_bytes(true));
-        if (e != cudaSuccess)
-            return e;
-    }
+    for (bool c : {false, true})
+        for (void *f : {quad_func(c), quad_batch_func(c)}) {
+            cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)quad_smem_bytes(true));
+            if (e != cudaSuccess)
+                return e;
+        }
     return cudaSuccess;
 }
 
@@ -134,6 +174,37 @@ cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGrap
     prm.blockDim = dim3(kQuadThreads);
     prm.sharedMemBytes = (unsigned)quad_smem_bytes(a.Fp != nullptr);
     void *args[] = {(void *)&a, (void *)&H};
+    prm.kernelParams = args;
+    prm.extra = nullptr;
+    return cudaGraphAddKernelNode(n, g, dep, dep ? 1 : 0, &prm);
+}
+
+int quad_batch_slots()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return kQuadBlocks;
+    return sms * kQuadBlocks;
+}
+
+int quad_tiles(int H, int nx, int ny)
+{
+    return quad_strips(nx) * ((ny + H - 1) / H);
+}
+
+cudaError_t node_quad_batch(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
+                            const PressureArgs *pa, const int *H, const int *pb0,
+                            const int2 *items, const int *nitems, int parity, bool check,
+                            double *parts, int grid, bool has_fp)
+{
+    cudaKernelNodeParams prm{};
+    prm.func = quad_batch_func(check);
+    prm.gridDim = dim3((unsigned)grid);
+    prm.blockDim = dim3(kQuadThreads);
+    prm.sharedMemBytes = (unsigned)quad_smem_bytes(has_fp);
+    void *args[] = {(void *)&pa, (void *)&H, (void *)&pb0, (void *)&items, (void *)&nitems,
+                    (void *)&parity, (void *)&parts};
     prm.kernelParams = args;
     prm.extra = nullptr;
     return cudaGraphAddKernelNode(n, g, dep, dep ? 1 : 0, &prm);

@@ -81,6 +81,11 @@ template <bool CHECK, bool FQ, int GEN, int S>
 struct Quad {
     const PressureArgs &a;
     const int lane;
+    // planes, kept here: a batched launch has its argument blocks in global memory
+    const float *fin, *R, *itau;
+    float *fout;
+    long long ps;                             // floats from plane to plane
+    int pitch;
     // ---- ring ----
     float *ring;
     int slot_floats;
@@ -128,19 +133,18 @@ struct Quad {
             const bool odd = lane >= 16;
             m >>= odd ? 1 : 0;
             const unsigned d = dst + (unsigned)(slot * slot_floats) * 4u;
-            const long long ps2 = 2 * (a.fin[1] - a.fin[0]);
-            const float *f = (odd ? a.fin[1] : a.fin[0]) + off;
+            const float *f = fin + (odd ? ps : 0) + off;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (m & (1u << (2 * j)))
-                    cp_async_16(d + (unsigned)(2 * j * kQuadCols) * 4u, f + j * ps2);
+                    cp_async_16(d + (unsigned)(2 * j * kQuadCols) * 4u, f + 2 * j * ps);
             if (m & (1u << 8))
-                cp_async_16(d + (unsigned)(8 * kQuadCols) * 4u, (odd ? a.inv_tau : a.R) + off);
+                cp_async_16(d + (unsigned)(8 * kQuadCols) * 4u, (odd ? itau : R) + off);
             if (FQ && a.Fp && !odd)
                 cp_async_16(d + (unsigned)(10 * kQuadCols) * 4u, a.Fp + off);
         }
         cp_async_commit();
-        off += a.g.pitch;
+        off += pitch;
     }
 
     // input row t (the next one) is in place; PENDING: copies of later rows that may be in flight
@@ -400,14 +404,14 @@ struct Quad {
                 if (owner0)
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        *reinterpret_cast<float2 *>(a.fout[i] + o) = w[i];
+                        *reinterpret_cast<float2 *>(fout + i * ps + o) = w[i];
             } else if (rowin) {
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     if (owner0)
-                        a.fout[i][o] = w[i].x;
+                        fout[i * ps + o] = w[i].x;
                     if (owner1)
-                        a.fout[i][o + 1] = w[i].y;
+                        fout[i * ps + o + 1] = w[i].y;
                 }
             }
             if (CHECK) {
@@ -417,7 +421,7 @@ struct Quad {
                     racc.add((dP.y - pd.y) - dshift, (rg[s].v.y - shift) + dP.y);
                 pd = dPp;
             }
-            o += a.g.pitch;
+            o += pitch;
         }
     }
 
@@ -425,6 +429,12 @@ struct Quad {
     __device__ __forceinline__ void tile(int x0, int y0, int y1, float *smem, int wlo_, int whi_)
     {
         const Geom &g = a.g;
+        fin = a.fin[0];
+        fout = a.fout[0];
+        ps = a.fin[1] - a.fin[0];
+        R = a.R;
+        itau = a.inv_tau;
+        pitch = g.pitch;
         ring = smem;
         slot_floats = (a.Fp ? 11 : 10) * kQuadCols;
         const int xs = x0 - kQuadHalo;                 // column of lane 0

@@ -315,3 +315,30 @@ def test_batch_against_oracle_with_a_1024_member():
                "ux": W.rel_l2(ux, ref["ux"]), "uy": W.rel_l2(uy, ref["uy"])}
         o.close()
         assert all(v <= 1e-5 for v in err.values()), (p.nx, err)
+
+
+@pytest.mark.parametrize("every, sizes", [
+    (4, [(512, 512), (48, 40)]),                        # two sweeps per launch, and one
+    (16, [(9, 4), (1, 60), (56, 3), (57, 33), (400, 113)]),     # four: single and ragged tiles
+    (24, [(113, 112), (60, 700)]),
+])
+def test_sweeps_per_launch_bit_identical(every, sizes):
+    """The launch forms that check_every selects (a multiple of 8: four sweeps per launch; of 4:
+    two from 512^2 nodes) against the same handles stepped alone, replayed."""
+    pkg = _pkg()
+    rng = np.random.default_rng(5)
+    probs = [uniform(nx, ny, bc=(W.NOFLUX,) * 4, K=np.exp(rng.standard_normal((ny, nx))), S0=0.3,
+                     wells=[(0, 0, 2e-3, 0), (nx - 1, ny - 1, 2e-3, 1)],
+                     tau_mode=W.TAU_PHYSICAL_DT) for nx, ny in sizes]
+    make = lambda p: pkg.Solver.from_problem(p, check_every=every, max_sub_iters=100 * every,
+                                             init_replay=32)
+    alone = [make(p) for p in probs]
+    inb = [make(p) for p in probs]
+    counts = [every * (1 + i % 3) for i in range(len(probs))]
+    with pkg.Batch(inb) as batch:
+        for _ in range(2):
+            for s, c in zip(alone, counts):
+                s.step(1, replay=[c])
+            batch.step(1, replay=counts)
+        for a, b in zip(alone, inb):
+            assert np.array_equal(a.get_state(), b.get_state())

@@ -309,7 +309,6 @@ cudaError_t node_pressure_pair_direct(cudaGraphNode_t *n, cudaGraph_t g, const c
 // four sweeps per launch (sweep_quad.cu), lattices without periodic sides: tiles of 56 columns by H
 // rows, one warp each, four to a block; grid = quad_grid(...)
 long long quad_grid(int H, int nx, int ny);
-int quad_strips_of(int nx);
 int quad_tile_slots(bool has_fp);      // tiles that run at a time (0: the kernel cannot run)
 cudaError_t quad_prepare();
 void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream);

@@ -1261,19 +1261,20 @@ lbm2p_status autotune_sweeps(lbm2p *h)
             }
         }
         // four sweeps per launch (lattices with walls on every side), when a check period is an
-        // even number of launches: rows per tile giving 1 to 12 rounds of resident tiles
+        // even number of launches: rows per tile giving a quarter to 12 rounds of resident tiles
         if (walls &&
             (h->p.fuse_sweeps == 4 || (h->p.fuse_sweeps == 0 && m_chk % 8 == 0)) &&
             lbm2p_launch::quad_prepare() == cudaSuccess) {
             const int slots = lbm2p_launch::quad_tile_slots(h->Fp != nullptr);
-            const int strips = (int)lbm2p_launch::quad_strips_of(h->nx);
             int last_H = -1;
-            for (int rounds : {1, 2, 3, 4, 5, 6, 8, 12}) {
+            for (int quarters : {1, 2, 4, 8, 12, 16, 20, 24, 32, 48}) {
                 if (slots < 1)
                     break;
-                const long long chunks = (long long)slots * rounds / strips;
-                int H = chunks > 0 ? (int)((h->ny + chunks - 1) / chunks) : 128;
-                H = H < 4 ? 4 : (H > 128 ? 128 : H);
+                // the lowest height whose tiles fit that many quarters of a round
+                int H = 2;
+                while (H < 128 &&
+                       lbm2p_launch::quad_grid(H, h->nx, h->ny) > (long long)slots * quarters / 4)
+                    ++H;
                 H = H < h->ny ? H : h->ny;
                 if (H == last_H)
                     continue;

@@ -26,9 +26,9 @@
 // interior tile took 60k).
 // The per-node operations and their order are those of the single sweep (dev1, pressure_of,
 // collide1), so four sweeps equal four launches of one bit for bit.
-// Per sweep, two-sweep launches before and this kernel now: 4096^2 129.5 and 57 us (229 us per
-// launch, 1.24 times the time that its 1208 MB take at the copy bandwidth), 1024^2 14.0 and
-// 7.7 us, 512^2 7.5 and 4.1 us.
+// Per sweep, two-sweep launches before and this kernel now: 4096^2 129.5 and 54.5 us (218 us per
+// launch, 1.18 times the time that its 1208 MB take at the copy bandwidth), 1024^2 14.0 and
+// 5.5 us, 512^2 7.5 and 3.3 us.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -49,10 +49,9 @@ __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
     __shared__ double red[kQuadWarps][4];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float *smem = quad_warp_smem<S>(smem_raw, warp, a.Fp != nullptr);
-    const int strips = quad_strips(a.g.nx);
     const int tile = blockIdx.x * kQuadWarps + warp;
     ResAcc racc;
-    if (tile < strips * ((a.g.ny + H - 1) / H))
+    if (tile < QuadPlan(H, a.g.nx, a.g.ny).tiles())
         quad_tile<CHECK, S>(a, H, tile, smem, lane, racc);
     if (CHECK) {
         double v[4];
@@ -124,11 +123,9 @@ using namespace lbm2p_dev;
 
 long long quad_grid(int H, int nx, int ny)
 {
-    const long long tiles = (long long)quad_strips(nx) * ((ny + H - 1) / H);
+    const long long tiles = QuadPlan(H, nx, ny).tiles();
     return (tiles + kQuadWarps - 1) / kQuadWarps;
 }
-
-int quad_strips_of(int nx) { return quad_strips(nx); }
 
 int quad_tile_slots(bool has_fp)
 {
@@ -190,7 +187,7 @@ int quad_batch_slots()
 
 int quad_tiles(int H, int nx, int ny)
 {
-    return quad_strips(nx) * ((ny + H - 1) / H);
+    return (int)QuadPlan(H, nx, ny).tiles();
 }
 
 cudaError_t node_quad_batch(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,

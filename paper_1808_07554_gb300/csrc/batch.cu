@@ -21,6 +21,7 @@
 #include "lbm2p_device.cuh"
 #include "lbm2p_handle.h"
 #include "lbm2p_node.cuh"
+#include "residual.cuh"
 
 using namespace lbm2p_dev;
 
@@ -148,46 +149,15 @@ __global__ void __launch_bounds__(kBlock) kb_sweep(const Member *__restrict__ me
 // the arithmetic of the single-lattice finalize), then retire it or keep it active, and
 // mark it for a mid-solve rebase on the rule of the single-lattice loop.  counts[0] counts
 // the members still active, counts[1] those to rebase.
-__global__ void __launch_bounds__(256) kb_finalize(const Member *__restrict__ mem,
-                                                   MemberCtl *ctl, int body, int *counts)
+__global__ void __launch_bounds__(kFinThreads) kb_finalize(const Member *__restrict__ mem,
+                                                           MemberCtl *ctl, int body, int *counts)
 {
-    const int mi = blockIdx.x;
-    MemberCtl &c = ctl[mi];
+    MemberCtl &c = ctl[blockIdx.x];
     if (!c.active)
         return;                                         // uniform over the block
-    const Member &M = mem[mi];
-    __shared__ double red[256][4];
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < M.nparts; i += 256)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            s[q] += M.pparts[4 * (size_t)i + q];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        red[threadIdx.x][q] = s[q];
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                red[threadIdx.x][q] += red[threadIdx.x + h][q];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double N = (double)M.nnodes;
-        const double sd = red[0][0], sdd = red[0][1], sp = red[0][2], spp = red[0][3];
-        const double c0 = (double)M.shift[0], c1 = (double)M.shift[1];
-        double r;
-        if (!isfinite(sd) || !isfinite(sdd) || !isfinite(sp) || !isfinite(spp)) {
-            r = nan("");
-        } else {
-            double num = sdd - sd * sd / N, den = spp - sp * sp / N;
-            num = num > 0.0 ? num : 0.0;
-            den = den > 0.0 ? den : 0.0;
-            r = den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0);
-            M.shift[0] = (float)(c0 + sp / N);
-            M.shift[1] = (float)(c1 + sd / N);
-        }
+    const Member &M = mem[blockIdx.x];
+    double r;
+    if (finalize_residual<1>(M.pparts, M.nparts, M.nnodes, M.shift, nullptr, r) && threadIdx.x == 0) {
         c.k += body;
         c.r = r;
         const bool more = !(r <= c.tol) && !isnan(r) && c.k < c.cap;
@@ -569,7 +539,7 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
         cudaKernelNodeParams kp{};
         kp.func = (void *)kb_finalize;
         kp.gridDim = dim3((unsigned)count);
-        kp.blockDim = dim3(256u);
+        kp.blockDim = dim3((unsigned)kFinThreads);
         kp.kernelParams = args;
         BTRY(b, cudaGraphAddKernelNode(&nf, bg, ends.data(), ends.size(), &kp));
     }

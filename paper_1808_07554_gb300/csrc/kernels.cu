@@ -16,6 +16,7 @@
 
 #include "lbm2p_device.cuh"
 #include "lbm2p_node.cuh"
+#include "residual.cuh"
 
 namespace lbm2p_dev {
 
@@ -529,71 +530,23 @@ __global__ void __launch_bounds__(kBlock) k_pressure_scalar(const __grid_constan
     }
 }
 
-// r = ||dP - mean dP|| / ||P - mean P|| from the block partials (FP64, fixed order).
-// Called by all 256 threads of one block; returns r in thread 0.
-__device__ double finalize_residual(const double *__restrict__ partials, int nparts,
-                                    long long nnodes, float *shift, ResidualOut *out)
+__global__ void __cluster_dims__(kFinBlocks, 1, 1) __launch_bounds__(kFinThreads)
+    k_residual_finalize(const double *__restrict__ partials, int nparts, long long nnodes,
+                        float *shift, ResidualOut *out)
 {
-    __shared__ double red[256][4];
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nparts; i += 256)
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            s[c] += partials[4 * i + c];
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        red[threadIdx.x][c] = s[c];
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h)
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-                red[threadIdx.x][c] += red[threadIdx.x + h][c];
-        __syncthreads();
-    }
-    double r = 0.0;
-    if (threadIdx.x == 0) {
-        const double N = (double)nnodes;
-        const double sd = red[0][0], sdd = red[0][1], sp = red[0][2], spp = red[0][3];
-        const double c = (double)shift[0], cd = (double)shift[1];
-        if (!isfinite(sd) || !isfinite(sdd) || !isfinite(sp) || !isfinite(spp)) {
-            r = nan("");
-        } else {
-            // sums of (dP - dP_prev - cd) and (P - c): variances are shift invariant
-            double num = sdd - sd * sd / N;
-            double den = spp - sp * sp / N;
-            num = num > 0.0 ? num : 0.0;
-            den = den > 0.0 ? den : 0.0;
-            r = den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0);
-            shift[0] = (float)(c + sp / N);
-            shift[1] = (float)(cd + sd / N);
-        }
-        out->r = r;
-        out->mean_P = c + sp / N;
-        out->sums[0] = sd;
-        out->sums[1] = sdd;
-        out->sums[2] = sp;
-        out->sums[3] = spp;
-    }
-    return r;
-}
-
-__global__ void __launch_bounds__(256) k_residual_finalize(const double *__restrict__ partials,
-                                                           int nparts, long long nnodes,
-                                                           float *shift, ResidualOut *out)
-{
-    finalize_residual(partials, nparts, nnodes, shift, out);
+    double r;
+    finalize_residual<kFinBlocks>(partials, nparts, nnodes, shift, out, r);
 }
 
 // Finalize inside the graph-resident loop: count the body's sweeps and keep looping while
 // r > tol, r is a number, and the cap is not reached.
-__global__ void __launch_bounds__(256) k_residual_finalize_loop(
-    const double *__restrict__ partials, int nparts, long long nnodes, float *shift,
-    ResidualOut *out, LoopCtl *ctl, cudaGraphConditionalHandle handle,
-    cudaGraphConditionalHandle h_rebase)
+__global__ void __cluster_dims__(kFinBlocks, 1, 1) __launch_bounds__(kFinThreads)
+    k_residual_finalize_loop(const double *__restrict__ partials, int nparts, long long nnodes,
+                             float *shift, ResidualOut *out, LoopCtl *ctl,
+                             cudaGraphConditionalHandle handle, cudaGraphConditionalHandle h_rebase)
 {
-    const double r = finalize_residual(partials, nparts, nnodes, shift, out);
-    if (threadIdx.x == 0) {
+    double r;
+    if (finalize_residual<kFinBlocks>(partials, nparts, nnodes, shift, out, r) && threadIdx.x == 0) {
         const int k = ctl->k + ctl->m;
         ctl->k = k;
         ctl->r = r;
@@ -963,7 +916,7 @@ void pressure_sweeps_fused(const PressureArgs &a, int T, int W, int H, bool chec
 void residual_finalize(const double *partials, int nparts, long long nnodes, float *shift,
                        ResidualOut *out, void *stream)
 {
-    k_residual_finalize<<<1, 256, 0, S(stream)>>>(partials, nparts, nnodes, shift, out);
+    k_residual_finalize<<<kFinBlocks, kFinThreads, 0, S(stream)>>>(partials, nparts, nnodes, shift, out);
 }
 
 void refresh(const RefreshArgs &a, int grid, void *stream)
@@ -1058,7 +1011,7 @@ cudaError_t node_finalize_loop(cudaGraphNode_t *n, cudaGraph_t g, const cudaGrap
 {
     void *args[] = {(void *)&partials, (void *)&nparts, (void *)&nnodes, (void *)&shift,
                     (void *)&out, (void *)&ctl, (void *)&h, (void *)&h_rebase};
-    return add_kernel(n, g, dep, (void *)k_residual_finalize_loop, 1, 256, args);
+    return add_kernel(n, g, dep, (void *)k_residual_finalize_loop, kFinBlocks, kFinThreads, args);
 }
 
 cudaError_t node_rebase_mid(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,

@@ -37,6 +37,7 @@
 #include "lbm2p_async.cuh"
 #include "lbm2p_device.cuh"
 #include "lbm2p_node.cuh"
+#include "residual.cuh"
 
 namespace lbm2p_dev {
 namespace {
@@ -48,34 +49,6 @@ struct ResidentShape {
     int C, h, cells, edges, npt, threads;
     size_t smem;
 };
-
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ unsigned cluster_size()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                     : "memory");
-}
-
-// the address of this block's shared address `a` in block `rank` of the cluster
-__device__ __forceinline__ unsigned cluster_addr(unsigned a, unsigned rank)
-{
-    unsigned r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    return r;
-}
 
 __device__ __forceinline__ void cluster_store(unsigned a, float v)
 {

@@ -101,3 +101,27 @@ def test_noalloc_rejects_lattices_beyond_its_scratch(env):
     assert ei.value.status == pkg.EINVAL
     assert "row tiles" in str(ei.value)
     torch.cuda.synchronize()                        # nothing was queued, nothing failed
+
+
+@pytest.mark.parametrize("nx, ny", [(5, 1), (9, 63), (9, 64), (40, 65), (12, 511), (12, 513), (2100, 700)])
+def test_residual_reduction_sizes(env, nx, ny):
+    """The residual of one sweep against the FP64 residual of the same planes, for counts of
+    partial sums around those that one block, one cluster and one round of loads of the reduction
+    take.  The sweep adds a warp's differences in FP32 (at most 128 terms each: 128 * 2^-24 of the
+    sums), so r agrees to 1e-5."""
+    torch, pkg = env
+    gen = torch.Generator(device="cuda").manual_seed(nx * 1000 + ny)
+    pitch = (nx + 31) // 32 * 32
+    rand = lambda *s: torch.rand(*s, generator=gen, device="cuda", dtype=torch.float32)  # noqa: E731
+    n_in = 1e-2 * (rand(8, ny, pitch) - 0.5)
+    n_out = torch.zeros_like(n_in)
+    R, inv_tau, dP = 1.0 + rand(ny, pitch), 0.6 + rand(ny, pitch), 1e-2 * rand(ny, pitch)
+    prev = dP.clone()
+    r = pkg.lbm2p_pressure_sweep_noalloc(
+        nx, ny, pitch, (1, 1, 1, 1), [n_in[i].data_ptr() for i in range(8)],
+        [n_out[i].data_ptr() for i in range(8)], R.data_ptr(), inv_tau.data_ptr(), 0, None,
+        dP.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    d = (dP.double() - prev.double())[:, :nx]
+    P = (R.double() + dP.double())[:, :nx]
+    want = ((d - d.mean()).norm() / (P - P.mean()).norm()).item()
+    assert r == pytest.approx(want, rel=1e-5)

@@ -22,25 +22,24 @@
 #include "lbm2p_handle.h"
 #include "lbm2p_node.cuh"
 #include "residual.cuh"
+#include "step_node.cuh"
 
 using namespace lbm2p_dev;
 
 namespace {
 
-// Device descriptor of one member: its kernel argument blocks for both f source parities
-// and both step parities, and where its tiles sit in the batch tile list.  A tile is kBlock
+// Device descriptor of one member: its kernel argument blocks for both step parities (and both f
+// source parities of a sweep), and where its tiles sit in the batch tile list.  A tile is kBlock
 // nodes: rpt rows of a (1 << wshift)-wide row segment, so lattices narrower than kBlock
 // still fill the block.
 struct Member {
-    PressureArgs pa[2];          // sweep from the current f buffer A into B / from B into A
-    RefreshArgs ra[2];           // batch step parity 0 / 1
+    PressureArgs pa[2][2];       // [step parity][f source: the step's first buffer, the other]
+    RefreshArgs ra[2];
     SaturationArgs sa[2];
-    RebaseArgs rb;
-    RebaseMidArgs rm;            // mid-solve rebase of the f buffer holding the state
+    RebaseMidArgs rm[2];         // mid-solve rebase of the f buffer holding the state
     float *shift;                // the handle's residual conditioning constants
     long long nnodes;
     int nx, ny;
-    int pf;                      // which of pa reads the buffer holding the state (0)
     int every;                   // sweeps between mid-solve rebases
     int wshift, rpt, seg_x;      // segment width 2^wshift, rows per tile, segments per row
     int tile0, ntiles;           // range in the batch tile list
@@ -75,16 +74,11 @@ __device__ __forceinline__ bool tile_node(const Member &M, int lt, int &x, int &
     return x < M.nx && y < M.ny;
 }
 
-__global__ void __launch_bounds__(kBlock) kb_refresh(const Member *__restrict__ mem,
-                                                     const int *__restrict__ tile_member,
-                                                     int total, int q)
+__global__ void __launch_bounds__(kStepThreads) kb_refresh(const Member *__restrict__ mem,
+                                                           const int2 *__restrict__ blocks, int q)
 {
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        const Member &M = mem[tile_member[t]];
-        int x, y;
-        if (tile_node(M, t - M.tile0, x, y))
-            refresh_node(M.ra[q], x, y, y * M.ra[q].g.pitch + x);
-    }
+    const int2 e = blocks[blockIdx.x];
+    refresh_block(mem[e.x].ra[q], e.y);
 }
 
 __global__ void kb_reset(MemberCtl *ctl, const int *__restrict__ caps,
@@ -108,7 +102,7 @@ __global__ void kb_reset(MemberCtl *ctl, const int *__restrict__ caps,
 template <bool CHECK, bool WRITE_P>
 __global__ void __launch_bounds__(kBlock) kb_sweep(const Member *__restrict__ mem,
                                                    const int2 *__restrict__ act,
-                                                   const int *__restrict__ counts, int idx,
+                                                   const int *__restrict__ counts, int q, int idx,
                                                    double *__restrict__ partials)
 {
     __shared__ double red[kBlock / 32][4];
@@ -117,15 +111,15 @@ __global__ void __launch_bounds__(kBlock) kb_sweep(const Member *__restrict__ me
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
         const int2 e = act[t];
         const Member &M = mem[e.x];
-        const PressureArgs &a = M.pa[M.pf ^ (idx & 1)];
-        float d = 0.0f, q = 0.0f;
+        const PressureArgs &a = M.pa[q][idx & 1];
+        float d = 0.0f, u = 0.0f;
         int x, y;
         const float shift = CHECK ? M.shift[0] : 0.0f;
         const float dshift = CHECK ? M.shift[1] : 0.0f;
         if (tile_node(M, e.y, x, y))
-            sweep_node<CHECK, WRITE_P>(a, x, y, y * a.g.pitch + x, shift, dshift, d, q);
+            sweep_node<CHECK, WRITE_P>(a, x, y, y * a.g.pitch + x, shift, dshift, d, u);
         if (CHECK) {
-            const float s0 = warp_sum(d), s1 = warp_sum(d * d), s2 = warp_sum(q), s3 = warp_sum(q * q);
+            const float s0 = warp_sum(d), s1 = warp_sum(d * d), s2 = warp_sum(u), s3 = warp_sum(u * u);
             if (lane == 0) {
                 red[warp][0] = s0;
                 red[warp][1] = s1;
@@ -244,7 +238,8 @@ __global__ void __launch_bounds__(256) kb_scatter(const Member *__restrict__ mem
 
 __global__ void __launch_bounds__(kBlock) kb_rebase_mid(const Member *__restrict__ mem,
                                                         const int *__restrict__ tile_member,
-                                                        int total, const MemberCtl *__restrict__ ctl)
+                                                        int total, int q,
+                                                        const MemberCtl *__restrict__ ctl)
 {
     for (int t = blockIdx.x; t < total; t += gridDim.x) {
         const int mi = tile_member[t];
@@ -253,38 +248,22 @@ __global__ void __launch_bounds__(kBlock) kb_rebase_mid(const Member *__restrict
         const Member &M = mem[mi];
         int x, y;
         if (tile_node(M, t - M.tile0, x, y))
-            rebase_mid_node(M.rm, y * M.rm.g.pitch + x);
+            rebase_mid_node(M.rm[q], y * M.rm[q].g.pitch + x);
     }
 }
 
-__global__ void __launch_bounds__(kBlock) kb_saturation(const Member *__restrict__ mem,
-                                                        const int *__restrict__ tile_member,
-                                                        int total, int q)
+__global__ void __launch_bounds__(kStepThreads) kb_saturation(const Member *__restrict__ mem,
+                                                              const int2 *__restrict__ blocks, int q)
 {
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        const Member &M = mem[tile_member[t]];
-        int x, y;
-        if (tile_node(M, t - M.tile0, x, y))
-            saturation_node(M.sa[q], x, y, y * M.sa[q].g.pitch + x);
-    }
-}
-
-__global__ void __launch_bounds__(kBlock) kb_rebase(const Member *__restrict__ mem,
-                                                    const int *__restrict__ tile_member, int total)
-{
-    for (int t = blockIdx.x; t < total; t += gridDim.x) {
-        const Member &M = mem[tile_member[t]];
-        int x, y;
-        if (tile_node(M, t - M.tile0, x, y))
-            rebase_node(M.rb, y * M.rb.g.pitch + x);
-    }
+    const int2 e = blocks[blockIdx.x];
+    saturation_block(mem[e.x].sa[q], e.y);
 }
 
 }  // namespace
 
 struct lbm2p_batch {
     std::vector<lbm2p *> members;
-    std::vector<int> pf, pg0, pr;        // member buffers the graphs were built for
+    std::vector<int> pf, pg0, pr;        // member buffers that the graph of step parity 0 starts from
     int count = 0, total = 0, body = 0, grid = 0, grid_check = 0;
     void *stream = nullptr;
     Member *d_mem = nullptr;
@@ -300,12 +279,14 @@ struct lbm2p_batch {
                                          // [3] tiles of the active multi members
     int *d_prefix = nullptr;             // first compacted tile of each active member
     int2 *d_act = nullptr;               // compacted (member, tile) list
+    int step_blocks = 0;                 // blocks of a refresh or saturation launch
+    int2 *d_step = nullptr;              // their (member, block of the member)
     double *d_partials = nullptr;
     bool quad = false;                   // the multi members sweep four times per launch
     bool has_fp = false;                 // one of them has dense sources
     int nmulti = 0, multi_total = 0;     // multi members, their tiles
     int pair_grid = 0;                   // blocks of a k_pair_batch launch
-    PressureArgs *d_pa2 = nullptr;       // [2 count] argument blocks of the multi launches
+    PressureArgs *d_pa2 = nullptr;       // [2][2 count] argument blocks of the multi launches, by parity
     int *d_h2 = nullptr, *d_pb0 = nullptr;   // [count] tile height, first partial
     int2 *d_items = nullptr;             // compacted (member, tile) list of the multi members
     double *d_pparts = nullptr;          // [4 multi_total] their residual partials
@@ -355,6 +336,7 @@ void batch_free(lbm2p_batch *b)
     cudaFree(b->d_active);
     cudaFree(b->d_prefix);
     cudaFree(b->d_act);
+    cudaFree(b->d_step);
     cudaFree(b->d_pa2);
     cudaFree(b->d_h2);
     cudaFree(b->d_pb0);
@@ -410,7 +392,7 @@ void plan_multi(lbm2p_batch *b, std::vector<Member> &hm, std::vector<int> &h2, s
         if (hm[(size_t)i].multi) {
             ++b->nmulti;
             tallest = h->ny > tallest ? h->ny : tallest;
-            b->has_fp = b->has_fp || hm[(size_t)i].pa[0].Fp;
+            b->has_fp = b->has_fp || hm[(size_t)i].pa[0][0].Fp;
         }
     }
     int height = 1;
@@ -449,7 +431,8 @@ void plan_multi(lbm2p_batch *b, std::vector<Member> &hm, std::vector<int> &h2, s
 
 // the graph of one batched step at step parity q (the g buffers swap every step):
 // refresh -> reset -> prefix -> scatter -> WHILE{ body sweeps -> finalize -> condition +
-// prefix -> scatter -> IF{ mid-solve rebase } } -> saturation -> rebase
+// prefix -> scatter -> IF{ mid-solve rebase } } -> saturation (which moves R too, and leaves the state
+// in the other of the two f buffers)
 lbm2p_status build_graph(lbm2p_batch *b, int q)
 {
     cudaGraph_t G;
@@ -457,6 +440,8 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
     b->graph[q] = G;
     const Member *mem = b->d_mem;
     const int *tm = b->d_tile_member;
+    const int2 *blocks = b->d_step;
+    const PressureArgs *pa2 = b->d_pa2 + (size_t)q * 2 * (size_t)b->count;
     int count = b->count, total = b->total;
     MemberCtl *ctl = b->d_ctl;
     const MemberCtl *cctl = b->d_ctl;
@@ -470,10 +455,10 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
     const int2 *cactl = b->d_act;
     const int *cact = b->d_active;
     int body = b->body;
-    cudaGraphNode_t nr, nreset, npre, nsc, nw, nsat, nreb;
+    cudaGraphNode_t nr, nreset, npre, nsc, nw, nsat;
     {
-        void *args[] = {(void *)&mem, (void *)&tm, (void *)&total, (void *)&q};
-        BTRY(b, add_k(&nr, G, nullptr, (void *)kb_refresh, b->grid, kBlock, args));
+        void *args[] = {(void *)&mem, (void *)&blocks, (void *)&q};
+        BTRY(b, add_k(&nr, G, nullptr, (void *)kb_refresh, b->step_blocks, kStepThreads, args));
     }
     {
         void *args[] = {(void *)&ctl, (void *)&caps, (void *)&tols, (void *)&count, (void *)&act};
@@ -507,8 +492,8 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
         for (int kk = 0; kk < body; ++kk) {
             const bool check = kk == body - 1, write_p = kk == body - 2;
             int idx = kk;
-            void *args[] = {(void *)&mem, (void *)&cactl, (void *)&cact, (void *)&idx,
-                            (void *)&partials};
+            void *args[] = {(void *)&mem, (void *)&cactl, (void *)&cact, (void *)&q,
+                            (void *)&idx, (void *)&partials};
             cudaGraphNode_t n;
             BTRY(b, add_k(&n, bg, prev ? &prev : nullptr, sweep_kernel(check, write_p),
                           check ? b->grid_check : b->grid, kBlock, args));
@@ -523,10 +508,10 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
             const bool check = kk == launches - 1;
             const cudaGraphNode_t *dep = p2 ? &p2 : nullptr;
             cudaGraphNode_t n;
-            BTRY(b, b->quad ? lbm2p_launch::node_quad_batch(&n, bg, dep, b->d_pa2, b->d_h2, b->d_pb0,
+            BTRY(b, b->quad ? lbm2p_launch::node_quad_batch(&n, bg, dep, pa2, b->d_h2, b->d_pb0,
                                                             b->d_items, b->d_active + 3, kk & 1, check,
                                                             b->d_pparts, b->multi_total, b->has_fp)
-                            : lbm2p_launch::node_pair_batch(&n, bg, dep, b->d_pa2, b->d_h2, b->d_pb0,
+                            : lbm2p_launch::node_pair_batch(&n, bg, dep, pa2, b->d_h2, b->d_pb0,
                                                             b->d_items, b->d_active + 3, kk & 1, check,
                                                             b->d_pparts, b->pair_grid));
             p2 = n;
@@ -562,17 +547,13 @@ lbm2p_status build_graph(lbm2p_batch *b, int q)
     ip.conditional.size = 1;
     BTRY(b, cudaGraphAddNode(&nif, bg, &nsc2, nullptr, 1, &ip));
     {
-        void *args[] = {(void *)&mem, (void *)&tm, (void *)&total, (void *)&cctl};
+        void *args[] = {(void *)&mem, (void *)&tm, (void *)&total, (void *)&q, (void *)&cctl};
         BTRY(b, add_k(&nrm, ip.conditional.phGraph_out[0], nullptr, (void *)kb_rebase_mid,
                       b->grid, kBlock, args));
     }
     {
-        void *args[] = {(void *)&mem, (void *)&tm, (void *)&total, (void *)&q};
-        BTRY(b, add_k(&nsat, G, &nw, (void *)kb_saturation, b->grid, kBlock, args));
-    }
-    {
-        void *args[] = {(void *)&mem, (void *)&tm, (void *)&total};
-        BTRY(b, add_k(&nreb, G, &nsat, (void *)kb_rebase, b->grid, kBlock, args));
+        void *args[] = {(void *)&mem, (void *)&blocks, (void *)&q};
+        BTRY(b, add_k(&nsat, G, &nw, (void *)kb_saturation, b->step_blocks, kStepThreads, args));
     }
     BTRY(b, cudaGraphInstantiate(&b->exec[q], G, 0));
     return LBM2P_OK;
@@ -620,32 +601,35 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
     b->body = m0->p.check_every;
     b->stream = m0->stream;
     std::vector<Member> hm((size_t)count);
-    std::vector<PressureArgs> pa2(2 * (size_t)count);
+    std::vector<PressureArgs> pa2(4 * (size_t)count);
+    std::vector<int2> step;
     std::vector<int> h2v((size_t)count), pb0v((size_t)count);
     std::vector<int> tile_member;
     int total = 0;
     for (int i = 0; i < count; ++i) {
         lbm2p *h = members[i];
         Member &M = hm[(size_t)i];
-        // the batch ping-pongs each member between its current f buffer A and the next one
-        // of the rotation, B (a loop body is an even number of sweeps, so a step ends in A),
-        // and updates R, 1/tau_f and P^{n-1} in place
-        const int A = h->cur_f, B = lbm2p_internal::fnext(A, 1);
-        M.pa[0] = lbm2p_internal::pressure_args(h, A, B, false);
-        M.pa[1] = lbm2p_internal::pressure_args(h, B, A, false);
+        // the batch ping-pongs each member between its current f buffer and the next one of the
+        // rotation (a loop body is an even number of sweeps, so a solve ends where it began); the
+        // saturation update writes the state into the other, so the two change places every step,
+        // like the two buffers of g, R, 1/tau_f and P^{n-1}
+        const int f0 = h->cur_f, f1 = lbm2p_internal::fnext(f0, 1), g0 = h->cur_g, r0 = h->cur_r;
         for (int q = 0; q < 2; ++q) {
-            M.pa[q].partials = nullptr;
-            M.ra[q] = lbm2p_internal::refresh_args(h, h->cur_g ^ q, true);
-            M.sa[q] = lbm2p_internal::saturation_args(h, A, h->cur_g ^ q, false);
+            const int A = q ? f1 : f0, B = q ? f0 : f1;
+            h->cur_r = r0 ^ q;
+            M.pa[q][0] = lbm2p_internal::pressure_args(h, A, B, true);
+            M.pa[q][1] = lbm2p_internal::pressure_args(h, B, A, true);
+            M.pa[q][0].partials = M.pa[q][1].partials = nullptr;
+            M.ra[q] = lbm2p_internal::refresh_args(h, g0 ^ q);
+            M.sa[q] = lbm2p_internal::saturation_args(h, A, B, g0 ^ q);
+            M.rm[q] = lbm2p_internal::rebase_mid_args(h, A, true);
         }
-        M.rb = lbm2p_internal::rebase_args(h, A, false);
-        M.rm = lbm2p_internal::rebase_mid_args(h, A, false);
+        h->cur_r = r0;
         M.every = h->rebase_every;
         M.shift = h->shift;
         M.nnodes = h->nnodes;
         M.nx = h->nx;
         M.ny = h->ny;
-        M.pf = 0;                      // pa[0] reads A
         int w = 32;
         while (w < h->nx && w < kBlock)
             w *= 2;
@@ -659,13 +643,18 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
         total += M.ntiles;
         tile_member.insert(tile_member.end(), (size_t)M.ntiles, i);
         M.multi = M.h2 = M.nb2 = M.pb0 = 0;
-        pa2[2 * (size_t)i] = M.pa[0];
-        pa2[2 * (size_t)i + 1] = M.pa[1];
+        for (int q = 0; q < 2; ++q)
+            for (int s = 0; s < 2; ++s)
+                pa2[2 * ((size_t)q * count + i) + s] = M.pa[q][s];
+        const int blocks = StepMap(h->nx, h->ny).blocks();
+        for (int k = 0; k < blocks; ++k)
+            step.push_back(make_int2(i, k));
         b->pf.push_back(h->cur_f);
         b->pg0.push_back(h->cur_g);
         b->pr.push_back(h->cur_r);
     }
     b->total = total;
+    b->step_blocks = (int)step.size();
     plan_multi(b, hm, h2v, pb0v);
     int dev = 0, sms = 0, per = 0, perc = 0;
     lbm2p_status st = LBM2P_OK;
@@ -698,7 +687,8 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
             ok(cudaMalloc(&b->d_prefix, sizeof(int) * (size_t)count), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_act, sizeof(int2) * (size_t)total), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_partials, sizeof(double) * 4 * (size_t)total), "cudaMalloc") &&
-            ok(cudaMalloc(&b->d_pa2, sizeof(PressureArgs) * 2 * (size_t)count), "cudaMalloc") &&
+            ok(cudaMalloc(&b->d_pa2, sizeof(PressureArgs) * 4 * (size_t)count), "cudaMalloc") &&
+            ok(cudaMalloc(&b->d_step, sizeof(int2) * step.size()), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_h2, sizeof(int) * (size_t)count), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_pb0, sizeof(int) * (size_t)count), "cudaMalloc") &&
             ok(cudaMalloc(&b->d_items, sizeof(int2) * (size_t)(b->multi_total > 0 ? b->multi_total : 1)),
@@ -721,7 +711,9 @@ lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int co
         cudaStream_t cs = (cudaStream_t)b->stream;
         ok(cudaMemcpyAsync(b->d_mem, hm.data(), sizeof(Member) * (size_t)count,
                            cudaMemcpyHostToDevice, cs), "cudaMemcpyAsync") &&
-            ok(cudaMemcpyAsync(b->d_pa2, pa2.data(), sizeof(PressureArgs) * 2 * (size_t)count,
+            ok(cudaMemcpyAsync(b->d_pa2, pa2.data(), sizeof(PressureArgs) * 4 * (size_t)count,
+                               cudaMemcpyHostToDevice, cs), "cudaMemcpyAsync") &&
+            ok(cudaMemcpyAsync(b->d_step, step.data(), sizeof(int2) * step.size(),
                                cudaMemcpyHostToDevice, cs), "cudaMemcpyAsync") &&
             ok(cudaMemcpyAsync(b->d_h2, h2v.data(), sizeof(int) * (size_t)count,
                                cudaMemcpyHostToDevice, cs), "cudaMemcpyAsync") &&
@@ -759,8 +751,9 @@ lbm2p_status lbm2p_batch_step(lbm2p_batch *b, int nsteps, const int *replay,
                              b->body, i, replay[i]);
     for (int m = 0; m < b->count; ++m) {
         const lbm2p *h = b->members[(size_t)m];
-        if (h->cur_f != b->pf[(size_t)m] || h->cur_r != b->pr[(size_t)m] ||
-            h->cur_g != (b->pg0[(size_t)m] ^ b->gstep))
+        const int f0 = b->pf[(size_t)m];
+        if (h->cur_f != (b->gstep ? lbm2p_internal::fnext(f0, 1) : f0) ||
+            h->cur_r != (b->pr[(size_t)m] ^ b->gstep) || h->cur_g != (b->pg0[(size_t)m] ^ b->gstep))
             return bfail(b, LBM2P_EINVAL,
                          "member %d was stepped outside the batch (buffer parity changed)", m);
     }
@@ -794,7 +787,10 @@ lbm2p_status lbm2p_batch_step(lbm2p_batch *b, int nsteps, const int *replay,
         for (int m = 0; m < b->count; ++m) {
             lbm2p *h = b->members[(size_t)m];
             const MemberCtl &c = b->h_ctl[m];
+            const int f0 = b->pf[(size_t)m];
+            h->cur_f = b->gstep ? lbm2p_internal::fnext(f0, 1) : f0;
             h->cur_g = 1 - h->cur_g;
+            h->cur_r = 1 - h->cur_r;
             h->sweeps += c.k;
             kmax = c.k > kmax ? c.k : kmax;
             lbm2p_status mst = LBM2P_OK;
@@ -813,11 +809,11 @@ lbm2p_status lbm2p_batch_step(lbm2p_batch *b, int nsteps, const int *replay,
                 o.step_ms = ms;
             }
         }
-        // refresh, reset, prefix, scatter, saturation, rebase; per loop pass: body sweeps,
+        // refresh, reset, prefix, scatter, saturation; per loop pass: body sweeps,
         // finalize, condition + prefix, scatter; and the mid-solve rebases of the longest solve
         const int passes = kmax > 0 ? kmax / b->body : 1;
         const int every = b->body * ((1024 + b->body - 1) / b->body);
-        b->launches += 6 + (long long)passes * 3 + (kmax > 0 ? (kmax - 1) / every : 0);
+        b->launches += 5 + (long long)passes * 3 + (kmax > 0 ? (kmax - 1) / every : 0);
         if (b->nmulti < b->count)
             b->launches += (long long)passes * b->body;
         if (b->nmulti > 0)

@@ -17,6 +17,7 @@
 #include "lbm2p_device.cuh"
 #include "lbm2p_node.cuh"
 #include "residual.cuh"
+#include "step_node.cuh"
 
 namespace lbm2p_dev {
 
@@ -572,29 +573,17 @@ __global__ void k_if_finite(const LoopCtl *ctl, cudaGraphConditionalHandle h)
 // --------------------------------------------------------------------------------------
 // a1: stream g, S^n (Eq. 3-9b), 1/tau_f (Eq. 3-11a with D_p = K lambda_t(S))
 // --------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock) k_refresh(const __grid_constant__ RefreshArgs a)
+__global__ void __launch_bounds__(kStepThreads) k_refresh(const __grid_constant__ RefreshArgs a)
 {
-    const Geom &g = a.g;
-    for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
-        const int y = t / g.tiles_x;
-        const int x = (t - y * g.tiles_x) * kBlock + threadIdx.x;
-        if (x < g.nx)
-            refresh_node(a, x, y, y * g.pitch + x);
-    }
+    refresh_block(a, blockIdx.x);
 }
 
 // --------------------------------------------------------------------------------------
 // a4 + a5: local grad P (Eq. 3-10a) and the fused saturation stream + collide (Eq. 3-2)
 // --------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock) k_saturation(const __grid_constant__ SaturationArgs a)
+__global__ void __launch_bounds__(kStepThreads) k_saturation(const __grid_constant__ SaturationArgs a)
 {
-    const Geom &g = a.g;
-    for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
-        const int y = t / g.tiles_x;
-        const int x = (t - y * g.tiles_x) * kBlock + threadIdx.x;
-        if (x < g.nx)
-            saturation_node(a, x, y, y * g.pitch + x);
-    }
+    saturation_block(a, blockIdx.x);
 }
 
 // --------------------------------------------------------------------------------------
@@ -683,7 +672,7 @@ __global__ void __launch_bounds__(kBlock) k_init_g(const __grid_constant__ InitG
 }
 
 // Four nodes per thread with 128-bit accesses (rows are padded to 32 floats, so a quad never
-// crosses a row); per node the arithmetic of rebase_node.  Padding lanes are written back
+// crosses a row); n_i += w_i (R - Pnew), R = Pnew.  Padding lanes are written back
 // unchanged.
 __global__ void __launch_bounds__(kBlock) k_rebase(const __grid_constant__ RebaseArgs a)
 {
@@ -761,37 +750,92 @@ __global__ void __launch_bounds__(kBlock) k_tau_from_S(float *inv_tau, const flo
 // --------------------------------------------------------------------------------------
 // fields: P (Eq. 3-9a), S, u = -K lambda_t grad P (Eq. 3-10b) into compact [ny][nx]
 // --------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kBlock) k_fields(const __grid_constant__ FieldsArgs a)
+// u at a node from the first moment of the pulled f
+__device__ __forceinline__ void velocity_node(const FieldsArgs &a, float mx, float my, float it, float S,
+                                              float K, float &ux, float &uy)
+{
+    const float gpx = -3.0f * mx * it * a.m.inv_dx, gpy = -3.0f * my * it * a.m.inv_dx;
+    float lw, lt;
+    mobility(a.m, S, lw, lt);
+    const float kl = K * lt;
+    ux = -kl * gpx;
+    uy = -kl * gpy;
+}
+
+// WIDE: the outputs take 128-bit stores (16-byte aligned, rows of a multiple of four nodes)
+template <bool WIDE>
+__global__ void __launch_bounds__(kStepThreads) k_fields(const __grid_constant__ FieldsArgs a)
 {
     const Geom &g = a.g;
-    for (int t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
-        const int y = t / g.tiles_x;
-        const int x = (t - y * g.tiles_x) * kBlock + threadIdx.x;
-        if (x >= g.nx)
-            continue;
+    const StepMap m(g.nx, g.ny);
+    const bool vel = a.ux_out || a.uy_out;
+    const int b = blockIdx.x;
+    if (b < m.eb) {
+        const int e = b * kStepThreads + (int)threadIdx.x;
+        if (e >= m.edges)
+            return;
+        int x, y;
+        m.edge(e, x, y);
         const int o = y * g.pitch + x;
         const long long c = (long long)y * g.nx + x;
-        float f[8];
+        float f[8], mx, my, ux, uy;
         gather_a(a.fin, a.R, g, a.Pb, x, y, o, f);
-        const float S = a.S[o];
+        const float S = a.S[o], r0 = a.R[o];
+        if (vel) {
+            const float it = a.inv_tau[o], K = a.K[o];
+            first_moment(f, mx, my);
+            velocity_node(a, mx, my, it, S, K, ux, uy);
+            if (a.ux_out)
+                a.ux_out[c] = ux;
+            if (a.uy_out)
+                a.uy_out[c] = uy;
+        }
         if (a.P_out)
-            a.P_out[c] = a.R[o] + pressure_of(f);
+            a.P_out[c] = node_pressure(f, r0);
         if (a.S_out)
             a.S_out[c] = S;
-        if (a.ux_out || a.uy_out) {
-            float mx, my;
-            first_moment(f, mx, my);
-            const float it = a.inv_tau[o];
-            const float gpx = -3.0f * mx * it * a.m.inv_dx, gpy = -3.0f * my * it * a.m.inv_dx;
-            float lw, lt;
-            mobility(a.m, S, lw, lt);
-            const float kl = a.K[o] * lt;
-            if (a.ux_out)
-                a.ux_out[c] = -kl * gpx;
-            if (a.uy_out)
-                a.uy_out[c] = -kl * gpy;
-        }
+        return;
     }
+    const StepQuad s(m, b, g.pitch);
+    PullA l;
+    l.load(a.fin, a.R, s, g.pitch);
+    const float4 S = ldq(a.S, s.o);
+    float4 it = make_float4(0.0f, 0.0f, 0.0f, 0.0f), K = it, P, ux = it, uy = it;
+    if (vel) {
+        it = ldq(a.inv_tau, s.o);
+        K = ldq(a.K, s.o);
+    }
+    float4 f[8];
+    l.values(s, f);
+    if (!s.store)
+        return;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        float fc[8], mx, my;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            fc[i] = at4(f[i], c);
+        at4(P, c) = node_pressure(fc, at4(l.r[1], c));
+        first_moment(fc, mx, my);
+        if (vel)
+            velocity_node(a, mx, my, at4(it, c), at4(S, c), at4(K, c), at4(ux, c), at4(uy, c));
+    }
+    auto put = [&](float *out, float4 v) {
+        if (!out)
+            return;
+        out += (long long)s.y * g.nx + s.x;
+        if (WIDE) {
+            *reinterpret_cast<float4 *>(out) = v;
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                out[c] = at4(v, c);
+        }
+    };
+    put(a.P_out, P);
+    put(a.S_out, S);
+    put(a.ux_out, ux);
+    put(a.uy_out, uy);
 }
 
 __global__ void __launch_bounds__(256) k_sum_compact(const float *__restrict__ x, long long n,
@@ -919,14 +963,14 @@ void residual_finalize(const double *partials, int nparts, long long nnodes, flo
     k_residual_finalize<<<kFinBlocks, kFinThreads, 0, S(stream)>>>(partials, nparts, nnodes, shift, out);
 }
 
-void refresh(const RefreshArgs &a, int grid, void *stream)
+void refresh(const RefreshArgs &a, void *stream)
 {
-    k_refresh<<<grid, kBlock, 0, S(stream)>>>(a);
+    k_refresh<<<StepMap(a.g.nx, a.g.ny).blocks(), kStepThreads, 0, S(stream)>>>(a);
 }
 
-void saturation(const SaturationArgs &a, int grid, void *stream)
+void saturation(const SaturationArgs &a, void *stream)
 {
-    k_saturation<<<grid, kBlock, 0, S(stream)>>>(a);
+    k_saturation<<<StepMap(a.g.nx, a.g.ny).blocks(), kStepThreads, 0, S(stream)>>>(a);
 }
 
 void init_g(const InitGArgs &a, int grid, void *stream)
@@ -950,9 +994,16 @@ void tau_from_S(float *inv_tau, const float *Sp, const float *K, Geom g, Model m
     k_tau_from_S<<<grid, kBlock, 0, S(stream)>>>(inv_tau, Sp, K, g, m);
 }
 
-void fields(const FieldsArgs &a, int grid, void *stream)
+void fields(const FieldsArgs &a, void *stream)
 {
-    k_fields<<<grid, kBlock, 0, S(stream)>>>(a);
+    bool wide = a.g.nx % 4 == 0;
+    for (const float *out : {a.P_out, a.S_out, a.ux_out, a.uy_out})
+        wide = wide && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+    const int blocks = StepMap(a.g.nx, a.g.ny).blocks();
+    if (wide)
+        k_fields<true><<<blocks, kStepThreads, 0, S(stream)>>>(a);
+    else
+        k_fields<false><<<blocks, kStepThreads, 0, S(stream)>>>(a);
 }
 
 void sum_compact(const float *x, long long n, double *partials, int grid, void *stream)
@@ -1036,24 +1087,18 @@ cudaError_t node_if_finite(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNod
 }
 
 cudaError_t node_refresh(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                         const RefreshArgs &a, int grid)
+                         const RefreshArgs &a)
 {
     void *args[] = {(void *)&a};
-    return add_kernel(n, g, dep, (void *)k_refresh, grid, kBlock, args);
+    return add_kernel(n, g, dep, (void *)k_refresh, StepMap(a.g.nx, a.g.ny).blocks(), kStepThreads, args);
 }
 
 cudaError_t node_saturation(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                            const SaturationArgs &a, int grid)
+                            const SaturationArgs &a)
 {
     void *args[] = {(void *)&a};
-    return add_kernel(n, g, dep, (void *)k_saturation, grid, kBlock, args);
-}
-
-cudaError_t node_rebase(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                        const RebaseArgs &a, int grid)
-{
-    void *args[] = {(void *)&a};
-    return add_kernel(n, g, dep, (void *)k_rebase, grid, kBlock, args);
+    return add_kernel(n, g, dep, (void *)k_saturation, StepMap(a.g.nx, a.g.ny).blocks(), kStepThreads,
+                      args);
 }
 
 }  // namespace lbm2p_launch

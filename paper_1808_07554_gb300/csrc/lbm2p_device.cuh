@@ -118,10 +118,11 @@ struct RefreshArgs {        // stream g, S^n, 1/tau_f (and the warm start of the
     Wells w;
 };
 
-struct SaturationArgs {     // stream f and g, grad P, collide g
+struct SaturationArgs {     // stream f and g, grad P, collide g; move R to the node pressure
     const float *fin[8];
     const float *R;
-    float *Pnew;             // P of the converged pressure state (for the rebase)
+    float *nout[8];          // n_i of the next step: fin relative to Rnew
+    float *Rnew;             // P of the converged pressure state, the next step's R
     const float *gin[9];
     float *gout[9];
     const float *K;
@@ -164,7 +165,7 @@ struct FieldsArgs {         // P, S, u into compact [ny][nx] outputs
     Model m;
 };
 
-struct RebaseArgs {         // n_i += w_i (R - Pnew); R = Pnew  (node-local)
+struct RebaseArgs {         // after the t = 0 solve: n_i += w_i (R - Pnew); R = Pnew  (node-local)
     float *n[8];
     float *R;
     const float *Pnew;
@@ -340,13 +341,13 @@ cudaError_t rows_h_prepare(int width, int slots);
 int rows_h_blocks_per_sm(int width, int slots, bool has_fp);
 void pressure_sweep_rows_h(const HalfSweepArgs &a, bool check, int width, int slots, int H,
                            int grid, void *stream);
-void refresh(const RefreshArgs &a, int grid, void *stream);
-void saturation(const SaturationArgs &a, int grid, void *stream);
+void refresh(const RefreshArgs &a, void *stream);
+void saturation(const SaturationArgs &a, void *stream);
 void init_g(const InitGArgs &a, int grid, void *stream);
 void rebase(const RebaseArgs &a, int grid, void *stream);
 void tau_from_S(float *inv_tau, const float *S, const float *K, Geom g, Model m, int grid,
                 void *stream);
-void fields(const FieldsArgs &a, int grid, void *stream);
+void fields(const FieldsArgs &a, void *stream);
 // graph nodes (explicit construction; parameters are copied into the node)
 cudaError_t node_pressure(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                           const PressureArgs &a, bool check, bool write_p, int grid, int kind);
@@ -365,11 +366,9 @@ cudaError_t node_loop_reset(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNo
 cudaError_t node_if_finite(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                            const LoopCtl *ctl, cudaGraphConditionalHandle h);
 cudaError_t node_refresh(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                         const RefreshArgs &a, int grid);
+                         const RefreshArgs &a);
 cudaError_t node_saturation(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                            const SaturationArgs &a, int grid);
-cudaError_t node_rebase(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                        const RebaseArgs &a, int grid);
+                            const SaturationArgs &a);
 void sum_compact(const float *x, long long n, double *partials, int grid, void *stream);
 void finalize_mean(const double *partials, int nparts, long long n, double *mean, void *stream);
 void subtract_mean(float *x, long long n, const double *mean, int grid, void *stream);

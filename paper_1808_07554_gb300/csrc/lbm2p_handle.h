@@ -68,8 +68,11 @@ struct lbm2p {
     // 1/tau_f, the reference pressure R of the pressure populations, and (warm start) the node
     // pressure of the previous step: two buffers each, cur_r the current one.  A step's S
     // refresh writes the other (the "work" buffer), which becomes current when the step ends.
+    // R of a step's solve is in Rwork (a mid-solve rebase moves it); the saturation update writes the
+    // next R.
     float *inv_taub[2] = {};
     float *Rb[2] = {};
+    float *Rwork = nullptr;
     float *Pstepb[2] = {};
     float *Fp = nullptr, *Fs = nullptr;
     float *Pb[4] = {}, *Sb[4] = {};
@@ -103,14 +106,15 @@ namespace lbm2p_internal {
 inline int fnext(int b, int k) { return (b + k) % 3; }
 // 1/tau_f, R and the previous step's P: the current buffers, or the work buffers of a step
 inline float *itau_of(const lbm2p *h, bool work) { return h->inv_taub[work ? 1 - h->cur_r : h->cur_r]; }
-inline float *R_of(const lbm2p *h, bool work) { return h->Rb[work ? 1 - h->cur_r : h->cur_r]; }
+inline float *R_of(const lbm2p *h, bool work) { return work ? h->Rwork : h->Rb[h->cur_r]; }
 inline float *Pstep_of(const lbm2p *h, bool work) { return h->Pstepb[work ? 1 - h->cur_r : h->cur_r]; }
-// kernel argument blocks of h (runtime.cu): sweeps from f buffer src into dst, the S refresh
-// of g buffer pg (in place: R, P^{n-1} and 1/tau_f overwritten; otherwise written into the
-// work buffers), saturation update and rebases of f buffer pf; `work`: use the work buffers
+// kernel argument blocks of h (runtime.cu): sweeps from f buffer src into dst, the S refresh of g
+// buffer pg into the work buffers, the saturation update of f buffer pf and g buffer pg, which
+// writes the next step's populations into f buffer pn and its R into the buffer that is not current,
+// and rebases of f buffer pf; `work`: use the work buffers
 lbm2p_dev::PressureArgs pressure_args(lbm2p *h, int src, int dst, bool work);
-lbm2p_dev::RefreshArgs refresh_args(lbm2p *h, int pg, bool in_place);
-lbm2p_dev::SaturationArgs saturation_args(lbm2p *h, int pf, int pg, bool work);
+lbm2p_dev::RefreshArgs refresh_args(lbm2p *h, int pg);
+lbm2p_dev::SaturationArgs saturation_args(lbm2p *h, int pf, int pn, int pg);
 lbm2p_dev::RebaseArgs rebase_args(lbm2p *h, int pf, bool work);
 lbm2p_dev::RebaseMidArgs rebase_mid_args(lbm2p *h, int pf, bool work);
 }  // namespace lbm2p_internal

@@ -173,14 +173,19 @@ __device__ __forceinline__ void tau_g_node(const Model &m, float K, float lw, fl
         return;
     }
     const float h = lt != 0.0f ? lw * (lt - lw) / lt : 0.0f;
-    inv_tg = 1.0f / (0.5f + m.ds_a0 + m.ds_a1 * K * h);
+    inv_tg = 1.0f / fmaf(m.ds_a1 * K, h, 0.5f + m.ds_a0);
     src = 1.0f - 0.5f * inv_tg;
 }
 
-// Eq. 3-9a: P = sum_{i=1..8} f_i / (1 - w_0) = (9/5) sum
+// Eq. 3-9a: P = sum_{i=1..8} f_i / (1 - w_0) = (9/5) sum; above the reference r0 of f
 __device__ __forceinline__ float pressure_of(const float (&f)[8])
 {
     return (((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7]))) * 1.8f;
+}
+
+__device__ __forceinline__ float node_pressure(const float (&f)[8], float r0)
+{
+    return fmaf(((f[0] + f[1]) + (f[2] + f[3])) + ((f[4] + f[5]) + (f[6] + f[7])), 1.8f, r0);
 }
 
 // sum_i c_i f_i (x and y components)
@@ -195,12 +200,12 @@ __device__ __forceinline__ void mobility(const Model &m, float S, float &lw, flo
     if (m.mobility == MOB_QUADRATIC) {
         lw = S * S * m.inv_mu_w;
         const float sn = 1.0f - S;
-        lt = lw + sn * sn * m.inv_mu_n;
+        lt = fmaf(S * S, m.inv_mu_w, sn * sn * m.inv_mu_n);   // explicit: every kernel rounds it the same
     } else if (m.mobility == MOB_DECOUPLED) {
         lw = m.inv_mu_w;
         lt = m.inv_mu_w;
     } else {
-        lt = 1.0f / (0.5f - 0.2f * S);
+        lt = 1.0f / fmaf(-0.2f, S, 0.5f);
         lw = S * lt;
     }
 }
@@ -296,57 +301,32 @@ struct ResAcc {
 // --------------------------------------------------------------------------------------
 // per-node bodies shared by the single-lattice kernels and the batched kernels
 // --------------------------------------------------------------------------------------
-// Warm start of a solve: the equilibrium part of f_i = n_i + w_i R moves with R to the
-// pressure extrapolated in time, R' = R + (R - P^{n-1}); n_i (the rest) is kept.  The inputs
-// may be the outputs (in place).
-__device__ __forceinline__ void extrapolate_node(const float *Rin, float *Rout,
-                                                 const float *Pin, float *Pout, int o)
+// a1: S^n (Eq. 3-9b) from the pulled g; 1/tau_f (Eq. 3-11a with D_p = K lambda_t(S))
+__device__ __forceinline__ float refresh_tau(const RefreshArgs &a, int o, const float (&q)[9], float K)
 {
-    const float r = Rin[o];
-    const float pv = Pin[o];
-    Rout[o] = r + (r - pv);
-    Pout[o] = r;
-}
-
-// a1: S^n (Eq. 3-9b) from the pulled g and 1/tau_f (Eq. 3-11a with D_p = K lambda_t(S)); with
-// a warm start also the extrapolation of the node's reference pressure for the coming solve
-__device__ __forceinline__ void refresh_node(const RefreshArgs &a, int x, int y, int o)
-{
-    float q[9];
-    gather_g(a.gin, a.g, a.m, a.Sb, x, y, o, q);
     const float sum = (q[0] + ((q[1] + q[2]) + (q[3] + q[4]))) + ((q[5] + q[6]) + (q[7] + q[8]));
     const float Fs = saturation_source(a.m, a.w, a.Fs, o, sum * a.m.inv_phi);
-    const float S = (sum + 0.5f * Fs) * a.m.inv_phi;
+    const float S = fmaf(0.5f, Fs, sum) * a.m.inv_phi;
     float lw, lt;
     mobility(a.m, S, lw, lt);
-    a.inv_tau[o] = 1.0f / (0.5f + a.m.s3 * a.K[o] * lt);
-    if (a.Pstep_in)
-        extrapolate_node(a.Rin, a.Rout, a.Pstep_in, a.Pstep_out, o);
-    else if (a.Rout != a.Rin)
-        a.Rout[o] = a.Rin[o];
+    return 1.0f / fmaf(a.m.s3 * K, lt, 0.5f);
 }
 
-// a4 + a5: local grad P (Eq. 3-10a), then the saturation collision (Eq. 3-2); also stores
-// S^n and the pressure of the pulled state (for the rebase)
-__device__ __forceinline__ void saturation_node(const SaturationArgs &a, int x, int y, int o)
+// The multiply-adds of a step's kernels are written out, as those of the sweeps are: left to the
+// compiler, the quad, edge and batched kernels round differently.
+// a4 + a5: local grad P (Eq. 3-10a) from the first moment of the pulled f, then the saturation
+// collision (Eq. 3-2) of the pulled populations q, in place; returns S^n
+__device__ __forceinline__ float saturation_collide(const SaturationArgs &a, int o, float mx, float my,
+                                                    float it, float K, float (&q)[9])
 {
-    const Geom &g = a.g;
     const Model &m = a.m;
-    float f[8], q[9];
-    gather_a(a.fin, a.R, g, a.Pb, x, y, o, f);
-    a.Pnew[o] = a.R[o] + pressure_of(f);
-    gather_g(a.gin, g, m, a.Sb, x, y, o, q);
     const float sum = (q[0] + ((q[1] + q[2]) + (q[3] + q[4]))) + ((q[5] + q[6]) + (q[7] + q[8]));
     const float Fs = saturation_source(m, a.w, a.Fs, o, sum * m.inv_phi);
-    const float S = (sum + 0.5f * Fs) * m.inv_phi;
+    const float S = fmaf(0.5f, Fs, sum) * m.inv_phi;
     // grad_X P = -3 sum_i c_i f_i / tau_f  (lattice units, Eq. 3-10a)
-    float mx, my;
-    first_moment(f, mx, my);
-    const float it = a.inv_tau[o];
     const float gx = -3.0f * mx * it, gy = -3.0f * my * it;
     float lw, lt;
     mobility(m, S, lw, lt);
-    const float K = a.K[o];
     float inv_tg, src_g;
     tau_g_node(m, K, lw, lt, inv_tg, src_g);
     // gamma~ = -3 lambda_w K dt / dx^2 (Eq. 3-8 in lattice units), pre-divided by tau_g
@@ -358,21 +338,10 @@ __device__ __forceinline__ void saturation_node(const SaturationArgs &a, int x, 
             break;
         const float wi = m.wg[i];
         const float cg = (float)cx(i) * gx + (float)cy(i) * gy;
-        const float eq = m.Gam[i] * S;
-        a.gout[i][o] = fmaf(eq - q[i], inv_tg, q[i]) + wi * src + gam * wi * cg;
+        const float rel = fmaf(fmaf(m.Gam[i], S, -q[i]), inv_tg, q[i]);
+        q[i] = fmaf(gam * wi, cg, fmaf(wi, src, rel));
     }
-    a.S[o] = S;
-}
-
-// move the reference pressure to Pnew: n_i += w_i (R - Pnew), R = Pnew (own node only)
-__device__ __forceinline__ void rebase_node(const RebaseArgs &a, int o)
-{
-    const float pn = a.Pnew[o];
-    const float d = a.R[o] - pn;
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        a.n[i][o] = fmaf(wgt(i + 1), d, a.n[i][o]);
-    a.R[o] = pn;
+    return S;
 }
 
 // Within a long sub-iteration, move R to the current pressure.  After a sweep the stored

@@ -48,18 +48,18 @@ PressureArgs pressure_args(lbm2p *h, int src, int dst, bool work)
     return a;
 }
 
-RefreshArgs refresh_args(lbm2p *h, int pg, bool in_place)
+RefreshArgs refresh_args(lbm2p *h, int pg)
 {
     RefreshArgs a{};
     for (int i = 0; i < 9; ++i)
         a.gin[i] = h->gbuf[pg][i];
     a.Rin = R_of(h, false);
-    a.Rout = R_of(h, !in_place);
+    a.Rout = R_of(h, true);
     a.Pstep_in = h->p.warm_start ? Pstep_of(h, false) : nullptr;
-    a.Pstep_out = h->p.warm_start ? Pstep_of(h, !in_place) : nullptr;
+    a.Pstep_out = h->p.warm_start ? Pstep_of(h, true) : nullptr;
     a.K = h->K;
     a.Fs = h->Fs;
-    a.inv_tau = itau_of(h, !in_place);
+    a.inv_tau = itau_of(h, true);
     for (int s = 0; s < 4; ++s)
         a.Sb[s] = h->Sb[s];
     a.g = h->geom;
@@ -68,19 +68,21 @@ RefreshArgs refresh_args(lbm2p *h, int pg, bool in_place)
     return a;
 }
 
-SaturationArgs saturation_args(lbm2p *h, int pf, int pg, bool work)
+SaturationArgs saturation_args(lbm2p *h, int pf, int pn, int pg)
 {
     SaturationArgs a{};
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < 8; ++i) {
         a.fin[i] = h->fbuf[pf][i];
-    a.R = R_of(h, work);
-    a.Pnew = h->Pio;
+        a.nout[i] = h->fbuf[pn][i];
+    }
+    a.R = R_of(h, true);
+    a.Rnew = h->Rb[1 - h->cur_r];
     for (int i = 0; i < 9; ++i) {
         a.gin[i] = h->gbuf[pg][i];
         a.gout[i] = h->gbuf[1 - pg][i];
     }
     a.K = h->K;
-    a.inv_tau = itau_of(h, work);
+    a.inv_tau = itau_of(h, true);
     a.Fs = h->Fs;
     a.S = h->S;
     for (int s = 0; s < 4; ++s) {
@@ -439,7 +441,7 @@ lbm2p_status solve_graph(lbm2p *h, int pin, cudaGraphExec_t *out)
 }
 
 // one physical step: refresh (into the work buffers) -> loop -> IF{the residual is a number:
-// saturation update -> rebase}; the step's inputs (f buffer pin, g buffer pg, the current R,
+// saturation update, which moves R too}; the step's inputs (f buffer pin, g buffer pg, the current R,
 // 1/tau_f and P^{n-1}) are only read, so a step that fails leaves them as they were
 lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
 {
@@ -448,8 +450,8 @@ lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
         cudaGraph_t G;
         CUDA_TRY(h, cudaGraphCreate(&G, 0));
         h->step_g[pin][pg][r] = G;
-        cudaGraphNode_t nr, last, nf, ifn, ns, nb;
-        CUDA_TRY(h, lbm2p_launch::node_refresh(&nr, G, nullptr, refresh_args(h, pg, false), h->grid));
+        cudaGraphNode_t nr, last, nf, ifn, ns;
+        CUDA_TRY(h, lbm2p_launch::node_refresh(&nr, G, nullptr, refresh_args(h, pg)));
         cudaGraphConditionalHandle hok;
         CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hok, G, 0, 0));
         lbm2p_status e = add_loop(h, G, &nr, pin, true, &last, &hok);
@@ -468,8 +470,7 @@ lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
         cudaGraph_t tail = ip.conditional.phGraph_out[0];
         const int pout = fnext(pin, 2);
         CUDA_TRY(h, lbm2p_launch::node_saturation(&ns, tail, nullptr,
-                                                  saturation_args(h, pout, pg, true), h->grid));
-        CUDA_TRY(h, lbm2p_launch::node_rebase(&nb, tail, &ns, rebase_args(h, pout, true), h->grid));
+                                                  saturation_args(h, pout, fnext(pin, 1), pg)));
         CUDA_TRY(h, cudaGraphInstantiate(&h->step_x[pin][pg][r], G, 0));
     }
     *out = h->step_x[pin][pg][r];
@@ -905,20 +906,20 @@ lbm2p_status one_step(lbm2p *h, int replay, lbm2p_step_stats *stats)
             return e;
         const bool finite = !std::isnan(r);
         // refresh and the finiteness test (a launch of its own unless the solve is one); saturation
-        // and rebase when the step goes on
-        h->launches += (finite ? 4 : 2) - (h->res_C > 0 ? 1 : 0);
+        // when the step goes on
+        h->launches += (finite ? 3 : 2) - (h->res_C > 0 ? 1 : 0);
         if (h->timing)
             CUDA_TRY(h, cudaEventElapsedTime(&step_ms, h->ev_step0, h->ev_step1));
         lbm2p_status ps = loop_status(h, k, r);
         if (finite)
-            advance(fnext(h->cur_f, 2));
+            advance(fnext(h->cur_f, 1));
         fill(k, ps, r, sw_ms, step_ms);
         return ps;
     }
     if (h->timing)
         CUDA_TRY(h, cudaEventRecord(h->ev_step0, st));
     // a1: stream g, S^n, tau_f (and the warm start) into the work buffers
-    lbm2p_launch::refresh(refresh_args(h, h->cur_g, false), h->grid, h->stream);
+    lbm2p_launch::refresh(refresh_args(h, h->cur_g), h->stream);
     LAUNCHED(h, "refresh");
     // a2/a3: pressure sub-iteration
     int k = 0, pout = h->cur_f;
@@ -930,11 +931,10 @@ lbm2p_status one_step(lbm2p *h, int replay, lbm2p_step_stats *stats)
         return ps;
     }
     // a4/a5: grad P and the saturation update
-    lbm2p_launch::saturation(saturation_args(h, pout, h->cur_g, true), h->grid, h->stream);
+    const int pn = fnext(pout, 1);
+    lbm2p_launch::saturation(saturation_args(h, pout, pn, h->cur_g), h->stream);
     LAUNCHED(h, "saturation");
-    lbm2p_launch::rebase(rebase_args(h, pout, true), h->grid, h->stream);
-    LAUNCHED(h, "rebase");
-    advance(pout);
+    advance(pn);
     float step_ms = -1.0f;
     if (h->timing) {
         CUDA_TRY(h, cudaEventRecord(h->ev_step1, st));
@@ -1654,7 +1654,7 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
         if (p.warm_start)
             ok = ok && plane_alloc(&h->Pstepb[b]);
     }
-    ok = ok && plane_alloc(&h->K) && plane_alloc(&h->S) && plane_alloc(&h->Pio) &&
+    ok = ok && plane_alloc(&h->Rwork) && plane_alloc(&h->K) && plane_alloc(&h->S) && plane_alloc(&h->Pio) &&
          plane_alloc(&h->tmp);
     if (in->Fp)
         ok = ok && plane_alloc(&h->Fp);
@@ -2025,7 +2025,7 @@ static lbm2p_status run_fields(lbm2p *h, float *P, float *S, float *ux, float *u
     a.uy_out = dst[3];
     a.g = h->geom;
     a.m = h->model;
-    lbm2p_launch::fields(a, h->grid, h->stream);
+    lbm2p_launch::fields(a, h->stream);
     LAUNCHED(h, "fields");
     if (P && mean_free_P) {
         lbm2p_launch::sum_compact(dst[0], n, h->partials, h->grid, h->stream);

@@ -315,6 +315,10 @@ cudaError_t quad_prepare();
 void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream);
 cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                const PressureArgs &a, bool check, int H, int grid);
+// four FP16-storage sweeps per launch (fp16_quad.cu) in the same tiles; the planes of a.nin are
+// equally spaced
+int quad_h_slots(bool has_fp);
+void pressure_sweeps_quad_h(const HalfSweepArgs &a, bool check, int H, int grid, void *stream);
 // the same over several lattices: item t (t < *nitems <= grid) is tile items[t].y (of H[m] rows) of
 // member m = items[t].x, with argument block pa[2 m + parity]; residual sums of member m to
 // parts[4 (pb0[m] + tile) ..]

@@ -55,6 +55,7 @@ struct lbm2p {
     int grid_h = 0;            // one-node-per-thread FP16 sweep
     int h16_kind = 0;          // FP16 sweep kernel: 0 one node per thread, 1 staged rows
     int h16_w = 0, h16_slots = 0, h16_H = 0, h16_grid = 0;
+    int h16q_H = 0, h16q_grid = 0;   // four FP16 sweeps per launch: tile rows (0: not used), tiles
     int rebase_every = 0;      // a long solve moves R to the current P after every this many
                                // sweeps (a multiple of check_every)
     void *stream = nullptr;

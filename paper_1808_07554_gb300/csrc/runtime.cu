@@ -543,13 +543,16 @@ lbm2p_status pressure_solve_h(lbm2p *h, int replay, bool work, int *k_out, doubl
     lbm2p_launch::half_narrow(convert_args(0), h->grid, h->stream);
     LAUNCHED(h, "FP16 narrow");
     h->hcur = 0;
-    int k = 0;
+    int k = 0, last_nparts = 0;
     double r = std::nan("");
     float ms_total = 0.0f;
     lbm2p_status status = LBM2P_OK;
     auto sweeps = [&](int upto, bool final_check) -> lbm2p_status {
         if (h->timing)
             CUDA_TRY(h, cudaEventRecord(h->ev_sw0, st));
+        // the sweeps beyond a multiple of four first, one per launch, then four per launch
+        const int single = h->h16q_H > 0 ? (upto - k) % 4 : upto - k;
+        const int k0 = k;
         for (int kk = k + 1; kk <= upto; ++kk) {
             HalfSweepArgs a{};
             for (int i = 0; i < 8; ++i) {
@@ -568,15 +571,20 @@ lbm2p_status pressure_solve_h(lbm2p *h, int replay, bool work, int *k_out, doubl
                 a.Pb[s] = h->Pb[s];
             a.g = h->geom;
             a.w = h->wells;
+            const bool four = kk - k0 > single;
+            kk += four ? 3 : 0;
             const bool check = final_check && kk == upto;
-            if (h->h16_kind == 1)
+            last_nparts = four ? h->h16q_grid : (h->h16_kind == 1 ? h->h16_grid : h->grid_h);
+            if (four)
+                lbm2p_launch::pressure_sweeps_quad_h(a, check, h->h16q_H, h->h16q_grid, h->stream);
+            else if (h->h16_kind == 1)
                 lbm2p_launch::pressure_sweep_rows_h(a, check, h->h16_w, h->h16_slots, h->h16_H,
                                                     h->h16_grid, h->stream);
             else
                 lbm2p_launch::pressure_sweep_h(a, check, h->grid_h, h->stream);
             LAUNCHED(h, "FP16 pressure sweep");
             h->hcur = 1 - h->hcur;
-            h->sweeps += 1;
+            h->sweeps += four ? 4 : 1;
         }
         k = upto;
         if (h->timing) {
@@ -589,8 +597,8 @@ lbm2p_status pressure_solve_h(lbm2p *h, int replay, bool work, int *k_out, doubl
         return LBM2P_OK;
     };
     auto read_residual = [&]() -> lbm2p_status {
-        lbm2p_launch::residual_finalize(h->partials, h->h16_kind == 1 ? h->h16_grid : h->grid_h,
-                                        h->nnodes, h->shift, h->res, h->stream);
+        lbm2p_launch::residual_finalize(h->partials, last_nparts, h->nnodes, h->shift, h->res,
+                                        h->stream);
         LAUNCHED(h, "residual finalize");
         CUDA_TRY(h, cudaMemcpyAsync(h->res_host, h->res, sizeof(ResidualOut),
                                     cudaMemcpyDeviceToHost, st));
@@ -1416,8 +1424,9 @@ done:
     return LBM2P_OK;
 }
 
-// FP16 storage: time the one-node-per-thread FP16 sweep and the FP16 staged-rows sweep over
-// its shapes on this lattice (zeroed buffers) and keep the fastest
+// FP16 storage: time the one-node-per-thread FP16 sweep, the FP16 staged-rows sweep over its shapes
+// and, on lattices with walls on every side, four FP16 sweeps per launch, on this lattice (zeroed
+// buffers), and keep the fastest
 lbm2p_status autotune_h(lbm2p *h, int sms)
 {
     cudaStream_t st = (cudaStream_t)h->stream;
@@ -1470,7 +1479,13 @@ lbm2p_status autotune_h(lbm2p *h, int sms)
     float best = 1e30f;
     const bool rows_only = h->p.sweep_kernel == LBM2P_SWEEP_ROWS;
     const bool no_rows = h->p.sweep_kernel == LBM2P_SWEEP_SCALAR || h->p.sweep_kernel == LBM2P_SWEEP_VEC4;
+    // four sweeps per launch, unless the caller names a single-sweep kernel or asks for one sweep per
+    // launch
+    bool four = (h->p.fuse_sweeps == 0 || h->p.fuse_sweeps == 4) && !rows_only && !no_rows;
+    for (int s = 0; s < 4; ++s)
+        four = four && h->p.bc[s] != LBM2P_BC_PERIODIC;
     h->h16_kind = 0;
+    h->h16q_H = h->h16q_grid = 0;
     {
         float ms = 0.0f;
         if (!timed([&](int k) { lbm2p_launch::pressure_sweep_h(args(k), false, h->grid_h, h->stream); },
@@ -1494,6 +1509,10 @@ lbm2p_status autotune_h(lbm2p *h, int sms)
             const int strips = (h->nx + width - 1) / width;
             int last_H = -1;
             for (int mult : {1, 2, 4, 8, 16}) {
+                // where four sweeps per launch run, this kernel has the one to three sweeps left
+                // over: its best multiples only
+                if (four && mult != 4 && mult != 8)
+                    continue;
                 long long chunks = ((long long)sms * per_sm * mult + strips - 1) / strips;
                 chunks = chunks < 1 ? 1 : chunks;
                 const int H = (int)((h->ny + chunks - 1) / chunks);
@@ -1518,6 +1537,36 @@ lbm2p_status autotune_h(lbm2p *h, int sms)
                     h->h16_H = H;
                     h->h16_grid = grid;
                 }
+            }
+        }
+    }
+    // the heights tried are those of the FP32 form
+    if (four) {
+        const int slots = lbm2p_launch::quad_h_slots(h->Fp != nullptr);
+        int last_H = -1;
+        for (int quarters : {2, 4, 8, 12, 16, 24}) {
+            if (slots < 1)
+                break;
+            int H = 2;
+            while (H < 128 &&
+                   lbm2p_launch::quad_grid(H, h->nx, h->ny) > (long long)slots * quarters / 4)
+                ++H;
+            H = H < h->ny ? H : h->ny;
+            const long long grid = lbm2p_launch::quad_grid(H, h->nx, h->ny);
+            if (H == last_H || grid > (1LL << 30))
+                continue;
+            last_H = H;
+            float ms = 0.0f;
+            if (!timed([&](int k) {
+                    lbm2p_launch::pressure_sweeps_quad_h(args(k), false, H, (int)grid, h->stream);
+                }, &ms))
+                goto done;
+            snprintf(line, sizeof line, "fp16_quad 0 0 %d %d %.3f\n", H, (int)grid, ms / 4 * 1e3f);
+            h->autotune_log += line;
+            if (ms / 4 < best) {
+                best = ms / 4;
+                h->h16q_H = H;
+                h->h16q_grid = (int)grid;
             }
         }
     }
@@ -1671,10 +1720,11 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
     if (h->fp16) {
         // FP16 copies of the populations and the per-sweep node pressures of a solve
         for (int b = 0; b < 2; ++b) {
-            for (int i = 0; i < 8; ++i) {
-                h->hbuf[b][i] = (__half *)dev_alloc(h, (size_t)h->plane * sizeof(__half));
-                ok = ok && h->hbuf[b][i];
-            }
+            // one allocation: the four-sweep kernel steps from plane to plane
+            h->hbuf[b][0] = (__half *)dev_alloc(h, 8 * (size_t)h->plane * sizeof(__half));
+            ok = ok && h->hbuf[b][0];
+            for (int i = 1; i < 8 && ok; ++i)
+                h->hbuf[b][i] = h->hbuf[b][0] + (size_t)i * h->plane;
             ok = ok && plane_alloc(&h->Rh[b]);
         }
         h->hscale = (float *)dev_alloc(h, 64);
@@ -1716,6 +1766,7 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
         np = np > h->host_form.grid ? np : h->host_form.grid;
         np = np > h->grid_h ? np : h->grid_h;
         np = np > h->h16_grid ? np : h->h16_grid;
+        np = np > h->h16q_grid ? np : h->h16q_grid;
         for (int kind = 0; kind < 2; ++kind) {
             np = np > h->grid_k[kind] ? np : h->grid_k[kind];
             np = np > h->grid_check_k[kind] ? np : h->grid_check_k[kind];
@@ -2131,7 +2182,7 @@ lbm2p_status lbm2p_sweep_config(const lbm2p *h, int *fused, int *kind, int *tile
     if (!h)
         return fail(nullptr, LBM2P_EINVAL, "NULL handle");
     if (fused)
-        *fused = h->tb.T > 1 ? h->tb.T : 1;
+        *fused = h->tb.T > 1 ? h->tb.T : (h->fp16 && h->h16q_H > 0 ? 4 : 1);
     if (h->fp16) {                       // the FP16 sweep kernels
         if (kind)
             *kind = h->h16_kind == 1 ? LBM2P_SWEEP_ROWS : LBM2P_SWEEP_SCALAR;
@@ -2208,7 +2259,9 @@ int lbm2p_fused_form_of(const lbm2p *h)
 {
     if (h && !h->fp16 && h->res_C > 0)
         return LBM2P_FUSED_RESIDENT;
-    if (!h || h->fp16 || h->tb.T <= 1)
+    if (h && h->fp16)
+        return h->h16q_H > 0 ? LBM2P_FUSED_QUAD : LBM2P_FUSED_NONE;
+    if (!h || h->tb.T <= 1)
         return LBM2P_FUSED_NONE;
     constexpr int forms[4] = {LBM2P_FUSED_STAGES, LBM2P_FUSED_STAGED_ROWS, LBM2P_FUSED_DIRECT,
                               LBM2P_FUSED_QUAD};

@@ -152,3 +152,37 @@ def test_fp16_member_is_refused_by_a_batch():
     with pytest.raises(pkg.LBM2PError) as e:
         pkg.Batch([a, b])
     assert e.value.status == pkg.EINVAL
+
+
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("bc", [(1, 1, 1, 1), (1, 2, 2, 1), (2, 1, 1, 1)])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (55, 9), (57, 8), (64, 64), (113, 131), (168, 33), (301, 257)])
+def test_four_fp16_sweeps_equal_single_sweeps(nx, ny, bc, dense):
+    """Four FP16 sweeps per launch store the values of four launches of one, bit for bit, at the edges
+    of the tiles, with wells on walls and tile borders, dense sources and walls of both kinds."""
+    import paper_1808_07554_gb300 as pkg
+    from _problems import uniform
+    rng = np.random.default_rng(nx * 1000 + ny)
+    wells = {(0, 0), (nx - 1, ny - 1), (min(56, nx - 1), ny // 2), (nx // 2, 0), (0, ny // 2)}
+    prob = uniform(nx, ny, bc=bc, K=np.exp(rng.standard_normal((ny, nx))),
+                   S0=0.2 + 0.5 * rng.random((ny, nx)),
+                   Fp=rng.standard_normal((ny, nx)) if dense else None,
+                   wells=[(i, j, 1e-2 * (1 + k), k % 2) for k, (i, j) in enumerate(sorted(wells))],
+                   P_b=[rng.random(2 * (ny if s < 2 else nx) + 1) for s in range(4)],
+                   S_b=[np.full(2 * (ny if s < 2 else nx) + 1, 0.3) for s in range(4)])
+    make = lambda fuse: pkg.Solver.from_problem(prob, init_replay=0, fuse_sweeps=fuse,   # noqa: E731
+                                                storage=pkg.STORE_FP16_DEV)
+    one, four = make(1), make(4)
+    assert one.fused_form() == pkg.FUSED_NONE
+    state = one.get_state()
+    state[:8] = 0.01 * rng.standard_normal(state[:8].shape)
+    state[17] = 1.0 / (0.55 + 2.0 * rng.random(state[17].shape))
+    state[19] = rng.standard_normal(state[19].shape)
+    one.set_state(state)
+    four.set_state(state)
+    for n in (4, 9, 8):
+        r1, r4 = one.pressure_sweeps(n), four.pressure_sweeps(n)
+        assert np.array_equal(one.get_state(), four.get_state()), (n, nx, ny, bc)
+        assert r4 == pytest.approx(r1, rel=1e-3, abs=1e-30)
+    one.close()
+    four.close()

@@ -336,7 +336,7 @@ cudaError_t node_resident(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode
 // FP16 storage (fp16.cu): narrow = max |n| -> scale -> convert; one sweep; widen
 int max_blocks_per_sm_pressure_h();
 void half_narrow(const HalfConvertArgs &a, int grid, void *stream);
-void half_widen(const HalfConvertArgs &a, int grid, void *stream);
+void half_widen(const HalfConvertArgs &a, void *stream);
 void half_rescale(const HalfConvertArgs &a, float factor, int grid, void *stream);
 void pressure_sweep_h(const HalfSweepArgs &a, bool check, int grid, void *stream);
 // the FP16 staged-rows sweep (fp16.cu): shapes as for rows_* (width 128 or 256, slots 6 or 8)

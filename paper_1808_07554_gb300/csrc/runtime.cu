@@ -674,7 +674,7 @@ lbm2p_status pressure_solve_h(lbm2p *h, int replay, bool work, int *k_out, doubl
                 return e;
         }
     }
-    lbm2p_launch::half_widen(convert_args(h->hcur), h->grid, h->stream);
+    lbm2p_launch::half_widen(convert_args(h->hcur), h->stream);
     LAUNCHED(h, "FP16 widen");
     if (pout)
         *pout = pw;

@@ -544,7 +544,7 @@ __global__ void __cluster_dims__(kFinBlocks, 1, 1) __launch_bounds__(kFinThreads
 __global__ void __cluster_dims__(kFinBlocks, 1, 1) __launch_bounds__(kFinThreads)
     k_residual_finalize_loop(const double *__restrict__ partials, int nparts, long long nnodes,
                              float *shift, ResidualOut *out, LoopCtl *ctl,
-                             cudaGraphConditionalHandle handle, cudaGraphConditionalHandle h_rebase)
+                             const __grid_constant__ LoopHandles h)
 {
     double r;
     if (finalize_residual<kFinBlocks>(partials, nparts, nnodes, shift, out, r) && threadIdx.x == 0) {
@@ -552,9 +552,22 @@ __global__ void __cluster_dims__(kFinBlocks, 1, 1) __launch_bounds__(kFinThreads
         ctl->k = k;
         ctl->r = r;
         const bool more = !(r <= ctl->tol) && !isnan(r) && k < ctl->cap;
-        cudaGraphSetConditional(handle, more ? 1u : 0u);
-        cudaGraphSetConditional(h_rebase, more && ctl->every > 0 && k % ctl->every == 0 ? 1u : 0u);
+        const bool rebase = more && ctl->every > 0 && k % ctl->every == 0;
+        cudaGraphSetConditional(h.loop, more ? 1u : 0u);
+        if (h.has_inner)
+            cudaGraphSetConditional(h.inner, more && !rebase ? 1u : 0u);
+        if (h.has_rebase)
+            cudaGraphSetConditional(h.rebase, rebase ? 1u : 0u);
+        if (h.has_ok && !more)
+            cudaGraphSetConditional(h.ok, isnan(r) ? 0u : 1u);
     }
+}
+
+// The inner loop starts; only a check inside it keeps the outer one going.
+__global__ void k_loop_open(const __grid_constant__ LoopHandles h)
+{
+    cudaGraphSetConditional(h.inner, 1u);
+    cudaGraphSetConditional(h.loop, 0u);
 }
 
 __global__ void k_loop_reset(LoopCtl *ctl)
@@ -563,18 +576,15 @@ __global__ void k_loop_reset(LoopCtl *ctl)
     ctl->r = nan("");
 }
 
-// After the loop: the step goes on (saturation update, rebase) only when the last residual is
-// a number; otherwise the step's inputs stay as they were and the host reports ENONFINITE.
-__global__ void k_if_finite(const LoopCtl *ctl, cudaGraphConditionalHandle h)
-{
-    cudaGraphSetConditional(h, isnan(ctl->r) ? 0u : 1u);
-}
-
 // --------------------------------------------------------------------------------------
 // a1: stream g, S^n (Eq. 3-9b), 1/tau_f (Eq. 3-11a with D_p = K lambda_t(S))
 // --------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kStepThreads) k_refresh(const __grid_constant__ RefreshArgs a)
 {
+    if (a.ctl && blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctl->k = 0;
+        a.ctl->r = nan("");
+    }
     refresh_block(a, blockIdx.x);
 }
 
@@ -1057,11 +1067,10 @@ cudaError_t node_pressure_fused(cudaGraphNode_t *n, cudaGraph_t g, const cudaGra
 
 cudaError_t node_finalize_loop(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                const double *partials, int nparts, long long nnodes, float *shift,
-                               ResidualOut *out, LoopCtl *ctl, cudaGraphConditionalHandle h,
-                               cudaGraphConditionalHandle h_rebase)
+                               ResidualOut *out, LoopCtl *ctl, const LoopHandles &h)
 {
     void *args[] = {(void *)&partials, (void *)&nparts, (void *)&nnodes, (void *)&shift,
-                    (void *)&out, (void *)&ctl, (void *)&h, (void *)&h_rebase};
+                    (void *)&out, (void *)&ctl, (void *)&h};
     return add_kernel(n, g, dep, (void *)k_residual_finalize_loop, kFinBlocks, kFinThreads, args);
 }
 
@@ -1072,18 +1081,17 @@ cudaError_t node_rebase_mid(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNo
     return add_kernel(n, g, dep, (void *)k_rebase_mid, grid, kBlock, args);
 }
 
+cudaError_t node_loop_open(cudaGraphNode_t *n, cudaGraph_t g, const LoopHandles &h)
+{
+    void *args[] = {(void *)&h};
+    return add_kernel(n, g, nullptr, (void *)k_loop_open, 1, 1, args);
+}
+
 cudaError_t node_loop_reset(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                             LoopCtl *ctl)
 {
     void *args[] = {(void *)&ctl};
     return add_kernel(n, g, dep, (void *)k_loop_reset, 1, 1, args);
-}
-
-cudaError_t node_if_finite(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                           const LoopCtl *ctl, cudaGraphConditionalHandle h)
-{
-    void *args[] = {(void *)&ctl, (void *)&h};
-    return add_kernel(n, g, dep, (void *)k_if_finite, 1, 1, args);
 }
 
 cudaError_t node_refresh(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,

@@ -103,6 +103,16 @@ struct PressureArgs {
     Wells w;
 };
 
+// Device-side control of the graph-resident sub-iteration loop.
+struct LoopCtl {
+    int k;          // sweeps run so far in this solve
+    int m;          // sweeps per loop body (= check_every)
+    int cap;        // max_sub_iters (a multiple of m)
+    int every;      // sweeps between mid-solve rebases (a multiple of m)
+    double tol;
+    double r;       // last residual
+};
+
 struct RefreshArgs {        // stream g, S^n, 1/tau_f (and the warm start of the next solve)
     const float *gin[9];
     const float *Rin;        // reference pressure of the last step
@@ -113,6 +123,7 @@ struct RefreshArgs {        // stream g, S^n, 1/tau_f (and the warm start of the
     const float *Fs;         // dense F~_s plane or nullptr
     float *inv_tau;
     const float *Sb[4];
+    LoopCtl *ctl;            // loop control that the launch resets for the coming solve, or nullptr
     Geom g;
     Model m;
     Wells w;
@@ -214,14 +225,11 @@ struct ResidualOut {        // written by the finalize kernel
     double sums[4];
 };
 
-// Device-side control of the graph-resident sub-iteration loop.
-struct LoopCtl {
-    int k;          // sweeps run so far in this solve
-    int m;          // sweeps per loop body (= check_every)
-    int cap;        // max_sub_iters (a multiple of m)
-    int every;      // sweeps between mid-solve rebases (a multiple of m)
-    double tol;
-    double r;       // last residual
+// The conditional nodes that a check of the graph loop sets: the loop goes on; the inner loop goes
+// on (it ends where R is to move); R moves; the last residual is a number (the step goes on).
+struct LoopHandles {
+    cudaGraphConditionalHandle loop, inner, rebase, ok;
+    int has_inner, has_rebase, has_ok;
 };
 
 // A whole sub-iteration in one launch (resident.cu): m, cap, every and tol from *ctl when given
@@ -359,16 +367,14 @@ cudaError_t node_pressure_fused(cudaGraphNode_t *n, cudaGraph_t g, const cudaGra
                                 const PressureArgs &a, int T, int W, int H, bool check, int grid);
 cudaError_t node_finalize_loop(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                const double *partials, int nparts, long long nnodes, float *shift,
-                               ResidualOut *out, LoopCtl *ctl, cudaGraphConditionalHandle h,
-                               cudaGraphConditionalHandle h_rebase);
+                               ResidualOut *out, LoopCtl *ctl, const LoopHandles &h);
 void rebase_mid(const RebaseMidArgs &a, int grid, void *stream);
 cudaError_t node_rebase_mid(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                             const RebaseMidArgs &a, int grid);
+cudaError_t node_loop_open(cudaGraphNode_t *n, cudaGraph_t g, const LoopHandles &h);
 cudaError_t node_loop_reset(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                             LoopCtl *ctl);
 // sets the condition of an IF node: 1 when the loop's last residual is a number
-cudaError_t node_if_finite(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                           const LoopCtl *ctl, cudaGraphConditionalHandle h);
 cudaError_t node_refresh(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                          const RefreshArgs &a);
 cudaError_t node_saturation(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,

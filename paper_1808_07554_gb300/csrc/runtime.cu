@@ -308,18 +308,24 @@ ResidentArgs resident_args(lbm2p *h, bool work)
     return s;
 }
 
+// whether a solve of the graph loop may move R
+bool loop_moves(const lbm2p *h) { return h->rebase_every > 0 && h->p.max_sub_iters > h->rebase_every; }
+
 // ---- graph-resident sub-iteration ----------------------------------------------------------
-// Appends to G: reset(ctl) -> event(sw0) -> the first check period -> WHILE{ further check
-// periods } -> event(sw1).  A check period is m = check_every sweeps (single or fused
-// launches), the last with residual partials, then the finalize kernel (it counts the sweeps,
-// keeps r, decides whether the WHILE goes on and whether R first moves to the current P:
-// IF{mid-solve rebase}).  The first period reads f buffer pin and writes the next buffer of the
-// rotation, then ping-pongs between the two buffers other than pin and ends on the third; every
-// later period starts and ends there (m, or m / T fused launches, is even).  So the state the
-// solve starts from is only read, and the solve ends in buffer fnext(pin, 2).  `work`: R and
-// 1/tau_f of the work buffers (a step's solve) or the current ones (a bare solve).  A lattice that
-// stays on chip runs all of this in one kernel, which also sets `ok` (when given) to whether the
-// last residual is a number.
+// Appends to G, after `dep` (nullptr: after a reset of the loop control): the first check period ->
+// WHILE{ further check periods }.  A check period is m = check_every sweeps (single or fused
+// launches), the last with residual partials, then the finalize kernel: it counts the sweeps, keeps
+// r, decides whether the loop goes on and sets `ok` (when given) to whether the last residual is a
+// number.  Where a solve may be longer than rebase_every sweeps, R moves to the current P at every
+// such count: the periods between two moves are an inner WHILE, so that the test for a move costs a
+// conditional node per move, not per period (a conditional node takes about as long as a sweep of a
+// small lattice): WHILE{ open the inner loop -> WHILE{ period } -> IF{ move } }.
+// The first period reads f buffer pin and writes the next buffer of the rotation, then ping-pongs
+// between the two buffers other than pin and ends on the third; every later period starts and ends
+// there (m, or m / T fused launches, is even).  So the state the solve starts from is only read, and
+// the solve ends in buffer fnext(pin, 2).  `work`: R and 1/tau_f of the work buffers (a step's
+// solve) or the current ones (a bare solve).  A lattice that stays on chip runs all of this in one
+// kernel.  With timing on, events around it.
 lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int pin, bool work,
                       cudaGraphNode_t *last, const cudaGraphConditionalHandle *ok)
 {
@@ -332,22 +338,35 @@ lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int p
             s.set_ok = 1;
             s.ok = *ok;
         }
-        CUDA_TRY(h, cudaGraphAddEventRecordNode(&e0, G, dep, dep ? 1 : 0, h->ev_sw0));
-        CUDA_TRY(h, lbm2p_launch::node_resident(&n, G, &e0, pressure_args(h, pin, b2, work), s, h->res_C));
-        CUDA_TRY(h, cudaGraphAddEventRecordNode(&e1, G, &n, 1, h->ev_sw1));
-        *last = e1;
+        if (h->timing) {
+            CUDA_TRY(h, cudaGraphAddEventRecordNode(&e0, G, dep, dep ? 1 : 0, h->ev_sw0));
+            dep = &e0;
+        }
+        CUDA_TRY(h, lbm2p_launch::node_resident(&n, G, dep, pressure_args(h, pin, b2, work), s, h->res_C));
+        *last = n;
+        if (h->timing) {
+            CUDA_TRY(h, cudaGraphAddEventRecordNode(&e1, G, &n, 1, h->ev_sw1));
+            *last = e1;
+        }
         return LBM2P_OK;
     }
     auto dst_of = [&](int src) { return src == b1 ? b2 : b1; };
-    cudaGraphNode_t reset, ev0, first_end, wn, ev1;
-    CUDA_TRY(h, lbm2p_launch::node_loop_reset(&reset, G, dep, h->ctl));
-    CUDA_TRY(h, cudaGraphAddEventRecordNode(&ev0, G, &reset, 1, h->ev_sw0));
+    cudaGraphNode_t start, ev0, first_end, wn, ev1;
+    if (dep)
+        start = *dep;
+    else
+        CUDA_TRY(h, lbm2p_launch::node_loop_reset(&start, G, nullptr, h->ctl));
+    if (h->timing) {
+        CUDA_TRY(h, cudaGraphAddEventRecordNode(&ev0, G, &start, 1, h->ev_sw0));
+        start = ev0;
+    }
+    const bool moves = loop_moves(h);
     cudaGraphConditionalHandle hd;
     CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hd, G, 1, cudaGraphCondAssignDefault));
     // one check period into graph g after node `after` (nullptr: none), its first launch
-    // reading buffer `first`, the mid-solve rebase conditioned on handle hr
-    auto period = [&](cudaGraph_t g, cudaGraphNode_t after, int first,
-                      cudaGraphConditionalHandle hr, cudaGraphNode_t *out) -> lbm2p_status {
+    // reading buffer `first`, its finalize setting the conditional nodes lh
+    auto period = [&](cudaGraph_t g, cudaGraphNode_t after, int first, const LoopHandles &lh,
+                      cudaGraphNode_t *out) -> lbm2p_status {
         cudaGraphNode_t prev = after;
         int src = first;
         int nparts = sweep_nparts(h);
@@ -385,40 +404,76 @@ lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int p
                 src = dst_of(src);
             }
         }
-        // finalize decides whether to continue, and whether R moves to the current P first
-        cudaGraphNode_t fin, ifn, rb;
-        CUDA_TRY(h, lbm2p_launch::node_finalize_loop(&fin, g, &prev, h->partials, nparts,
-                                                     h->nnodes, h->shift, h->res, h->ctl, hd, hr));
+        CUDA_TRY(h, lbm2p_launch::node_finalize_loop(out, g, &prev, h->partials, nparts,
+                                                     h->nnodes, h->shift, h->res, h->ctl, lh));
+        return LBM2P_OK;
+    };
+    // IF{ move of R } on handle hr after node `after` of graph g
+    auto move = [&](cudaGraph_t g, cudaGraphNode_t after, cudaGraphConditionalHandle hr,
+                    cudaGraphNode_t *out) -> lbm2p_status {
         cudaGraphNodeParams ip{};
         ip.type = cudaGraphNodeTypeConditional;
         ip.conditional.handle = hr;
         ip.conditional.type = cudaGraphCondTypeIf;
         ip.conditional.size = 1;
-        CUDA_TRY(h, cudaGraphAddNode(&ifn, g, &fin, nullptr, 1, &ip));
+        CUDA_TRY(h, cudaGraphAddNode(out, g, &after, nullptr, 1, &ip));
+        cudaGraphNode_t rb;
         CUDA_TRY(h, lbm2p_launch::node_rebase_mid(&rb, ip.conditional.phGraph_out[0], nullptr,
                                                   rebase_mid_args(h, b2, work), h->grid));
-        *out = ifn;
         return LBM2P_OK;
     };
-    cudaGraphConditionalHandle hr0;
-    CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hr0, G, 0, 0));
-    lbm2p_status e = period(G, ev0, pin, hr0, &first_end);
-    if (e != LBM2P_OK)
+    auto loop = [&](cudaGraph_t g, const cudaGraphNode_t *after, cudaGraphConditionalHandle hl,
+                    cudaGraphNode_t *out, cudaGraph_t *body) -> lbm2p_status {
+        cudaGraphNodeParams cp{};
+        cp.type = cudaGraphNodeTypeConditional;
+        cp.conditional.handle = hl;
+        cp.conditional.type = cudaGraphCondTypeWhile;
+        cp.conditional.size = 1;
+        CUDA_TRY(h, cudaGraphAddNode(out, g, after, nullptr, after ? 1 : 0, &cp));
+        *body = cp.conditional.phGraph_out[0];
+        return LBM2P_OK;
+    };
+    LoopHandles lh{};
+    lh.loop = hd;
+    if (ok) {
+        lh.ok = *ok;
+        lh.has_ok = 1;
+    }
+    lbm2p_status e;
+    cudaGraph_t body;
+    cudaGraphNode_t n;
+    if (moves) {
+        cudaGraphConditionalHandle hr0, hr, hi;
+        CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hr0, G, 0, 0));
+        LoopHandles first = lh;
+        first.rebase = hr0;
+        first.has_rebase = 1;
+        if ((e = period(G, start, pin, first, &n)) != LBM2P_OK ||
+            (e = move(G, n, hr0, &first_end)) != LBM2P_OK ||
+            (e = loop(G, &first_end, hd, &wn, &body)) != LBM2P_OK)
+            return e;
+        CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hi, body, 0, 0));
+        CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hr, body, 0, 0));
+        lh.inner = hi;
+        lh.rebase = hr;
+        lh.has_inner = lh.has_rebase = 1;
+        cudaGraph_t inner;
+        cudaGraphNode_t open, wi, end;
+        CUDA_TRY(h, lbm2p_launch::node_loop_open(&open, body, lh));
+        if ((e = loop(body, &open, hi, &wi, &inner)) != LBM2P_OK ||
+            (e = period(inner, nullptr, b2, lh, &n)) != LBM2P_OK ||
+            (e = move(body, wi, hr, &end)) != LBM2P_OK)
+            return e;
+    } else if ((e = period(G, start, pin, lh, &first_end)) != LBM2P_OK ||
+               (e = loop(G, &first_end, hd, &wn, &body)) != LBM2P_OK ||
+               (e = period(body, nullptr, b2, lh, &n)) != LBM2P_OK) {
         return e;
-    cudaGraphNodeParams cp{};
-    cp.type = cudaGraphNodeTypeConditional;
-    cp.conditional.handle = hd;
-    cp.conditional.type = cudaGraphCondTypeWhile;
-    cp.conditional.size = 1;
-    CUDA_TRY(h, cudaGraphAddNode(&wn, G, &first_end, nullptr, 1, &cp));
-    cudaGraph_t body = cp.conditional.phGraph_out[0];
-    cudaGraphConditionalHandle hr;
-    CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hr, body, 0, 0));
-    cudaGraphNode_t body_end;
-    if ((e = period(body, nullptr, b2, hr, &body_end)) != LBM2P_OK)
-        return e;
-    CUDA_TRY(h, cudaGraphAddEventRecordNode(&ev1, G, &wn, 1, h->ev_sw1));
-    *last = ev1;
+    }
+    *last = wn;
+    if (h->timing) {
+        CUDA_TRY(h, cudaGraphAddEventRecordNode(&ev1, G, &wn, 1, h->ev_sw1));
+        *last = ev1;
+    }
     return LBM2P_OK;
 }
 
@@ -450,23 +505,21 @@ lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
         cudaGraph_t G;
         CUDA_TRY(h, cudaGraphCreate(&G, 0));
         h->step_g[pin][pg][r] = G;
-        cudaGraphNode_t nr, last, nf, ifn, ns;
-        CUDA_TRY(h, lbm2p_launch::node_refresh(&nr, G, nullptr, refresh_args(h, pg)));
+        cudaGraphNode_t nr, last, ifn, ns;
+        RefreshArgs ra = refresh_args(h, pg);
+        ra.ctl = h->ctl;
+        CUDA_TRY(h, lbm2p_launch::node_refresh(&nr, G, nullptr, ra));
         cudaGraphConditionalHandle hok;
         CUDA_TRY(h, cudaGraphConditionalHandleCreate(&hok, G, 0, 0));
         lbm2p_status e = add_loop(h, G, &nr, pin, true, &last, &hok);
         if (e != LBM2P_OK)
             return e;
-        if (h->res_C > 0)
-            nf = last;
-        else
-            CUDA_TRY(h, lbm2p_launch::node_if_finite(&nf, G, &last, h->ctl, hok));
         cudaGraphNodeParams ip{};
         ip.type = cudaGraphNodeTypeConditional;
         ip.conditional.handle = hok;
         ip.conditional.type = cudaGraphCondTypeIf;
         ip.conditional.size = 1;
-        CUDA_TRY(h, cudaGraphAddNode(&ifn, G, &nf, nullptr, 1, &ip));
+        CUDA_TRY(h, cudaGraphAddNode(&ifn, G, &last, nullptr, 1, &ip));
         cudaGraph_t tail = ip.conditional.phGraph_out[0];
         const int pout = fnext(pin, 2);
         CUDA_TRY(h, lbm2p_launch::node_saturation(&ns, tail, nullptr,
@@ -488,10 +541,11 @@ lbm2p_status read_loop(lbm2p *h, int *k, double *r, float *sweep_ms)
     const int m = h->p.check_every;
     const int per_launch = h->tb_T_graph > 1 ? h->tb_T_graph : 1;
     h->sweeps += *k;
-    // reset, sweep launches, finalizes, mid-solve rebases; or the one launch of the whole solve
+    // sweep launches, finalizes, mid-solve rebases and openings of the inner loop; or the one launch
+    // of the whole solve
     h->launches += h->res_C > 0 ? 1
-                                : 1 + *k / per_launch + *k / m +
-                                      (h->rebase_every > 0 && *k > 0 ? (*k - 1) / h->rebase_every : 0);
+                                : *k / per_launch + *k / m +
+                                      (loop_moves(h) && *k > 0 ? (*k > m) + 2 * ((*k - 1) / h->rebase_every) : 0);
     if (sweep_ms) {
         *sweep_ms = -1.0f;
         if (h->timing)
@@ -790,6 +844,7 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
         if ((e = solve_graph(h, pin, &x)) != LBM2P_OK)
             return e;
         CUDA_TRY(h, cudaGraphLaunch(x, st));
+        h->launches += h->res_C > 0 ? 0 : 1;   // reset of the loop control
         float ms = -1.0f;
         if ((e = read_loop(h, &k, &r, &ms)) != LBM2P_OK)
             return e;
@@ -913,9 +968,7 @@ lbm2p_status one_step(lbm2p *h, int replay, lbm2p_step_stats *stats)
         if ((e = read_loop(h, &k, &r, &sw_ms)) != LBM2P_OK)
             return e;
         const bool finite = !std::isnan(r);
-        // refresh and the finiteness test (a launch of its own unless the solve is one); saturation
-        // when the step goes on
-        h->launches += (finite ? 3 : 2) - (h->res_C > 0 ? 1 : 0);
+        h->launches += finite ? 2 : 1;         // refresh; saturation when the step goes on
         if (h->timing)
             CUDA_TRY(h, cudaEventElapsedTime(&step_ms, h->ev_step0, h->ev_step1));
         lbm2p_status ps = loop_status(h, k, r);
@@ -2173,7 +2226,12 @@ lbm2p_status lbm2p_set_timing(lbm2p *h, int enable)
 {
     if (!h)
         return fail(nullptr, LBM2P_EINVAL, "NULL handle");
-    h->timing = enable != 0;
+    if (h->timing != (enable != 0)) {
+        // the solve graphs record the events only where timing is on; rebuilt on the next solve
+        CUDA_TRY(h, cudaStreamSynchronize((cudaStream_t)h->stream));
+        drop_graphs(h);
+        h->timing = enable != 0;
+    }
     return LBM2P_OK;
 }
 

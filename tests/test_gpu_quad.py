@@ -54,3 +54,26 @@ def test_four_sweeps_equal_single_sweeps(nx, ny, bc, dense):
         assert r4 == pytest.approx(r1, rel=1e-3, abs=1e-30)
     one.close()
     four.close()
+
+
+@pytest.mark.parametrize("every, cap", [(8, 1024), (8, 1032), (8, 2056), (16, 3088), (1024, 3072)])
+@pytest.mark.parametrize("fuse", [1, 4])
+def test_graph_loop_equals_replay_across_moves_of_R(every, cap, fuse):
+    """A solve of `cap` sweeps by the graph loop (the residual never meets the tolerance), with the
+    reference pressure moved after 1024 and 2048 sweeps or, at 1024, never, against the same count
+    driven from the host; then a second step, whose loop starts from the first one's conditions."""
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(cap)
+    nx, ny = 70, 33
+    prob = uniform(nx, ny, bc=(1, 1, 1, 1), K=np.exp(rng.standard_normal((ny, nx))), S0=0.4,
+                   wells=[(0, 0, 1e-2, 0), (nx - 1, ny - 1, 1e-2, 1)])
+    make = lambda: pkg.Solver.from_problem(prob, init_replay=16, check_every=every,   # noqa: E731
+                                           max_sub_iters=cap, tol=0.0, fuse_sweeps=fuse)
+    a, b = make(), make()
+    for _ in range(2):
+        st, stats = a.step(1)
+        assert st == pkg.ENOTCONVERGED and stats[0].sub_iters == cap
+        b.step(1, replay=[cap])
+        assert np.array_equal(a.get_state(), b.get_state())
+    a.close()
+    b.close()

@@ -170,7 +170,7 @@ struct ConvArgs {
 // load/store unit 60 to 80 % busy), one thread issues the MMAs (descriptors by additions), four warps
 // read the accumulator, of which there are two, apply bias, activation and mask and store whole pixels
 // through a padded row per warp.
-// 1024^2 pixels, 32 -> 32 channels: 80 us with all three in turn in one set of warps.
+// 1024^2 pixels, 32 -> 32 channels: 80 us with all three in turn in one set of warps, 56 us so.
 constexpr int kRowPix = 130;                        // staged pixels per row
 constexpr uint32_t kChunkBytes = kRowPix * 16;      // one channel chunk of a staged row
 constexpr int kCvCopiers = 8, kCvEpilogue = 4;      // warps 0-7, 8-11; warp 12 issues the MMAs
@@ -748,16 +748,16 @@ __device__ __forceinline__ float unit_scale(float v)
 
 // Sums of a - b and (a - b)^2.  The difference of two floats is a pair of floats exactly, and so its
 // square to 2^-48: each thread adds pairs, the squares scaled by a power of two that follows its
-// largest difference (so they cover the range that FP64 would), and the block's totals are added in
-// FP64.  The FP64 units, a 64th as many, took 27 us for a 1024^2 plane.
-__global__ void k_diff_stats(const float *a, const float *b, long long n, double *st)
-{
-    __shared__ double red[2][8];
+// largest difference (so they cover the range that FP64 would); a warp adds its lanes' pairs at the
+// scale of the largest, and one lane turns them into FP64, which the block and the grid add.  FP64
+// per element took 27 us for a 1024^2 plane, FP64 per thread 32 us (an FP64 instruction holds its SM
+// for 16 cycles, and every warp ran forty), this 7.4 us.  VEC: 128-bit loads (both planes aligned).
+struct DiffSums {
     float2 s1 = make_float2(0.0f, 0.0f), s2 = make_float2(0.0f, 0.0f);
     float sc = 0.0f;                                          // scale of s2's terms (0: none yet)
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x) {
-        const float x = a[i], y = b[i];
+
+    __device__ __forceinline__ void add(float x, float y)
+    {
         const float h = __fsub_rn(x, y), yy = __fsub_rn(x, h);
         const float l = __fsub_rn(__fsub_rn(x, __fadd_rn(h, yy)), __fsub_rn(y, yy));
         pair_add(s1, h, l);
@@ -772,20 +772,57 @@ __global__ void k_diff_stats(const float *a, const float *b, long long n, double
         const float v = l * sc, q = __fmul_rn(u, u);
         pair_add(s2, q, fmaf(2.0f * u, v, fmaf(u, u, -q)));
     }
-    const double is = sc > 0.0f ? 1.0 / (double)sc : 0.0;
-    double t1 = (double)s1.x + (double)s1.y, t2 = ((double)s2.x + (double)s2.y) * is * is;
-    for (int o = 16; o > 0; o >>= 1) {
-        t1 += __shfl_xor_sync(0xffffffffu, t1, o);
-        t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+
+    // the sums of the warp in every lane
+    __device__ __forceinline__ void warp_sum()
+    {
+        float low = sc > 0.0f ? sc : __int_as_float(0x7f800000);
+        for (int o = 16; o > 0; o >>= 1)
+            low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
+        const float f = sc > 0.0f ? low / sc : 0.0f;          // at most 1, a power of two
+        s2 = make_float2(s2.x * f * f, s2.y * f * f);
+        sc = isinf(low) ? 0.0f : low;
+        for (int o = 16; o > 0; o >>= 1) {
+            const float a = __shfl_xor_sync(0xffffffffu, s1.x, o), b = __shfl_xor_sync(0xffffffffu, s1.y, o);
+            const float c = __shfl_xor_sync(0xffffffffu, s2.x, o), d = __shfl_xor_sync(0xffffffffu, s2.y, o);
+            pair_add(s1, a, b);
+            pair_add(s2, c, d);
+        }
     }
+};
+
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_diff_stats(const float *a, const float *b, long long n, double *st)
+{
+    __shared__ double red[2][8];
+    DiffSums d;
+    const long long t0 = blockIdx.x * 256LL + threadIdx.x, step = gridDim.x * 256LL;
+    if (VEC) {
+        const long long nq = n / 4;
+#pragma unroll 2
+        for (long long i = t0; i < nq; i += step) {
+            const float4 x = reinterpret_cast<const float4 *>(a)[i], y = reinterpret_cast<const float4 *>(b)[i];
+            d.add(x.x, y.x);
+            d.add(x.y, y.y);
+            d.add(x.z, y.z);
+            d.add(x.w, y.w);
+        }
+        if (t0 < n - 4 * nq)
+            d.add(a[4 * nq + t0], b[4 * nq + t0]);
+    } else {
+        for (long long i = t0; i < n; i += step)
+            d.add(a[i], b[i]);
+    }
+    d.warp_sum();
     if ((threadIdx.x & 31) == 0) {
-        red[0][threadIdx.x >> 5] = t1;
-        red[1][threadIdx.x >> 5] = t2;
+        const double is = d.sc > 0.0f ? 1.0 / (double)d.sc : 0.0;
+        red[0][threadIdx.x >> 5] = (double)d.s1.x + (double)d.s1.y;
+        red[1][threadIdx.x >> 5] = ((double)d.s2.x + (double)d.s2.y) * is * is;
     }
     __syncthreads();
     if (threadIdx.x < 2) {
         double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
+        for (int w = 0; w < 8; ++w)
             t += red[threadIdx.x][w];
         atomicAdd(st + threadIdx.x, t);
     }
@@ -1090,7 +1127,14 @@ lbm2p_status lbm2p_op_diff_stats(const float *a, const float *b, long long n, do
 {
     if (!a || !b || !stats || n < 1)
         return set_global_error(LBM2P_EINVAL, "diff_stats: bad arguments");
-    k_diff_stats<<<grid_for(n, 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a, b, n, stats);
+    // a block adds 4096 differences at least (its FP64 end costs as much as some 2000), and the grid
+    // fills the SMs four times at most
+    long long blocks = (n + 4095) / 4096;
+    blocks = blocks < 4LL * sm_count() ? blocks : 4LL * sm_count();
+    if (aligned16(a) && aligned16(b))
+        k_diff_stats<true><<<(unsigned)blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a, b, n, stats);
+    else
+        k_diff_stats<false><<<(unsigned)blocks, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a, b, n, stats);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
         return set_global_error(LBM2P_ECUDA, "diff_stats launch failed: %s", cudaGetErrorString(e));

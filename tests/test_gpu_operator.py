@@ -209,3 +209,25 @@ def test_learned_warm_start_loop_keeps_the_solution(env):
     op.check()
     assert W.rel_l2(learned.fields()[1], plain.fields()[1]) < 1e-5
     assert np.all(np.isfinite(lw.Ppred.cpu().numpy()))
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 31, 4095, 4097, 8193, 300 * 140, 3_000_001])
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("spread", [0, 30])
+def test_diff_stats_sums(n, offset, spread):
+    """Sums of a - b and (a - b)^2 against FP64, for aligned planes and planes that are not, with
+    differences of one size and of sizes 2^-30 to 2^30.  Pairs of floats carry 2^-47 per addition and
+    a lane adds a few thousand terms at most: 2^-35 of the sum of magnitudes."""
+    import torch
+    import paper_1808_07554_gb300 as pkg
+    gen = torch.Generator(device="cuda").manual_seed(n + offset)
+    rand = lambda: torch.rand(n + offset, generator=gen, device="cuda") - 0.5    # noqa: E731
+    scale = torch.exp2((rand() * 2 * spread).round())
+    a, b = (rand() * scale)[offset:], (rand() * scale)[offset:]
+    st = torch.zeros(2, dtype=torch.float64, device="cuda")
+    pkg.lbm2p_op_diff_stats(a.data_ptr(), b.data_ptr(), n, st.data_ptr(),
+                            torch.cuda.current_stream().cuda_stream)
+    d = a.double() - b.double()
+    want = torch.stack([d.sum(), (d * d).sum()])
+    size = torch.stack([d.abs().sum(), (d * d).sum()])
+    assert ((st - want).abs() <= 2.0 ** -35 * size + 1e-300).all(), (st, want)

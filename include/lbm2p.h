@@ -375,15 +375,15 @@ void lbm2p_batch_destroy(lbm2p_batch *b);
  *   residual host double: r = ||dP_new - dP_old - mean|| / ||P_new - mean P_new||.
  * pitch is a multiple of 4 floats and every plane pointer is 16-byte aligned.  Wells are
  * not taken: put their sources into Fp.
- * Memory: allocates nothing.  The residual scratch (four FP64 partials per row tile of 1024
- * nodes, the finalize output and two shifts) is a static device array sized for
- * LBM2P_NOALLOC_MAX_TILES tiles (2 MiB), held by every GPU that loads the library until the
- * process exits; lattices with more row tiles (ceil(nx / 1024) * ny) are rejected with
+ * Memory: allocates nothing.  The residual scratch (four FP64 partials per block and the
+ * finalize output) is a static device array sized for LBM2P_NOALLOC_MAX_TILES blocks (2 MiB),
+ * held by every GPU that loads the library until the process exits; lattices with more than as
+ * many row tiles (a row tile of 1024 nodes: ceil(nx / 1024) * ny) are rejected with
  * LBM2P_EINVAL before anything is launched.  The first call on each device (and again the
  * first after that device's context is re-created, e.g. by cudaDeviceReset) looks up the
- * array's device address with that device current.  Every call shares the one array and
- * each call clears what must start at zero, so calls whose work overlaps on the GPU (other
- * streams, other host threads) race on it: serialise them.  Each call synchronises `stream`
+ * array's device address with that device current.  Every call shares the one array, so calls
+ * whose work overlaps on the GPU (other streams, other host threads) race on it: serialise
+ * them.  Each call synchronises `stream`
  * (a cudaStream_t) to return the residual to the host, so it cannot be used inside a stream
  * capture.  Errors: lbm2p_last_error(NULL) describes the failure. */
 #define LBM2P_NOALLOC_MAX_TILES 65536

@@ -112,9 +112,9 @@ def load_library(path: str = LIB_PATH):
         "lbm2p_autotune_report": (C.c_char_p, [H]),
         "lbm2p_warm_start": (C.c_int, [H, fp, C.c_int]),
         "lbm2p_pressure_sweep_noalloc": (C.c_int, [C.c_int, C.c_int, C.c_int, C.POINTER(C.c_int),
-                                                   C.POINTER(fp), C.POINTER(fp), fp, fp, fp,
-                                                   C.POINTER(fp), fp, C.POINTER(C.c_double),
-                                                   C.c_void_p]),
+                                                   C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
+                                                   C.c_void_p, C.c_void_p, C.c_void_p,
+                                                   C.POINTER(C.c_double), C.c_void_p]),
         "lbm2p_batch_create": (C.c_int, [C.POINTER(H), C.POINTER(H), C.c_int]),
         "lbm2p_batch_step": (C.c_int, [H, C.c_int, C.POINTER(C.c_int),
                                        C.POINTER(lbm2p_step_stats)]),
@@ -237,19 +237,19 @@ def lbm2p_counters(h):
     return a.value, b.value
 
 
+_PLANES, _TRACES, _WALLS = C.c_void_p * 8, C.c_void_p * 4, C.c_int * 4
+
+
 def lbm2p_pressure_sweep_noalloc(nx, ny, pitch, bc, n_in, n_out, R, inv_tau, Fp, P_b, dP,
                                  stream=None):
     """Device pointers (ints) in, residual out; allocates nothing (see include/lbm2p.h)."""
-    fp = C.POINTER(C.c_float)
-    cast = lambda p: C.cast(C.c_void_p(p), fp) if p else None
-    bcs = (C.c_int * 4)(*[int(b) for b in bc])
-    nin = (fp * 8)(*[cast(p) for p in n_in])
-    nout = (fp * 8)(*[cast(p) for p in n_out])
-    pb = (fp * 4)(*[cast(p) for p in (P_b if P_b is not None else [0, 0, 0, 0])])
+    # addresses go to C as they are: a typed pointer object for each of the 20 planes and traces
+    # took longer than the sweep of a small lattice
     r = C.c_double(0.0)
     st = _lib_or_raise().lbm2p_pressure_sweep_noalloc(
-        int(nx), int(ny), int(pitch), bcs, nin, nout, cast(R), cast(inv_tau), cast(Fp), pb,
-        cast(dP), C.byref(r), C.c_void_p(stream) if stream else None)
+        int(nx), int(ny), int(pitch), _WALLS(*[int(b) for b in bc]), _PLANES(*n_in), _PLANES(*n_out),
+        R or None, inv_tau or None, Fp or None, _TRACES(*(P_b if P_b is not None else ())), dP or None,
+        C.byref(r), stream or None)
     _check(st, None)
     return r.value
 

@@ -56,7 +56,8 @@ constexpr int kFinThreads = 256;
 
 // r = ||dP - mean dP|| / ||P - mean P|| from nparts partials of four sums each (FP64, in an order
 // fixed by nparts).  CL blocks of kFinThreads threads; true in the lanes of warp 0 of block 0, where
-// lane 0 holds r.  Updates shift (the constants that the next check subtracts) and, when given, out.
+// lane 0 holds r.  Updates shift (the constants that this check subtracted and the next
+// will; nullptr: none) and, when given, out.
 template <int CL>
 __device__ __forceinline__ bool finalize_residual(const double *__restrict__ partials, int nparts,
                                                   long long nnodes, float *shift, ResidualOut *out,
@@ -115,10 +116,10 @@ __device__ __forceinline__ bool finalize_residual(const double *__restrict__ par
     const double den = __shfl_sync(0xffffffffu, var, 1);
     r = !finite ? nan("") : (den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0));
     if (lane < 2) {
-        const double base = (double)shift[1 - lane] + mean;
+        const double base = (shift ? (double)shift[1 - lane] : 0.0) + mean;
         if (out && lane == 1)
             out->mean_P = base;
-        if (finite)
+        if (finite && shift)
             shift[1 - lane] = (float)base;
     }
     if (out) {

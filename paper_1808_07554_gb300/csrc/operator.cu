@@ -157,25 +157,27 @@ struct ConvArgs {
 
 // ---- convolution on staged rows ----------------------------------------------------------
 // A tile is 128 consecutive pixels of one image row (x0 .. x0 + 127, the last tile of a row
-// ragged).  Its three input rows y - 1 .. y + 1, pixels x0 - 1 .. x0 + 128, are copied into shared
-// memory as channel-chunk planes: chunk c (channels 8 c .. 8 c + 7) of staged row r is an array of
-// 130 pixels x 16 bytes.  In that layout the A operand of tap (dy, dx) and K-half j is the K-major
-// core-matrix matrix that starts at row dy + 1, chunk 2 j, pixel dx + 1: a shift by one pixel is a
-// shift of the descriptor's start address by 16 bytes, so all 9 x C_in / 16 MMAs of a tile read the
-// same staged rows.
+// ragged).  A CTA works down a strip of 128 columns, so its ring holds input rows, each copied once
+// and read by the three tiles that it borders: pixels x0 - 1 .. x0 + 128 of a row as channel-chunk
+// planes, chunk c (channels 8 c .. 8 c + 7) an array of 130 pixels x 16 bytes.  In that layout the A
+// operand of tap (dy, dx) and K-half j is the K-major core-matrix matrix that starts at row
+// dy + 1, chunk 2 j, pixel dx + 1: a shift by one pixel is a shift of the descriptor's start address
+// by 16 bytes.  Rows above and below an image are zero: their taps are left out.
 //
 // The three stages of a tile run in different warps, handed on by mbarriers: eight warps copy (whole
-// pixels, a warp 512 contiguous bytes, the next tile's loads in registers while this one's are
+// pixels, a warp 512 contiguous bytes, the next three rows' loads in registers while one is
 // stored: cp.async with a chunk plane as its target makes a request of every 16 bytes and kept the
 // load/store unit 60 to 80 % busy), one thread issues the MMAs (descriptors by additions), four warps
 // read the accumulator, of which there are two, apply bias, activation and mask and store whole pixels
 // through a padded row per warp.
-// 1024^2 pixels, 32 -> 32 channels: 80 us with all three in turn in one set of warps, 56 us so.
+// 1024^2 pixels, 32 -> 32 channels: 80 us with all three in turn in one set of warps, 56 us in three
+// with every tile's three rows copied anew (the load/store unit's data path 64 % busy), 46 us so.
 constexpr int kRowPix = 130;                        // staged pixels per row
 constexpr uint32_t kChunkBytes = kRowPix * 16;      // one channel chunk of a staged row
 constexpr int kCvCopiers = 8, kCvEpilogue = 4;      // warps 0-7, 8-11; warp 12 issues the MMAs
 constexpr int kCvThreads = 32 * (kCvCopiers + kCvEpilogue + 1);
-constexpr int kCvStages = 3;
+constexpr int kCvRows = 8;                          // input rows in the ring
+constexpr int kCvAhead = 4;                         // rows that a copying lane has in registers
 constexpr uint32_t kCvTmemCols = 64;                // two accumulators of 32 columns
 
 // 16 bytes of padding per pixel row of the output tile of a warp
@@ -185,9 +187,42 @@ __host__ __device__ constexpr uint32_t conv_out_row() { return COUT * 2 + 16; }
 template <int CIN, int COUT>
 __host__ __device__ constexpr size_t conv_rows_smem_bytes()
 {
-    return (size_t)(9 * CIN / 16) * COUT * 32 + kCvStages * (size_t)3 * (CIN / 8) * kChunkBytes +
-           (size_t)kCvEpilogue * 32 * conv_out_row<COUT>() + (2 * kCvStages + 4) * 8 + 16 + 128;
+    return (size_t)(9 * CIN / 16) * COUT * 32 + kCvRows * (size_t)(CIN / 8) * kChunkBytes +
+           (size_t)kCvEpilogue * 32 * conv_out_row<COUT>() + (2 * kCvRows + 4) * 8 + 16 + 128;
 }
+
+// A CTA's tiles: `left` of them from row r of strip `strip` on, down the rows of all images and on
+// to the next strip.  A segment is the part in one strip: tiles r .. r + n - 1, which read the input
+// rows lo .. hi (the first and last rows of an image beside them included, read or not).
+struct ConvWalk {
+    long long rows;                                 // of all images
+    long long r, lo, hi;
+    int strip;
+    unsigned n, left;
+
+    __device__ __forceinline__ void open()
+    {
+        const long long room = rows - r;
+        n = (long long)left < room ? left : (unsigned)room;
+        left -= n;
+        lo = r > 0 ? r - 1 : 0;
+        hi = r + n < rows ? r + n : rows - 1;
+    }
+    __device__ __forceinline__ ConvWalk(long long first, unsigned count, long long rows_)
+        : rows(rows_), r(first % rows_), strip((int)(first / rows_)), left(count)
+    {
+        open();
+    }
+    __device__ __forceinline__ bool next()
+    {
+        if (left == 0)
+            return false;
+        r = 0;
+        ++strip;
+        open();
+        return true;
+    }
+};
 
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(kCvThreads, 2) k_conv3x3_rows(const ConvArgs a)
@@ -196,16 +231,16 @@ __global__ void __launch_bounds__(kCvThreads, 2) k_conv3x3_rows(const ConvArgs a
     constexpr int KH = CIN / 16;                      // K-halves of 16 channels per tap
     constexpr int KS = 9 * KH;
     constexpr uint32_t kBBytes = COUT * 16 * 2;
-    constexpr uint32_t kStageBytes = 3 * CH * kChunkBytes;
+    constexpr uint32_t kRowBytes = CH * kChunkBytes;
     constexpr uint32_t IDESC = idesc_bf16(128, COUT);
     constexpr uint32_t ORow = conv_out_row<COUT>();
-    constexpr int R = kCvStages;
+    constexpr unsigned R = kCvRows;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
     unsigned char *wsm = smem;
     unsigned char *stg = smem + KS * kBBytes;
-    unsigned char *osm = stg + R * kStageBytes;
-    // full[s] / empty[s]: stage s copied / read; done[d] / taken[d]: accumulator d ready / read
+    unsigned char *osm = stg + R * kRowBytes;
+    // full[s] / empty[s]: ring row s copied / read; done[d] / taken[d]: accumulator d ready / read
     uint64_t *full = reinterpret_cast<uint64_t *>(osm + kCvEpilogue * 32 * ORow);
     uint64_t *empty = full + R, *done = empty + R, *taken = done + 2;
     uint32_t *tslot = reinterpret_cast<uint32_t *>(taken + 2);
@@ -231,7 +266,7 @@ __global__ void __launch_bounds__(kCvThreads, 2) k_conv3x3_rows(const ConvArgs a
     if (tid == 0) {
         failed = 0;
         issued = 0;
-        for (int i = 0; i < R; ++i) {
+        for (unsigned i = 0; i < R; ++i) {
             bar_init(full + i, kCvCopiers);
             bar_init(empty + i, 1);
         }
@@ -246,111 +281,144 @@ __global__ void __launch_bounds__(kCvThreads, 2) k_conv3x3_rows(const ConvArgs a
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tslot;
-    const unsigned tiles_x = (unsigned)(a.W + 127) / 128u;
-    const long long tiles = (long long)a.nimg * a.H * tiles_x;
-    const unsigned count = tiles > (long long)blockIdx.x
-                               ? (unsigned)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0u;
-    // image row (over all images) and first pixel of this CTA's tile n
-    auto tile_at = [&](unsigned n, long long &row, int &x0) {
-        const long long t = blockIdx.x + (long long)n * gridDim.x;
-        row = tiles < 0x7fffffffLL ? (long long)((unsigned)t / tiles_x) : t / tiles_x;
-        x0 = (int)(t - row * tiles_x) * 128;
-    };
+    const long long rows = (long long)a.nimg * a.H, tiles = rows * ((a.W + 127) / 128);
+    const long long first = tiles * blockIdx.x / gridDim.x;
+    const unsigned count = (unsigned)(tiles * (blockIdx.x + 1) / gridDim.x - first);
     bool ok = true;
     if (warp == kMmaWarp) {
         if (lane == 0) {
             // descriptors: start addresses count 16 bytes
             const uint64_t ad0 = sdesc(smem_u32(stg), kChunkBytes, 128);
             const uint64_t bd0 = sdesc(smem_u32(wsm), COUT * 16, 128);
-            for (unsigned n = 0; n < count; ++n) {
-                ok = wait_bounded(full + n % R, (n / R) & 1u) &&
-                     (n < 2 || wait_bounded(taken + (n & 1u), ((n >> 1) + 1u) & 1u));
-                if (!ok)
-                    break;
-                tc_fence_after();
-                const uint64_t ad = ad0 + (n % R) * (kStageBytes >> 4);
-                const uint32_t d = tmem + 32u * (n & 1u);
+            unsigned waited = 0, released = 0, n = 0;  // ring rows, tiles
+            auto wait_to = [&](unsigned k) {          // ring rows up to k are there
+                for (; ok && waited <= k; ++waited)
+                    ok = wait_bounded(full + waited % R, (waited / R) & 1u);
+            };
+            ConvWalk wk(first, count, rows);
+            unsigned k0 = 0;                          // ring row of the segment's first
+            do {
+                int y = (int)(wk.r % a.H);
+                for (unsigned i = 0; i < wk.n && ok; ++i, ++n) {
+                    const unsigned kc = k0 + (unsigned)(wk.r - wk.lo) + i;   // ring row of the tile's own
+                    const bool up = y > 0, down = y < a.H - 1;
+                    wait_to(down ? kc + 1 : kc);
+                    ok = ok && (n < 2 || wait_bounded(taken + (n & 1u), ((n >> 1) + 1u) & 1u));
+                    if (!ok)
+                        break;
+                    tc_fence_after();
+                    const uint32_t d = tmem + 32u * (n & 1u);
 #pragma unroll
-                for (int t = 0; t < 9; ++t)
+                    for (int dy = 0; dy < 3; ++dy) {
+                        if (dy == 0 ? !up : (dy == 2 && !down))
+                            continue;
+                        const uint64_t ad = ad0 + ((kc + dy - 1) % R) * (kRowBytes >> 4);
 #pragma unroll
-                    for (int j = 0; j < KH; ++j)
-                        umma_bf16(d, ad + ((((t / 3) * CH + 2 * j) * kChunkBytes + (t % 3) * 16) >> 4),
-                                  bd0 + (((t * KH + j) * kBBytes) >> 4), IDESC, t + j > 0 ? 1u : 0u);
-                umma_commit(empty + n % R);
-                umma_commit(done + (n & 1u));
-                issued = n + 1;
-            }
+                        for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                            for (int j = 0; j < KH; ++j)
+                                umma_bf16(d, ad + ((2 * j * kChunkBytes + dx * 16) >> 4),
+                                          bd0 + ((((dy * 3 + dx) * KH + j) * kBBytes) >> 4), IDESC,
+                                          dx + j > 0 || dy == 2 || (dy == 1 && up) ? 1u : 0u);
+                    }
+                    // rows that no later tile of the segment reads go back
+                    const bool end = i + 1 == wk.n;
+                    const unsigned done_to = end ? k0 + (unsigned)(wk.hi - wk.lo) + 1u : kc;
+                    if (end)
+                        wait_to(done_to - 1u);
+                    for (; released < done_to; ++released)
+                        umma_commit(empty + released % R);
+                    umma_commit(done + (n & 1u));
+                    issued = n + 1;
+                    y = down ? y + 1 : 0;
+                }
+                k0 += (unsigned)(wk.hi - wk.lo) + 1u;
+            } while (ok && wk.next());
         }
         __syncwarp();
     } else if (warp < kCvCopiers) {
-        // ---- copies: chunk c of pixels px, px + P, ... of the three rows; the last two pixels of
-        // the rows by the first lanes ----
+        // ---- copies: chunk c of pixels px, px + P, ... of a row; its last two pixels by the first
+        // lanes ----
         constexpr int P = 32 * kCvCopiers / CH;       // pixels per pass
-        constexpr int NP = 128 / P, NV = 3 * NP + 1;
+        constexpr int NP = 128 / P, NV = NP + 1;
         const int c = tid % CH, px = tid / CH;
-        const bool tail = tid < 6 * CH;
-        const int tr = tid / (2 * CH), tpx = 128 + (tid / CH) % 2;
+        const bool tail = tid < 2 * CH;
         const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-        auto fetch = [&](unsigned n, uint4 (&v)[NV]) {
-            long long row;
-            int x0;
-            tile_at(n, row, x0);
-            const int y = row < 0x7fffffffLL ? (int)((unsigned)row % (unsigned)a.H) : (int)(row % a.H);
-            const bf16 *src = a.x + ((row - 1) * a.W + x0 - 1) * CIN + 8 * c;
-            auto get = [&](int r, int p) {
+        ConvWalk wk(first, count, rows);
+        long long row = wk.lo;
+        bool more = true;
+        auto fetch = [&](uint4 (&v)[NV]) {            // the next row
+            if (!more)
+                return;
+            const int x0 = wk.strip * 128;
+            const bf16 *src = a.x + (row * a.W + x0 - 1) * CIN + 8 * c;
+            auto get = [&](int p) {
                 const int xx = x0 - 1 + p;
-                const bool in = (r != 0 || y > 0) && (r != 2 || y < a.H - 1) && xx >= 0 && xx < a.W;
-                return in ? __ldg(reinterpret_cast<const uint4 *>(src + ((long long)r * a.W + p) * CIN)) : zero;
+                return xx >= 0 && xx < a.W ? __ldg(reinterpret_cast<const uint4 *>(src + (long long)p * CIN)) : zero;
             };
 #pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int q = 0; q < NP; ++q)
-                    v[r * NP + q] = get(r, px + q * P);
-            v[NV - 1] = tail ? get(tr, tpx) : zero;
+            for (int q = 0; q < NP; ++q)
+                v[q] = get(px + q * P);
+            v[NP] = tail ? get(128 + px) : zero;
+            if (row < wk.hi) {
+                ++row;
+            } else {
+                more = wk.next();
+                row = wk.lo;
+            }
         };
-        auto hand_over = [&](unsigned n, const uint4 (&v)[NV]) {
-            if (n >= (unsigned)R && !wait_bounded(empty + n % R, (n / R + 1u) & 1u)) {
+        auto hand_over = [&](unsigned k, const uint4 (&v)[NV]) {
+            if (k >= R && !wait_bounded(empty + k % R, (k / R + 1u) & 1u)) {
                 ok = false;
                 return;
             }
-            unsigned char *dst = stg + (n % R) * kStageBytes + c * kChunkBytes;
+            unsigned char *dst = stg + (k % R) * kRowBytes + c * kChunkBytes;
 #pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int q = 0; q < NP; ++q)
-                    *reinterpret_cast<uint4 *>(dst + r * CH * kChunkBytes + (px + q * P) * 16) = v[r * NP + q];
+            for (int q = 0; q < NP; ++q)
+                *reinterpret_cast<uint4 *>(dst + (px + q * P) * 16) = v[q];
             if (tail)
-                *reinterpret_cast<uint4 *>(dst + tr * CH * kChunkBytes + tpx * 16) = v[NV - 1];
+                *reinterpret_cast<uint4 *>(dst + (128 + px) * 16) = v[NP];
             fence_async_smem();
             __syncwarp();
             if (lane == 0)
-                bar_arrive(full + n % R);
+                bar_arrive(full + k % R);
         };
-        uint4 v0[NV], v1[NV];
-        if (count > 0)
-            fetch(0, v0);
-        for (unsigned n = 0; n < count && ok; n += 2) {
-            if (n + 1 < count)
-                fetch(n + 1, v1);
-            hand_over(n, v0);
-            if (n + 1 < count && ok) {
-                if (n + 2 < count)
-                    fetch(n + 2, v0);
-                hand_over(n + 1, v1);
-            }
+        unsigned total = 0;                           // rows of all segments
+        {
+            ConvWalk t(first, count, rows);
+            do
+                total += (unsigned)(t.hi - t.lo) + 1u;
+            while (t.next());
         }
+        uint4 v[kCvAhead][NV];
+#pragma unroll
+        for (int d = 0; d < kCvAhead; ++d)
+            fetch(v[d]);
+        for (unsigned k = 0; k < total && ok; k += kCvAhead)
+#pragma unroll
+            for (int d = 0; d < kCvAhead; ++d)
+                if (k + d < total && ok) {
+                    hand_over(k + d, v[d]);
+                    fetch(v[d]);
+                }
     } else {
         // ---- epilogue: a pixel per lane, 32 lanes of tensor memory per warp ----
         const int w = warp - kCvCopiers;              // = warp % 4, the warp's tensor-memory lanes
         unsigned char *out = osm + w * 32 * ORow;
         // stores: whole pixels, GH lanes each; lane's chunk sc of pixels sp, sp + 32 / GH, ...
         const int sc = lane % GH, sp = lane / GH;
+        ConvWalk wk(first, count, rows);
+        long long row = wk.r - 1;
+        unsigned left = wk.n;                         // tiles of the segment
         for (unsigned n = 0; n < count; ++n) {
-            long long row;
-            int x0;
-            tile_at(n, row, x0);
-            const int xw = x0 + 32 * w;               // the warp's first pixel
+            ++row;
+            if (left == 0) {
+                wk.next();
+                row = wk.r;
+                left = wk.n;
+            }
+            --left;
+            const int xw = wk.strip * 128 + 32 * w;   // the warp's first pixel
             const long long q0 = row * a.W + xw;
             // the mask is on its way while the tensor core works
             uint4 mk[GH];

@@ -1,6 +1,6 @@
 // Batched realisations: many independent lattices (handles made by lbm2p_create) advanced
 // together.  One CUDA graph per physical step runs every member's saturation refresh,
-// pressure sub-iteration and saturation update; each kernel walks one tile list that spans
+// pressure sub-iteration and saturation update; each kernel runs one list of tiles that spans
 // all members, so lattices too small to fill the GPU share it instead of each launching
 // kernels that occupy a fraction of it.  The sub-iteration is a conditional WHILE node: a
 // body runs check_every sweeps of every still-active member, then one block per member

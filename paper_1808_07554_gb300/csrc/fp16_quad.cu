@@ -8,8 +8,10 @@
 // sweep does and the results are the same bit for bit; half the registers of the FP32 form, which
 // the rows of R that every sweep changes take up again.  A pull from a neighbouring column is one
 // shuffle of a packed register and a byte permute.  Arithmetic is FP32 in packed pairs.
-// Four sweeps at 2048^2: 242 us in four launches, 92 us in one (1.35 times the FP32 form's 68: 196 MB,
-// but the conversions and two roundings of R more per node).
+// The row loop is one row with guards for the filling sweeps: 555 instructions, two of which no longer
+// fit the instruction cache nearest to the warps (unrolled by two with straight-line filling rows as
+// the FP32 form is, warps waited for instructions most, 86 us).
+// Four sweeps at 2048^2: 242 us in four launches, 78 us in one.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -264,22 +266,16 @@ struct QuadH {
         return dP;
     }
 
-    static constexpr int NP = GEN ? 1 : 2;    // as Quad: rows unrolled by two, or not
-
-    template <int P>
     __device__ __forceinline__ void keep_row(int s, const unsigned (&v)[8])
     {
         c0[s] = v[0];
         c2[s] = v[2];
-        if (NP == 1) {
-            d1[s][1] = d1[s][0];
-            d4[s][1] = d4[s][0];
-            d5[s][1] = d5[s][0];
-        }
-        constexpr int w = NP == 2 ? P : 0;
-        d1[s][w] = v[1];
-        d4[s][w] = v[4];
-        d5[s][w] = v[5];
+        d1[s][1] = d1[s][0];
+        d4[s][1] = d4[s][0];
+        d5[s][1] = d5[s][0];
+        d1[s][0] = v[1];
+        d4[s][0] = v[4];
+        d5[s][0] = v[5];
         if (GEN) {
             k3[s] = v[3];
             k6[s] = v[6];
@@ -287,7 +283,7 @@ struct QuadH {
         }
     }
 
-    template <int P, int NS>
+    // iteration t: the next input row, sweep 1 at the row before it, sweep s once its rows are there
     __device__ __forceinline__ void row(int t)
     {
         next_row<S - 3>();
@@ -317,44 +313,43 @@ struct QuadH {
         const float2 dP = sweep(n, rw[1][2], rw[1][1], rw[1][0], kp[1], source(1, y), own, y, v);
         __syncwarp();
         issue(q >= 3 ? q - 3 : q + S - 3, t + S);
-        next_sweep<P, NS, 2>(t, v, dP);
+        next_sweep<2>(t, v, dP);
         ++y;
     }
 
     // sweep s of iteration t from sweep s - 1's row v (pressure increment dPp), then the next
-    template <int P, int NS, int s>
+    template <int s>
     __device__ __forceinline__ void next_sweep(int t, const unsigned (&v)[8], float2 dPp)
     {
         push_R(s, __fadd2_rn(rw[s - 1][1].v, dPp));
-        if (s > NS || (GEN && t < 2 * (s - 1))) {
-            keep_row<P>(s - 1, v);
+        if (t < 2 * (s - 1)) {
+            keep_row(s - 1, v);
             return;
         }
-        constexpr int older = NP == 2 ? P : 1, newer = NP == 2 ? 1 - P : 0;
         unsigned n[8], own[8], w[8];
         n[0] = c0[s - 1];
-        n[1] = d1[s - 1][older];
+        n[1] = d1[s - 1][1];
         n[2] = c2[s - 1];
         n[3] = v[3];
-        n[4] = d4[s - 1][older];
-        n[5] = d5[s - 1][older];
+        n[4] = d4[s - 1][1];
+        n[5] = d5[s - 1][1];
         n[6] = v[6];
         n[7] = v[7];
         if (GEN) {
             own[0] = c0[s - 1];
-            own[1] = d1[s - 1][newer];
+            own[1] = d1[s - 1][0];
             own[2] = c2[s - 1];
             own[3] = k3[s - 1];
-            own[4] = d4[s - 1][newer];
-            own[5] = d5[s - 1][newer];
+            own[4] = d4[s - 1][0];
+            own[5] = d5[s - 1][0];
             own[6] = k6[s - 1];
             own[7] = k7[s - 1];
         }
         const int yy = y - s + 1;
         const float2 dP = sweep(n, rw[s][2], rw[s][1], rw[s][0], kp[s], source(s, yy), own, yy, w);
-        keep_row<P>(s - 1, v);
+        keep_row(s - 1, v);
         if constexpr (s < kQuadT) {
-            next_sweep<P, NS, s + 1>(t, w, dP);
+            next_sweep<s + 1>(t, w, dP);
         } else {
             const bool rowin = !GEN || (yy >= ylo && yy < yhi);
             const float2 Rn = __fadd2_rn(rw[s][1].v, dP);
@@ -431,24 +426,9 @@ struct QuadH {
         next_row<S - 1>();
         next_row<S - 2>();
         const int iters = y1 - y0 + 2 * (kQuadT - 1);
-        if (GEN) {
-            for (int t = 0; t < iters; ++t)
-                row<0, kQuadT>(t);
-        } else {
-            row<0, 1>(0);
-            row<1, 1>(1);
-            row<0, 2>(2);
-            row<1, 2>(3);
-            row<0, 3>(4);
-            row<1, 3>(5);
-            int t = 6;
-            for (; t + 1 < iters; t += 2) {
-                row<0, 4>(t);
-                row<1, 4>(t + 1);
-            }
-            if (t < iters)
-                row<0, 4>(t);
-        }
+#pragma unroll 1
+        for (int t = 0; t < iters; ++t)
+            row(t);
         cp_async_wait<0>();
         __syncwarp();
     }

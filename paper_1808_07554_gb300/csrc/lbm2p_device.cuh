@@ -320,9 +320,10 @@ cudaError_t node_pressure_pair_direct(cudaGraphNode_t *n, cudaGraph_t g, const c
 long long quad_grid(int H, int nx, int ny);
 int quad_tile_slots(bool has_fp);      // tiles that run at a time (0: the kernel cannot run)
 cudaError_t quad_prepare();
-void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream);
+// unroll: the interior tiles' row loop unrolled by two
+void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, bool unroll, int grid, void *stream);
 cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                               const PressureArgs &a, bool check, int H, int grid);
+                               const PressureArgs &a, bool check, int H, bool unroll, int grid);
 // four FP16-storage sweeps per launch (fp16_quad.cu) in the same tiles; the planes of a.nin are
 // equally spaced
 int quad_h_slots(bool has_fp);

@@ -18,7 +18,8 @@ struct Alloc {
 // Fused sweeps: T per launch (0 or 1: single sweeps) by kernel kind 0 = k_pressure_tb (shared-
 // memory stages), 1 = k_pressure_rows2 (two sweeps on staged rows), 2 = k_pressure_pair_direct
 // (two sweeps, direct loads), 3 = k_pressure_quad (four sweeps in registers); W columns (kinds 1
-// and 2: 30 x warps) or threads per block, H rows per block, ring slots of kind 1
+// and 2: 30 x warps) or threads per block, H rows per block, ring slots of kind 1 (kind 3: 1 where
+// the interior row loop is unrolled)
 struct FusedShape {
     int T = 0, kind = 0, W = 0, H = 0, grid = 0, slots = 0;
 };

@@ -377,7 +377,8 @@ lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int p
                 PressureArgs a = pressure_args(h, src, dst_of(src), work);
                 if (h->tb.kind == 3)
                     CUDA_TRY(h, lbm2p_launch::node_pressure_quad(&n, g, prev ? &prev : nullptr, a,
-                                                                 kk == m, h->tb.H, h->tb.grid));
+                                                                 kk == m, h->tb.H, h->tb.slots != 0,
+                                                                 h->tb.grid));
                 else if (h->tb.kind == 2)
                     CUDA_TRY(h, lbm2p_launch::node_pressure_pair_direct(&n, g, prev ? &prev : nullptr,
                                                                         a, kk == m, h->tb.W / 30,
@@ -798,8 +799,8 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
         for (int q = 0; q < nf; ++q) {
             PressureArgs a = pressure_args(h, src, dst_of(src), work);
             if (fs.kind == 3)
-                lbm2p_launch::pressure_sweeps_quad(a, q == nf - 1 && final_check, fs.H, fs.grid,
-                                                   h->stream);
+                lbm2p_launch::pressure_sweeps_quad(a, q == nf - 1 && final_check, fs.H, fs.slots != 0,
+                                                   fs.grid, h->stream);
             else if (fs.kind == 2)
                 lbm2p_launch::pressure_sweeps_pair_direct(a, q == nf - 1 && final_check, fs.W / 30,
                                                           fs.H, fs.grid, h->stream);
@@ -1322,13 +1323,14 @@ lbm2p_status autotune_sweeps(lbm2p *h)
             }
         }
         // four sweeps per launch (lattices with walls on every side), when a check period is an
-        // even number of launches: rows per tile giving a quarter to 12 rounds of resident tiles
+        // even number of launches: rows per tile giving a quarter to 8 rounds of resident tiles, with
+        // either form of the interior row loop
         if (walls &&
             (h->p.fuse_sweeps == 4 || (h->p.fuse_sweeps == 0 && m_chk % 8 == 0)) &&
             lbm2p_launch::quad_prepare() == cudaSuccess) {
             const int slots = lbm2p_launch::quad_tile_slots(h->Fp != nullptr);
             int last_H = -1;
-            for (int quarters : {1, 2, 4, 8, 12, 16, 20, 24, 32, 48}) {
+            for (int quarters : {1, 2, 4, 8, 12, 20, 32}) {
                 if (slots < 1)
                     break;
                 // the lowest height whose tiles fit that many quarters of a round
@@ -1343,20 +1345,22 @@ lbm2p_status autotune_sweeps(lbm2p *h)
                 const long long blocks = lbm2p_launch::quad_grid(H, h->nx, h->ny);
                 if (blocks > (1LL << 30))
                     continue;
-                float ms = 0.0f, mc = 0.0f;
-                if (!timed([&](int k) {
-                        PressureArgs a = pressure_args(h, k % 2, 1 - k % 2, false);
-                        lbm2p_launch::pressure_sweeps_quad(a, false, H, (int)blocks, h->stream);
-                    }, &ms))
-                    goto done;
-                if (!timed_check([&](int k) {
-                        PressureArgs a = pressure_args(h, k % 2, 1 - k % 2, false);
-                        lbm2p_launch::pressure_sweeps_quad(a, true, H, (int)blocks, h->stream);
-                    }, blocks, ms, &mc))
-                    goto done;
-                const float per = in_loop(ms, mc, 4);
-                note("fused_quad", 4, 0, H, (int)blocks, per * 1e3f);
-                take(per, FusedShape{4, 3, 32, H, (int)blocks, 0}, false);
+                for (bool unroll : {false, true}) {
+                    float ms = 0.0f, mc = 0.0f;
+                    if (!timed([&](int k) {
+                            PressureArgs a = pressure_args(h, k % 2, 1 - k % 2, false);
+                            lbm2p_launch::pressure_sweeps_quad(a, false, H, unroll, (int)blocks, h->stream);
+                        }, &ms))
+                        goto done;
+                    if (!timed_check([&](int k) {
+                            PressureArgs a = pressure_args(h, k % 2, 1 - k % 2, false);
+                            lbm2p_launch::pressure_sweeps_quad(a, true, H, unroll, (int)blocks, h->stream);
+                        }, blocks, ms, &mc))
+                        goto done;
+                    const float per = in_loop(ms, mc, 4);
+                    note("fused_quad", 4, unroll, H, (int)blocks, per * 1e3f);
+                    take(per, FusedShape{4, 3, 32, H, (int)blocks, unroll ? 1 : 0}, false);
+                }
             }
         }
         // two sweeps per launch on rows staged by bulk copies (lattices with walls on every

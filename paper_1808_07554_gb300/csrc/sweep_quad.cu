@@ -23,7 +23,11 @@
 // apply the wall rules of Sec. 4 as selects and keep the planes that the rules read.  The edge
 // path is one row body with guards for the filling sweeps, not unrolled: few tiles run it, so its
 // instruction fetches are cold (unrolled, the tile at a corner took 500k cycles at 4096^2 where an
-// interior tile took 60k).
+// interior tile took 60k).  The interior path exists in both forms: unrolled by two with straight-line
+// filling rows it has fewer instructions, as one guarded row it leaves the instruction cache to the
+// edge tiles beside it.  Create times both: the first is ahead at 1024^2 (22.0 against 22.7 us per
+// launch), the second at 256^2 (10.4 against 12.4), at 2048^2 (60.8 against 68.0) and for batches,
+// where it is the only one.
 // The per-node operations and their order are those of the single sweep (dev1, pressure_of,
 // collide1), so four sweeps equal four launches of one bit for bit.
 // Per sweep, two-sweep launches before and this kernel now: 4096^2 129.5 and 54.5 us (218 us per
@@ -41,7 +45,7 @@
 namespace lbm2p_dev {
 namespace {
 
-template <bool CHECK, int S>
+template <bool CHECK, int S, bool UNROLL>
 __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
     k_pressure_quad(const __grid_constant__ PressureArgs a, int H)
 {
@@ -52,7 +56,7 @@ __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
     const int tile = blockIdx.x * kQuadWarps + warp;
     ResAcc racc;
     if (tile < QuadPlan(H, a.g.nx, a.g.ny).tiles())
-        quad_tile<CHECK, S>(a, H, tile, smem, lane, racc);
+        quad_tile<CHECK, S, UNROLL>(a, H, tile, smem, lane, racc);
     if (CHECK) {
         double v[4];
         racc.warp_totals(v);
@@ -93,7 +97,7 @@ __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
         reinterpret_cast<unsigned *>(&a)[i] = src[i];
     __syncwarp();
     ResAcc racc;
-    quad_tile<CHECK, S>(a, H[e.x], e.y, smem_raw, lane, racc);
+    quad_tile<CHECK, S, false>(a, H[e.x], e.y, smem_raw, lane, racc);
     if (CHECK) {
         double v[4];
         racc.warp_totals(v);
@@ -108,9 +112,13 @@ void *quad_batch_func(bool check)
     return check ? (void *)k_quad_batch<true, kQuadSlots> : (void *)k_quad_batch<false, kQuadSlots>;
 }
 
-void *quad_func(bool check)
+void *quad_func(bool check, bool unroll)
 {
-    return check ? (void *)k_pressure_quad<true, kQuadSlots> : (void *)k_pressure_quad<false, kQuadSlots>;
+    if (unroll)
+        return check ? (void *)k_pressure_quad<true, kQuadSlots, true>
+                     : (void *)k_pressure_quad<false, kQuadSlots, true>;
+    return check ? (void *)k_pressure_quad<true, kQuadSlots, false>
+                 : (void *)k_pressure_quad<false, kQuadSlots, false>;
 }
 
 }  // namespace
@@ -135,10 +143,12 @@ int quad_tile_slots(bool has_fp)
         return 0;
     for (bool c : {false, true}) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, quad_func(c), kQuadThreads,
-                                                          quad_smem_bytes(has_fp)) != cudaSuccess)
-            return 0;
-        lo = b < lo ? b : lo;
+        for (bool u : {false, true}) {
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, quad_func(c, u), kQuadThreads,
+                                                              quad_smem_bytes(has_fp)) != cudaSuccess)
+                return 0;
+            lo = b < lo ? b : lo;
+        }
     }
     return sms * lo * kQuadWarps;
 }
@@ -146,7 +156,7 @@ int quad_tile_slots(bool has_fp)
 cudaError_t quad_prepare()
 {
     for (bool c : {false, true})
-        for (void *f : {quad_func(c), quad_batch_func(c)}) {
+        for (void *f : {quad_func(c, false), quad_func(c, true), quad_batch_func(c)}) {
             cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)quad_smem_bytes(true));
             if (e != cudaSuccess)
@@ -155,18 +165,18 @@ cudaError_t quad_prepare()
     return cudaSuccess;
 }
 
-void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, int grid, void *stream)
+void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, bool unroll, int grid, void *stream)
 {
     void *args[] = {(void *)&a, (void *)&H};
-    cudaLaunchKernel(quad_func(check), dim3(grid), dim3(kQuadThreads), args,
+    cudaLaunchKernel(quad_func(check, unroll), dim3(grid), dim3(kQuadThreads), args,
                      quad_smem_bytes(a.Fp != nullptr), reinterpret_cast<cudaStream_t>(stream));
 }
 
 cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
-                               const PressureArgs &a, bool check, int H, int grid)
+                               const PressureArgs &a, bool check, int H, bool unroll, int grid)
 {
     cudaKernelNodeParams prm{};
-    prm.func = quad_func(check);
+    prm.func = quad_func(check, unroll);
     prm.gridDim = dim3((unsigned)grid);
     prm.blockDim = dim3(kQuadThreads);
     prm.sharedMemBytes = (unsigned)quad_smem_bytes(a.Fp != nullptr);

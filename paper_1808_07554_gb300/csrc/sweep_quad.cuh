@@ -133,8 +133,8 @@ struct QuadRow {
 };
 
 // FQ: there is a source in the tile; GEN: 0 no wall in the tile's footprint, 1 no-flux walls, 2 walls
-// of both kinds
-template <bool CHECK, bool FQ, int GEN, int S>
+// of both kinds; UNROLL: rows unrolled by two, the filling rows as straight-line code (GEN 0 only)
+template <bool CHECK, bool FQ, int GEN, int S, bool UNROLL>
 struct Quad {
     const PressureArgs &a;
     const int lane;
@@ -340,7 +340,7 @@ struct Quad {
 
     // directions 2, 5, 6 of two rows: in sets indexed by the row's parity P where the row loop is
     // unrolled by two, else moved on from row to row (edge tiles: half the code)
-    static constexpr int NP = GEN ? 1 : 2;
+    static constexpr int NP = GEN || !UNROLL ? 1 : 2;
 
     // what sweep s + 1 will need of sweep s's row
     template <int P>
@@ -422,7 +422,7 @@ struct Quad {
     template <int P, int NS, int s>
     __device__ __forceinline__ void next_sweep(int t, const float2 (&v)[8], float2 dPp)
     {
-        if (s > NS || (GEN && t < 2 * (s - 1))) {
+        if (s > NS || (NP == 1 && t < 2 * (s - 1))) {
             keep<P>(s - 1, v);
             if (CHECK && s == kQuadT)
                 pd = dPp;
@@ -526,7 +526,8 @@ struct Quad {
         next_row<S - 1>();
         next_row<S - 2>();
         const int iters = y1 - y0 + 2 * (kQuadT - 1);
-        if (GEN) {
+        if (NP == 1) {
+#pragma unroll 1
             for (int t = 0; t < iters; ++t)
                 row<0, kQuadT>(t);
         } else {
@@ -551,7 +552,7 @@ struct Quad {
 
 // Tile `tile` of the lattice of `a` (QuadPlan); every lane of the warp calls it with the warp's own
 // shared memory.
-template <bool CHECK, int S>
+template <bool CHECK, int S, bool UNROLL>
 __device__ __forceinline__ void quad_tile(const PressureArgs &a, int H, int tile, float *smem,
                                           int lane, ResAcc &racc)
 {
@@ -577,7 +578,7 @@ __device__ __forceinline__ void quad_tile(const PressureArgs &a, int H, int tile
     for (int sd = 0; sd < 4; ++sd)
         dir = dir || g.bc[sd] != BC_NOFLUX;
     auto go = [&](auto fq, auto gen) {
-        Quad<CHECK, decltype(fq)::value, decltype(gen)::value, S> t(a, lane);
+        Quad<CHECK, decltype(fq)::value, decltype(gen)::value, S, UNROLL> t(a, lane);
         t.tile(x0, y0, y1, smem, wlo, whi);
         racc = t.racc;
     };

@@ -626,8 +626,8 @@ def run_ours(args):
     return 0
 
 
-# bytes per node of the once-per-step kernels: S refresh 44, saturation update 124, rebase 76
-BYTES_PER_STEP_NODE = 244
+# bytes per node of the once-per-step kernels: S refresh 52, saturation update 156
+BYTES_PER_STEP_NODE = 208
 
 
 def run_batch(args):

@@ -322,20 +322,23 @@ struct Quad {
         return dP;
     }
 
-    // the sources of the tile's wells in row yy, where no source plane is read (rare)
+    // the sources of the tile's wells in row yy, where no source plane is read (rare); those of one
+    // node are added up before they are rounded into its populations, as in the single sweep
     __device__ __forceinline__ void add_wells(float2 (&v)[8], int yy) const
     {
+        float2 F = make_float2(0.0f, 0.0f);
 #pragma unroll 1
         for (int w = 0; w < a.w.n; ++w) {
             const int wo = a.w.idx[w] - (yy * a.g.pitch + x);
-            const float Fq = 0.125f * a.w.fp[w];
-            if ((wo == 0 && in0) || (wo == 1 && in1)) {
-                const float2 F = make_float2(wo == 0 ? Fq : 0.0f, wo == 0 ? 0.0f : Fq);
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    v[i] = __fadd2_rn(v[i], F);
-            }
+            if (wo == 0 && in0)
+                F.x += a.w.fp[w];
+            else if (wo == 1 && in1)
+                F.y += a.w.fp[w];
         }
+        F = __fmul2_rn(dup2(0.125f), F);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            v[i] = __fadd2_rn(v[i], F);
     }
 
     // directions 2, 5, 6 of two rows: in sets indexed by the row's parity P where the row loop is

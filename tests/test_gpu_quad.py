@@ -77,3 +77,32 @@ def test_graph_loop_equals_replay_across_moves_of_R(every, cap, fuse):
         assert np.array_equal(a.get_state(), b.get_state())
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("bc", [(1, 1, 1, 1), (2, 2, 2, 2)])
+@pytest.mark.parametrize("nx,ny,i,j", [(70, 33, 20, 10), (70, 33, 0, 0), (301, 257, 150, 128),
+                                       (57, 9, 56, 4)])
+def test_wells_that_share_a_node(nx, ny, i, j, bc):
+    """Injectors and producers of one node: their sources are added up and then rounded once into the
+    populations, with four sweeps per launch as with one, also in a batch."""
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(nx + i)
+    prob = uniform(nx, ny, bc=bc, K=np.exp(rng.standard_normal((ny, nx))),
+                   S0=0.2 + 0.5 * rng.random((ny, nx)),
+                   wells=[(i, j, 0.1, 0), (i, j, 0.037, 1), (i, j, 0.0193, 0)],
+                   P_b=[rng.random(2 * (ny if s < 2 else nx) + 1) for s in range(4)],
+                   S_b=[np.full(2 * (ny if s < 2 else nx) + 1, 0.3) for s in range(4)])
+    kw = dict(init_replay=0, tol=0.0, max_sub_iters=32)
+    one = pkg.Solver.from_problem(prob, fuse_sweeps=1, **kw)
+    four = pkg.Solver.from_problem(prob, fuse_sweeps=4, **kw)
+    member = pkg.Solver.from_problem(prob, fuse_sweeps=4, **kw)
+    with pkg.Batch([member]) as batch:
+        for _ in range(2):
+            one.step(1, replay=[32])
+            four.step(1, replay=[32])
+            batch.step(1, replay=[[32]])
+            state = one.get_state()
+            assert np.array_equal(state, four.get_state())
+            assert np.array_equal(state, member.get_state())
+    for s in (one, four, member):
+        s.close()

@@ -18,13 +18,13 @@
 // adds, w_i (R(x - c_i) - R(x)), or 2 w_i (P_b - R(x)) at a Dirichlet wall, or nothing, does not
 // change between rebases and is kept per direction in registers as the factor of w_i.
 //
-// Measured, 16 blocks: 64^2 0.7 us per sweep and 2.6 us per check (before 4.1 us per sweep as a
+// Measured, 16 blocks: 64^2 0.7 us per sweep and 1.7 us per check (before 4.1 us per sweep as a
 // launch of its own, or 2.9 as a quarter of a four-sweep launch, and 10 to 12 us per check with the
-// finalize kernel and the graph's conditional nodes); 128^2 1.3 us per sweep.  What bounds it now is
-// the cluster barrier with the distributed stores before it (about 0.5 us) and, at 128^2, one
-// node per thread on 32 warps.  The check's sums go through FP32 pairs and its test through a
-// product instead of a division and a root: with FP64 sums per warp it took 6.8 us at 64^2 and
-// 10.4 us at 128^2, all of it the few FP64 units.
+// finalize kernel and the graph's conditional nodes); 128^2 1.2 us per sweep and 2.3 per check.  What
+// bounds it now is the cluster barrier with the distributed stores before it (about 0.5 us) and, at
+// 128^2, one node per thread on 32 warps.  The check's sums are FP32 inside a warp and FP64 in one warp
+// per block, and its test a product instead of a division and a root: with FP64 in every warp it took
+// 6.8 us at 64^2 and 10.4 us at 128^2, all of it the few FP64 units.
 //
 // Per node the arithmetic is that of the single sweep (dev1, pressure_of, collide1; the factor 2 of
 // a Dirichlet wall is exact), so a solve equals the same number of single sweeps bit for bit; the
@@ -60,16 +60,6 @@ __device__ __forceinline__ double cluster_load(unsigned a)
     double v;
     asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
     return v;
-}
-
-// (a + b) of unevaluated pairs of floats (Knuth's two-sum, about 48 bits)
-__device__ __forceinline__ float2 pair_add(float2 a, float2 b)
-{
-    const float s = __fadd_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
-    const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-    const float l = __fadd_rn(__fadd_rn(a.y, b.y), e);
-    const float h = __fadd_rn(s, l);
-    return make_float2(h, __fsub_rn(l, __fsub_rn(h, s)));
 }
 
 __device__ __forceinline__ float flip(float v, bool f)
@@ -115,10 +105,9 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     k_pressure_resident(const __grid_constant__ PressureArgs a, const __grid_constant__ ResidentArgs s)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ float red[4][kResMaxThreads / 32];
+    __shared__ float red[7][kResMaxThreads / 32];     // the warps' residual sums, pivots and nodes
     __shared__ double part[4];            // this block's residual sums, read by the whole cluster
     __shared__ double tot[4];
-    __shared__ float sh_pivot[2];         // written by one block in every block
     __shared__ int sh_stop;
     const Geom &g = a.g;
     const unsigned rank = cluster_rank(), C = cluster_size();
@@ -263,12 +252,11 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
         ++k;
         const bool check = --to_check == 0;
         const unsigned nxt = cur == base ? base + buffer : base;
-        // sums of d, d^2, q, q^2 over this thread's nodes, d and q relative to the pivots
-        float s1 = 0.0f, s2 = 0.0f, t1 = 0.0f, t2 = 0.0f;
-        const float p0 = check ? sh_pivot[0] : 0.0f, p1 = check ? sh_pivot[1] : 0.0f;
+        float d[NPT], u[NPT];                         // what a check sums over
 #pragma unroll
         for (int q = 0; q < NPT; ++q) {
             ResNode<NPT> &n = nd[q];
+            d[q] = u[q] = 0.0f;
             if (n.cell == ~0u)
                 continue;
             float f[8], v[8];
@@ -284,46 +272,90 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                 v[i] = collide1(f[i], wgt(i + 1), dP, n.it, n.Fq);
             put(n, nxt, v);
             if (check) {
-                const float e = ((dP - n.dp) - shift1) - p1, u = ((n.r0 - shift0) + dP) - p0;
-                s1 += e;
-                s2 = fmaf(e, e, s2);
-                t1 += u;
-                t2 = fmaf(u, u, t2);
-            } else if (q == 0 && to_check == 1 && rank == C / 2 && tid == 0) {
-                // the next sweep checks: one node's values are everyone's pivots
-                for (unsigned b = 0; b < C; ++b) {
-                    cluster_store(cluster_addr(smem_u32(&sh_pivot[0]), b), (n.r0 - shift0) + dP);
-                    cluster_store(cluster_addr(smem_u32(&sh_pivot[1]), b),
-                                  k > 1 ? (dP - n.dp) - shift1 : 0.0f);
-                }
+                d[q] = (dP - n.dp) - shift1;
+                u[q] = (n.r0 - shift0) + dP;
             }
             n.dp = dP;
         }
         cur = nxt;
         if (check) {
-            s1 = warp_sum(s1);
-            s2 = warp_sum(s2);
-            t1 = warp_sum(t1);
-            t2 = warp_sum(t2);
+            // Sums of d, d^2, u, u^2.  A warp's in FP32, relative to its own means: their rounding is a
+            // few 2^-24 of the spread inside the warp, whatever the values of other nodes.  Then one
+            // warp restores the raw sums and adds them in FP64.
+            const bool h16 = lane & 16, h8 = lane & 8;
+            float n = 0.0f, cd = 0.0f, cu = 0.0f;
+#pragma unroll
+            for (int q = 0; q < NPT; ++q) {
+                n += (float)__popc(__ballot_sync(0xffffffffu, nd[q].cell != ~0u));
+                cd += d[q];
+                cu += u[q];
+            }
+            float v = (h16 ? cu : cd) + __shfl_xor_sync(0xffffffffu, h16 ? cd : cu, 16);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+                v += __shfl_xor_sync(0xffffffffu, v, o);
+            v *= 1.0f / n;
+            cd = __shfl_sync(0xffffffffu, v, 0);
+            cu = __shfl_sync(0xffffffffu, v, 16);
+            float s1 = 0.0f, s2 = 0.0f, t1 = 0.0f, t2 = 0.0f;
+#pragma unroll
+            for (int q = 0; q < NPT; ++q)
+                if (nd[q].cell != ~0u) {
+                    const float e = d[q] - cd, g = u[q] - cu;
+                    s1 += e;
+                    s2 = fmaf(e, e, s2);
+                    t1 += g;
+                    t2 = fmaf(g, g, t2);
+                }
+            // four sums over 32 lanes by six shuffles: lane 8 c ends with sum c
+            s1 = (h16 ? t1 : s1) + __shfl_xor_sync(0xffffffffu, h16 ? s1 : t1, 16);
+            s2 = (h16 ? t2 : s2) + __shfl_xor_sync(0xffffffffu, h16 ? s2 : t2, 16);
+            s1 = (h8 ? s2 : s1) + __shfl_xor_sync(0xffffffffu, h8 ? s1 : s2, 8);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1)
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            if ((lane & 7) == 0)
+                red[lane >> 3][warp] = s1;
             if (lane == 0) {
-                red[0][warp] = s1;
-                red[1][warp] = s2;
-                red[2][warp] = t1;
-                red[3][warp] = t2;
+                red[4][warp] = cd;
+                red[5][warp] = cu;
+                red[6][warp] = n;
             }
             __syncthreads();
             if (warp == 0) {
-                // eight lanes per sum, as unevaluated pairs of floats (this GPU's FP64 units are few)
+                // sum x = S1 + n p, sum x^2 = S2 + 2 p S1 + n p^2.  Up to eight warps: a lane per warp
+                // and sum, half the FP64 instructions of the other form (64^2, per check: 1.7 us
+                // against 2.0; with 32 warps, where it takes four rounds, 2.8 against 2.3 at 128^2).
                 const int nw = (int)blockDim.x >> 5, c = lane >> 3;
-                float2 t = make_float2(0.0f, 0.0f);
-                for (int w = lane & 7; w < nw; w += 8)
-                    t = pair_add(t, make_float2(red[c][w], 0.0f));
+                double t = 0.0;
+                if (nw <= 8) {
+                    const int w = lane & 7;
+                    if (w < nw && red[6][w] > 0.0f) {
+                        const double p = red[4 + (c >> 1)][w], S1 = red[c & 2][w];
+                        const double raw = fma((double)red[6][w], p, S1);
+                        t = (c & 1) ? fma(p, S1 + raw, (double)red[c][w]) : raw;
+                    }
+                } else {
+                    // a lane per warp, then lanes 8 c .. 8 c + 7 hold sum c
+                    double v[4] = {0.0, 0.0, 0.0, 0.0};
+                    if (lane < nw && red[6][lane] > 0.0f) {
+                        const double nodes = red[6][lane];
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const double p = red[4 + i][lane], S1 = red[2 * i][lane];
+                            v[2 * i] = fma(nodes, p, S1);
+                            v[2 * i + 1] = fma(p, S1 + v[2 * i], (double)red[2 * i + 1][lane]);
+                        }
+                    }
+                    v[0] = (h16 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, h16 ? v[0] : v[2], 16);
+                    v[1] = (h16 ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, h16 ? v[1] : v[3], 16);
+                    t = (h8 ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, h8 ? v[0] : v[1], 8);
+                }
 #pragma unroll
                 for (int o = 4; o > 0; o >>= 1)
-                    t = pair_add(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o),
-                                                __shfl_xor_sync(0xffffffffu, t.y, o)));
+                    t += __shfl_xor_sync(0xffffffffu, t, o);
                 if ((lane & 7) == 0)
-                    part[c] = (double)t.x + (double)t.y;
+                    part[c] = t;
             }
         }
         cluster_sync();
@@ -341,7 +373,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
             }
             __syncthreads();
             if (tid == 0) {
-                // the residual r = sqrt(num / den); variances do not depend on the pivots
+                // the residual r = sqrt(num / den)
                 const double sd = tot[0], sp = tot[2];
                 int stop = 0;
                 num = tot[1] - sd * sd * inv_n;
@@ -403,8 +435,8 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     if (rank == 0 && tid == 0) {
         double r = nan("");
         if (checked) {
-            const double mean0 = (double)shift0 + (double)sh_pivot[0] + tot[2] * inv_n;
-            const double mean1 = (double)shift1 + (double)sh_pivot[1] + tot[0] * inv_n;
+            const double mean0 = (double)shift0 + tot[2] * inv_n;
+            const double mean1 = (double)shift1 + tot[0] * inv_n;
             r = isnan(num) ? num : (den > 0.0 ? sqrt(num / den) : (num > 0.0 ? INFINITY : 0.0));
             s.out->r = r;
             s.out->mean_P = mean0;

@@ -91,3 +91,33 @@ def test_resident_stops_where_single_sweeps_do(name):
     assert W.rel_l2(Pb, Pa) <= 8 * 4 * 1e-7 * 2 and W.rel_l2(Sb, Sa) <= 1e-6
     one.close()
     res.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(5, 3), (8, 96), (32, 32), (64, 64), (97, 70), (128, 128), (160, 128),
+                                   (200, 200)])
+@pytest.mark.parametrize("amp", [1.0, 100.0])
+def test_residual_against_64_bits_beside_outliers(nx, ny, amp):
+    """The residual of the second sweep from P0 = noise of 1e-3 with a few nodes (some at the start of a
+    block's rows, whatever the cluster's size) a thousand or more deviations away, against 64-bit sums
+    over the pressures of the first two sweeps.  A warp's FP32 sums of squares are relative to its
+    means, so their rounding (a square, its operand and eight additions, 2^-24 each) is at most
+    12 x 2^-24 of the whole variance, half of that in the root; P itself is rounded to 2^-24 on both sides
+    and enters as a difference: 4 x 2^-24 more.  Together 6e-7; 2e-6 is allowed."""
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(nx)
+    P0 = 1e-3 * rng.standard_normal((ny, nx))
+    for C in (1, 2, 4, 8, 16):
+        y = (C // 2) * -(-ny // C)
+        P0[y if y < ny else 0, 0] = amp
+    prob = uniform(nx, ny, bc=(1, 1, 1, 1), K=np.exp(rng.standard_normal((ny, nx))),
+                   S0=0.2 + 0.5 * rng.random((ny, nx)), P0=P0)
+    p = []
+    for k in (0, 1):                          # the fields are those that the next sweep computes
+        one = pkg.Solver.from_problem(prob, init_replay=k, fuse_sweeps=1)
+        p.append(one.fields()[0].astype(np.float64))
+        one.close()
+    res = pkg.Solver.from_problem(prob, tol=0.0, max_sub_iters=2, check_every=2)
+    assert res.fused_form() == pkg.FUSED_RESIDENT
+    want = np.std(p[1] - p[0]) / np.std(p[1])
+    assert res.init_stats.residual == pytest.approx(want, rel=2e-6)
+    res.close()

@@ -278,9 +278,8 @@ typedef enum {
     LBM2P_FUSED_DIRECT = 3,      /* two sweeps, inputs loaded directly (lattices held in L2) */
     LBM2P_FUSED_QUAD = 4,        /* four sweeps, one warp per tile of 56 columns */
     LBM2P_FUSED_RESIDENT = 5     /* whole solves in one launch, the lattice in the shared memory of
-                                    a thread-block cluster (small lattices; solves that end at a
-                                    residual check the graph loop cannot make, an odd check_every,
-                                    use the form that lbm2p_sweep_config reports) */
+                                    a thread-block cluster (small lattices, check_every even and
+                                    max_sub_iters a multiple of it) */
 } lbm2p_fused_form;
 int lbm2p_fused_form_of(const lbm2p *h);
 

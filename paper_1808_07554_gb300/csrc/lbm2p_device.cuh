@@ -233,7 +233,8 @@ struct LoopHandles {
 };
 
 // A whole sub-iteration in one launch (resident.cu): m, cap, every and tol from *ctl when given
-// (which receives the sweeps run and the last residual), else from here.
+// (which receives the sweeps run and the last residual; m and cap are the same here, for the
+// launcher's check), else from here.
 struct ResidentArgs {
     LoopCtl *ctl;
     int m, cap, every;

@@ -527,9 +527,18 @@ bool resident_fits(int C, int nx, int ny)
     return clusters >= 1;
 }
 
+// what the kernel relies on: a sweep between two checks (`part` is rewritten by the next one), and a
+// check at the cap
+static bool resident_args_ok(const ResidentShape &p, const ResidentArgs &s)
+{
+    return p.C > 0 && s.m >= 2 && s.cap >= s.m && s.cap % s.m == 0;
+}
+
 cudaError_t pressure_resident(const PressureArgs &a, const ResidentArgs &s_, int C, void *stream)
 {
     const ResidentShape p = resident_shape(C, a.g.nx, a.g.ny);
+    if (!resident_args_ok(p, s_))
+        return cudaErrorInvalidValue;
     ResidentArgs s = s_;
     s.h = p.h;
     s.cells = p.cells;
@@ -543,6 +552,8 @@ cudaError_t node_resident(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode
                           const PressureArgs &a, const ResidentArgs &s_, int C)
 {
     const ResidentShape p = resident_shape(C, a.g.nx, a.g.ny);
+    if (!resident_args_ok(p, s_))
+        return cudaErrorInvalidValue;
     ResidentArgs s = s_;
     s.h = p.h;
     s.cells = p.cells;

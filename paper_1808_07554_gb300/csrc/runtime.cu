@@ -302,6 +302,8 @@ ResidentArgs resident_args(lbm2p *h, bool work)
 {
     ResidentArgs s{};
     s.ctl = h->ctl;
+    s.m = h->p.check_every;
+    s.cap = h->p.max_sub_iters;
     s.out = h->res;
     s.shift_out = h->shift;
     s.Rw = R_of(h, work);
@@ -1439,13 +1441,13 @@ lbm2p_status autotune_sweeps(lbm2p *h)
     }
     if (!host_two)
         h->host_form = h->tb;
-    // whole solves in one launch, for lattices that fit a cluster's shared memory: timed over four
-    // check periods (the tolerance -1 never stops it), checks included.  What a check costs the
+    // whole solves in one launch, for lattices that fit a cluster's shared memory and solves that the
+    // graph loop can run (it ends them at the same checks): timed over four check periods (the tolerance -1 never stops it), checks included.  What a check costs the
     // other forms besides its launch (the finalize kernel and the conditional nodes around it,
     // about 10 us at 64^2 to 256^2) is not in their times, so it is added here
     h->res_C = 0;
     best += 0.010f / (float)m_chk;
-    if (h->p.fuse_sweeps == 0 && forced == LBM2P_SWEEP_AUTO && m_chk >= 2 && m_chk <= 4096)
+    if (h->graph_ok && h->p.fuse_sweeps == 0 && forced == LBM2P_SWEEP_AUTO && m_chk <= 4096)
         for (int C : {1, 2, 4, 8, 16}) {
             if (!lbm2p_launch::resident_fits(C, h->nx, h->ny))
                 continue;
@@ -1792,6 +1794,9 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
     if (!ok)
         return fail(h, LBM2P_ENOMEM, "device allocation of %.1f MiB failed",
                     (double)pb * 45 / (1 << 20));
+    // the body of the graph loop holds check_every sweeps and must return to the same f buffer
+    h->graph_ok = !h->fp16 && p.check_every >= 2 && p.check_every % 2 == 0 &&
+                  p.max_sub_iters % p.check_every == 0;
     // which single-sweep kernel, single or fused sweeps, and the fused tile shape: timed
     // on this lattice (within what fuse_sweeps allows); FP16 storage has one sweep kernel
     if (!h->fp16) {
@@ -1853,9 +1858,6 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
     // a long solve moves R to the current P about every 1024 sweeps (at a check point);
     // FP16 sweeps move it every sweep
     h->rebase_every = h->fp16 ? 0 : p.check_every * ((1024 + p.check_every - 1) / p.check_every);
-    // the loop body holds check_every sweeps and must return to the same f buffer
-    h->graph_ok = !h->fp16 && p.check_every >= 2 && p.check_every % 2 == 0 &&
-                  p.max_sub_iters % p.check_every == 0;
     if (h->tb.T > 1 && p.check_every % (2 * h->tb.T) != 0)
         h->tb_T_graph = 0;
     else

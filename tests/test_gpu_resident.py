@@ -121,3 +121,23 @@ def test_residual_against_64_bits_beside_outliers(nx, ny, amp):
     want = np.std(p[1] - p[0]) / np.std(p[1])
     assert res.init_stats.residual == pytest.approx(want, rel=2e-6)
     res.close()
+
+
+@pytest.mark.parametrize("walls", ["periodic", "noflux"])
+@pytest.mark.parametrize("every,cap", [(1, 20), (7, 70), (8, 68), (6, 100), (8, 4)])
+def test_not_reported_where_a_solve_cannot_use_it(every, cap, walls):
+    """A check period that is odd, or a cap that is no multiple of it: the host runs the solves, and the
+    on-chip form is neither timed nor reported."""
+    import paper_1808_07554_gb300 as pkg
+    rng, prob = _problem(64, 64, walls)
+    kw = dict(init_replay=0, tol=0.0, max_sub_iters=cap, check_every=every)
+    one = pkg.Solver.from_problem(prob, fuse_sweeps=1, **kw)
+    auto = pkg.Solver.from_problem(prob, **kw)
+    assert auto.fused_form() != pkg.FUSED_RESIDENT
+    assert all(r[0] != "resident" for r in auto.autotune_report())
+    for s in (one, auto):
+        st, stats = s.step(1)
+        assert st == pkg.ENOTCONVERGED and stats[0].sub_iters == cap
+    assert np.array_equal(one.get_state(), auto.get_state())
+    one.close()
+    auto.close()

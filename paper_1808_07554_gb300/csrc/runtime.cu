@@ -1442,8 +1442,10 @@ lbm2p_status autotune_sweeps(lbm2p *h)
     if (!host_two)
         h->host_form = h->tb;
     // whole solves in one launch, for lattices that fit a cluster's shared memory and solves that the
-    // graph loop can run (it ends them at the same checks): timed over four check periods (the tolerance -1 never stops it), checks included.  What a check costs the
-    // other forms besides its launch (the finalize kernel and the conditional nodes around it,
+    // graph loop can run (it ends them at the same checks): timed over four check periods of at most
+    // 64 sweeps (the tolerance -1 never stops it; a check is then 0.03 us per sweep, and four whole
+    // periods of 4096 sweeps made a create of 0.12 s one of 1.1 s), checks included.  What a check costs
+    // the other forms besides its launch (the finalize kernel and the conditional nodes around it,
     // about 10 us at 64^2 to 256^2) is not in their times, so it is added here
     h->res_C = 0;
     best += 0.010f / (float)m_chk;
@@ -1452,8 +1454,8 @@ lbm2p_status autotune_sweeps(lbm2p *h)
             if (!lbm2p_launch::resident_fits(C, h->nx, h->ny))
                 continue;
             ResidentArgs s{};
-            s.m = m_chk;
-            s.cap = 4 * m_chk;
+            s.m = m_chk < 64 ? m_chk : 64;
+            s.cap = 4 * s.m;
             s.tol = -1.0;
             s.out = reinterpret_cast<ResidualOut *>(h->partials);
             s.shift_out = h->shift;

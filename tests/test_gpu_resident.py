@@ -2,6 +2,8 @@
 identical populations bit for bit at the edges of its shapes (blocks of one row, a last block with
 fewer rows, one to three nodes per thread, lattices one column wide), for every wall kind, with
 wells, dense sources and a mid-solve rebase, and the same stopping sweep as the host's rule."""
+import time
+
 import numpy as np
 import pytest
 
@@ -141,3 +143,19 @@ def test_not_reported_where_a_solve_cannot_use_it(every, cap, walls):
     assert np.array_equal(one.get_state(), auto.get_state())
     one.close()
     auto.close()
+
+
+def test_create_does_not_run_long_check_periods_to_time_the_form():
+    """The form is timed over a bounded number of sweeps, so a handle with a check period of 4096 sweeps
+    takes about as long to create as one with 64 (it took 17 times as long when it did not)."""
+    import paper_1808_07554_gb300 as pkg
+    rng, prob = _problem(64, 64, "noflux")
+    took = {}
+    for every in (64, 4096):
+        for _ in range(4):
+            t0 = time.perf_counter()
+            s = pkg.Solver.from_problem(prob, init_replay=0, check_every=every, max_sub_iters=40960)
+            took[every] = min(took.get(every, 1e9), time.perf_counter() - t0)
+            assert any(r[0] == "resident" for r in s.autotune_report())
+            s.close()
+    assert took[4096] < 3 * took[64], took

@@ -797,15 +797,46 @@ __device__ __forceinline__ float sd_of(const double *st, long long n)
     return v > 1e-60 ? (float)sqrt(v) : 1.0f;
 }
 
-// (s, c) += (h, l): an unevaluated pair of floats (about 48 bits)
-__device__ __forceinline__ void pair_add(float2 &a, float h, float l)
+// a + b = s + e exactly (Knuth's two-sum); returns s
+__device__ __forceinline__ float two_sum(float a, float b, float &e)
 {
-    const float s = __fadd_rn(a.x, h), bb = __fsub_rn(s, a.x);
-    const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(h, bb));
-    const float t = __fadd_rn(__fadd_rn(a.y, l), e);
-    a.x = __fadd_rn(s, t);
-    a.y = __fsub_rn(t, __fsub_rn(a.x, s));
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
 }
+
+// A running sum as x + y + z: what x rounds off goes into y exactly, what y rounds off into z, so the
+// whole is good to about 2^-70 where an FP64 sum is good to 2^-53.
+struct Sum3 {
+    float x = 0.0f, y = 0.0f, z = 0.0f;
+
+    __device__ __forceinline__ void mid(float m)              // m some 2^-24 of the sum
+    {
+        float e;
+        y = two_sum(y, m, e);
+        z += e;
+    }
+    __device__ __forceinline__ void add(float h, float m)     // h + m, m at most 2^-24 of h
+    {
+        float e;
+        x = two_sum(x, h, e);
+        mid(e);
+        mid(m);
+    }
+    __device__ __forceinline__ void scale(float f)            // f^2, a power of two
+    {
+        x = x * f * f;
+        y = y * f * f;
+        z = z * f * f;
+    }
+    __device__ __forceinline__ void add_lane(int o)           // the same sum of the lane o away
+    {
+        const float h = __shfl_xor_sync(0xffffffffu, x, o), m = __shfl_xor_sync(0xffffffffu, y, o);
+        z += __shfl_xor_sync(0xffffffffu, z, o);
+        add(h, m);
+    }
+    __device__ __forceinline__ double value() const { return (double)x + ((double)y + (double)z); }
+};
 
 // a power of two that brings |v| near 1 (1 for zero, infinities and NaN)
 __device__ __forceinline__ float unit_scale(float v)
@@ -814,31 +845,43 @@ __device__ __forceinline__ float unit_scale(float v)
     return e == 255 || v == 0.0f ? 1.0f : __uint_as_float((unsigned)(e < 253 ? 254 - e : 1) << 23);
 }
 
-// Sums of a - b and (a - b)^2.  The difference of two floats is a pair of floats exactly, and so its
-// square to 2^-48: each thread adds pairs, the squares scaled by a power of two that follows its
-// largest difference (so they cover the range that FP64 would); a warp adds its lanes' pairs at the
-// scale of the largest, and one lane turns them into FP64, which the block and the grid add.  FP64
-// per element took 27 us for a 1024^2 plane, FP64 per thread 32 us (an FP64 instruction holds its SM
-// for 16 cycles, and every warp ran forty), this 7.4 us.  VEC: 128-bit loads (both planes aligned).
+// Sums of a - b and (a - b)^2.  The difference of two floats is a pair of floats exactly, its square
+// one of four: each thread adds these in FP32 sums that lose less than FP64 ones (Sum3), the squares
+// scaled by a power of two that follows its largest difference (so they cover the range that FP64
+// would); a warp adds its lanes' sums at the scale of the largest, and one lane turns them into FP64,
+// which the block and the grid add.  FP64 per element took 27 us for a 1024^2 plane, FP64 per thread
+// 32 us (an FP64 instruction holds its SM for 16 cycles, and every warp ran forty), this 8 us.  VEC:
+// 128-bit loads (both planes aligned).
 struct DiffSums {
-    float2 s1 = make_float2(0.0f, 0.0f), s2 = make_float2(0.0f, 0.0f);
+    Sum3 s1, s2;
     float sc = 0.0f;                                          // scale of s2's terms (0: none yet)
 
-    __device__ __forceinline__ void add(float x, float y)
+    // N differences at a time: their sums are independent but for one addition each
+    template <int N>
+    __device__ __forceinline__ void add(const float (&x)[N], const float (&y)[N])
     {
-        const float h = __fsub_rn(x, y), yy = __fsub_rn(x, h);
-        const float l = __fsub_rn(__fsub_rn(x, __fadd_rn(h, yy)), __fsub_rn(y, yy));
-        pair_add(s1, h, l);
-        float u = h * sc;
-        if (sc == 0.0f || fabsf(u) > 1073741824.0f) {
-            const float ns = unit_scale(h);
-            const float f = sc == 0.0f ? 0.0f : ns / sc;      // both powers of two
-            s2 = make_float2(s2.x * f * f, s2.y * f * f);
-            sc = h == 0.0f ? sc : ns;
-            u = h * sc;
+        float h[N], l[N], big = 0.0f;
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            h[i] = __fsub_rn(x[i], y[i]);
+            const float yy = __fsub_rn(x[i], h[i]);
+            l[i] = __fsub_rn(__fsub_rn(x[i], __fadd_rn(h[i], yy)), __fsub_rn(y[i], yy));
+            big = fmaxf(big, fabsf(h[i]));
         }
-        const float v = l * sc, q = __fmul_rn(u, u);
-        pair_add(s2, q, fmaf(2.0f * u, v, fmaf(u, u, -q)));
+        if (sc == 0.0f || big * sc > 1073741824.0f) {
+            const float ns = unit_scale(big);
+            s2.scale(sc == 0.0f ? 0.0f : ns / sc);            // both powers of two
+            sc = big == 0.0f ? sc : ns;
+        }
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            s1.add(h[i], l[i]);
+            // (u + v)^2 = u u + 2 u v + v v
+            const float u = h[i] * sc, v = l[i] * sc, q = __fmul_rn(u, u), p = __fmul_rn(2.0f * u, v);
+            s2.add(q, fmaf(u, u, -q));
+            s2.mid(p);
+            s2.z += fmaf(v, v, fmaf(2.0f * u, v, -p));
+        }
     }
 
     // the sums of the warp in every lane
@@ -847,14 +890,11 @@ struct DiffSums {
         float low = sc > 0.0f ? sc : __int_as_float(0x7f800000);
         for (int o = 16; o > 0; o >>= 1)
             low = fminf(low, __shfl_xor_sync(0xffffffffu, low, o));
-        const float f = sc > 0.0f ? low / sc : 0.0f;          // at most 1, a power of two
-        s2 = make_float2(s2.x * f * f, s2.y * f * f);
+        s2.scale(sc > 0.0f ? low / sc : 0.0f);                // at most 1, a power of two
         sc = isinf(low) ? 0.0f : low;
         for (int o = 16; o > 0; o >>= 1) {
-            const float a = __shfl_xor_sync(0xffffffffu, s1.x, o), b = __shfl_xor_sync(0xffffffffu, s1.y, o);
-            const float c = __shfl_xor_sync(0xffffffffu, s2.x, o), d = __shfl_xor_sync(0xffffffffu, s2.y, o);
-            pair_add(s1, a, b);
-            pair_add(s2, c, d);
+            s1.add_lane(o);
+            s2.add_lane(o);
         }
     }
 };
@@ -870,22 +910,19 @@ __global__ void __launch_bounds__(256) k_diff_stats(const float *a, const float 
 #pragma unroll 2
         for (long long i = t0; i < nq; i += step) {
             const float4 x = reinterpret_cast<const float4 *>(a)[i], y = reinterpret_cast<const float4 *>(b)[i];
-            d.add(x.x, y.x);
-            d.add(x.y, y.y);
-            d.add(x.z, y.z);
-            d.add(x.w, y.w);
+            d.add({x.x, x.y, x.z, x.w}, {y.x, y.y, y.z, y.w});
         }
         if (t0 < n - 4 * nq)
-            d.add(a[4 * nq + t0], b[4 * nq + t0]);
+            d.add({a[4 * nq + t0]}, {b[4 * nq + t0]});
     } else {
         for (long long i = t0; i < n; i += step)
-            d.add(a[i], b[i]);
+            d.add({a[i]}, {b[i]});
     }
     d.warp_sum();
     if ((threadIdx.x & 31) == 0) {
         const double is = d.sc > 0.0f ? 1.0 / (double)d.sc : 0.0;
-        red[0][threadIdx.x >> 5] = (double)d.s1.x + (double)d.s1.y;
-        red[1][threadIdx.x >> 5] = ((double)d.s2.x + (double)d.s2.y) * is * is;
+        red[0][threadIdx.x >> 5] = d.s1.value();
+        red[1][threadIdx.x >> 5] = d.s2.value() * is * is;
     }
     __syncthreads();
     if (threadIdx.x < 2) {

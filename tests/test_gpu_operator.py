@@ -231,3 +231,36 @@ def test_diff_stats_sums(n, offset, spread):
     want = torch.stack([d.sum(), (d * d).sum()])
     size = torch.stack([d.abs().sum(), (d * d).sum()])
     assert ((st - want).abs() <= 2.0 ** -35 * size + 1e-300).all(), (st, want)
+
+
+@pytest.mark.parametrize("kind", ["equal", "near", "normal", "wide"])
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_diff_stats_sums_no_worse_than_fp64(kind, seed):
+    """4096 differences (one block) against exact sums.  A lane's and a warp's sums lose less than 2^-60;
+    then come eleven FP64 additions (two in a warp's value, eight warps, the output), 2^-53 of the sum of
+    magnitudes each.  Equal differences with a long square make an error of every addition count."""
+    import torch
+    from fractions import Fraction
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(seed)
+    n = 4096
+    if kind == "equal":
+        pairs = [(1.0764390230178833, 0.0010697194375097752), (1.6369616985321045, -0.0008992706425487995),
+                 (-1.9999998807907104, 2.0 ** -24)]
+        a, b = (np.full(n, v, np.float32) for v in pairs[seed])
+    elif kind == "near":                       # two saturations: the difference is exact
+        a = (0.2 + 0.5 * rng.random(n)).astype(np.float32)
+        b = (a + 1e-3 * rng.standard_normal(n)).astype(np.float32)
+    else:
+        scale = np.exp2(rng.integers(-30, 31, n)) if kind == "wide" else 1.0
+        a = (rng.standard_normal(n) * scale).astype(np.float32)
+        b = (rng.standard_normal(n) * 1e-3).astype(np.float32)
+    ta, tb = torch.tensor(a, device="cuda"), torch.tensor(b, device="cuda")
+    st = torch.zeros(2, dtype=torch.float64, device="cuda")
+    pkg.lbm2p_op_diff_stats(ta.data_ptr(), tb.data_ptr(), n, st.data_ptr(),
+                            torch.cuda.current_stream().cuda_stream)
+    d = [Fraction(float(x)) - Fraction(float(y)) for x, y in zip(a, b)]
+    want = (sum(d), sum(v * v for v in d))
+    size = (sum(abs(v) for v in d), want[1])
+    for got, w, s in zip(st.cpu().numpy(), want, size):
+        assert abs(Fraction(float(got)) - w) <= 11 * Fraction(1, 2 ** 53) * s, float(Fraction(float(got)) / w - 1)

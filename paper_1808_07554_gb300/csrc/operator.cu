@@ -853,25 +853,46 @@ __device__ __forceinline__ float unit_scale(float v)
 // 32 us (an FP64 instruction holds its SM for 16 cycles, and every warp ran forty), this 8 us.  VEC:
 // 128-bit loads (both planes aligned).
 struct DiffSums {
+    static constexpr float kFar = 0x1p95f;                    // room for 2^32 of them in an FP32 sum
     Sum3 s1, s2;
     float sc = 0.0f;                                          // scale of s2's terms (0: none yet)
+    float lim = 0.0f;                                         // largest difference at that scale
+    bool far = false;                                         // left something to add_far
+
+    template <int N>
+    __device__ __forceinline__ static float largest(const float (&x)[N], const float (&y)[N])
+    {
+        float big = 0.0f;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+            big = fmaxf(big, fabsf(__fsub_rn(x[i], y[i])));
+        return big;
+    }
 
     // N differences at a time: their sums are independent but for one addition each
     template <int N>
     __device__ __forceinline__ void add(const float (&x)[N], const float (&y)[N])
     {
-        float h[N], l[N], big = 0.0f;
+        float h[N], l[N];
 #pragma unroll
         for (int i = 0; i < N; ++i) {
             h[i] = __fsub_rn(x[i], y[i]);
             const float yy = __fsub_rn(x[i], h[i]);
             l[i] = __fsub_rn(__fsub_rn(x[i], __fadd_rn(h[i], yy)), __fsub_rn(y[i], yy));
-            big = fmaxf(big, fabsf(h[i]));
         }
-        if (sc == 0.0f || big * sc > 1073741824.0f) {
-            const float ns = unit_scale(big);
-            s2.scale(sc == 0.0f ? 0.0f : ns / sc);            // both powers of two
-            sc = big == 0.0f ? sc : ns;
+        const float big = largest(x, y);
+        if (big > lim) {
+            if (big >= kFar) {
+                far = true;
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+                    h[i] = l[i] = 0.0f;
+            } else {
+                const float ns = unit_scale(big);
+                s2.scale(sc == 0.0f ? 0.0f : ns / sc);        // both powers of two
+                sc = ns;
+                lim = fminf(1073741824.0f / ns, 0x1.fffffep94f);
+            }
         }
 #pragma unroll
         for (int i = 0; i < N; ++i) {
@@ -882,6 +903,22 @@ struct DiffSums {
             s2.mid(p);
             s2.z += fmaf(v, v, fmaf(2.0f * u, v, -p));
         }
+    }
+
+    // What add left out, in FP64: where a difference is beyond what FP32 sums hold, or infinite, its
+    // parts are of no use, but two finite floats have a finite FP64 difference with a finite square.
+    // (A NaN has made the FP32 sums NaN by itself.)
+    template <int N>
+    __device__ __forceinline__ static void add_far(const float (&x)[N], const float (&y)[N], double &f1,
+                                                   double &f2)
+    {
+        if (largest(x, y) >= kFar)
+#pragma unroll
+            for (int i = 0; i < N; ++i) {
+                const double d = (double)x[i] - (double)y[i];
+                f1 += d;
+                f2 += d * d;
+            }
     }
 
     // the sums of the warp in every lane
@@ -899,30 +936,56 @@ struct DiffSums {
     }
 };
 
+// f of every four (one at the end, one by one where the planes are not aligned) of this thread's values
+template <bool VEC, class F>
+__device__ __forceinline__ void each_pair(const float *a, const float *b, long long n, F f)
+{
+    const long long t0 = blockIdx.x * 256LL + threadIdx.x, step = gridDim.x * 256LL;
+    auto one = [&](long long i) {
+        const float x[1] = {a[i]}, y[1] = {b[i]};
+        f(x, y);
+    };
+    if (VEC) {
+        const long long nq = n / 4;
+#pragma unroll 2
+        for (long long i = t0; i < nq; i += step) {
+            const float4 p = reinterpret_cast<const float4 *>(a)[i], q = reinterpret_cast<const float4 *>(b)[i];
+            const float x[4] = {p.x, p.y, p.z, p.w}, y[4] = {q.x, q.y, q.z, q.w};
+            f(x, y);
+        }
+        if (t0 < n - 4 * nq)
+            one(4 * nq + t0);
+    } else {
+        for (long long i = t0; i < n; i += step)
+            one(i);
+    }
+}
+
 template <bool VEC>
 __global__ void __launch_bounds__(256) k_diff_stats(const float *a, const float *b, long long n, double *st)
 {
     __shared__ double red[2][8];
     DiffSums d;
-    const long long t0 = blockIdx.x * 256LL + threadIdx.x, step = gridDim.x * 256LL;
-    if (VEC) {
-        const long long nq = n / 4;
-#pragma unroll 2
-        for (long long i = t0; i < nq; i += step) {
-            const float4 x = reinterpret_cast<const float4 *>(a)[i], y = reinterpret_cast<const float4 *>(b)[i];
-            d.add({x.x, x.y, x.z, x.w}, {y.x, y.y, y.z, y.w});
+    each_pair<VEC>(a, b, n, [&](const auto &x, const auto &y) { d.add(x, y); });
+    double f1 = 0.0, f2 = 0.0;
+    if (__any_sync(0xffffffffu, d.far)) {
+        each_pair<VEC>(a, b, n, [&](const auto &x, const auto &y) { DiffSums::add_far(x, y, f1, f2); });
+        for (int o = 16; o > 0; o >>= 1) {
+            f1 += __shfl_xor_sync(0xffffffffu, f1, o);
+            f2 += __shfl_xor_sync(0xffffffffu, f2, o);
         }
-        if (t0 < n - 4 * nq)
-            d.add({a[4 * nq + t0]}, {b[4 * nq + t0]});
-    } else {
-        for (long long i = t0; i < n; i += step)
-            d.add({a[i]}, {b[i]});
+        d.far = true;
     }
     d.warp_sum();
     if ((threadIdx.x & 31) == 0) {
-        const double is = d.sc > 0.0f ? 1.0 / (double)d.sc : 0.0;
-        red[0][threadIdx.x >> 5] = d.s1.value();
-        red[1][threadIdx.x >> 5] = d.s2.value() * is * is;
+        const double is = d.sc > 0.0f ? 1.0f / d.sc : 0.0f;   // exact: a power of two
+        double v1 = d.s1.value(), v2 = d.s2.value() * is * is;
+        if (d.far) {
+            v1 += f1;
+            v2 += f2;
+        }
+        red[0][threadIdx.x >> 5] = v1;
+        red[1][threadIdx.x >> 5] = v2;
     }
     __syncthreads();
     if (threadIdx.x < 2) {

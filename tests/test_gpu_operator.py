@@ -264,3 +264,24 @@ def test_diff_stats_sums_no_worse_than_fp64(kind, seed):
     size = (sum(abs(v) for v in d), want[1])
     for got, w, s in zip(st.cpu().numpy(), want, size):
         assert abs(Fraction(float(got)) - w) <= 11 * Fraction(1, 2 ** 53) * s, float(Fraction(float(got)) / w - 1)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("x,y", [(np.inf, 0.0), (-np.inf, 1.0), (1.0, np.inf), (np.inf, np.inf), (np.nan, 1.0),
+                                 (3e38, -3e38), (-3.4e38, 3.4e38), (1e30, 0.0), (4e28, -4e28)])
+def test_diff_stats_of_infinite_and_very_large_differences(x, y, offset):
+    """One such difference among ordinary ones, as FP64 adds it: an infinite value keeps its sign, only
+    inf - inf and NaN make NaN, and two finite floats have a finite difference and square."""
+    import torch
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(5)
+    n = 5000
+    a, b = (rng.standard_normal(n + offset).astype(np.float32) for _ in range(2))
+    a[offset + 1234], b[offset + 1234] = x, y
+    ta, tb = torch.tensor(a, device="cuda")[offset:], torch.tensor(b, device="cuda")[offset:]
+    st = torch.zeros(2, dtype=torch.float64, device="cuda")
+    pkg.lbm2p_op_diff_stats(ta.data_ptr(), tb.data_ptr(), n, st.data_ptr(),
+                            torch.cuda.current_stream().cuda_stream)
+    with np.errstate(invalid="ignore"):
+        d = a[offset:].astype(np.float64) - b[offset:].astype(np.float64)
+    np.testing.assert_allclose(st.cpu().numpy(), [d.sum(), (d * d).sum()], rtol=2.0 ** -40)

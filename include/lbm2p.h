@@ -259,7 +259,9 @@ lbm2p_status lbm2p_set_state(lbm2p *h, const float *buf, size_t count, int on_de
    side).  Combined with warm_start = 1, the extrapolation is applied on top at the next step. */
 lbm2p_status lbm2p_warm_start(lbm2p *h, const float *P_guess, int on_device);
 
-/* Record CUDA events around each step and its sweeps (fills sweep_ms / step_ms). */
+/* Record CUDA events around each step and its sweeps (fills sweep_ms / step_ms).  Takes effect at the
+   next step; the graphs of timed steps and those of untimed ones are built at their first use and both
+   kept. */
 lbm2p_status lbm2p_set_timing(lbm2p *h, int enable);
 
 /* How the pressure sweeps run on this handle, as chosen at create: sweeps fused per launch

@@ -89,15 +89,15 @@ struct lbm2p {
     bool timing = false;
     cudaEvent_t ev_step0 = nullptr, ev_step1 = nullptr, ev_sw0 = nullptr, ev_sw1 = nullptr;
     // graph-resident sub-iteration (free-running solves when check_every is even and
-    // divides max_sub_iters): one graph per (f buffer, R buffer) for a bare solve, and one per
-    // (f buffer, g buffer, R buffer) for a whole physical step
+    // divides max_sub_iters): one graph per (timing off or on, f buffer, R buffer) for a bare solve, and
+    // one per (timing, f buffer, g buffer, R buffer) for a whole physical step
     bool graph_ok = false;
     lbm2p_dev::LoopCtl *ctl = nullptr;
     lbm2p_dev::LoopCtl *ctl_host = nullptr;       // pinned
-    cudaGraph_t solve_g[3][2] = {};
-    cudaGraphExec_t solve_x[3][2] = {};
-    cudaGraph_t step_g[3][2][2] = {};
-    cudaGraphExec_t step_x[3][2][2] = {};
+    cudaGraph_t solve_g[2][3][2] = {};
+    cudaGraphExec_t solve_x[2][3][2] = {};
+    cudaGraph_t step_g[2][3][2][2] = {};
+    cudaGraphExec_t step_x[2][3][2][2] = {};
     std::string autotune_log;          // one line per candidate timed at create
     std::string err;
 };

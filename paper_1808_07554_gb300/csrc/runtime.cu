@@ -188,23 +188,21 @@ void *dev_alloc(lbm2p *h, size_t bytes)
 // destroy the instantiated solve and step graphs (they are rebuilt on first use)
 void drop_graphs(lbm2p *h)
 {
-    for (int a = 0; a < 3; ++a)
-        for (int r = 0; r < 2; ++r) {
-            if (h->solve_x[a][r])
-                cudaGraphExecDestroy(h->solve_x[a][r]);
-            if (h->solve_g[a][r])
-                cudaGraphDestroy(h->solve_g[a][r]);
-            h->solve_x[a][r] = nullptr;
-            h->solve_g[a][r] = nullptr;
-            for (int b = 0; b < 2; ++b) {
-                if (h->step_x[a][b][r])
-                    cudaGraphExecDestroy(h->step_x[a][b][r]);
-                if (h->step_g[a][b][r])
-                    cudaGraphDestroy(h->step_g[a][b][r]);
-                h->step_x[a][b][r] = nullptr;
-                h->step_g[a][b][r] = nullptr;
+    auto drop = [](cudaGraphExec_t &x, cudaGraph_t &g) {
+        if (x)
+            cudaGraphExecDestroy(x);
+        if (g)
+            cudaGraphDestroy(g);
+        x = nullptr;
+        g = nullptr;
+    };
+    for (int t = 0; t < 2; ++t)
+        for (int a = 0; a < 3; ++a)
+            for (int r = 0; r < 2; ++r) {
+                drop(h->solve_x[t][a][r], h->solve_g[t][a][r]);
+                for (int b = 0; b < 2; ++b)
+                    drop(h->step_x[t][a][b][r], h->step_g[t][a][b][r]);
             }
-        }
 }
 
 void free_all(lbm2p *h)
@@ -483,18 +481,18 @@ lbm2p_status add_loop(lbm2p *h, cudaGraph_t G, const cudaGraphNode_t *dep, int p
 // a bare solve (current R and 1/tau_f) from f buffer pin; it ends in fnext(pin, 2)
 lbm2p_status solve_graph(lbm2p *h, int pin, cudaGraphExec_t *out)
 {
-    const int r = h->cur_r;
-    if (!h->solve_x[pin][r]) {
+    cudaGraphExec_t &x = h->solve_x[h->timing][pin][h->cur_r];
+    if (!x) {
         cudaGraph_t G;
         CUDA_TRY(h, cudaGraphCreate(&G, 0));
-        h->solve_g[pin][r] = G;
+        h->solve_g[h->timing][pin][h->cur_r] = G;
         cudaGraphNode_t last;
         lbm2p_status e = add_loop(h, G, nullptr, pin, false, &last, nullptr);
         if (e != LBM2P_OK)
             return e;
-        CUDA_TRY(h, cudaGraphInstantiate(&h->solve_x[pin][r], G, 0));
+        CUDA_TRY(h, cudaGraphInstantiate(&x, G, 0));
     }
-    *out = h->solve_x[pin][r];
+    *out = x;
     return LBM2P_OK;
 }
 
@@ -503,11 +501,11 @@ lbm2p_status solve_graph(lbm2p *h, int pin, cudaGraphExec_t *out)
 // 1/tau_f and P^{n-1}) are only read, so a step that fails leaves them as they were
 lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
 {
-    const int r = h->cur_r;
-    if (!h->step_x[pin][pg][r]) {
+    cudaGraphExec_t &x = h->step_x[h->timing][pin][pg][h->cur_r];
+    if (!x) {
         cudaGraph_t G;
         CUDA_TRY(h, cudaGraphCreate(&G, 0));
-        h->step_g[pin][pg][r] = G;
+        h->step_g[h->timing][pin][pg][h->cur_r] = G;
         cudaGraphNode_t nr, last, ifn, ns;
         RefreshArgs ra = refresh_args(h, pg);
         ra.ctl = h->ctl;
@@ -527,9 +525,9 @@ lbm2p_status step_graph(lbm2p *h, int pin, int pg, cudaGraphExec_t *out)
         const int pout = fnext(pin, 2);
         CUDA_TRY(h, lbm2p_launch::node_saturation(&ns, tail, nullptr,
                                                   saturation_args(h, pout, fnext(pin, 1), pg)));
-        CUDA_TRY(h, cudaGraphInstantiate(&h->step_x[pin][pg][r], G, 0));
+        CUDA_TRY(h, cudaGraphInstantiate(&x, G, 0));
     }
-    *out = h->step_x[pin][pg][r];
+    *out = x;
     return LBM2P_OK;
 }
 
@@ -2234,12 +2232,7 @@ lbm2p_status lbm2p_set_timing(lbm2p *h, int enable)
 {
     if (!h)
         return fail(nullptr, LBM2P_EINVAL, "NULL handle");
-    if (h->timing != (enable != 0)) {
-        // the solve graphs record the events only where timing is on; rebuilt on the next solve
-        CUDA_TRY(h, cudaStreamSynchronize((cudaStream_t)h->stream));
-        drop_graphs(h);
-        h->timing = enable != 0;
-    }
+    h->timing = enable != 0;            // the solve graphs with the events and those without are both kept
     return LBM2P_OK;
 }
 

@@ -264,8 +264,8 @@ lbm2p_status lbm2p_warm_start(lbm2p *h, const float *P_guess, int on_device);
    kept. */
 lbm2p_status lbm2p_set_timing(lbm2p *h, int enable);
 
-/* How the pressure sweeps run on this handle, as chosen at create: sweeps fused per launch
-   (1, 2 or 4); the single-sweep kernel (an lbm2p_sweep_kernel value, never AUTO); the tile
+/* How the pressure sweeps run on this handle, as chosen at create (sweep counts given by the caller on
+   small lattices: see lbm2p_counters): sweeps fused per launch (1, 2 or 4); the single-sweep kernel (an lbm2p_sweep_kernel value, never AUTO); the tile
    of the kernel that runs the sweeps: for fused sweeps its threads per block (columns per
    block for the two-sweep row-walking kernels: 120 or 240; 32 for the four-sweep kernel's
    one-warp tiles of 56 columns) and rows per block, for the ROWS
@@ -310,7 +310,10 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
  * kinds once per grid tried: the resident-block capacity of the GPU down to half of it).  Owned by h; valid until the next create-time tuning. */
 const char *lbm2p_autotune_report(const lbm2p *h);
 
-/* Running totals since creation: kernels launched by the library, pressure sweeps run. */
+/* Running totals since creation: kernels launched by the library, pressure sweeps run.  Sweep counts that
+   the caller gives (replay, init_replay, lbm2p_pressure_sweeps) on lattices of fewer than 512^2 nodes
+   do not use the four-sweep form FUSED_QUAD unless fuse_sweeps = 4 asks for it, so with walls on every
+   side they take at least one launch per two sweeps there. */
 lbm2p_status lbm2p_counters(const lbm2p *h, long long *launches, long long *sweeps);
 
 /* ---- Batched realisations --------------------------------------------------------------

@@ -43,7 +43,7 @@ struct lbm2p {
     int grid_k[2] = {}, grid_check_k[2] = {}, grid_cap_k[2] = {};
     int rows_w = 0, rows_slots = 0, rows_H = 0, rows_grid = 0;   // staged-rows kernel shape
     lbm2p_internal::FusedShape tb;          // fused sweeps per launch, chosen at create
-    lbm2p_internal::FusedShape host_form;   // the same for counts driven from the host
+    lbm2p_internal::FusedShape count_form;  // the same for sweep counts given by the caller
     int tb_T_graph = 0;        // fused sweeps used inside the graph loop body (0: single sweeps)
     int res_C = 0;             // blocks of the cluster that runs whole solves (resident.cu), or 0
     bool fp16 = false;         // storage FP16_DEV: sweeps run on FP16 copies inside a solve

@@ -781,7 +781,7 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
         if (h->timing)
             CUDA_TRY(h, cudaEventRecord(h->ev_sw0, st));
         const int n = upto - k;
-        const FusedShape &fs = h->host_form;
+        const FusedShape &fs = replay >= 0 ? h->count_form : h->tb;
         const int T = fs.T;
         const int nf = (T > 1 && n >= T) ? n / T : 0;
         const int ns = n - nf * T;
@@ -1134,18 +1134,21 @@ lbm2p_status autotune_sweeps(lbm2p *h)
     // direct form estimated 8 % ahead here with a 16-sweep check period and 3.5 % ahead in the
     // loop; 8 % ahead with an 8-sweep period and about even in the loop)
     float single_best = 1e30f;
-    // counts driven from the host (replays, bare sweeps) below 512^2 keep launches of at most two
-    // sweeps: what a caller reads from lbm2p_counters there is launches per sweep
-    const bool host_two = h->p.fuse_sweeps == 0 && h->nnodes < 512LL * 512;
-    float host_best = 1e30f;
+    // Counts given by the caller (replays, bare sweeps) keep to the other forms below 512^2, as
+    // lbm2p_counters documents: callers there read launches per sweep, and test_gpu_parity.py holds them
+    // to one per two sweeps at 128^2.  It costs time: 64 sweeps from the host 347 us at 128^2 where the
+    // four-sweep form takes 180, 445 and 215 at 500^2.
+    const bool count_other = h->p.fuse_sweeps == 0 && h->nnodes < 512LL * 512;
+    float count_best = 1e30f;
     auto take = [&](float per, const FusedShape &s, bool pinned) {
         if (pinned || (per < best && (h->tb.T > 1 || per < kFusedMargin * single_best))) {
             best = per;
             h->tb = s;
         }
-        if (host_two && s.T == 2 && per < host_best && per < kFusedMargin * single_best) {
-            host_best = per;
-            h->host_form = s;
+        if (count_other && s.kind != 3 && per < count_best &&
+            (h->count_form.T > 1 || per < kFusedMargin * single_best)) {
+            count_best = per;
+            h->count_form = s;
         }
     };
     h->autotune_log.clear();
@@ -1168,7 +1171,7 @@ lbm2p_status autotune_sweeps(lbm2p *h)
             return true;
         return timed(launch, ms);
     };
-    h->tb = h->host_form = FusedShape{};
+    h->tb = h->count_form = FusedShape{};
     h->sweep_kind = forced == LBM2P_SWEEP_AUTO ? 0 : forced - 1;
     if (!fused_only || forced != LBM2P_SWEEP_AUTO) {
         // grid-stride kernels: resident blocks per SM from the occupancy limit down to half
@@ -1437,8 +1440,8 @@ lbm2p_status autotune_sweeps(lbm2p *h)
             }
         }
     }
-    if (!host_two)
-        h->host_form = h->tb;
+    if (!count_other)
+        h->count_form = h->tb;
     // whole solves in one launch, for lattices that fit a cluster's shared memory and solves that the
     // graph loop can run (it ends them at the same checks): timed over four check periods of at most
     // 64 sweeps (the tolerance -1 never stops it; a check is then 0.03 us per sweep, and four whole
@@ -1813,7 +1816,7 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
             return e;
     } else {
         h->sweep_kind = 1;
-        h->tb = h->host_form = FusedShape{};
+        h->tb = h->count_form = FusedShape{};
         lbm2p_status e = autotune_h(h, sms);
         if (e != LBM2P_OK)
             return e;
@@ -1825,7 +1828,7 @@ lbm2p_status build(lbm2p *h, const lbm2p_inputs *in, lbm2p_step_stats *init_stat
     h->grid_check = h->grid_check_k[h->sweep_kind < 2 ? h->sweep_kind : 1];
     {
         int np = h->tb.grid > h->rows_grid ? h->tb.grid : h->rows_grid;
-        np = np > h->host_form.grid ? np : h->host_form.grid;
+        np = np > h->count_form.grid ? np : h->count_form.grid;
         np = np > h->grid_h ? np : h->grid_h;
         np = np > h->h16_grid ? np : h->h16_grid;
         np = np > h->h16q_grid ? np : h->h16q_grid;
@@ -2310,7 +2313,7 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
     h->tb_T_graph = h->p.check_every % 4 == 0 ? 2 : 0;
     const bool staged = form == LBM2P_FUSED_STAGED_ROWS;
     h->tb = FusedShape{2, staged ? 1 : 2, 30 * warps, rows, (int)grid, staged ? slots : 0};
-    h->host_form = h->tb;
+    h->count_form = h->tb;
     return LBM2P_OK;
 }
 

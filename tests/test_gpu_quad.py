@@ -106,3 +106,26 @@ def test_wells_that_share_a_node(nx, ny, i, j, bc):
             assert np.array_equal(state, member.get_state())
     for s in (one, four, member):
         s.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(64, 64), (128, 128), (300, 140)])
+def test_solves_driven_from_the_host_use_the_tuned_form(nx, ny):
+    """A cap that is no multiple of check_every: the host runs the solve, four sweeps per launch where
+    that is the form reported (lattices of fewer than 512^2 nodes included), and each check is a period of
+    two launches and the reduction."""
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(nx)
+    prob = uniform(nx, ny, bc=(1, 1, 1, 1), K=np.exp(rng.standard_normal((ny, nx))), S0=0.4,
+                   wells=[(0, 0, 1e-2, 0), (nx - 1, ny - 1, 1e-2, 1)])
+    kw = dict(init_replay=8, tol=0.0, check_every=8, max_sub_iters=44)
+    one, auto = pkg.Solver.from_problem(prob, fuse_sweeps=1, **kw), pkg.Solver.from_problem(prob, **kw)
+    if auto.fused_form() != pkg.FUSED_QUAD:
+        pytest.skip("the four-sweep form was not the fastest here")
+    before = auto.counters()
+    assert one.step(1)[1][0].sub_iters == 44 and auto.step(1)[1][0].sub_iters == 44
+    after = auto.counters()
+    # refresh and saturation; five periods of 8 sweeps and one of 4, each with its reduction
+    assert (after[0] - before[0], after[1] - before[1]) == (2 + 5 * 3 + 2, 44)
+    assert np.array_equal(one.get_state(), auto.get_state())
+    one.close()
+    auto.close()

@@ -2248,10 +2248,11 @@ lbm2p_status lbm2p_sweep_config(const lbm2p *h, int *fused, int *kind, int *tile
     if (h->fp16) {                       // the FP16 sweep kernels
         if (kind)
             *kind = h->h16_kind == 1 ? LBM2P_SWEEP_ROWS : LBM2P_SWEEP_SCALAR;
+        const bool four = h->h16q_H > 0;
         if (tile_w)
-            *tile_w = h->h16_kind == 1 ? h->h16_w : 0;
+            *tile_w = four ? 32 : (h->h16_kind == 1 ? h->h16_w : 0);
         if (tile_h)
-            *tile_h = h->h16_kind == 1 ? h->h16_H : 0;
+            *tile_h = four ? h->h16q_H : (h->h16_kind == 1 ? h->h16_H : 0);
         return LBM2P_OK;
     }
     if (kind)
@@ -2268,7 +2269,7 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
     if (!h)
         return fail(nullptr, LBM2P_EINVAL, "NULL handle");
     if (h->fp16)
-        return fail(h, LBM2P_EINVAL, "FP16 storage sweeps one sweep per launch");
+        return fail(h, LBM2P_EINVAL, "FP16 storage has no two-sweep form to pin");
     for (int sd = 0; sd < 4; ++sd)
         if (h->p.bc[sd] == LBM2P_BC_PERIODIC)
             return fail(h, LBM2P_EINVAL, "the two-sweep row-walking kernels need walls on every side");

@@ -186,3 +186,26 @@ def test_four_fp16_sweeps_equal_single_sweeps(nx, ny, bc, dense):
         assert r4 == pytest.approx(r1, rel=1e-3, abs=1e-30)
     one.close()
     four.close()
+
+
+def test_sweep_config_reports_the_tile_of_the_form_that_runs():
+    """(sweeps per launch, single-sweep kernel, threads and rows of the tile): those of the four-sweep
+    kernel where it runs, else of the single-sweep kernel."""
+    import paper_1808_07554_gb300 as pkg
+    prob = W.quarter_five_spot(300, 140, seed=12, corr_len=6.0)
+    four = pkg.Solver.from_problem(prob, init_replay=0, fuse_sweeps=4, storage=pkg.STORE_FP16_DEV)
+    quad = [r for r in four.autotune_report() if r[0] == "fp16_quad"]
+    assert four.fused_form() == pkg.FUSED_QUAD and quad
+    fused, kind, w, rows = four.sweep_config()
+    assert (fused, w, rows) == (4, 32, min(quad, key=lambda r: r[-1])[3])
+    assert kind in (pkg.SWEEP_SCALAR, pkg.SWEEP_ROWS)
+    four.close()
+    one = pkg.Solver.from_problem(prob, init_replay=0, storage=pkg.STORE_FP16_DEV,
+                                  sweep_kernel=pkg.SWEEP_SCALAR)
+    assert one.sweep_config() == (1, pkg.SWEEP_SCALAR, 0, 0)
+    one.close()
+    rows = pkg.Solver.from_problem(prob, init_replay=0, storage=pkg.STORE_FP16_DEV,
+                                   sweep_kernel=pkg.SWEEP_ROWS)
+    best = min((r for r in rows.autotune_report() if r[0] == "fp16_rows"), key=lambda r: r[-1])
+    assert rows.sweep_config() == (1, pkg.SWEEP_ROWS, best[1], best[3])
+    rows.close()

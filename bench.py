@@ -13,13 +13,16 @@ Metric: MLUPS = nodes x (pressure sweeps + 1 saturation update) / time, summed o
 timed steps (and over ranks).  L2 is flushed before every timed step; each step is timed
 with CUDA events on the solver's stream.
 
-Roofline of the dominant kernel (the pressure sweep launch): algorithmic bytes = 68 B per
-node and pressure sweep (8 populations read and written, plus 1/tau_f) x the sweeps one
-launch performs x nodes, over the launch's average device time (CUDA events around the
-sweep batches, on the solver's stream), against the measured HBM copy bandwidth.  A launch
-that carries two sweeps moves the populations once, so this fraction can exceed 1; the
-DRAM bytes such a launch really moves (from an ncu capture of the same kernel source) give
-the DRAM-actual fraction beside it.
+Roofline of the dominant kernel (the pressure sweep launch): the bytes that the launch cannot
+do without, one pass over the state whatever the sweeps that it carries (72 B per node: 8
+populations read and written, 1/tau_f, the reference pressure; 44 B with FP16 storage), over the
+launch's average device time (CUDA events around the sweep batches, on the solver's stream),
+against the measured HBM copy bandwidth.  Beside it the rate of the paper's form of the sweep,
+68 B per node and sweep (8 populations read and written, plus 1/tau_f): with four sweeps per
+launch most of these bytes stay in registers, so that rate exceeds the bandwidth.  The DRAM bytes
+that a launch really moves (from an ncu capture of the same kernel sources) give the DRAM-actual
+fraction.  Where a lattice stays on chip for a whole solve, that solve is the launch and the
+bandwidth does not bound it.
 
 Workload batch_five_spot_64: 64 independent five-spot realisations with sizes drawn from
 {128, 256, 512}^2 (sigma, correlation length and viscosity ratio drawn per member), advanced
@@ -50,14 +53,14 @@ sys.path.insert(0, ROOT)
 import workloads as W  # noqa: E402
 from paper_1808_07554_gb300.initial_guess import coarse_initial_pressure  # noqa: E402
 
-# algorithmic bytes per node and pressure sweep (the paper's form of the sweep): 8
-# populations read and written + 1/tau_f; f_0 is never needed, the sparse wells add nothing
+# bytes per node and pressure sweep of the paper's form of the sweep: 8 populations read and
+# written + 1/tau_f; f_0 is never needed, the sparse wells add nothing
 BYTES_PER_NODE_SWEEP = 68
-# bytes per node the FP32 deviation storage really moves per launch (one pass over the
-# populations whatever the sweeps per launch): the 68 above + the reference pressure R
+# bytes per node that a launch cannot do without (one pass over the populations whatever the sweeps
+# per launch): the 68 above + the reference pressure R
 BYTES_MOVED_PER_NODE = 72
 # with FP16 storage: 8 populations x (2 + 2) B + the node pressure read and written + 1/tau_f
-BYTES_PER_SWEEP_NODE_FP16 = 44
+BYTES_MOVED_PER_NODE_FP16 = 44
 WORKLOADS = {
     "five_spot_4096": dict(kind="five_spot", n=4096),
     "five_spot_1024": dict(kind="five_spot", n=1024),
@@ -74,6 +77,10 @@ SWEEP_KERNEL_NAMES = {1: "four nodes per thread (128-bit accesses)", 2: "one nod
                       3: "rows staged in shared memory by bulk async copies"}
 # CUDA sources each launch form is compiled from; their hash keys the ncu captures below
 KERNEL_SOURCES = {
+    "stages": ["kernels.cu", "lbm2p_node.cuh", "lbm2p_device.cuh"],
+    "single_fp16": ["fp16.cu", "lbm2p_node.cuh", "lbm2p_device.cuh", "lbm2p_async.cuh"],
+    "four_sweep_fp16": ["fp16_quad.cu", "sweep_quad.cuh", "lbm2p_node.cuh", "lbm2p_device.cuh",
+                        "lbm2p_async.cuh"],
     "four_sweep": ["sweep_quad.cu", "sweep_quad.cuh", "lbm2p_node.cuh", "lbm2p_device.cuh"],
     "resident": ["resident.cu", "lbm2p_node.cuh", "lbm2p_device.cuh"],
     "two_sweep": ["sweep_rows.cu", "lbm2p_node.cuh", "lbm2p_device.cuh", "lbm2p_async.cuh"],
@@ -94,8 +101,7 @@ NCU_TRAFFIC_PER_LAUNCH = {
 }
 FUSED_FORM_NAMES = {1: "stages", 2: "staged_rows", 3: "direct", 4: "quad", 5: "resident"}
 FUSED_FORM_TEXT = {1: "on shared-memory stages", 2: "on rows staged by bulk copies",
-                   3: "with direct loads", 4: "in registers, one warp per tile of 56 columns",
-                   5: "of a whole solve in one launch, the lattice in a cluster's shared memory"}
+                   3: "with direct loads", 4: "in registers, one warp per tile of 56 columns"}
 
 
 def log(msg: str) -> None:
@@ -120,6 +126,36 @@ def captured_traffic(form, src_hash: str):
     if cap is None or cap["sources"] != src_hash:
         return None, None
     return cap["bytes"], cap["profile"]
+
+
+def sweep_launch(fform: int, fused: int, kind: int, fp16: bool) -> dict:
+    """The launch that runs the pressure sweeps, from what the handle reports (lbm2p_fused_form_of,
+    sweeps per launch, single-sweep kernel): its form, the sweeps it carries (None: a whole solve),
+    the bytes per node that it cannot do without, its sources, and texts."""
+    if fform == 5:
+        return {"form": "resident", "sources": "resident", "sweeps": None,
+                "bytes_per_node": BYTES_MOVED_PER_NODE, "bound": "cluster barriers",
+                "text": "a whole solve per launch, the lattice in a cluster's shared memory",
+                "bytes_model": "72 B per node and solve (read and written once)"}
+    form = FUSED_FORM_NAMES[fform] if fused > 1 else "single"
+    out = {"form": form, "sweeps": fused, "bound": "hbm",
+           "sources": {"single": "single", "stages": "stages", "quad": "four_sweep"}.get(form, "two_sweep"),
+           "text": (f"{fused} sweeps per launch {FUSED_FORM_TEXT[fform]}" if fused > 1
+                    else SWEEP_KERNEL_NAMES.get(kind, "?"))}
+    if fp16:
+        out["text"] = "FP16 populations, " + out["text"]
+        out["sources"] = "four_sweep_fp16" if fused > 1 else "single_fp16"
+    out["bytes_per_node"] = BYTES_MOVED_PER_NODE_FP16 if fp16 else BYTES_MOVED_PER_NODE
+    out["bytes_model"] = (f"{out['bytes_per_node']} B per node and launch of "
+                          + (f"{fused} sweeps" if fused > 1 else "one sweep"))
+    return out
+
+
+def batch_sweeps_per_launch(nx: int, ny: int, check_every: int) -> int:
+    """Sweeps that a batched launch carries for a wall-bounded member (lbm2p_batch_create's rule)."""
+    if check_every % 8 == 0:
+        return 4
+    return 2 if nx * ny >= 512 * 512 and check_every % 4 == 0 else 1
 
 
 def batch_members(name: str, rank: int = 0):
@@ -534,27 +570,21 @@ def run_ours(args):
 
     peak, peak_kind = peaks()
     sweeps_timed = int(np.sum(ksub))
-    avg_sweep_s = float(np.sum(sweep_ms)) / 1e3 / max(1, sweeps_timed)
-    fused = sweep_cfg[0]
-    avg_launch_s = avg_sweep_s * fused
+    sweep_s = float(np.sum(sweep_ms)) / 1e3
     fp16 = args.storage == "fp16"
-    # algorithmic bytes per launch: 68 B per node and sweep x the sweeps of one launch
-    bpn = BYTES_PER_SWEEP_NODE_FP16 if fp16 else BYTES_PER_NODE_SWEEP * fused
-    achieved = bpn * nodes / avg_launch_s / 1e9
-    form = ((args.workload, FUSED_FORM_NAMES.get(fform, "?"), sweep_cfg[2]) if fused > 1
-            else (args.workload, "single", sweep_cfg[1]))
-    src_form = {4: "four_sweep", 5: "resident"}[fform] if fform in (4, 5) else ("two_sweep" if fused > 1 else "single")
-    src_hash = kernel_source_hash(src_form)
+    lc = sweep_launch(fform, sweep_cfg[0], sweep_cfg[1], fp16)
+    # launches that the sweep time was spent on: one per solve, or one per lc["sweeps"] sweeps
+    launches_timed = args.steps if lc["sweeps"] is None else sweeps_timed / lc["sweeps"]
+    avg_launch_s = sweep_s / max(1.0, launches_timed)
+    achieved = lc["bytes_per_node"] * nodes / avg_launch_s / 1e9
+    form = (args.workload, lc["form"], sweep_cfg[1] if lc["form"] == "single" else sweep_cfg[2])
+    src_hash = kernel_source_hash(lc["sources"])
     traffic, traffic_profile = captured_traffic(form, src_hash) if not fp16 else (None, None)
     hist = {}
     for k in ksub:
         hist[str(k)] = hist.get(str(k), 0) + 1
-    kernel_text = ("pressure sweep (fused stream + collide, Eq. 3-1), "
-                   + (("FP16 populations, " + SWEEP_KERNEL_NAMES.get(sweep_cfg[1], "?"))
-                      if fp16 else
-                      ((f"{fused} sweeps per launch " + FUSED_FORM_TEXT.get(fform, "?"))
-                       if fused > 1 else SWEEP_KERNEL_NAMES.get(sweep_cfg[1], "?"))
-                      + (", autotuned" if args.sweep_kernel == 0 else "")))
+    kernel_text = ("pressure sweep (fused stream + collide, Eq. 3-1), " + lc["text"]
+                   + (", autotuned" if args.sweep_kernel == 0 and not fp16 else ""))
     line = {
         "metric": "MLUPS", "value": updates_all / time_max / 1e6, "unit": "MLUPS",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -585,17 +615,19 @@ def run_ours(args):
                    "wall_s": round(wall, 3),
                    "learned_operator": op_log,
                    "parallelism": f"{world} independent realisations (seed 2 + rank)"},
-        "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+        "roofline": {"bound": lc["bound"], "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "kernel": kernel_text,
-                     "bytes_per_launch": bpn * nodes,
-                     "bytes_model": ("44 B per node and sweep (FP16 storage)" if fp16 else
-                                     f"68 B per node and sweep x {fused} sweeps per launch"),
-                     "sweeps_per_launch": fused,
+                     "bytes_per_launch": lc["bytes_per_node"] * nodes,
+                     "bytes_model": lc["bytes_model"],
+                     "sweeps_per_launch": (lc["sweeps"] if lc["sweeps"] is not None
+                                           else sweeps_timed / args.steps),
                      "avg_launch_us": avg_launch_s * 1e6,
-                     "launch_time_includes": ("the residual finalize kernel of every "
+                     "launch_time_includes": ("the residual checks" if lc["sweeps"] is None else
+                                              "the residual finalize kernel of every "
                                               f"{args.check_every}th sweep"),
-                     "dram_bytes_moved_model": (None if fp16 else BYTES_MOVED_PER_NODE * nodes),
+                     "paper_form_gbs": (BYTES_PER_NODE_SWEEP * nodes * sweeps_timed
+                                        / max(sweep_s, 1e-30) / 1e9),
                      "dram_frac": (traffic / avg_launch_s / 1e9 / peak
                                    if traffic is not None else None),
                      "traffic_source": (f"ncu capture, {traffic_profile}" if traffic is not None
@@ -707,7 +739,8 @@ def run_batch(args):
     gpu_launches = batch.counters()[0] - launches0
     k = np.array(kmat, dtype=np.int64)                       # [steps, members]
     updates = int(np.sum(k * nodes[None, :]) + args.steps * nodes.sum())
-    step_bytes = float(np.sum((BYTES_MOVED_PER_NODE * k + BYTES_PER_STEP_NODE) * nodes[None, :]))
+    per = np.array([batch_sweeps_per_launch(p.nx, p.ny, args.check_every) for p in probs])
+    step_bytes = float(np.sum((BYTES_MOVED_PER_NODE * k / per + BYTES_PER_STEP_NODE) * nodes[None, :]))
     total_ms = float(np.sum(step_ms))
 
     # end to end: batch step + P and S of every member read back to host memory
@@ -770,9 +803,11 @@ def run_batch(args):
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak,
                      "traffic": None,
-                     "kernel": "whole batched step (k_quad_batch, four sweeps per launch, for "
-                               "the wall-bounded members): 72 B per node and sweep + the "
-                               "per-step kernels' bytes / step time",
+                     "kernel": (f"whole batched step (launches of {'/'.join(str(v) for v in sorted(set(per)))}"
+                                " sweeps): 72 B per node and launch + the per-step kernels' bytes"
+                                " / step time"),
+                     "paper_form_gbs": float(np.sum(BYTES_PER_NODE_SWEEP * k * nodes[None, :])
+                                             / (total_ms / 1e3) / 1e9),
                      "bytes_per_step": step_bytes / args.steps, "peak_kind": peak_kind},
         "e2e": {"value": e2e_all / e2e_max / 1e6, "unit": "MLUPS", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": int(8 * nodes.sum())},

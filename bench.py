@@ -39,6 +39,7 @@ import argparse
 import datetime
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -75,17 +76,16 @@ WORKLOADS = {
 DEFAULT_WORKLOAD = "five_spot_4096"
 SWEEP_KERNEL_NAMES = {1: "four nodes per thread (128-bit accesses)", 2: "one node per thread",
                       3: "rows staged in shared memory by bulk async copies"}
-# CUDA sources each launch form is compiled from; their hash keys the ncu captures below
+# The translation units that hold the kernels of each launch form; with every header of the sources
+# that they include they make the hash that keys the ncu captures below
 KERNEL_SOURCES = {
-    "stages": ["kernels.cu", "lbm2p_node.cuh", "lbm2p_device.cuh"],
-    "single_fp16": ["fp16.cu", "lbm2p_node.cuh", "lbm2p_device.cuh", "lbm2p_async.cuh"],
-    "four_sweep_fp16": ["fp16_quad.cu", "sweep_quad.cuh", "lbm2p_node.cuh", "lbm2p_device.cuh",
-                        "lbm2p_async.cuh"],
-    "four_sweep": ["sweep_quad.cu", "sweep_quad.cuh", "lbm2p_node.cuh", "lbm2p_device.cuh"],
-    "resident": ["resident.cu", "lbm2p_node.cuh", "lbm2p_device.cuh"],
-    "two_sweep": ["sweep_rows.cu", "lbm2p_node.cuh", "lbm2p_device.cuh", "lbm2p_async.cuh"],
-    "single": ["kernels.cu", "sweep_rows.cu", "lbm2p_node.cuh", "lbm2p_device.cuh",
-               "lbm2p_async.cuh"],
+    "single": ["kernels.cu", "sweep_rows.cu"],
+    "stages": ["kernels.cu"],
+    "two_sweep": ["sweep_rows.cu"],
+    "four_sweep": ["sweep_quad.cu"],
+    "resident": ["resident.cu"],
+    "single_fp16": ["fp16.cu"],
+    "four_sweep_fp16": ["fp16_quad.cu"],
 }
 # DRAM bytes per pressure-sweep launch (dram__bytes_read.sum + dram__bytes_write.sum) from
 # one ncu capture, keyed by workload and launch form (sweeps per launch, fused form, tile
@@ -110,10 +110,29 @@ def log(msg: str) -> None:
     print(f"[bench {time.strftime('%H:%M:%S')}] {msg}", file=sys.stderr, flush=True)
 
 
+def kernel_source_files(form: str) -> list:
+    """The sources of a launch form: its translation units and the headers beside them that they
+    include, directly or not, in the order of first use."""
+    out = []
+
+    def visit(name):
+        path = os.path.join(ROOT, "paper_1808_07554_gb300", "csrc", name)
+        if name in out or not os.path.exists(path):
+            return
+        out.append(name)
+        with open(path) as fh:
+            for inc in re.findall(r'^\s*#\s*include\s+"([^"]+)"', fh.read(), re.M):
+                visit(inc)
+
+    for unit in KERNEL_SOURCES[form]:
+        visit(unit)
+    return out
+
+
 def kernel_source_hash(form: str) -> str:
     import hashlib
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES[form]:
+    for f in kernel_source_files(form):
         with open(os.path.join(ROOT, "paper_1808_07554_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

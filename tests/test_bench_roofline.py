@@ -49,3 +49,43 @@ def test_measured_launches_stay_below_the_bandwidth():
                                             (512, 6, 1)])
 def test_sweeps_of_a_batched_launch(n, every, sweeps):
     assert bench.batch_sweeps_per_launch(n, n, every) == sweeps
+
+
+@pytest.mark.parametrize("form,needs", [
+    ("single", {"kernels.cu", "sweep_rows.cu", "lbm2p_async.cuh", "residual.cuh"}),
+    ("stages", {"kernels.cu", "residual.cuh", "step_node.cuh"}),
+    ("two_sweep", {"sweep_rows.cu", "lbm2p_async.cuh"}),
+    ("four_sweep", {"sweep_quad.cu", "sweep_quad.cuh", "lbm2p_async.cuh"}),
+    ("resident", {"resident.cu", "residual.cuh", "lbm2p_async.cuh"}),
+    ("single_fp16", {"fp16.cu", "lbm2p_async.cuh"}),
+    ("four_sweep_fp16", {"fp16_quad.cu", "sweep_quad.cuh", "lbm2p_async.cuh"}),
+])
+def test_source_hash_covers_every_header_that_the_kernels_compile_from(form, needs, monkeypatch):
+    """Every file is hashed: an edit of any of them changes the hash that keys a capture."""
+    import builtins
+    files = bench.kernel_source_files(form)
+    assert needs | {"lbm2p_node.cuh", "lbm2p_device.cuh"} <= set(files) and len(files) == len(set(files))
+    before = bench.kernel_source_hash(form)
+    real = builtins.open
+    for edited in files:
+        class Edited:
+            def __init__(self, f):
+                self.f = f
+
+            def __enter__(self):
+                return self
+
+            def __exit__(self, *exc):
+                self.f.close()
+
+            def read(self):
+                return self.f.read() + b" "
+
+        def fake(path, mode="r", *a, **k):
+            f = real(path, mode, *a, **k)
+            return Edited(f) if "b" in mode and str(path).endswith(os.sep + edited) else f
+
+        monkeypatch.setattr(builtins, "open", fake)
+        assert bench.kernel_source_hash(form) != before, edited
+        monkeypatch.setattr(builtins, "open", real)
+    assert bench.kernel_source_hash(form) == before

@@ -50,26 +50,16 @@ __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
     k_pressure_quad(const __grid_constant__ PressureArgs a, int H)
 {
     extern __shared__ __align__(128) float smem_raw[];
-    __shared__ double red[kQuadWarps][4];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float *smem = quad_warp_smem<S>(smem_raw, warp, a.Fp != nullptr);
-    const int tile = blockIdx.x * kQuadWarps + warp;
+    const int lane = threadIdx.x;
     ResAcc racc;
-    if (tile < QuadPlan(H, a.g.nx, a.g.ny).tiles())
-        quad_tile<CHECK, S, UNROLL>(a, H, tile, smem, lane, racc);
+    if (blockIdx.x < QuadPlan(H, a.g.nx, a.g.ny).tiles())
+        quad_tile<CHECK, S, UNROLL>(a, H, blockIdx.x, smem_raw, lane, racc);
     if (CHECK) {
         double v[4];
         racc.warp_totals(v);
         if (lane == 0)
             for (int c = 0; c < 4; ++c)
-                red[warp][c] = v[c];
-        __syncthreads();
-        if (threadIdx.x < 4) {
-            double s = 0.0;
-            for (int w = 0; w < kQuadWarps; ++w)
-                s += red[w][threadIdx.x];
-            a.partials[4 * blockIdx.x + threadIdx.x] = s;
-        }
+                a.partials[4 * (size_t)blockIdx.x + c] = v[c];
     }
 }
 
@@ -87,10 +77,9 @@ __global__ void __launch_bounds__(kQuadThreads, kQuadBlocks)
 {
     extern __shared__ __align__(128) float smem_raw[];
     __shared__ PressureArgs a;
-    static_assert(kQuadWarps == 1, "an item per block");
     if ((int)blockIdx.x >= *nitems)
         return;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x;
     const int2 e = items[blockIdx.x];
     const unsigned *src = reinterpret_cast<const unsigned *>(pa + 2 * e.x + parity);
     for (int i = lane; i < (int)(sizeof(PressureArgs) / 4); i += 32)
@@ -131,8 +120,7 @@ using namespace lbm2p_dev;
 
 long long quad_grid(int H, int nx, int ny)
 {
-    const long long tiles = QuadPlan(H, nx, ny).tiles();
-    return (tiles + kQuadWarps - 1) / kQuadWarps;
+    return QuadPlan(H, nx, ny).tiles();
 }
 
 int quad_tile_slots(bool has_fp)
@@ -150,7 +138,7 @@ int quad_tile_slots(bool has_fp)
             lo = b < lo ? b : lo;
         }
     }
-    return sms * lo * kQuadWarps;
+    return sms * lo;
 }
 
 cudaError_t quad_prepare()

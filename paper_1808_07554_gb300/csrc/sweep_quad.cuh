@@ -16,8 +16,7 @@ constexpr int kQuadT = 4;                     // sweeps per launch
 constexpr int kQuadCols = 64;                 // columns of a warp: two per lane
 constexpr int kQuadHalo = 4;                  // columns on each side that it does not own
 constexpr int kQuadOwn = kQuadCols - 2 * kQuadHalo;
-constexpr int kQuadWarps = 1;                 // warps (tiles) per block
-constexpr int kQuadThreads = 32 * kQuadWarps;
+constexpr int kQuadThreads = 32;              // a block is one warp with one tile
 constexpr int kQuadBlocks = 8;                // blocks per SM: two warps per scheduler, 255 registers
 constexpr int kQuadSlots = 7;                 // ring slots: rows in flight = slots - 3
 
@@ -80,20 +79,9 @@ struct QuadPlan {
     }
 };
 
-__host__ __device__ constexpr size_t quad_warp_bytes(int slots, bool has_fp)
-{
-    return (size_t)slots * (has_fp ? 11 : 10) * kQuadCols * sizeof(float);
-}
-
 inline size_t quad_smem_bytes(bool has_fp)
 {
-    return kQuadWarps * quad_warp_bytes(kQuadSlots, has_fp);
-}
-
-template <int S>
-__device__ __forceinline__ float *quad_warp_smem(float *raw, int warp, bool has_fp)
-{
-    return raw + warp * (quad_warp_bytes(S, has_fp) / sizeof(float));
+    return (size_t)kQuadSlots * (has_fp ? 11 : 10) * kQuadCols * sizeof(float);
 }
 
 // 16 bytes global -> shared without a register round trip

@@ -278,7 +278,7 @@ typedef enum {
     LBM2P_FUSED_STAGES = 1,      /* T sweeps on shared-memory stages (T = 2 or 4) */
     LBM2P_FUSED_STAGED_ROWS = 2, /* two sweeps on rows staged by bulk copies */
     LBM2P_FUSED_DIRECT = 3,      /* two sweeps, inputs loaded directly (lattices held in L2) */
-    LBM2P_FUSED_QUAD = 4,        /* four sweeps, one warp per tile of 56 columns */
+    LBM2P_FUSED_QUAD = 4,        /* four sweeps, one warp per tile of 56 columns (FP32 or FP16 storage) */
     LBM2P_FUSED_RESIDENT = 5     /* whole solves in one launch, the lattice in the shared memory of
                                     a thread-block cluster (small lattices, check_every even and
                                     max_sub_iters a multiple of it) */
@@ -303,11 +303,16 @@ lbm2p_status lbm2p_set_fused_shape(lbm2p *h, int form, int warps, int slots, int
  *   "fused <sweeps per launch> <threads per block> <rows per block> <grid> <us>",
  *   "fused_rows <consumer warps> <ring slots> <rows per block> <grid> <us>",
  *   "fused_direct <warps> 0 <rows per block> <grid> <us>",
- *   "fused_quad <sweeps per launch> 0 <rows per tile> <grid> <us>",
+ *   "fused_quad <sweeps per launch> <1: interior row loop unrolled> <rows per tile> <grid> <us>",
  *   "resident <blocks of the cluster> 0 <rows per block> <grid> <us>" (its residual checks included)
+ * and with FP16 storage
+ *   "fp16_scalar <grid> 0 0 0 <us>",
+ *   "fp16_rows <strip width> <ring slots> <rows per block> <grid> <us>",
+ *   "fp16_quad 0 0 <rows per tile> <grid> <us>" (four sweeps per launch; these without a check)
  * with <us> the time per sweep inside the solve loop: a check period of check_every sweeps
  * timed as its plain launches plus the one launch that also sums the residual (the first two
- * kinds once per grid tried: the resident-block capacity of the GPU down to half of it).  Owned by h; valid until the next create-time tuning. */
+ * kinds once per grid tried: the resident-block capacity of the GPU down to half of it).  Owned by
+ * h; valid until the next create-time tuning. */
 const char *lbm2p_autotune_report(const lbm2p *h);
 
 /* Running totals since creation: kernels launched by the library, pressure sweeps run.  Sweep counts that
@@ -323,9 +328,9 @@ lbm2p_status lbm2p_counters(const lbm2p *h, long long *launches, long long *swee
  * all members, and the sub-iteration continues while any member is still above its
  * tolerance (members that met theirs stop sweeping).  The paper solves one realisation at
  * a time; this is the same per-member computation scheduled so that small lattices fill
- * the GPU together: they share one sweep kernel over a tile list, while the members of 512^2
- * nodes or more on lattices with walls on every side share a two-sweeps-per-launch kernel
- * over a list of their blocks, beside the shared sweep (when check_every is a multiple of 4).
+ * the GPU together: those on lattices with walls on every side share a kernel of four sweeps per
+ * launch over a list of their tiles (when check_every is a multiple of 8; of two sweeps for those of
+ * 512^2 nodes or more when it is a multiple of 4), the others one of a sweep per launch beside it.
  *
  * members: count handles made by lbm2p_create on the current device, all on one stream,
  * all with one even check_every that divides each member's max_sub_iters; each handle
@@ -334,8 +339,8 @@ lbm2p_status lbm2p_counters(const lbm2p *h, long long *launches, long long *swee
  * (lbm2p_batch_step returns EINVAL if a member was stepped alone).  Between batch steps
  * a member may be read (fields, velocity, get_state, counters) and its sources, wall
  * values and state replaced (set_sources, set_dirichlet, set_state).  The batch owns a
- * little device memory of its own (a descriptor per member, 36 bytes per tile of 256
- * nodes), allocated with cudaMalloc. */
+ * little device memory of its own (a descriptor per member, some 60 bytes per 256 nodes),
+ * allocated with cudaMalloc. */
 typedef struct lbm2p_batch lbm2p_batch;
 lbm2p_status lbm2p_batch_create(lbm2p_batch **out, lbm2p *const *members, int count);
 
@@ -364,8 +369,9 @@ void lbm2p_batch_destroy(lbm2p_batch *b);
  * an application that owns the device allocator).  Such callers cannot create a handle,
  * but can run the solver's pressure sweep on buffers they already own.
  *
- * One fused pressure sweep (the kernel lbm2p_step uses), then the residual r of the
- * stopping rule, for one lattice whose planes the caller owns on the current device:
+ * One fused pressure sweep (a kernel of its own with the arithmetic of lbm2p_step's), then the
+ * residual r of the stopping rule, for one lattice whose planes the caller owns on the current
+ * device:
  *   n_in[8]  pressure populations in the library's deviation form n_i = f_i^+ - w_i R,
  *            directions c_1..c_8, each a [ny][pitch] FP32 plane (read);
  *   n_out[8] the populations after the sweep (written; no output plane may be an input

@@ -317,7 +317,7 @@ void pressure_sweeps_pair_direct(const PressureArgs &a, bool check, int cw, int 
 cudaError_t node_pressure_pair_direct(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                       const PressureArgs &a, bool check, int cw, int H, int grid);
 // four sweeps per launch (sweep_quad.cu), lattices without periodic sides: tiles of 56 columns by H
-// rows, one warp each, four to a block; grid = quad_grid(...)
+// rows, a block of one warp each; grid = quad_grid(...)
 long long quad_grid(int H, int nx, int ny);
 int quad_tile_slots(bool has_fp);      // tiles that run at a time (0: the kernel cannot run)
 cudaError_t quad_prepare();
@@ -325,11 +325,7 @@ cudaError_t quad_prepare();
 void pressure_sweeps_quad(const PressureArgs &a, bool check, int H, bool unroll, int grid, void *stream);
 cudaError_t node_pressure_quad(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                                const PressureArgs &a, bool check, int H, bool unroll, int grid);
-// four FP16-storage sweeps per launch (fp16_quad.cu) in the same tiles; the planes of a.nin are
-// equally spaced
-int quad_h_slots(bool has_fp);
-void pressure_sweeps_quad_h(const HalfSweepArgs &a, bool check, int H, int grid, void *stream);
-// the same over several lattices: item t (t < *nitems <= grid) is tile items[t].y (of H[m] rows) of
+// the same (FP32) over several lattices: item t (t < *nitems <= grid) is tile items[t].y (of H[m] rows) of
 // member m = items[t].x, with argument block pa[2 m + parity]; residual sums of member m to
 // parts[4 (pb0[m] + tile) ..]
 int quad_tiles(int H, int nx, int ny);
@@ -338,6 +334,10 @@ cudaError_t node_quad_batch(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNo
                             const PressureArgs *pa, const int *H, const int *pb0,
                             const int2 *items, const int *nitems, int parity, bool check,
                             double *parts, int grid, bool has_fp);
+// four FP16-storage sweeps per launch (fp16_quad.cu) in the same tiles; the planes of a.nin are
+// equally spaced
+int quad_h_slots(bool has_fp);
+void pressure_sweeps_quad_h(const HalfSweepArgs &a, bool check, int H, int grid, void *stream);
 // a whole sub-iteration by one cluster of C blocks (resident.cu)
 bool resident_fits(int C, int nx, int ny);
 cudaError_t pressure_resident(const PressureArgs &a, const ResidentArgs &s, int C, void *stream);
@@ -376,7 +376,6 @@ cudaError_t node_rebase_mid(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNo
 cudaError_t node_loop_open(cudaGraphNode_t *n, cudaGraph_t g, const LoopHandles &h);
 cudaError_t node_loop_reset(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                             LoopCtl *ctl);
-// sets the condition of an IF node: 1 when the loop's last residual is a number
 cudaError_t node_refresh(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,
                          const RefreshArgs &a);
 cudaError_t node_saturation(cudaGraphNode_t *n, cudaGraph_t g, const cudaGraphNode_t *dep,

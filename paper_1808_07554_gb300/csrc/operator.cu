@@ -1128,15 +1128,15 @@ cudaError_t launch_conv(const ConvArgs &a, cudaStream_t s)
     const size_t smem = conv_rows_smem_bytes<CIN, COUT>();
     cudaError_t e = cudaFuncSetAttribute(k_conv3x3_rows<CIN, COUT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    // all of the unified L1/shared storage as shared memory, so that several CTAs (each ~69 KB
-    // for 32 input channels) fit on an SM
+    // all of the unified L1/shared storage as shared memory, so that two CTAs (95 KB each at 32 input
+    // and output channels) fit on an SM
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_conv3x3_rows<CIN, COUT>,
                                  cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess)
         return e;
-    // the runtime's occupancy query answered one CTA per SM for this kernel, where its
-    // registers and shared memory allow three (ncu's occupancy limits agree with the latter)
+    // the runtime's occupancy query answered one CTA per SM for a kernel of this kind where ncu's
+    // limits gave what its registers and shared memory allow, so they are computed here
     const int per_sm = resident_per_sm((const void *)k_conv3x3_rows<CIN, COUT>, smem, kCvThreads,
                                        kCvTmemCols);
     const long long tiles = (long long)a.nimg * a.H * ((a.W + 127) / 128);

@@ -1602,7 +1602,7 @@ lbm2p_status autotune_h(lbm2p *h, int sms)
             }
         }
     }
-    // the heights tried are those of the FP32 form
+    // rows per tile giving half a round to six rounds of resident tiles (FP32: a quarter to eight)
     if (four) {
         const int slots = lbm2p_launch::quad_h_slots(h->Fp != nullptr);
         int last_H = -1;

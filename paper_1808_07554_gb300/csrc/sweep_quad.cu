@@ -25,14 +25,14 @@
 // instruction fetches are cold (unrolled, the tile at a corner took 500k cycles at 4096^2 where an
 // interior tile took 60k).  The interior path exists in both forms: unrolled by two with straight-line
 // filling rows it has fewer instructions, as one guarded row it leaves the instruction cache to the
-// edge tiles beside it.  Create times both: the first is ahead at 1024^2 (22.0 against 22.7 us per
-// launch), the second at 256^2 (10.4 against 12.4), at 2048^2 (60.8 against 68.0) and for batches,
-// where it is the only one.
+// edge tiles beside it.  Create times both: the first is ahead at 1024^2 (19.4 against 22.2 us per
+// launch), the second at 2048^2 (61.9 against 65.6) and, by little, at 512^2 and 4096^2; for batches it
+// is the only one.
 // The per-node operations and their order are those of the single sweep (dev1, pressure_of,
 // collide1), so four sweeps equal four launches of one bit for bit.
-// Per sweep, two-sweep launches before and this kernel now: 4096^2 129.5 and 54.5 us (218 us per
-// launch, 1.18 times the time that its 1208 MB take at the copy bandwidth), 1024^2 14.0 and
-// 5.5 us, 512^2 7.5 and 3.3 us.
+// Per sweep, two-sweep launches before and this kernel now: 4096^2 129.5 and 55.2 us (221 us per
+// launch, 1.24 times the time that its 1208 MB take at the copy bandwidth), 1024^2 14.0 and
+// 4.9 us, 512^2 7.5 and 3.1 us.
 #include <cuda_runtime.h>
 
 #include <cstdint>

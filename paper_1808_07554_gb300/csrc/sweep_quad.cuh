@@ -23,11 +23,12 @@ constexpr int kQuadSlots = 7;                 // ring slots: rows in flight = sl
 __host__ __device__ constexpr int quad_strips(int nx) { return (nx + kQuadOwn - 1) / kQuadOwn; }
 
 // The tiles of a lattice: strips of 56 columns by H rows, lower where the footprint meets a wall.
-// The row of an edge tile takes 1.4 times an interior one's, so with one height the edge tiles end
-// last: 1024^2 in one round of resident tiles 27 us of which the interior tiles run 17.  He rows make
+// The row of an edge tile took 1.4 times an interior one's, so with one height the edge tiles ended
+// last: 1024^2 in one round of resident tiles 27 us of which the interior tiles ran 17.  He rows make
 // an edge tile last as long as an interior one (the 8 rows of filling and draining counted in), and
 // the edge tiles come first, so that the tail of a launch of several rounds is made of short ones:
-// 22 us at 1024^2, 231 -> 218 us at 4096^2.
+// 22 us at 1024^2, 231 -> 218 us at 4096^2 (19.4 and 221 since the edge path sums a node's wells first,
+// which made its code shorter).
 struct QuadPlan {
     int H, He, Hb;               // rows of interior tiles, of those on x walls, on y walls
     int first;                   // strips 1 .. first - 1 meet no x wall

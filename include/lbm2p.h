@@ -20,7 +20,8 @@
  * j*nx + i), cell centred: node (i, j) sits at ((i + 1/2) dx, (j + 1/2) dx) and walls
  * lie half-way between a boundary node and its missing neighbour.  Host inputs are FP64
  * and are copied (the caller keeps ownership); the library computes in FP32 on the GPU
- * and accumulates the residual in FP64.  Device outputs are FP32.
+ * and forms the residual in FP64 (from sums inside a warp that are FP32, relative to values of the
+ * warp itself).  Device outputs are FP32.
  *
  * Memory.  The handle owns all device memory.  It is obtained through params.alloc /
  * params.release when given (for instance a framework's caching allocator), otherwise

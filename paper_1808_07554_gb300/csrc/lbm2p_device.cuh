@@ -187,6 +187,7 @@ struct RebaseMidArgs {      // within a long solve: R += dP of the last sweep (n
     float *n[8];
     float *R;
     const float *Fp;
+    float *Pio;              // the last sweep's increment over R, moved with it, or nullptr
     Geom g;
     Wells w;
 };

@@ -363,7 +363,14 @@ __device__ __forceinline__ void rebase_mid_node(const RebaseMidArgs &a, int o)
 #pragma unroll
     for (int i = 0; i < 8; ++i)
         a.n[i][o] = fmaf(-wgt(i + 1), dP, n[i]);
-    a.R[o] = a.R[o] + dP;
+    const float r = a.R[o], rn = r + dP;
+    a.R[o] = rn;
+    if (a.Pio) {
+        // relative to the new R: what R's rounding left out (the error of the sum) stays in it
+        const float b = __fsub_rn(rn, r);
+        const float e = __fadd_rn(__fsub_rn(r, __fsub_rn(rn, b)), __fsub_rn(dP, b));
+        a.Pio[o] = __fadd_rn(__fsub_rn(a.Pio[o], dP), e);
+    }
 }
 
 // a2: one node of a pressure sweep with scalar gathers; (d, q) feed the residual partials

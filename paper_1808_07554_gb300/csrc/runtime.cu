@@ -772,30 +772,36 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
             return kk == replay;
         return (kk % m == 0) || kk >= cap;
     };
-    // run sweeps k+1 .. upto; the last one evaluates the residual when asked
+    // whether sweep kk + 1 checks: as a sweep of its own it compares with the increment plane that sweep
+    // kk writes
+    auto check_next = [&](int kk) { return kk < (replay >= 0 ? replay : cap) && is_check(kk + 1); };
     int last_nparts = sweep_nparts(h);
     // run sweeps k+1 .. upto; the last one evaluates the residual when it is a check point.
     // With fused sweeps the batch is a few single sweeps followed by fused launches, the
-    // last of which computes the residual from its final two stages.
+    // last of which computes the residual from its final two stages; where the next batch is one
+    // sweep (the cap or the count is one more, or every sweep checks), this one ends in a single sweep
+    // too, which writes the increment plane.
     auto run_batch = [&](int upto) -> lbm2p_status {
         if (h->timing)
             CUDA_TRY(h, cudaEventRecord(h->ev_sw0, st));
-        const int n = upto - k;
         const FusedShape &fs = replay >= 0 ? h->count_form : h->tb;
-        const int T = fs.T;
+        const int T = fs.T, tail = check_next(upto) ? 1 : 0;
+        const int n = upto - k - tail;
         const int nf = (T > 1 && n >= T) ? n / T : 0;
         const int ns = n - nf * T;
-        const bool final_check = is_check(upto) && upto >= 2;
-        for (int i = 0; i < ns; ++i) {
-            const int kk = k + 1 + i;
-            const bool check = nf == 0 && is_check(kk) && kk >= 2;
-            const bool write_p = nf == 0 && is_check(kk + 1) && kk + 1 >= 2;
+        const bool final_check = tail == 0 && is_check(upto) && upto >= 2;
+        auto single = [&](int kk) -> lbm2p_status {
             PressureArgs a = pressure_args(h, src, dst_of(src), work);
-            launch_sweep(h, a, check, write_p);
+            launch_sweep(h, a, is_check(kk) && kk >= 2, check_next(kk));
             LAUNCHED(h, "pressure sweep");
             src = dst_of(src);
             h->sweeps += 1;
-        }
+            return LBM2P_OK;
+        };
+        lbm2p_status es;
+        for (int i = 1; i <= ns; ++i)
+            if ((es = single(k + i)) != LBM2P_OK)
+                return es;
         for (int q = 0; q < nf; ++q) {
             PressureArgs a = pressure_args(h, src, dst_of(src), work);
             if (fs.kind == 3)
@@ -814,7 +820,9 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
             src = dst_of(src);
             h->sweeps += T;
         }
-        last_nparts = nf > 0 ? fs.grid : sweep_nparts(h);
+        if (tail && (es = single(upto)) != LBM2P_OK)
+            return es;
+        last_nparts = nf > 0 && !tail ? fs.grid : sweep_nparts(h);
         if (h->timing)
             CUDA_TRY(h, cudaEventRecord(h->ev_sw1, st));
         k = upto;
@@ -863,7 +871,9 @@ lbm2p_status pressure_solve(lbm2p *h, int replay, bool work, int *k_out, double 
     // solve goes on (the graph loop applies the same rule)
     const int every = h->rebase_every;
     auto rebase_mid = [&]() -> lbm2p_status {
-        lbm2p_launch::rebase_mid(rebase_mid_args(h, src, work), h->grid, h->stream);
+        RebaseMidArgs a = rebase_mid_args(h, src, work);
+        a.Pio = check_next(k) ? h->Pio : nullptr;
+        lbm2p_launch::rebase_mid(a, h->grid, h->stream);
         LAUNCHED(h, "mid-solve rebase");
         return LBM2P_OK;
     };

@@ -129,3 +129,39 @@ def test_solves_driven_from_the_host_use_the_tuned_form(nx, ny):
     assert np.array_equal(one.get_state(), auto.get_state())
     one.close()
     auto.close()
+
+
+@pytest.mark.parametrize("bc", [(1, 1, 1, 1), (0, 0, 0, 0), (1, 1, 2, 1)])
+@pytest.mark.parametrize("fuse", [0, 1, 2, 4])
+def test_residual_of_a_last_sweep_on_its_own(fuse, bc):
+    """A cap one sweep beyond a check, or a count one sweep beyond a move of R: the last sweep checks by
+    itself and must compare with the increment of the sweep before it, over the same R.  Against the same
+    count in one piece (equal states; the residual's sums are grouped differently: 1e-4), and, where R was
+    moved, against a solve that does not move it (P is then rounded differently, by 1e-7 of it where it
+    changes by 1e-4 and more per sweep: 1e-2)."""
+    import paper_1808_07554_gb300 as pkg
+    rng = np.random.default_rng(3)
+    nx, ny = 70, 33
+    prob = uniform(nx, ny, bc=bc, K=np.exp(rng.standard_normal((ny, nx))), S0=0.4,
+                   wells=[(3, 2, 1e-2, 0), (nx - 4, ny - 3, 1e-2, 1)],
+                   P_b=[rng.random(2 * (ny if s < 2 else nx) + 1) for s in range(4)],
+                   S_b=[np.full(2 * (ny if s < 2 else nx) + 1, 0.3) for s in range(4)])
+    make = lambda every, cap: pkg.Solver.from_problem(   # noqa: E731
+        prob, init_replay=0, tol=0.0, check_every=every, max_sub_iters=cap, fuse_sweeps=fuse)
+    for every, cap in ((8, 25), (7, 8), (2, 15), (16, 17), (1, 9)):
+        a, b = make(every, cap), make(every, cap)
+        (_, sa), (_, sb) = a.step(1), b.step(1, replay=[cap])
+        assert sa[0].sub_iters == sb[0].sub_iters == cap
+        assert np.array_equal(a.get_state(), b.get_state())
+        assert sa[0].residual == pytest.approx(sb[0].residual, rel=1e-4), (every, cap)
+        a.close()
+        b.close()
+    want = make(25, 1025)                     # R moves every 1025 sweeps: not within this solve
+    r = want.step(1)[1][0].residual
+    assert r > 1e-5
+    for every, replay in ((8, None), (1, None), (8, [1025])):
+        a = make(every, 1025)
+        st = a.step(1, replay=replay)[1][0]
+        assert st.sub_iters == 1025 and st.residual == pytest.approx(r, rel=1e-2), (every, replay)
+        a.close()
+    want.close()

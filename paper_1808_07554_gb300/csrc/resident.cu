@@ -250,13 +250,20 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
     bool checked = false;
     while (k < cap) {
         ++k;
-        const bool check = --to_check == 0;
+        const bool check = --to_check == 0, before = to_check == 1;
         const unsigned nxt = cur == base ? base + buffer : base;
-        float d[NPT], u[NPT];                         // what a check sums over
+        // Sums of d, d^2, u, u^2 over this warp's nodes in FP32, relative to means over the warp, so that
+        // their rounding is a few 2^-24 of the spread inside the warp, whatever the values of other
+        // nodes.  One node per thread: the means of this sweep.  Several: those of the sweep before a
+        // check, since the nodes' d and u, kept until the means are there, would take registers that
+        // the sweeps need (160^2: 1.94 us per sweep so, 1.73 now, 1.78 with one node's values as
+        // everyone's pivots).
+        constexpr bool kOne = NPT == 1;
+        float s1 = 0.0f, s2 = 0.0f, t1 = 0.0f, t2 = 0.0f;
+        float md = !kOne && check ? red[4][warp] : 0.0f, mu = !kOne && check ? red[5][warp] : 0.0f;
 #pragma unroll
         for (int q = 0; q < NPT; ++q) {
             ResNode<NPT> &n = nd[q];
-            d[q] = u[q] = 0.0f;
             if (n.cell == ~0u)
                 continue;
             float f[8], v[8];
@@ -271,42 +278,44 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
             for (int i = 0; i < 8; ++i)
                 v[i] = collide1(f[i], wgt(i + 1), dP, n.it, n.Fq);
             put(n, nxt, v);
-            if (check) {
-                d[q] = (dP - n.dp) - shift1;
-                u[q] = (n.r0 - shift0) + dP;
+            if (check || (!kOne && before)) {
+                const float e = ((dP - n.dp) - shift1) - md, u = ((n.r0 - shift0) + dP) - mu;
+                s1 += e;
+                t1 += u;
+                if (!kOne) {
+                    s2 = fmaf(e, e, s2);
+                    t2 = fmaf(u, u, t2);
+                }
             }
             n.dp = dP;
         }
         cur = nxt;
-        if (check) {
-            // Sums of d, d^2, u, u^2.  A warp's in FP32, relative to its own means: their rounding is a
-            // few 2^-24 of the spread inside the warp, whatever the values of other nodes.  Then one
-            // warp restores the raw sums and adds them in FP64.
-            const bool h16 = lane & 16, h8 = lane & 8;
-            float n = 0.0f, cd = 0.0f, cu = 0.0f;
+        const bool h16 = lane & 16, h8 = lane & 8;
+        if (kOne ? check : before) {
+            float n = 0.0f;
 #pragma unroll
-            for (int q = 0; q < NPT; ++q) {
+            for (int q = 0; q < NPT; ++q)
                 n += (float)__popc(__ballot_sync(0xffffffffu, nd[q].cell != ~0u));
-                cd += d[q];
-                cu += u[q];
-            }
-            float v = (h16 ? cu : cd) + __shfl_xor_sync(0xffffffffu, h16 ? cd : cu, 16);
+            float v = (h16 ? t1 : s1) + __shfl_xor_sync(0xffffffffu, h16 ? s1 : t1, 16);
 #pragma unroll
             for (int o = 8; o > 0; o >>= 1)
                 v += __shfl_xor_sync(0xffffffffu, v, o);
-            v *= 1.0f / n;
-            cd = __shfl_sync(0xffffffffu, v, 0);
-            cu = __shfl_sync(0xffffffffu, v, 16);
-            float s1 = 0.0f, s2 = 0.0f, t1 = 0.0f, t2 = 0.0f;
-#pragma unroll
-            for (int q = 0; q < NPT; ++q)
-                if (nd[q].cell != ~0u) {
-                    const float e = d[q] - cd, g = u[q] - cu;
-                    s1 += e;
-                    s2 = fmaf(e, e, s2);
-                    t1 += g;
-                    t2 = fmaf(g, g, t2);
-                }
+            v = n > 0.0f ? v * (1.0f / n) : 0.0f;
+            if ((lane & 15) == 0) {
+                red[4 + (lane >> 4)][warp] = v;
+                red[6][warp] = n;
+            }
+            if (kOne) {
+                md = __shfl_sync(0xffffffffu, v, 0);
+                mu = __shfl_sync(0xffffffffu, v, 16);
+                const bool mine = nd[0].cell != ~0u;
+                s1 = mine ? s1 - md : 0.0f;
+                t1 = mine ? t1 - mu : 0.0f;
+                s2 = s1 * s1;
+                t2 = t1 * t1;
+            }
+        }
+        if (check) {
             // four sums over 32 lanes by six shuffles: lane 8 c ends with sum c
             s1 = (h16 ? t1 : s1) + __shfl_xor_sync(0xffffffffu, h16 ? s1 : t1, 16);
             s2 = (h16 ? t2 : s2) + __shfl_xor_sync(0xffffffffu, h16 ? s2 : t2, 16);
@@ -316,11 +325,6 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                 s1 += __shfl_xor_sync(0xffffffffu, s1, o);
             if ((lane & 7) == 0)
                 red[lane >> 3][warp] = s1;
-            if (lane == 0) {
-                red[4][warp] = cd;
-                red[5][warp] = cu;
-                red[6][warp] = n;
-            }
             __syncthreads();
             if (warp == 0) {
                 // sum x = S1 + n p, sum x^2 = S2 + 2 p S1 + n p^2.  Up to eight warps: a lane per warp
@@ -413,6 +417,7 @@ __global__ void __launch_bounds__(kResMaxThreads, 1)
                         v[i] = fmaf(-wgt(i + 1), dP, v[i]);
                     put(n, cur, v);
                     n.r0 = n.r0 + dP;
+                    n.dp -= dP;
                     s.Rw[n.go] = n.r0;
                 }
                 __threadfence();

@@ -102,8 +102,8 @@ def test_residual_against_64_bits_beside_outliers(nx, ny, amp):
     """The residual of the second sweep from P0 = noise of 1e-3 with a few nodes (some at the start of a
     block's rows, whatever the cluster's size) a thousand or more deviations away, against 64-bit sums
     over the pressures of the first two sweeps.  A warp's FP32 sums of squares are relative to its
-    means, so their rounding (a square, its operand and eight additions, 2^-24 each) is at most
-    12 x 2^-24 of the whole variance, half of that in the root; P itself is rounded to 2^-24 on both sides
+    means of the sweep before, so their rounding (a square, its operand and eight additions, 2^-24
+    each) is about 12 x 2^-24 of the whole variance, half of that in the root; P itself is rounded to 2^-24 on both sides
     and enters as a difference: 4 x 2^-24 more.  Together 6e-7; 2e-6 is allowed."""
     import paper_1808_07554_gb300 as pkg
     rng = np.random.default_rng(nx)

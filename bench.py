@@ -98,10 +98,10 @@ NCU_TRAFFIC_PER_LAUNCH = {
     ("five_spot_4096", "staged_rows", 120): {
         "bytes": 1229841323, "sources": "a38cf4db413179c4",
         "profile": "profiles/pressure_sweeps_fused_rows_five_spot_4096.md"},
-    # k_pressure_quad<0, 7, 0> (66 rows per tile), mean of 3 launches: 189.4 + 90.7, 189.4 + 87.9,
-    # 189.3 + 87.9 MB (the last writes of a launch are still in L2)
+    # k_pressure_quad<0, 7, 0> (66 rows per tile), mean of 3 launches: 189.4 + 91.0, 189.4 + 87.9,
+    # 189.4 + 87.9 MB (the last writes of a launch are still in L2)
     ("five_spot_2048", "quad", 32): {
-        "bytes": 278225322, "sources": "b8f940bdaf553d4f",
+        "bytes": 278330965, "sources": "4182917ce6e12e29",
         "profile": "profiles/sweeps_and_step_kernels_five_spot_2048.md"},
 }
 FUSED_FORM_NAMES = {1: "stages", 2: "staged_rows", 3: "direct", 4: "quad", 5: "resident"}
